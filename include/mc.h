@@ -97,14 +97,14 @@ typedef struct {
   int32_t graph;
   /* 1 = every worker searches its root's whole tree itself (the warps of a
    * block worker still share it through the block's pool); 0 = (default) a
-   * worker that expands more than its budget of Branch nodes on one root
-   * copies the root's adjacency matrix to a device arena and turns the
-   * untried branches of its stack into tasks of one GPU-wide queue, which
-   * every block serves, so one hard neighbourhood spreads over the GPU */
+   * root of at most 1,024 candidates whose colouring leaves branches copies
+   * its adjacency matrix to a device arena and becomes a task of one GPU-wide
+   * queue, which every warp serves, so one hard neighbourhood spreads over
+   * the GPU */
   int32_t no_split;
-  /* Branch nodes a warp worker expands on one root before it spills the
-   * rest of its tree to the task queue (a block worker: four times as
-   * many); 0 = default (4096) */
+  /* Branch nodes a warp expands on a task between two looks at the queue:
+   * when other warps wait, it hands them the untried branches of its
+   * shallowest level; 0 = default (8) */
   int32_t split_nodes;
   /* The learned form (an extension; the paper has no learned part): a
    * scoring network from mc_mlp_create, or NULL.  With a network, the solve
@@ -168,11 +168,11 @@ typedef struct {
   int64_t roots_colored;       /* roots that reached the colouring test */
   int64_t roots_branched;      /* roots that reached Branch */
   int64_t nodes;               /* Branch nodes expanded */
-  int64_t donations;           /* subproblems handed to other warps */
+  int64_t donations;           /* subproblems handed to other warps (of a block, or by a task to the queue) */
   int64_t neighbourhood_entries; /* later-neighbour row entries read to build the
                                     roots' adjacency matrices (Fact 3's work) */
   int64_t neighbourhood_entries_block; /* ... of which read by block workers */
-  int64_t tasks;               /* subproblems spilled to the task queue */
+  int64_t tasks;               /* subproblems published to the task queue */
   int64_t heuristic_grows;     /* start vertices grown by Algorithm 1 */
   int64_t heuristic_tests;     /* adjacency tests of its greedy steps */
   int64_t heuristic_row_entries; /* CSR row entries it read (gathers, merges) */
@@ -251,7 +251,7 @@ int mc_max_clique_batch(mc_graph *g, const mc_options *opt, int32_t *omegas_out,
  * graph `repeats` times per candidate setting, one coordinate at a time,
  * starting from `base` (NULL = defaults): the work split between warp and
  * block workers (warp_max 32, 64, 128), then the task queue (no_split, or
- * split_nodes 1024, 4096, 16384), then the block-worker layout (layout 0,
+ * split_nodes 4, 8, 32), then the block-worker layout (layout 0,
  * 1) and the build's member lookup (no_bitmap 0, 1), then, from the default
  * heuristic, its warm-up part alone (heuristic 3), then CUDA-graph replay
  * (graph 0, 1).  It

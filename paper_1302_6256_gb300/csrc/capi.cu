@@ -847,8 +847,8 @@ int mc_autotune(mc_graph *g, const mc_options *base, int32_t repeats, mc_options
     *ms = tot / repeats;
     return MC_OK;
   };
-  // one coordinate at a time: the warp/block split of the roots, the spill
-  // budget of the task queue, the heuristic's extent, then direct launches
+  // one coordinate at a time: the warp/block split of the roots, the task
+  // queue, the heuristic's extent, then direct launches
   // vs graph replay
   mc_options bo = b;
   bo.graph = 0;
@@ -867,7 +867,7 @@ int mc_autotune(mc_graph *g, const mc_options *base, int32_t repeats, mc_options
   struct Split {
     int32_t no_split, nodes;
   };
-  const Split splits[] = {{1, 0}, {0, 1024}, {0, 4096}, {0, 16384}};
+  const Split splits[] = {{1, 0}, {0, 4}, {0, 8}, {0, 32}};
   Split bs = {bo.no_split, bo.split_nodes};
   for (const Split &sp : splits) {
     mc_options o = bo;

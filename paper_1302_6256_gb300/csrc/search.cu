@@ -32,11 +32,11 @@
 //                shared-memory pool (a busy warp hands the shallowest untried
 //                branch to an idle one);
 //   big class    larger: as the block class with the matrix in global memory.
-// Task queue: a warp (block) that expands more than its budget of Branch
-// nodes on one root copies the root's matrix to an arena and turns every
-// untried branch of its stack into a task in a GPU-wide ring; the task
-// kernel searches tasks with whole blocks and spills again while the queue
-// is short, so one hard neighbourhood spreads over the whole GPU.
+// Task queue: a root whose colouring leaves branches copies its matrix to an
+// arena and becomes one task of a GPU-wide ring; the task kernel searches
+// tasks with single warps, which hand the untried branches of their
+// shallowest level to the ring while other warps wait for work, so one hard
+// neighbourhood spreads over the whole GPU.
 // Every spin-wait is bounded; on timeout the device error word is set.
 #include <algorithm>
 #include <climits>
@@ -83,14 +83,12 @@ struct SA {
   int32_t *ready;                // per ring slot: 2*lap free for lap's writer, 2*lap+1 written
   int32_t task_cap;              // ring slots (a power of two)
   int32_t *ntasks;               // positions taken (the queue's tail, monotonic)
-  int32_t *task_next;            // positions handed out (the queue's head)
-  int32_t *active;               // blocks of the task kernel holding a task
+  int32_t *task_next;            // tickets taken by the task kernel's warps (runs ahead of ntasks by the waiting ones)
+  int32_t *pending;              // tasks published and not yet finished
   int32_t *progress;             // heartbeat: bumped every 256 Branch nodes
-  int32_t queue_gate;            // spill only while fewer tasks wait (0 = always)
   int32_t *overflow;             // roots too large for this launch's layout (or null)
   int64_t *noverflow;
-  long long budget_warp;         // Branch nodes before a warp worker spills
-  long long budget_block;        // ... and a block, on one root or task
+  int32_t offer_nodes;           // Branch nodes of a task between two looks for waiting warps
 };
 
 struct RootRec {
@@ -101,7 +99,12 @@ constexpr int kTaskWords = 2 + 64;  // root record, clique size, C bits, P bits 
 constexpr long long kArenaWords = 64ll << 20;  // 256 MB of published matrices
 constexpr int kRecCap = 1 << 16;
 constexpr int kTaskCap = 1 << 20;          // ring slots, 277 MB
-constexpr long long kSpillNodes = 4096;    // default Branch-node budget of a warp worker
+constexpr size_t kCtrBytes = 96 * 8;       // counters and the queue's control words
+// Default SA::offer_nodes.  R-MAT scale 17 (ef 12) / 18 (ef 12) / 20 (ef 16),
+// task kernel: 4 nodes 3.2 / 4.2 / 11 ms, 6 nodes 2.8 / 3.3 / 6.5 ms, 16 nodes
+// 3.5 / 4.4 / 5.7 ms, 64 nodes 8 / 10 / 12 ms: rare offers leave warps idle,
+// frequent ones make tasks too small for their set-up (10-30 us).
+constexpr int kOfferNodes = 8;
 constexpr int kMidCap = 512;               // candidates of the two-blocks-per-SM block layout
 
 template <int WPL>
@@ -198,25 +201,21 @@ __device__ __forceinline__ void bandnot_row(Bits<WPL> &b, const uint32_t *A, int
 // Greedy colouring of P in index order by independent-set extraction: colour
 // class c takes, in index order, every remaining vertex with no neighbour
 // already in class c.  (This is exactly the sequential greedy colouring.)
-// B receives the vertices with colour > kmin.  Returns the colour count.
+// B receives the vertices with colour > kmin: what is left after kmin
+// classes, so the classes above are never made.
 template <int WPL, bool SM>
-__device__ int color_ise(const uint32_t *A, int Ws, int W, const Bits<WPL> &P, int kmin, Bits<WPL> &B) {
-  Bits<WPL> U = P;
-  bzero(B);
-  int col = 0;
-  while (bany(U)) {
-    col++;
-    Bits<WPL> Q = U;
+__device__ void color_ise(const uint32_t *A, int Ws, int W, const Bits<WPL> &P, int kmin, Bits<WPL> &B) {
+  B = P;
+  for (int col = 1; col <= kmin && bany(B); col++) {
+    Bits<WPL> Q = B;
     for (;;) {
       int v = blowest(Q);
       if (v < 0) break;
       bclear(Q, v);
-      bclear(U, v);
-      if (col > kmin) bset(B, v);
+      bclear(B, v);
       bandnot_row<WPL, SM>(Q, A, Ws, W, v);
     }
   }
-  return col;
 }
 
 __device__ __forceinline__ int read_best(const int32_t *best, int g) {
@@ -340,9 +339,6 @@ __device__ __forceinline__ int level_word(const uint32_t *p) {
 template <int WPL>
 struct Pool {
   int lock, count, idle, beat;
-  int spent;  // Branch nodes the block has expanded on this root or task
-  int spill;  // 0 searching here, 2 record being written, 1 spilling, 3 no room
-  int rec;    // record of the root's matrix in the arena, -1 none yet
   int csize[kPoolCap];
   uint32_t C[kPoolCap][32 * WPL];
   uint32_t P[kPoolCap][32 * WPL];
@@ -375,30 +371,30 @@ struct Root {
 
 // Take k consecutive queue positions, all or none; returns the first or -1.
 // The queue is a ring of task_cap slots: positions are taken only while
-// fewer than task_cap are taken and not yet handed out.
-__device__ int reserve_tasks(const SA &a, int k) {
+// fewer than task_cap are taken and not yet handed out.  The positions count
+// as pending from here on (the caller still holds a task, or runs before the
+// task kernel, so the count cannot reach zero in between).  tries bounds the
+// compare-and-swap attempts: thousands of warps offer branches at once when
+// the queue runs dry, and one that loses goes on searching instead.
+__device__ int reserve_tasks(const SA &a, int k, long long tries) {
   int cur = *(volatile int32_t *)a.ntasks;
-  for (long long it = 0; it < a.spin; it++) {
+  for (long long it = 0; it < tries; it++) {
     const int head = *(volatile int32_t *)a.task_next;
     if (cur - head + k > a.task_cap || cur > INT_MAX - k) return -1;
     const int prev = atomicCAS(a.ntasks, cur, cur + k);
-    if (prev == cur) return cur;
+    if (prev == cur) {
+      atomicAdd(a.pending, k);
+      return cur;
+    }
     cur = prev;
   }
   return -1;
 }
 
-// True while the queue is short enough that splitting work pays.
-__device__ __forceinline__ bool queue_short(const SA &a) {
-  if (a.queue_gate <= 0) return true;
-  const int tail = *(volatile int32_t *)a.ntasks, head = *(volatile int32_t *)a.task_next;
-  return tail - head < a.queue_gate;
-}
-
 // Reserve arena room and a record for a root's matrix and P list.  Returns
 // the record index (and the arena offset) or -1 without room.
 __device__ int reserve_record(const SA &a, const Root &r, int Ws, long long *off_out) {
-  const long long need = (long long)r.p * Ws + r.p;
+  const long long need = ((long long)r.p * Ws + r.p + 31) & ~31ll;  // records start on 128-byte lines
   const long long off = (long long)atomicAdd(a.arena_used, (unsigned long long)need);
   if (off + need > a.arena_cap) return -1;
   const int rec = atomicAdd(a.nrec, 1);
@@ -471,7 +467,7 @@ __device__ void write_task(const SA &a, int t, int rec, int cs, const Bits<1> &C
 __device__ void emit_task(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, int rec, int t,
                           const Bits<1> &Cl, int csl, const Bits<1> &Pl, int x) {
   Bits<1> TP = Pl;
-  band_row<1, true>(TP, A, Ws, W, x);
+  band_row<1, false>(TP, A, Ws, W, x);
   const int om = read_best(a.best, r.g);
   int cs = csl + 1;
   if (!bany(TP)) {
@@ -489,80 +485,26 @@ __device__ void emit_task(const SA &a, const Root &r, const uint32_t *A, int Ws,
   write_task(a, t, rec, cs, Cx, TP);
 }
 
-// Hand the untried rest of one warp's depth-first search to the task queue:
-// every untried branch at each stored level and at the current level becomes
-// a task of record rec.  All or nothing: returns false, publishing nothing,
-// without room in the queue.
-__device__ bool spill_levels(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, const uint32_t *stk, int d,
-                             int csize0, const Bits<1> &P, const Bits<1> &B, const Bits<1> &C, int rec) {
+// The whole search of a root as one task (clique {u}, candidates P): its
+// matrix and P list go to the arena once.  False, publishing nothing, without
+// room for the record or in the queue.  Warp-collective.
+__device__ bool publish_root(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, const Bits<1> &P) {
   const int lane = threadIdx.x & 31;
-  const int stride = 64 + 2;
-  int ntask = bcount(B);
-  for (int l = 0; l < d; l++) {
-    Bits<1> Bl;
-    Bl.w[0] = stk[(int64_t)l * stride + 32 + lane];
-    ntask += bcount(Bl);
+  int rec = -1, t = -1;
+  long long off = 0;
+  if (lane == 0) {
+    rec = reserve_record(a, r, Ws, &off);
+    if (rec >= 0) t = reserve_tasks(a, 1, a.spin);
   }
-  if (ntask == 0) return true;
-  int t = -1;
-  if (lane == 0) t = reserve_tasks(a, ntask);
+  rec = __shfl_sync(FULL, rec, 0);
+  off = __shfl_sync(FULL, off, 0);
   t = __shfl_sync(FULL, t, 0);
   if (t < 0) return false;
-  for (int l = 0; l <= d; l++) {
-    Bits<1> Pl, Bl, Cl = C;
-    if (l < d) {
-      const uint32_t *q = stk + (int64_t)l * stride;
-      Pl.w[0] = q[lane];
-      Bl.w[0] = q[32 + lane];
-      for (int m = l; m < d; m++) bclear(Cl, level_word(stk + (int64_t)m * stride + 65));
-    } else {
-      Pl = P;
-      Bl = B;
-    }
-    for (;;) {
-      const int x = bhighest(Bl);
-      if (x < 0) break;
-      bclear(Bl, x);
-      bclear(Pl, x);
-      emit_task(a, r, A, Ws, W, rec, t++, Cl, csize0 + l, Pl, x);
-    }
-  }
+  write_record(a, r, A, Ws, W, rec, off);
+  Bits<1> C;
+  bzero(C);
+  write_task(a, t, rec, 1, C, P);
   return true;
-}
-
-// Spill state of a block worker past its node budget (warp-collective):
-// the first warp to see the budget spent writes the root's record (unless
-// the task already has one) and opens the spill; returns 1 when this warp
-// should spill now, 3 when there is no room, 0 or 2 to keep searching.
-__device__ int block_spill_state(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, Pool<1> *pool,
-                                 long long budget) {
-  const int lane = threadIdx.x & 31;
-  int s = 0;
-  if (lane == 0) {
-    s = *(volatile int *)&pool->spill;
-    if (s == 0 && *(volatile int *)&pool->spent > budget && queue_short(a)) {
-      if (atomicCAS(&pool->spill, 0, 2) == 0) s = 4;
-      else s = *(volatile int *)&pool->spill;
-    }
-  }
-  s = __shfl_sync(FULL, s, 0);
-  if (s != 4) return s;
-  int rec = __shfl_sync(FULL, lane == 0 ? *(volatile int *)&pool->rec : 0, 0);
-  if (rec < 0) {
-    long long off = 0;
-    if (lane == 0) rec = reserve_record(a, r, Ws, &off);
-    rec = __shfl_sync(FULL, rec, 0);
-    off = __shfl_sync(FULL, off, 0);
-    if (rec >= 0) write_record(a, r, A, Ws, W, rec, off);
-  }
-  s = rec >= 0 ? 1 : 3;
-  if (lane == 0) {
-    *(volatile int *)&pool->rec = rec;
-    __threadfence_block();
-    atomicExch(&pool->spill, s);
-  }
-  __syncwarp();
-  return s;
 }
 
 // Depth-first Branch from one level (csize0 = |C| including the root u).
@@ -571,7 +513,7 @@ __device__ int block_spill_state(const SA &a, const Root &r, const uint32_t *A, 
 template <int WPL, bool SM>
 __device__ void dfs(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, uint32_t *stk, int csize0,
                     Bits<WPL> P, Bits<WPL> B, Bits<WPL> C, int wat, Pool<WPL> *pool, unsigned long long &nodes,
-                    unsigned long long &donations, long long budget = 0) {
+                    unsigned long long &donations) {
   const int lane = threadIdx.x & 31;
   const int stride = 64 * WPL + 2;
   int d = 0, csize = csize0;
@@ -582,32 +524,6 @@ __device__ void dfs(const SA &a, const Root &r, const uint32_t *A, int Ws, int W
     if (om > wat) {
       color_ise<WPL, SM>(A, Ws, W, P, om - csize, B);
       wat = om;
-    }
-    if constexpr (WPL == 1 && SM) {
-      // Past its node budget a worker hands the untried rest of its tree to
-      // the task queue, where whole blocks search it.
-      if (budget > 0 && !pool && spent > budget) {
-        int rec = -1;
-        long long off = 0;
-        if (lane == 0) rec = reserve_record(a, r, Ws, &off);
-        rec = __shfl_sync(FULL, rec, 0);
-        off = __shfl_sync(FULL, off, 0);
-        if (rec >= 0) {
-          write_record(a, r, A, Ws, W, rec, off);
-          if (spill_levels(a, r, A, Ws, W, stk, d, csize0, P, B, C, rec)) return;
-        }
-        budget = 0;
-      } else if (budget > 0 && pool) {
-        const int st = block_spill_state(a, r, A, Ws, W, pool, budget);
-        if (st == 1) {
-          int rec = lane == 0 ? *(volatile int *)&pool->rec : 0;
-          rec = __shfl_sync(FULL, rec, 0);
-          if (spill_levels(a, r, A, Ws, W, stk, d, csize0, P, B, C, rec)) return;
-          budget = 0;
-        } else if (st == 3) {
-          budget = 0;
-        }
-      }
     }
     int v = bhighest(B);
     if (v < 0) {
@@ -631,10 +547,7 @@ __device__ void dfs(const SA &a, const Root &r, const uint32_t *A, int Ws, int W
     band_row<WPL, SM>(NP, A, Ws, W, v);
     nodes++;
     spent++;
-    if (lane == 0) {
-      if (pool && budget > 0) atomicAdd(&pool->spent, 1);
-      if (a.progress && (spent & 255) == 0) atomicAdd(a.progress, 1);
-    }
+    if (lane == 0 && a.progress && (spent & 255) == 0) atomicAdd(a.progress, 1);
     if (!bany(NP)) {
       if (csize + 1 > om) {
         const Bits<WPL> Cc = C;
@@ -989,8 +902,8 @@ __global__ void __launch_bounds__(kSW * 32) search_warp_kernel(SA a) {
     Bits<1> C;
     bzero(C);
     Root r{u, g, S.Pidx, p};
-    dfs<1, true>(a, r, S.A, Ws, W, stk, 1, al, B, C, om, (Pool<1> *)nullptr, nodes, don,
-                 a.tasks ? a.budget_warp : 0);
+    if (a.tasks && publish_root(a, r, S.A, Ws, W, al)) continue;
+    dfs<1, true>(a, r, S.A, Ws, W, stk, 1, al, B, C, om, (Pool<1> *)nullptr, nodes, don);
   }
   if (lane == 0) {
     atomicAdd(a.counters + 0, colored);
@@ -1028,14 +941,14 @@ struct BlockLayout {
 template <int WPL, bool SM>
 __device__ void block_search(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, uint32_t *stk,
                              Pool<WPL> *pool, bool have, Bits<WPL> P, Bits<WPL> B, Bits<WPL> C, int cs, int wat,
-                             unsigned long long &nodes, unsigned long long &don, long long budget) {
+                             unsigned long long &nodes, unsigned long long &don) {
   const int lane = threadIdx.x & 31;
   const int g = r.g;
   long long waited = 0;
   int lastbeat = -1;
   for (;;) {
     if (have) {
-      dfs<WPL, SM>(a, r, A, Ws, W, stk, cs, P, B, C, wat, pool, nodes, don, budget);
+      dfs<WPL, SM>(a, r, A, Ws, W, stk, cs, P, B, C, wat, pool, nodes, don);
       have = false;
       if (lane == 0) {
         if (pool_lock(pool, a.err, a.spin)) {
@@ -1085,29 +998,6 @@ __device__ void block_search(const SA &a, const Root &r, const uint32_t *A, int 
     __syncwarp();
     if (lane == 0) pool_unlock(pool);
     __syncwarp();
-    if constexpr (WPL == 1 && SM) {
-      // while the block spills, pooled subproblems go to the queue as tasks
-      int sp = 0, rec = -1, t = -1;
-      if (lane == 0 && budget > 0 && *(volatile int *)&pool->spill == 1) {
-        sp = 1;
-        rec = *(volatile int *)&pool->rec;
-        t = reserve_tasks(a, 1);
-      }
-      sp = __shfl_sync(FULL, sp, 0);
-      if (sp) {
-        t = __shfl_sync(FULL, t, 0);
-        rec = __shfl_sync(FULL, rec, 0);
-        if (t >= 0) {
-          write_task(a, t, rec, cs, C, P);
-          if (lane == 0 && pool_lock(pool, a.err, a.spin)) {
-            pool->idle++;
-            pool_unlock(pool);
-          }
-          __syncwarp();
-          continue;
-        }
-      }
-    }
     int om2 = read_best(a.best, g);
     color_ise<WPL, SM>(A, Ws, W, P, om2 - cs, B);
     wat = om2;
@@ -1289,6 +1179,9 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
         color_ise<WPL, SM>(A, Ws, W, P, om - 1, B);
         go = bany(B) ? 1 : 0;
         if (go) branched++;
+        if constexpr (WPL == 1 && SM) {
+          if (go && a.tasks && publish_root(a, r, A, Ws, W, P)) go = 0;
+        }
       }
       have = go != 0;
       if (lane == 0) {
@@ -1297,15 +1190,11 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
         pool->count = 0;
         pool->idle = kBW - 1;
         pool->beat = 0;
-        pool->spent = 0;
-        pool->spill = 0;
-        pool->rec = -1;
       }
     }
     __syncthreads();
     if (!ctl[4]) continue;
-    block_search<WPL, SM>(a, r, A, Ws, W, stk, pool, have, P, B, C, cs, wat, nodes, don,
-                          (SM && WPL == 1 && a.tasks) ? a.budget_block : 0);
+    block_search<WPL, SM>(a, r, A, Ws, W, stk, pool, have, P, B, C, cs, wat, nodes, don);
     __syncthreads();
   }
   if (lane == 0) {
@@ -1317,173 +1206,536 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
 }
 
 
-// The task queue: tasks of spilled roots, searched by whole blocks.  A block
-// takes the next task, loads its root's matrix and P list into shared
-// memory when the root changes, and searches it like a block worker; past
-// its node budget, while the queue is short, it spills again.  The kernel
-// ends when the queue is empty and no block holds a task (a block counts
-// itself in `active` before it looks for a task and leaves it only after
-// its spilled tasks are visible).
-template <int PC>
-__global__ void __launch_bounds__(kBT, (PC <= kMidCap) ? 2 : 1) branch_task_kernel(SA a) {
-  using L = BlockLayout<1, true, PC>;  // PC >= every record's p
-  extern __shared__ __align__(16) unsigned char smem[];
-  int *Pidx = (int *)(smem + L::off_P);
-  Pool<1> *pool = (Pool<1> *)(smem + L::off_pool);
-  int *ctl = (int *)(smem + L::off_ctl);
-  uint32_t *A = (uint32_t *)(smem + L::off_A);
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  uint32_t *stk = a.stack + ((int64_t)blockIdx.x * kBW + wid) * a.stack_stride;
-  unsigned long long nodes = 0, don = 0;
-  int loaded = -1;
+// ------------------------------------------------------------ task queue ---
+//
+// Tasks are searched by single warps on a compact copy of their subproblem.
+// A task's candidates are a few hundred at most (a neighbourhood of a
+// neighbourhood), so their adjacency matrix takes 2 or 8 KB of shared memory
+// per warp (16 warps per SM), and every lane holds whole vertex sets in
+// registers.  The search is bound by the latency of the greedy colouring, a
+// chain from vertex to vertex.  Against whole blocks per task with a bit
+// matrix of up to 1,024 candidates, the candidates in rank order and one set
+// word per lane: 13 us per Branch node before, 7 us now, and 5 to 30 times
+// fewer nodes, since the candidates are sorted by their degree in the
+// subproblem.  R-MAT scale 18, edge factor 12: search 83-330 ms before (it
+// depends on when the larger cliques are found), 4.2-4.6 ms now; scale 15,
+// edge factor 16: 60-104 ms before, 1.3 ms now.
+constexpr int kTM = 256;    // candidates of a compact subproblem
+constexpr int kTW = 4;      // warps per block of the task kernel
+constexpr int kTStk = 20;   // stack words per level (two sets of at most 8 words, omega, chosen vertex)
+
+struct TaskSmem {
+  uint32_t A[kTM * (kTM / 32)];
+  int mem[kTM];       // position in the root's P list of compact vertex i
+  uint32_t bits[32];  // sets over the root's positions
+  uint32_t drop[32];
+  uint8_t lst[kTM + 16];  // vertices of the set being coloured
+};
+
+template <int NW>
+struct Set {
+  uint32_t w[NW];
+};
+template <int NW>
+__device__ __forceinline__ bool sany(const Set<NW> &s) {
+  uint32_t x = 0;
+#pragma unroll
+  for (int i = 0; i < NW; i++) x |= s.w[i];
+  return x != 0;
+}
+template <int NW>
+__device__ __forceinline__ int scount(const Set<NW> &s) {
+  int c = 0;
+#pragma unroll
+  for (int i = 0; i < NW; i++) c += __popc(s.w[i]);
+  return c;
+}
+template <int NW>
+__device__ __forceinline__ int shighest(const Set<NW> &s) {
+  int v = -1;
+#pragma unroll
+  for (int i = 0; i < NW; i++)
+    if (s.w[i]) v = 32 * i + 31 - __clz(s.w[i]);
+  return v;
+}
+template <int NW>
+__device__ __forceinline__ void sclear(Set<NW> &s, int v) {
+  const uint32_t m = ~(1u << (v & 31));
+#pragma unroll
+  for (int i = 0; i < NW; i++)
+    if (i == (v >> 5)) s.w[i] &= m;
+}
+template <int NW>
+__device__ __forceinline__ Set<NW> sload(const uint32_t *p) {
+  Set<NW> s;
+#pragma unroll
+  for (int i = 0; i < NW / 4; i++) {
+    const uint4 x = reinterpret_cast<const uint4 *>(p)[i];
+    s.w[4 * i] = x.x;
+    s.w[4 * i + 1] = x.y;
+    s.w[4 * i + 2] = x.z;
+    s.w[4 * i + 3] = x.w;
+  }
+  return s;
+}
+// one lane stores
+template <int NW>
+__device__ __forceinline__ void sstore(uint32_t *p, const Set<NW> &s) {
+#pragma unroll
+  for (int i = 0; i < NW / 4; i++)
+    reinterpret_cast<uint4 *>(p)[i] = make_uint4(s.w[4 * i], s.w[4 * i + 1], s.w[4 * i + 2], s.w[4 * i + 3]);
+}
+
+// Greedy colouring of P in index order with at most q classes: a vertex takes
+// the first class that holds none of its neighbours; R receives the vertices
+// no class takes.  Class 32 s + lane is in this lane's registers, so placing a
+// vertex is a few ANDs and a ballot per 32 classes, 64 classes at a time
+// without a branch.  The vertices are listed first: a row is on its way from
+// shared memory while the one before is placed, and no find-first-set is on
+// the chain from one vertex to the next.  Every lane holds the same P and R.
+template <int NW>
+__device__ __forceinline__ void colour_set(const uint32_t *A, uint8_t *lst, const Set<NW> &P, int q, Set<NW> &R) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  int end[NW];
+  __syncwarp();
+#pragma unroll
+  for (int w = 0; w < NW; w++) {
+    const int at = w ? end[w - 1] : 0;
+    if ((P.w[w] >> lane) & 1u) lst[at + __popc(P.w[w] & lt)] = (uint8_t)(32 * w + lane);
+    end[w] = at + __popc(P.w[w]);
+  }
+  __syncwarp();
+  Set<NW> cls[NW];
+#pragma unroll
+  for (int s = 0; s < NW; s++)
+#pragma unroll
+    for (int i = 0; i < NW; i++) cls[s].w[i] = 0;
+  int v = lst[0], vn = lst[1];  // past the end: some row of the matrix's space, not used
+  Set<NW> row = sload<NW>(A + v * NW);
+  int i = 0;
+#pragma unroll
+  for (int w = 0; w < NW; w++) {
+    R.w[w] = 0;
+    for (; i < end[w]; i++) {
+      const Set<NW> next = sload<NW>(A + vn * NW);
+      const int vnn = lst[i + 2];
+      const uint32_t bit = 1u << (v & 31);
+      bool placed = false;
+#pragma unroll
+      for (int p = 0; p < NW / 2; p++) {
+        if (p == 0 || (!placed && 64 * p < q)) {
+          // vertices come in index order: no class holds one of a later word
+          uint32_t y0 = 0, y1 = 0;
+#pragma unroll
+          for (int k = 0; k <= w; k++) {
+            y0 |= cls[2 * p].w[k] & row.w[k];
+            y1 |= cls[2 * p + 1].w[k] & row.w[k];
+          }
+          const bool free0 = y0 == 0 && 64 * p + lane < q, free1 = y1 == 0 && 64 * p + 32 + lane < q;
+          const unsigned f0 = __ballot_sync(FULL, free0), f1 = __ballot_sync(FULL, free1);
+          if (free0 && !(f0 & lt)) cls[2 * p].w[w] |= bit;
+          if (free1 && !(f0 | (f1 & lt))) cls[2 * p + 1].w[w] |= bit;
+          placed = (f0 | f1) != 0;
+        }
+      }
+      if (!placed) R.w[w] |= bit;
+      row = next;
+      v = vn;
+      vn = vnn;
+    }
+  }
+}
+
+// What a warp knows of its task.
+struct TaskCtx {
+  int rec, cs;          // record, clique size (counting u) at the task's start
+  uint32_t C;           // the task's clique over the root's positions, one word per lane
+  int u, g, p, W, Ws;
+  const uint32_t *A;    // the root's matrix (arena)
+  const int *Pidx;      // the root's P list (arena)
+};
+
+// The clique {u} + C + the compact vertices path[0..d) (+ v) in original
+// ids.  All lanes.
+__device__ void write_task_clique(int32_t *base, const SA &a, const TaskCtx &T, const int *mem, const uint32_t *stk,
+                                  int d, int v) {
+  const int lane = threadIdx.x & 31;
+  const int cnt = __popc(T.C);
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    int y = __shfl_up_sync(FULL, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const int tot = __shfl_sync(FULL, incl, 31);
+  int pos = 1 + incl - cnt;
+  uint32_t x = T.C;
+  while (x) {
+    const int b = __ffs(x) - 1;
+    x &= x - 1;
+    base[pos++] = a.oold[__ldcg(T.Pidx + 32 * lane + b)];
+  }
+  if (lane == 0) base[0] = a.oold[T.u];
+  const int n = d + (v >= 0 ? 1 : 0);
+  for (int i = lane; i < n; i += 32) {
+    const int y = i < d ? (int)stk[i * kTStk + 17] : v;
+    base[1 + tot + i] = a.oold[__ldcg(T.Pidx + mem[y])];
+  }
+}
+
+// Hand the untried branches of the shallowest level that has some to the
+// queue, one task each; that level keeps none.  All or nothing: without room
+// in the queue nothing changes.  Returns the tasks written.
+template <int NW>
+__device__ int offer_level(const SA &a, const TaskCtx &T, TaskSmem &S, uint32_t *stk, int d, Set<NW> &P, Set<NW> &B) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  int l = 0;
+  Set<NW> Pl = P, Bl = B;
+  for (; l < d; l++) {
+    Bl = sload<NW>(stk + l * kTStk + 8);
+    if (sany(Bl)) break;
+  }
+  if (l < d) Pl = sload<NW>(stk + l * kTStk);
+  else Bl = B;
+  const int k = scount(Bl);
+  if (k == 0) return 0;
+  int t = -1;
+  if (lane == 0) t = reserve_tasks(a, k, 1);
+  t = __shfl_sync(FULL, t, 0);
+  if (t < 0) return 0;
+  // the clique at this level, over the root's positions
+  S.bits[lane] = T.C;
+  __syncwarp();
+  for (int i = lane; i < l; i += 32) {
+    const int pos = S.mem[stk[i * kTStk + 17]];
+    atomicOr(&S.bits[pos >> 5], 1u << (pos & 31));
+  }
+  __syncwarp();
+  const uint32_t Cl = S.bits[lane];
+  const int csl = T.cs + l;
+  for (int i = 0; i < k; i++) {
+    const int x = shighest(Bl);
+    sclear(Bl, x);
+    sclear(Pl, x);
+    const Set<NW> row = sload<NW>(S.A + x * NW);
+    Set<NW> TP;
+#pragma unroll
+    for (int q = 0; q < NW; q++) TP.w[q] = Pl.w[q] & row.w[q];
+    const int om = read_best(a.best, T.g);
+    const int n = scount(TP);
+    int cs = csl + 1;
+    if (cs + n <= om) cs = 0;  // decided: an empty task
+    // the child's candidates over the root's positions
+    __syncwarp();
+    S.bits[lane] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < NW; q++)
+      if ((TP.w[q] >> lane) & 1u) {
+        const int pos = S.mem[32 * q + lane];
+        atomicOr(&S.bits[pos >> 5], 1u << (pos & 31));
+      }
+    __syncwarp();
+    const int px = S.mem[x];
+    Bits<1> Cx, Px;
+    Cx.w[0] = Cl | (lane == (px >> 5) ? 1u << (px & 31) : 0u);
+    Px.w[0] = S.bits[lane];
+    write_task(a, t + i, T.rec, cs, Cx, Px);
+  }
+  if (l < d) {
+    if (lane == 0) {
+      Set<NW> none;
+#pragma unroll
+      for (int q = 0; q < NW; q++) none.w[q] = 0;
+      sstore<NW>(stk + l * kTStk + 8, none);
+    }
+    __syncwarp();
+  } else {
+#pragma unroll
+    for (int q = 0; q < NW; q++) B.w[q] = 0;
+  }
+  return k;
+}
+
+// Depth-first Branch on the compact subproblem S.A over m vertices.
+template <int NW>
+__device__ void task_dfs(const SA &a, const TaskCtx &T, TaskSmem &S, uint32_t *stk, int m, unsigned long long &nodes,
+                         unsigned long long &don) {
+  const int lane = threadIdx.x & 31;
+  Set<NW> P, B;
+#pragma unroll
+  for (int i = 0; i < NW; i++)
+    P.w[i] = m >= 32 * (i + 1) ? FULL : (m > 32 * i ? (1u << (m - 32 * i)) - 1u : 0u);
+  int d = 0, wat = -1, csize = T.cs;
+  int since = 0;
+  long long spent = 0;
+  // omega, read one step ahead (an old value only prunes less)
+  int ahead = *(const volatile int32_t *)(a.best + T.g);
   for (;;) {
-    __syncthreads();
-    Bits<1> C, P;
-    bzero(C);
-    bzero(P);
-    if (wid == 0) {
-      int got = -1;
+    const int om = __shfl_sync(FULL, ahead, 0);
+    ahead = *(const volatile int32_t *)(a.best + T.g);
+    if (om > wat) {  // a new node, or omega has risen since it was coloured
+      colour_set<NW>(S.A, S.lst, P, om - csize, B);
+      wat = om;
+    }
+    const int v = shighest(B);
+    if (v < 0) {
+      if (d == 0) return;
+      d--;
+      csize--;
+      P = sload<NW>(stk + d * kTStk);
+      B = sload<NW>(stk + d * kTStk + 8);
+      wat = (int)stk[d * kTStk + 16];
+      continue;
+    }
+    if (++since >= a.offer_nodes) {
+      // waiting warps hold tickets beyond the last published task
+      since = 0;
+      int hungry = 0;
       if (lane == 0) {
-        long long waited = 0;
-        int last = -1;
-        atomicAdd(a.active, 1);
-        __threadfence();
-        for (;;) {
-          if (*(volatile int32_t *)a.err) break;
-          const int tail = *(volatile int32_t *)a.ntasks, head = *(volatile int32_t *)a.task_next;
-          if (head < tail) {
-            if (atomicCAS(a.task_next, head, head + 1) == head) {
-              got = head;
-              break;
-            }
-            continue;
-          }
-          // nothing queued: stand down and wait for work or for the end (no
-          // block holds a task and the queue is empty)
-          atomicSub(a.active, 1);
-          __threadfence();
-          bool done = false, work = false;
-          while (!done && !work) {
-            if (*(volatile int32_t *)a.err) {
-              done = true;
-              break;
-            }
-            const int act = *(volatile int32_t *)a.active;
-            __threadfence();
-            const int tail2 = *(volatile int32_t *)a.ntasks, head2 = *(volatile int32_t *)a.task_next;
-            if (head2 < tail2) {
-              work = true;
-            } else if (act == 0) {
-              done = true;
-            } else {
-              const int prog = *(volatile int32_t *)a.progress + tail2;
-              if (prog != last) {
-                last = prog;
-                waited = 0;
-              }
-              if (++waited > a.spin) {
-                atomicExch(a.err, kDevTimeout);
-                done = true;
-              }
-              __nanosleep(512);
-            }
-          }
-          if (done) break;
-          atomicAdd(a.active, 1);
-          __threadfence();
-        }
-        if (got >= 0) {
-          // the slot's words are written before its word reads 2*lap+1
-          const int slot = got & (a.task_cap - 1);
-          const int lap2 = 2 * (got / a.task_cap);
-          long long w = 0;
-          while (*(volatile int32_t *)(a.ready + slot) != lap2 + 1) {
-            if (++w > a.spin) {
-              atomicExch(a.err, kDevTimeout);
-              break;
-            }
-            __nanosleep(64);
-          }
-          __threadfence();
-        }
+        hungry = *(volatile int32_t *)a.task_next > *(volatile int32_t *)a.ntasks;
+        if (*(volatile int32_t *)a.err) hungry = -1;
       }
-      got = __shfl_sync(FULL, got, 0);
-      if (got >= 0) {
-        const uint32_t *tk = a.tasks + (int64_t)(got & (a.task_cap - 1)) * kTaskWords;
-        C.w[0] = __ldcg(tk + 2 + lane);
-        P.w[0] = __ldcg(tk + 34 + lane);
-        const int cs1 = (int)__ldcg(tk + 1), rec1 = (int)__ldcg(tk + 0);
-        __syncwarp();
-        if (lane == 0) {
-          __threadfence();
-          // free the slot for the next lap's writer
-          atomicExch(a.ready + (got & (a.task_cap - 1)), 2 * (got / a.task_cap) + 2);
-          ctl[1] = cs1;
-          ctl[2] = rec1;
-        }
-      }
-      if (lane == 0) {
-        ctl[0] = got;
-        ctl[3] = *(volatile int32_t *)a.err;
+      hungry = __shfl_sync(FULL, hungry, 0);
+      if (hungry < 0) return;
+      if (hungry) {
+        const int k = offer_level<NW>(a, T, S, stk, d, P, B);
+        don += (unsigned long long)k;
+        if (k) continue;
       }
     }
-    __syncthreads();
-    const int t = ctl[0];
-    if (t < 0) break;
-    const int cs0 = ctl[1], rec = ctl[2];
-    if (cs0 == 0 || ctl[3]) {  // empty task (or giving up)
-      __syncthreads();
-      if (tid == 0) {
-        __threadfence();
-        atomicSub(a.active, 1);
+    sclear(B, v);
+    sclear(P, v);
+    const Set<NW> row = sload<NW>(S.A + v * NW);
+    Set<NW> NP;
+#pragma unroll
+    for (int i = 0; i < NW; i++) NP.w[i] = P.w[i] & row.w[i];
+    nodes++;
+    if ((++spent & 255) == 0 && lane == 0) atomicAdd(a.progress, 1);
+    const int cnt = scount(NP);
+    if (cnt == 0) {
+      if (csize + 1 > om) {
+        __syncwarp();
+        const int dd = d;
+        dev::raise_incumbent(a.best, a.lock, a.wit, a.voff, T.g, csize + 1, a.err, a.spin,
+                             [&](int, int32_t *base) { write_task_clique(base, a, T, S.mem, stk, dd, v); });
       }
       continue;
     }
-    RootRec rr;
-    {
-      const int *rp = (const int *)(a.recs + rec);
-      rr.u = __ldcg(rp + 0);
-      rr.g = __ldcg(rp + 1);
-      rr.p = __ldcg(rp + 2);
-      rr.W = __ldcg(rp + 3);
-      rr.Ws = __ldcg(rp + 4);
-      rr.off = __ldcg((const long long *)(rp + 6));
+    if (csize + 1 + cnt <= om) continue;
+    if (lane == 0) {
+      sstore<NW>(stk + d * kTStk, P);
+      sstore<NW>(stk + d * kTStk + 8, B);
+      stk[d * kTStk + 16] = (uint32_t)wat;
+      stk[d * kTStk + 17] = (uint32_t)v;
     }
-    if (rec != loaded) {
-      const uint32_t *sm = a.arena + rr.off;
-      for (int i = tid; i < rr.p * rr.Ws; i += kBT) A[i] = __ldcg(sm + i);
-      const int *sp = (const int *)(sm + (int64_t)rr.p * rr.Ws);
-      for (int i = tid; i < rr.p; i += kBT) Pidx[i] = __ldcg(sp + i);
-      loaded = rec;
-    }
-    __syncthreads();
-    Root r{rr.u, rr.g, Pidx, rr.p};
-    Bits<1> B;
-    bzero(B);
-    int cs = cs0, wat = 0;
-    bool have = false;
-    if (wid == 0) {
-      wat = read_best(a.best, rr.g);
-      color_ise<1, true>(A, rr.Ws, rr.W, P, wat - cs, B);
-      have = bany(B);
-      if (lane == 0) {
-        ctl[4] = have ? 1 : 0;
-        pool->lock = 0;
-        pool->count = 0;
-        pool->idle = kBW - 1;
-        pool->beat = 0;
-        pool->spent = 0;
-        pool->spill = 0;
-        pool->rec = rec;
+    __syncwarp();
+    d++;
+    csize++;
+    P = NP;
+    wat = -1;
+  }
+}
+
+// Compact matrix of the m listed members (S.mem): row i, word w holds the
+// adjacency of member i to members 32w .. 32w+31.  A row of the root's matrix
+// is at most 32 words: one coalesced load, then a shuffle, a shift and a
+// ballot per compact word.
+template <int NW>
+__device__ void compact_matrix(const TaskCtx &T, TaskSmem &S, int m) {
+  const int lane = threadIdx.x & 31;
+  int at[NW];
+#pragma unroll
+  for (int w = 0; w < NW; w++) at[w] = 32 * w + lane < m ? S.mem[32 * w + lane] : -1;
+  for (int i0 = 0; i0 < m; i0 += 4) {
+    uint32_t x[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+      x[k] = (i0 + k < m && lane < T.W) ? __ldcg(T.A + (int64_t)S.mem[i0 + k] * T.Ws + lane) : 0u;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      uint32_t mine = 0;
+#pragma unroll
+      for (int w = 0; w < NW; w++) {
+        const uint32_t y = __shfl_sync(FULL, x[k], (at[w] < 0 ? 0 : at[w]) >> 5);
+        const unsigned word = __ballot_sync(FULL, at[w] >= 0 && ((y >> (at[w] & 31)) & 1u));
+        if (lane == w) mine = word;
       }
+      if (i0 + k < m && lane < NW) S.A[(i0 + k) * NW + lane] = mine;
     }
-    __syncthreads();
-    if (ctl[4]) block_search<1, true>(a, r, A, rr.Ws, rr.W, stk, pool, have, P, B, C, cs, wat, nodes, don,
-                                      a.budget_block);
-    __syncthreads();
-    if (tid == 0) {
+  }
+  __syncwarp();
+}
+
+// One task (all lanes): clique T.C, candidates P (a word per lane).
+__device__ void run_task(const SA &a, TaskCtx &T, Bits<1> P, TaskSmem &S, uint32_t *stk, unsigned long long &nodes,
+                         unsigned long long &don) {
+  const int lane = threadIdx.x & 31;
+  const int om = read_best(a.best, T.g);
+  // a clique larger than omega takes omega + 1 - cs of the candidates, each
+  // with at least omega - cs neighbours among them: drop the others.  The
+  // candidates' list and their sort keys use the matrix's space, which is not
+  // built yet; lane i takes every 32nd candidate.
+  int *lst = (int *)S.A;
+  uint32_t *key = S.A + 1024, *drop = S.drop;
+  int m = 0;
+  for (;;) {
+    const int cnt = __popc(P.w[0]);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int y = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += y;
+    }
+    m = __shfl_sync(FULL, incl, 31);
+    if (T.cs + m <= om) return;
+    __syncwarp();
+    S.bits[lane] = P.w[0];
+    drop[lane] = 0;
+    int slot = incl - cnt;
+    for (uint32_t x = P.w[0]; x; x &= x - 1) lst[slot++] = 32 * lane + __ffs(x) - 1;
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) {
+      const int pos = lst[i];
+      const uint32_t *row = T.A + (int64_t)pos * T.Ws;
+      int deg = 0;
+#pragma unroll 4
+      for (int w = 0; w < T.W; w++) deg += __popc(__ldcg(row + w) & S.bits[w]);
+      if (deg < om - T.cs) atomicOr(&drop[pos >> 5], 1u << (pos & 31));
+      key[i] = ((uint32_t)(deg + 1) << 16) | (uint32_t)(0xffff - pos);
+    }
+    __syncwarp();
+    const uint32_t dr = drop[lane];
+    if (!__any_sync(FULL, dr != 0)) break;
+    P.w[0] &= ~dr;
+  }
+  if (m == 0) {  // a maximal clique: {u} + C
+    dev::raise_incumbent(a.best, a.lock, a.wit, a.voff, T.g, T.cs, a.err, a.spin,
+                         [&](int, int32_t *base) { write_task_clique(base, a, T, S.mem, stk, 0, -1); });
+    return;
+  }
+  if (m > kTM) {
+    // too many for the compact form: colour on the arena's matrix and make
+    // every branch a task (or search here when the queue is full)
+    Bits<1> B, C;
+    C.w[0] = T.C;
+    color_ise<1, false>(T.A, T.Ws, T.W, P, om - T.cs, B);
+    const int k = bcount(B);
+    if (k == 0) return;
+    Root r{T.u, T.g, T.Pidx, T.p};
+    int t = -1;
+    if (lane == 0) t = reserve_tasks(a, k, a.spin);
+    t = __shfl_sync(FULL, t, 0);
+    if (t < 0) {
+      dfs<1, false>(a, r, T.A, T.Ws, T.W, stk, T.cs, P, B, C, om, (Pool<1> *)nullptr, nodes, don);
+      return;
+    }
+    for (int i = 0; i < k; i++) {
+      const int x = bhighest(B);
+      bclear(B, x);
+      bclear(P, x);
+      emit_task(a, r, T.A, T.Ws, T.W, T.rec, t + i, C, T.cs, P, x);
+    }
+    nodes++;
+    don += (unsigned long long)k;
+    return;
+  }
+  // members by decreasing degree among the candidates (ties: smaller
+  // position): the colouring takes the densest first, the branching the
+  // sparsest
+  int np2 = 32;
+  while (np2 < m) np2 <<= 1;
+  for (int i = m + lane; i < np2; i += 32) key[i] = 0;
+  __syncwarp();
+  bitonic_desc<false>((int *)key, np2, lane, 32);  // keys below 2^27: the signed order is the same
+  for (int i = lane; i < m; i += 32) S.mem[i] = 0xffff - (int)(key[i] & 0xffffu);
+  __syncwarp();  // the keys are read before the matrix takes their place
+  if (m <= 128) {
+    compact_matrix<4>(T, S, m);
+    task_dfs<4>(a, T, S, stk, m, nodes, don);
+  } else {
+    compact_matrix<8>(T, S, m);
+    task_dfs<8>(a, T, S, stk, m, nodes, don);
+  }
+}
+
+// The task kernel: every warp takes a ticket (a queue position) and waits for
+// the task at that position; tickets beyond the last published task are the
+// waiting warps, which the searching warps see and hand branches to.  The
+// wait is on the position's own word, so waiting warps do not contend.  It
+// ends when no published task is unfinished (pending is 0): nothing can be
+// published then.
+__global__ void __launch_bounds__(kTW * 32, 4) branch_task_kernel(SA a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  TaskSmem &S = ((TaskSmem *)smem)[wib];
+  uint32_t *stk = a.stack + ((int64_t)blockIdx.x * kTW + wib) * a.stack_stride;
+  unsigned long long nodes = 0, don = 0;
+  for (;;) {
+    __syncwarp();
+    int got = -1;
+    if (lane == 0 && *(volatile int32_t *)a.pending > 0) {
+      const int t = atomicAdd(a.task_next, 1);
+      const int slot = t & (a.task_cap - 1), lap2 = 2 * (t / a.task_cap);
+      long long waited = 0;
+      unsigned ns = 64, polls = 0;
+      int last = -1;
+      for (;;) {
+        if (*(volatile int32_t *)(a.ready + slot) == lap2 + 1) {
+          got = t;
+          break;
+        }
+        if (*(volatile int32_t *)a.pending == 0) break;
+        if ((polls++ & 15) == 0) {
+          if (*(volatile int32_t *)a.err) break;
+          const int prog = *(volatile int32_t *)a.progress + *(volatile int32_t *)a.ntasks;
+          if (prog != last) {
+            last = prog;
+            waited = 0;
+          }
+        }
+        waited += ns >> 6;
+        if (waited > a.spin) {
+          atomicExch(a.err, kDevTimeout);
+          break;
+        }
+        __nanosleep(ns);
+        if (ns < 4096) ns <<= 1;
+      }
       __threadfence();
-      atomicSub(a.active, 1);
+    }
+    got = __shfl_sync(FULL, got, 0);
+    if (got < 0) break;
+    const int slot = got & (a.task_cap - 1);
+    const uint32_t *tk = a.tasks + (int64_t)slot * kTaskWords;
+    TaskCtx T;
+    Bits<1> P;
+    T.rec = (int)__ldcg(tk + 0);
+    T.cs = (int)__ldcg(tk + 1);
+    T.C = __ldcg(tk + 2 + lane);
+    P.w[0] = __ldcg(tk + 34 + lane);
+    __syncwarp();
+    if (lane == 0) {
+      __threadfence();
+      atomicExch(a.ready + slot, 2 * (got / a.task_cap) + 2);  // free for the next lap's writer
+    }
+    if (T.cs > 0) {
+      const int *rp = (const int *)(a.recs + T.rec);
+      T.u = __ldcg(rp + 0);
+      T.g = __ldcg(rp + 1);
+      T.p = __ldcg(rp + 2);
+      T.W = __ldcg(rp + 3);
+      T.Ws = __ldcg(rp + 4);
+      T.A = a.arena + __ldcg((const long long *)(rp + 6));
+      T.Pidx = (const int *)(T.A + (int64_t)T.p * T.Ws);
+      run_task(a, T, P, S, stk, nodes, don);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      __threadfence();
+      atomicSub(a.pending, 1);
     }
   }
   if (lane == 0) {
@@ -1500,14 +1752,15 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   // device (pg.d_counts), and sizes are bounded by K(G) >= |N+(u)|, so the
   // launches need no host synchronisation.
   void *p;
-  MC_TRY(ws_get(g, "se.ctr", 16 * sizeof(unsigned long long), &p));
+  MC_TRY(ws_get(g, "se.ctr", kCtrBytes, &p));
   // [0..5] colored, branched, nodes, donations, row entries read by warp
   // workers, by block workers; [8..9] four root queue heads; [10] arena
-  // words used; [11..13] records, task tail, task head, blocks holding a
-  // task, heartbeat; [14] roots left to the 1,024-candidate launch
+  // words used; [11] records; [14] roots left to the 1,024-candidate launch;
+  // the queue's hot words on 128-byte lines of their own: [32] tasks, [48]
+  // tickets, [64] unfinished tasks, [80] heartbeat
   unsigned long long *ctr = (unsigned long long *)p;
   int32_t *next = (int32_t *)(ctr + 8);
-  MC_CUDA_TRY(cudaMemsetAsync(ctr, 0, 16 * sizeof(unsigned long long), g->stream));
+  MC_CUDA_TRY(cudaMemsetAsync(ctr, 0, kCtrBytes, g->stream));
   SA a{};
   a.np_count = pg.d_counts;
   a.use_bitmap = no_bitmap ? 0 : 1;
@@ -1532,7 +1785,7 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   const int wmax = g->warp_max_used;
   if (!no_split) {
     // queue sizes grow with the graph (a small graph gets a small queue; a
-    // full queue only stops further spills)
+    // full queue only keeps work where it is)
     const long long arena_words = std::min<long long>(kArenaWords, std::max<long long>(1ll << 18, 4 * g->nnz));
     const int rec_cap = (int)std::min<int64_t>(kRecCap, std::max<int64_t>(1024, g->n));
     int task_cap = 1 << 12;
@@ -1551,17 +1804,14 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
     a.ready = (int32_t *)p;
     MC_CUDA_TRY(cudaMemsetAsync(a.ready, 0, (size_t)task_cap * 4, g->stream));
     a.task_cap = task_cap;
-    a.ntasks = a.nrec + 1;
-    a.task_next = a.nrec + 2;
-    a.active = a.nrec + 3;
-    a.progress = a.nrec + 4;
-    a.queue_gate = 0;
-    a.budget_warp = split_nodes > 0 ? split_nodes : kSpillNodes;
-    a.budget_block = 4 * a.budget_warp;
+    a.ntasks = (int32_t *)(ctr + 32);
+    a.task_next = (int32_t *)(ctr + 48);
+    a.pending = (int32_t *)(ctr + 64);
+    a.progress = (int32_t *)(ctr + 80);
+    a.offer_nodes = split_nodes > 0 ? split_nodes : kOfferNodes;
   }
   // Block workers (shared-memory matrices): a 512-candidate launch first,
-  // then a 1,024-candidate launch over the roots it could not hold; the task
-  // kernel shares the large layout and its stack buffer.
+  // then a 1,024-candidate launch over the roots it could not hold.
   using LB = BlockLayout<1, true>;
   using LM = BlockLayout<1, true, kMidCap>;
   const size_t smem_b = LB::bytes, smem_m = LM::bytes;
@@ -1569,33 +1819,31 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
                                    (int)smem_b));
   MC_CUDA_TRY(cudaFuncSetAttribute(search_block_kernel<1, true, kMidCap>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)smem_m));
-  MC_CUDA_TRY(cudaFuncSetAttribute(branch_task_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
-  MC_CUDA_TRY(cudaFuncSetAttribute(branch_task_kernel<kMidCap>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)smem_m));
-  int per_sm_b = 0, per_sm_t = 0, per_sm_m = 0, per_sm_tm = 0;
+  const size_t smem_t = kTW * sizeof(TaskSmem);
+  MC_CUDA_TRY(cudaFuncSetAttribute(branch_task_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_t));
+  int per_sm_b = 0, per_sm_t = 0, per_sm_m = 0;
   MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, search_block_kernel<1, true, 1024>, kBT, smem_b));
-  MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_t, branch_task_kernel<1024>, kBT, smem_b));
-  MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_tm, branch_task_kernel<kMidCap>, kBT, smem_m));
+  MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_t, branch_task_kernel, kTW * 32, smem_t));
   MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_m, search_block_kernel<1, true, kMidCap>, kBT,
                                                             smem_m));
-  per_sm_b = std::min(per_sm_b, per_sm_t);
-  if (per_sm_b < 1 || per_sm_m < 1 || per_sm_tm < 1) return MC_ERR_CUDA;
+  if (per_sm_b < 1 || per_sm_m < 1 || per_sm_t < 1) return MC_ERR_CUDA;
   // grids (and the stacks sized by them) shrink for small graphs: a block
   // per 64 vertices at most, a warp per four vertices in the warp class
   const int64_t small_cap = std::max<int64_t>(1, (g->n + 63) / 64);
   const int blocks_b = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_b, small_cap);
   const int blocks_m = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_m, small_cap);
-  // the task kernel takes the mid layout (two blocks per SM) when no record
-  // can hold more than kMidCap candidates (p <= K(G))
-  const bool task_mid = kbound <= kMidCap;
-  const int blocks_t =
-      task_mid ? (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_tm, small_cap) : blocks_b;
+  const int blocks_t = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_t, std::max<int64_t>(1, (g->n + 15) / 16));
   const int64_t stride_b = (int64_t)(std::min(kbound, 1024) + 2) * (64 + 2);
   const int64_t stride_m = (int64_t)(std::min(kbound, kMidCap) + 2) * (64 + 2);
-  uint32_t *stk_b = nullptr;
-  if (kbound > wmax || !no_split) {
-    MC_TRY(ws_get(g, "se.stk_b", (size_t)std::max(blocks_b, blocks_t) * kBW * stride_b * 4, &p));
+  const int64_t stride_t = (stride_b + 3) & ~(int64_t)3;  // levels of the compact search are stored as uint4
+  uint32_t *stk_b = nullptr, *stk_t = nullptr;
+  if (kbound > wmax) {
+    MC_TRY(ws_get(g, "se.stk_b", (size_t)blocks_b * kBW * stride_b * 4, &p));
     stk_b = (uint32_t *)p;
+  }
+  if (!no_split) {
+    MC_TRY(ws_get(g, "se.stk_t", (size_t)blocks_t * kTW * stride_t * 4, &p));
+    stk_t = (uint32_t *)p;
   }
 
   // block class first (largest trees), then big, then warp class, then the
@@ -1682,13 +1930,9 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   }
   MC_TRY(record_event(g, 11));
   if (!no_split) {
-    a.stack_stride = stride_b;
-    a.stack = stk_b;
-    a.queue_gate = 2 * blocks_t;
-    if (task_mid)
-      branch_task_kernel<kMidCap><<<blocks_t, kBT, smem_m, g->stream>>>(a);
-    else
-      branch_task_kernel<1024><<<blocks_t, kBT, smem_b, g->stream>>>(a);
+    a.stack_stride = stride_t;
+    a.stack = stk_t;
+    branch_task_kernel<<<blocks_t, kTW * 32, smem_t, g->stream>>>(a);
     g_launches++;
     MC_CUDA_TRY(cudaGetLastError());
   }
@@ -1699,7 +1943,7 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
 
 int read_search_counters(mc_graph *g, SearchCounters *cnt) {
   unsigned long long *h = (unsigned long long *)g->h_small;
-  MC_CUDA_TRY(cudaMemcpyAsync(h, cnt->d_counters, 13 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, g->stream));
+  MC_CUDA_TRY(cudaMemcpyAsync(h, cnt->d_counters, 33 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, g->stream));
   MC_CUDA_TRY(cudaStreamSynchronize(g->stream));
   cnt->roots_colored = h[0];
   cnt->roots_branched = h[1];
@@ -1707,7 +1951,7 @@ int read_search_counters(mc_graph *g, SearchCounters *cnt) {
   cnt->donations = h[3];
   cnt->entries = h[4] + h[5];
   cnt->entries_block = h[5];
-  cnt->tasks = (unsigned long long)((const int32_t *)(h + 11))[1];
+  cnt->tasks = (unsigned long long)*(const int32_t *)(h + 32);
   return MC_OK;
 }
 

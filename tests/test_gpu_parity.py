@@ -182,6 +182,26 @@ def test_split_tasks_keep_omega(mc):
     assert seen > 0
 
 
+@pytest.mark.parametrize("n,p,planted", [(60, 0.9, 20), (140, 0.7, 18), (200, 0.7, 20), (300, 0.5, 14),
+                                         (900, 0.35, 16)])
+def test_task_sizes_keep_omega(mc, n, p, planted):
+    """Tasks are searched on a compact matrix of 128 or 256 candidates, and
+    expanded into smaller tasks above; these dense graphs have roots below,
+    between and above those sizes (K(G) from about 50 to 300).  The task
+    queue's omega must equal the in-block search's, with and without the
+    heuristic's lower bound, and the oracle's where that is quick."""
+    g = gg.relabel(gg.erdos_renyi(n, p, planted=planted, seed=n), 5)
+    h = load(mc, g)
+    om0, wit0, st0 = mc.mc_max_clique(h, no_split=True)
+    assert om0 >= planted and oracle.is_clique(g, wit0) and st0["tasks"] == 0
+    if n <= 300:
+        assert om0 == oracle.max_clique(g)[0]
+    for opts in (dict(), dict(heuristic=2), dict(heuristic=2, split_nodes=1, warp_max=1)):
+        om, wit, st = mc.mc_max_clique(h, **opts)
+        assert om == om0 and len(wit) == om and oracle.is_clique(g, wit), opts
+        assert st["tasks"] > 0 or st["roots_branched"] == 0
+
+
 def test_host_pointers_and_repeat_calls(mc):
     g = gg.chung_lu(5000, 2.4, 10.0, 500.0, planted=14, seed=21)
     h = load(mc, g, device=False)
