@@ -68,6 +68,7 @@ struct SA {
   int32_t *next;            // root grab counter
   uint32_t *stack;          // per-warp DFS stacks
   int64_t stack_stride;     // words per warp stack
+  int64_t small_stack;      // task kernel: offset of the compact search's levels in it
   uint32_t *gmat;           // per-block global matrix (big class)
   int64_t gmat_stride;      // words per block matrix
   int32_t neigh_cores;
@@ -934,6 +935,76 @@ struct BlockLayout {
   static constexpr size_t bytes = off_A + (SM ? (size_t)PCAP * WSMAX * 4 : 0);
 };
 
+// A block's root as a task: the candidates left by the core test, sorted by
+// decreasing degree among them, with their adjacency in that order (the
+// colouring of the task's upper levels takes the densest first too).  All
+// threads; keys: room for the next power of two above p, ctl: two words.
+// False, publishing nothing, without room.
+__device__ bool publish_sorted(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, const uint32_t *al,
+                               uint32_t *keys, int *ctl) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  int np2 = 32;
+  while (np2 < r.p) np2 <<= 1;
+  int m = 0;
+  for (int w = 0; w < W; w++) m += __popc(al[w]);
+  for (int i = tid; i < np2; i += kBT) {
+    uint32_t key = 0;
+    if (i < r.p && ((al[i >> 5] >> (i & 31)) & 1u)) {
+      int deg = 0;
+      for (int w = 0; w < W; w++) deg += __popc(A[i * Ws + w] & al[w]);
+      key = ((uint32_t)(deg + 1) << 16) | (uint32_t)(0xffff - i);
+    }
+    keys[i] = key;
+  }
+  const int Wm = (m + 31) >> 5, Wsm = Wm | 1;
+  if (tid == 0) {
+    const Root rm{r.u, r.g, r.Pidx, m};
+    long long off = 0;
+    int t = -1;
+    const int rec = reserve_record(a, rm, Wsm, &off);
+    if (rec >= 0) t = reserve_tasks(a, 1, a.spin);
+    ctl[0] = t;
+    ctl[1] = rec;
+    if (t >= 0) {
+      RootRec rr;
+      rr.u = r.u;
+      rr.g = r.g;
+      rr.p = m;
+      rr.W = Wm;
+      rr.Ws = Wsm;
+      rr.pad = 0;
+      rr.off = off;
+      a.recs[rec] = rr;
+    }
+  }
+  __syncthreads();
+  if (ctl[0] < 0) return false;
+  bitonic_desc<true>((int *)keys, np2, tid, kBT);
+  uint32_t *dm = a.arena + a.recs[ctl[1]].off;
+  int *dp = (int *)(dm + (int64_t)m * Wsm);
+  for (int i = wid; i < m; i += kBW) {
+    const uint32_t *row = A + (int64_t)(0xffff - (int)(keys[i] & 0xffffu)) * Ws;
+    uint32_t mine = 0;
+    for (int w = 0; w < Wm; w++) {
+      const int j = 32 * w + lane;
+      const int at = j < m ? 0xffff - (int)(keys[j] & 0xffffu) : 0;
+      const unsigned word = __ballot_sync(FULL, j < m && ((row[at >> 5] >> (at & 31)) & 1u));
+      if (lane == w) mine = word;
+    }
+    if (lane < Wm) dm[(int64_t)i * Wsm + lane] = mine;
+  }
+  for (int i = tid; i < m; i += kBT) dp[i] = r.Pidx[0xffff - (int)(keys[i] & 0xffffu)];
+  __threadfence();
+  __syncthreads();
+  if (wid == 0) {
+    Bits<1> C, P;
+    bzero(C);
+    P.w[0] = m >= 32 * (lane + 1) ? FULL : (m > 32 * lane ? (1u << (m - 32 * lane)) - 1u : 0u);
+    write_task(a, ctl[0], ctl[1], 1, C, P);
+  }
+  return true;
+}
+
 // The warps of a block search one root (or one task) together: warps that
 // hold work run the depth-first Branch and hand untried branches to idle
 // warps through the block's pool; the call returns when the pool is empty
@@ -1179,9 +1250,6 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
         color_ise<WPL, SM>(A, Ws, W, P, om - 1, B);
         go = bany(B) ? 1 : 0;
         if (go) branched++;
-        if constexpr (WPL == 1 && SM) {
-          if (go && a.tasks && publish_root(a, r, A, Ws, W, P)) go = 0;
-        }
       }
       have = go != 0;
       if (lane == 0) {
@@ -1194,6 +1262,10 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
     }
     __syncthreads();
     if (!ctl[4]) continue;
+    if constexpr (WPL == 1 && SM) {
+      // (the hash table's space is free: the matrix is built)
+      if (a.tasks && publish_sorted(a, r, A, Ws, W, al, (uint32_t *)hk, ctl + 8)) continue;
+    }
     block_search<WPL, SM>(a, r, A, Ws, W, stk, pool, have, P, B, C, cs, wat, nodes, don);
     __syncthreads();
   }
@@ -1220,6 +1292,12 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
 // subproblem.  R-MAT scale 18, edge factor 12: search 83-330 ms before (it
 // depends on when the larger cliques are found), 4.2-4.6 ms now; scale 15,
 // edge factor 16: 60-104 ms before, 1.3 ms now.
+// Subproblems above 256 candidates are searched depth first by the warp on the
+// root's matrix until a child fits; publishing every branch of such a node
+// instead (breadth first) let the queue fill with them before omega rose: two
+// of 40 R-MAT scale-20 graphs then took 36 and 85 s, now none of 129 takes
+// more than 65 ms.  Block roots are published with their candidates sorted by
+// degree, so that these levels are coloured densest first as well.
 constexpr int kTM = 256;    // candidates of a compact subproblem
 constexpr int kTW = 4;      // warps per block of the task kernel
 constexpr int kTStk = 20;   // stack words per level (two sets of at most 8 words, omega, chosen vertex)
@@ -1354,7 +1432,10 @@ struct TaskCtx {
   int u, g, p, W, Ws;
   const uint32_t *A;    // the root's matrix (arena)
   const int *Pidx;      // the root's P list (arena)
+  uint32_t *lev;        // levels of more than kTM candidates (kBigLev words each) ...
+  int nlev;             // ... and how many there are
 };
+constexpr int kBigLev = 66;  // two sets of 32 words, omega at the colouring, chosen vertex
 
 // The clique {u} + C + the compact vertices path[0..d) (+ v) in original
 // ids.  All lanes.
@@ -1459,6 +1540,38 @@ __device__ int offer_level(const SA &a, const TaskCtx &T, TaskSmem &S, uint32_t 
   return k;
 }
 
+// The same for the levels above the compact form, of which the first `chosen`
+// have a chosen vertex in T's clique; returns the tasks written.
+__device__ __noinline__ int offer_big(const SA &a, const TaskCtx &T, int chosen) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  for (int l = 0; l < T.nlev; l++) {
+    uint32_t *q = T.lev + (int64_t)l * kBigLev;
+    Bits<1> Pl, Bl, Cl;
+    Bl.w[0] = q[32 + lane];
+    const int k = bcount(Bl);
+    if (k == 0) continue;
+    int t = -1;
+    if (lane == 0) t = reserve_tasks(a, k, 1);
+    t = __shfl_sync(FULL, t, 0);
+    if (t < 0) return 0;
+    Pl.w[0] = q[lane];
+    Cl.w[0] = T.C;
+    for (int i = l; i < chosen; i++) bclear(Cl, level_word(T.lev + (int64_t)i * kBigLev + 65));
+    const Root r{T.u, T.g, T.Pidx, T.p};
+    for (int i = 0; i < k; i++) {
+      const int x = bhighest(Bl);
+      bclear(Bl, x);
+      bclear(Pl, x);
+      emit_task(a, r, T.A, T.Ws, T.W, T.rec, t + i, Cl, T.cs - (chosen - l), Pl, x);
+    }
+    q[32 + lane] = 0;
+    __syncwarp();
+    return k;
+  }
+  return 0;
+}
+
 // Depth-first Branch on the compact subproblem S.A over m vertices.
 template <int NW>
 __device__ void task_dfs(const SA &a, const TaskCtx &T, TaskSmem &S, uint32_t *stk, int m, unsigned long long &nodes,
@@ -1501,7 +1614,8 @@ __device__ void task_dfs(const SA &a, const TaskCtx &T, TaskSmem &S, uint32_t *s
       hungry = __shfl_sync(FULL, hungry, 0);
       if (hungry < 0) return;
       if (hungry) {
-        const int k = offer_level<NW>(a, T, S, stk, d, P, B);
+        int k = offer_big(a, T, T.nlev);
+        if (k == 0) k = offer_level<NW>(a, T, S, stk, d, P, B);
         don += (unsigned long long)k;
         if (k) continue;
       }
@@ -1569,18 +1683,18 @@ __device__ void compact_matrix(const TaskCtx &T, TaskSmem &S, int m) {
   __syncwarp();
 }
 
-// One task (all lanes): clique T.C, candidates P (a word per lane).
-__device__ void run_task(const SA &a, TaskCtx &T, Bits<1> P, TaskSmem &S, uint32_t *stk, unsigned long long &nodes,
-                         unsigned long long &don) {
+// Candidates that can be in a clique larger than omega with T's clique: omega
+// + 1 - cs of them are needed, each with at least omega - cs neighbours among
+// them; the others are dropped until none is.  Returns how many are left (0:
+// decided; a maximal clique {u} + C larger than omega was raised).  Their sort
+// keys (degree, then smaller position) are left in S.A + 1024.
+__device__ int prune_candidates(const SA &a, const TaskCtx &T, Bits<1> &P, TaskSmem &S) {
   const int lane = threadIdx.x & 31;
   const int om = read_best(a.best, T.g);
-  // a clique larger than omega takes omega + 1 - cs of the candidates, each
-  // with at least omega - cs neighbours among them: drop the others.  The
-  // candidates' list and their sort keys use the matrix's space, which is not
-  // built yet; lane i takes every 32nd candidate.
+  // the candidates' list and keys use the matrix's space, which is not built
+  // yet; lane i takes every 32nd candidate
   int *lst = (int *)S.A;
-  uint32_t *key = S.A + 1024, *drop = S.drop;
-  int m = 0;
+  uint32_t *key = S.A + 1024;
   for (;;) {
     const int cnt = __popc(P.w[0]);
     int incl = cnt;
@@ -1589,11 +1703,16 @@ __device__ void run_task(const SA &a, TaskCtx &T, Bits<1> P, TaskSmem &S, uint32
       int y = __shfl_up_sync(FULL, incl, o);
       if (lane >= o) incl += y;
     }
-    m = __shfl_sync(FULL, incl, 31);
-    if (T.cs + m <= om) return;
+    const int m = __shfl_sync(FULL, incl, 31);
+    if (T.cs + m <= om) return 0;
+    if (m == 0) {
+      dev::raise_incumbent(a.best, a.lock, a.wit, a.voff, T.g, T.cs, a.err, a.spin,
+                           [&](int, int32_t *base) { write_task_clique(base, a, T, S.mem, nullptr, 0, -1); });
+      return 0;
+    }
     __syncwarp();
     S.bits[lane] = P.w[0];
-    drop[lane] = 0;
+    S.drop[lane] = 0;
     int slot = incl - cnt;
     for (uint32_t x = P.w[0]; x; x &= x - 1) lst[slot++] = 32 * lane + __ffs(x) - 1;
     __syncwarp();
@@ -1603,48 +1722,23 @@ __device__ void run_task(const SA &a, TaskCtx &T, Bits<1> P, TaskSmem &S, uint32
       int deg = 0;
 #pragma unroll 4
       for (int w = 0; w < T.W; w++) deg += __popc(__ldcg(row + w) & S.bits[w]);
-      if (deg < om - T.cs) atomicOr(&drop[pos >> 5], 1u << (pos & 31));
+      if (deg < om - T.cs) atomicOr(&S.drop[pos >> 5], 1u << (pos & 31));
       key[i] = ((uint32_t)(deg + 1) << 16) | (uint32_t)(0xffff - pos);
     }
     __syncwarp();
-    const uint32_t dr = drop[lane];
-    if (!__any_sync(FULL, dr != 0)) break;
+    const uint32_t dr = S.drop[lane];
+    if (!__any_sync(FULL, dr != 0)) return m;
     P.w[0] &= ~dr;
   }
-  if (m == 0) {  // a maximal clique: {u} + C
-    dev::raise_incumbent(a.best, a.lock, a.wit, a.voff, T.g, T.cs, a.err, a.spin,
-                         [&](int, int32_t *base) { write_task_clique(base, a, T, S.mem, stk, 0, -1); });
-    return;
-  }
-  if (m > kTM) {
-    // too many for the compact form: colour on the arena's matrix and make
-    // every branch a task (or search here when the queue is full)
-    Bits<1> B, C;
-    C.w[0] = T.C;
-    color_ise<1, false>(T.A, T.Ws, T.W, P, om - T.cs, B);
-    const int k = bcount(B);
-    if (k == 0) return;
-    Root r{T.u, T.g, T.Pidx, T.p};
-    int t = -1;
-    if (lane == 0) t = reserve_tasks(a, k, a.spin);
-    t = __shfl_sync(FULL, t, 0);
-    if (t < 0) {
-      dfs<1, false>(a, r, T.A, T.Ws, T.W, stk, T.cs, P, B, C, om, (Pool<1> *)nullptr, nodes, don);
-      return;
-    }
-    for (int i = 0; i < k; i++) {
-      const int x = bhighest(B);
-      bclear(B, x);
-      bclear(P, x);
-      emit_task(a, r, T.A, T.Ws, T.W, T.rec, t + i, C, T.cs, P, x);
-    }
-    nodes++;
-    don += (unsigned long long)k;
-    return;
-  }
-  // members by decreasing degree among the candidates (ties: smaller
-  // position): the colouring takes the densest first, the branching the
-  // sparsest
+}
+
+// Search T's clique with its m pruned candidates (at most kTM) on a compact
+// matrix, the members by decreasing degree among the candidates: the
+// colouring takes the densest first, the branching the sparsest.
+__device__ __forceinline__ void search_compact(const SA &a, const TaskCtx &T, int m, TaskSmem &S, uint32_t *stk,
+                                               unsigned long long &nodes, unsigned long long &don) {
+  const int lane = threadIdx.x & 31;
+  uint32_t *key = S.A + 1024;
   int np2 = 32;
   while (np2 < m) np2 <<= 1;
   for (int i = m + lane; i < np2; i += 32) key[i] = 0;
@@ -1661,6 +1755,83 @@ __device__ void run_task(const SA &a, TaskCtx &T, Bits<1> P, TaskSmem &S, uint32
   }
 }
 
+// One task (all lanes): clique T.C, candidates P (a word per lane).  Nodes of
+// more than kTM candidates are searched depth first on the arena's matrix (a
+// set word per lane, rows of one 128-byte line), until a child fits the
+// compact form.
+__device__ void run_task(const SA &a, TaskCtx &T, Bits<1> P, TaskSmem &S, uint32_t *stk, unsigned long long &nodes,
+                         unsigned long long &don) {
+  const int lane = threadIdx.x & 31;
+  T.nlev = 0;
+  for (;;) {
+    // a new node: P with T's clique
+    const int m = prune_candidates(a, T, P, S);
+    if (m > kTM) {
+      uint32_t *q = T.lev + (int64_t)T.nlev * kBigLev;
+      q[lane] = P.w[0];
+      if (lane == 0) q[64] = (uint32_t)-1;  // not coloured yet
+      T.nlev++;
+    } else {
+      if (m > 0) search_compact(a, T, m, S, stk, nodes, don);
+      if (T.nlev == 0) return;
+      Bits<1> C;
+      C.w[0] = T.C;
+      bclear(C, level_word(T.lev + (int64_t)(T.nlev - 1) * kBigLev + 65));
+      T.C = C.w[0];
+      T.cs--;
+    }
+    // the next branch of the deepest level that has one
+    for (;;) {
+      __syncwarp();
+      if (__shfl_sync(FULL, lane == 0 ? *(volatile int32_t *)a.err : 0, 0)) return;
+      uint32_t *q = T.lev + (int64_t)(T.nlev - 1) * kBigLev;
+      Bits<1> LP, LB;
+      LP.w[0] = q[lane];
+      LB.w[0] = q[32 + lane];
+      const int om = read_best(a.best, T.g);
+      if (om > level_word(q + 64)) {
+        color_ise<1, false>(T.A, T.Ws, T.W, LP, om - T.cs, LB);
+        __syncwarp();
+        q[32 + lane] = LB.w[0];
+        if (lane == 0) q[64] = (uint32_t)om;
+        __syncwarp();
+      }
+      int hungry = 0;
+      if (lane == 0) hungry = *(volatile int32_t *)a.task_next > *(volatile int32_t *)a.ntasks;
+      if (__shfl_sync(FULL, hungry, 0)) {
+        const int k = offer_big(a, T, T.nlev - 1);  // the deepest level has chosen none yet
+        don += (unsigned long long)k;
+        LB.w[0] = q[32 + lane];
+      }
+      const int v = bhighest(LB);
+      if (v >= 0) {
+        bclear(LB, v);
+        bclear(LP, v);
+        q[lane] = LP.w[0];
+        q[32 + lane] = LB.w[0];
+        if (lane == 0) q[65] = (uint32_t)v;
+        __syncwarp();
+        P = LP;
+        band_row<1, false>(P, T.A, T.Ws, T.W, v);
+        nodes++;
+        if (lane == 0 && (nodes & 15) == 0) atomicAdd(a.progress, 1);
+        Bits<1> C;
+        C.w[0] = T.C;
+        bset(C, v);
+        T.C = C.w[0];
+        T.cs++;
+        break;
+      }
+      if (--T.nlev == 0) return;
+      Bits<1> C;
+      C.w[0] = T.C;
+      bclear(C, level_word(T.lev + (int64_t)(T.nlev - 1) * kBigLev + 65));
+      T.C = C.w[0];
+      T.cs--;
+    }
+  }
+}
+
 // The task kernel: every warp takes a ticket (a queue position) and waits for
 // the task at that position; tickets beyond the last published task are the
 // waiting warps, which the searching warps see and hand branches to.  The
@@ -1671,7 +1842,8 @@ __global__ void __launch_bounds__(kTW * 32, 4) branch_task_kernel(SA a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   TaskSmem &S = ((TaskSmem *)smem)[wib];
-  uint32_t *stk = a.stack + ((int64_t)blockIdx.x * kTW + wib) * a.stack_stride;
+  uint32_t *lev = a.stack + ((int64_t)blockIdx.x * kTW + wib) * a.stack_stride;
+  uint32_t *stk = lev + a.small_stack;
   unsigned long long nodes = 0, don = 0;
   for (;;) {
     __syncwarp();
@@ -1711,6 +1883,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) branch_task_kernel(SA a) {
     const int slot = got & (a.task_cap - 1);
     const uint32_t *tk = a.tasks + (int64_t)slot * kTaskWords;
     TaskCtx T;
+    T.lev = lev;
     Bits<1> P;
     T.rec = (int)__ldcg(tk + 0);
     T.cs = (int)__ldcg(tk + 1);
@@ -1835,7 +2008,8 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   const int blocks_t = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_t, std::max<int64_t>(1, (g->n + 15) / 16));
   const int64_t stride_b = (int64_t)(std::min(kbound, 1024) + 2) * (64 + 2);
   const int64_t stride_m = (int64_t)(std::min(kbound, kMidCap) + 2) * (64 + 2);
-  const int64_t stride_t = (stride_b + 3) & ~(int64_t)3;  // levels of the compact search are stored as uint4
+  // levels above the compact form, then those of the compact form (uint4)
+  const int64_t stride_t = ((stride_b + 3) & ~(int64_t)3) + (int64_t)kTStk * (std::min(kbound, kTM) + 2);
   uint32_t *stk_b = nullptr, *stk_t = nullptr;
   if (kbound > wmax) {
     MC_TRY(ws_get(g, "se.stk_b", (size_t)blocks_b * kBW * stride_b * 4, &p));
@@ -1931,6 +2105,7 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   MC_TRY(record_event(g, 11));
   if (!no_split) {
     a.stack_stride = stride_t;
+    a.small_stack = (stride_b + 3) & ~(int64_t)3;
     a.stack = stk_t;
     branch_task_kernel<<<blocks_t, kTW * 32, smem_t, g->stream>>>(a);
     g_launches++;
