@@ -1,4 +1,6 @@
-// Core numbers by a bucketed parallel peel (Section 3: K(v) is the largest k
+// Core numbers.  Graphs of up to kLocalMaxNnz entries: kcore_local_kernel
+// (below); larger ones, and small ones of long cascades:
+// a bucketed parallel peel (Section 3: K(v) is the largest k
 // such that v lies in the k-core; the peel removes, level by level, every
 // vertex whose remaining degree is at most k).
 //
@@ -37,6 +39,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cmath>
 #include <mutex>
 
 namespace mc {
@@ -104,7 +107,8 @@ __device__ __forceinline__ void barrier_snap(KcoreCtl *ctl, unsigned nblocks, in
 }
 
 __global__ void degree_init_kernel(int64_t n, const int64_t *__restrict__ rp, int32_t *__restrict__ deg,
-                                   int32_t *__restrict__ core, int32_t *__restrict__ maxdeg) {
+                                   int32_t *__restrict__ core, int32_t *__restrict__ maxdeg, const int32_t *skip) {
+  if (skip && *skip) return;
   int local = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     int d = (int)(rp[v + 1] - rp[v]);
@@ -374,7 +378,9 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_peel_kernel(int64_t n, cons
                                                                  const int32_t *__restrict__ ci, int32_t *deg,
                                                                  int32_t *core, int32_t *order, int32_t *live0,
                                                                  int32_t *live1, long long *wq, KcoreCtl *ctl,
-                                                                 int32_t *err, long long spin_limit, int nocheck) {
+                                                                 int32_t *err, long long spin_limit, int nocheck,
+                                                                 const int32_t *skip) {
+  if (skip && *skip) return;  // the order is made already
   __shared__ int bmin;
   extern __shared__ __align__(16) unsigned char s_pool[];
   BlockPool *bp = (BlockPool *)s_pool;
@@ -537,7 +543,9 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_peel_kernel(int64_t n, cons
 // order unwritten: such entries are skipped and reported, never used as an
 // index.
 __global__ void peel_pos_kernel(int64_t n, const int32_t *__restrict__ order, int32_t *__restrict__ pos,
-                                const int32_t *__restrict__ core, int32_t *__restrict__ maxcore, int32_t *err) {
+                                const int32_t *__restrict__ core, int32_t *__restrict__ maxcore, int32_t *err,
+                                const int32_t *skip) {
+  if (skip && *skip) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     int v = order[i];
     if (v < 0 || (int64_t)v >= n) {
@@ -546,6 +554,617 @@ __global__ void peel_pos_kernel(int64_t n, const int32_t *__restrict__ order, in
     }
     pos[v] = (int32_t)i;
     if (i == n - 1) *maxcore = core[v];  // the peel order is nondecreasing in K
+  }
+}
+
+// ------------------------------------------------------------------------
+// Core numbers by local updates, then the order shell by shell.
+//
+// Up to kLocalMaxNnz entries the level-by-level peel is bound by latency: a
+// level costs a grid barrier and a chain of dependent steps per generation of
+// its cascade, and graphs have hundreds of levels (258 at R-MAT scale 22).
+// This kernel runs all levels at once, in two parts (the H-index operator
+// converges to the core numbers: Lue, Zhou, Zhang and Stanley 2016; as a
+// distributed algorithm: Montresor, De Pellegrini and Miorandi 2013):
+//   values  every vertex holds an upper bound h of its core number, at first
+//           min(degree, sqrt(entries)); a vertex whose support (neighbours
+//           with a bound of at least h) may have fallen below h takes the
+//           largest k with at least k neighbours of bound >= k.  A step
+//           evaluates the listed vertices, and after a barrier the lowered
+//           ones list the neighbours they no longer support.  18 to 45 steps.
+//   order   with K known, the shells are peeled side by side: a vertex leaves
+//           in the first round in which at most K(v) of its neighbours of core
+//           number >= K(v) have not left in an earlier round; positions go by
+//           shell, then by round.  Each vertex has at most K(v) neighbours
+//           after it, so this is a degeneracy order.  13 to 43 rounds.
+// Rows of at most 32 entries are read by a warp four at a time, rows of up to
+// kLocalWarpRow by a warp, longer ones by a block; a new value is found in
+// one pass over the row from a histogram of the values just below h.  A step
+// of few vertices takes 4-12 us (two barriers and six dependent L2 accesses);
+// in all the rows are read about 17 times.  Graphs that need more than
+// kLocalSteps steps or rounds (long paths) are left to the peel.
+//
+// The peel / this kernel: Chung-Lu 20,000 vertices 1.42 / 0.46 ms, R-MAT scale
+// 15 2.1 / 0.58, scale 18 (edge factor 12) 3.5 / 1.5, scale 20 5.7 / 5.0,
+// Chung-Lu 1,000,003 vertices (35 M entries, K(G) = 438) 14.8 / 4.3.  Above
+// kLocalMaxNnz the repeated reads cost more than the peel's barriers.
+// ------------------------------------------------------------------------
+
+constexpr int64_t kLocalMaxNnz = 40000000;
+constexpr int kLocalSteps = 256;
+constexpr int kLocalWarpRow = 2048;
+constexpr int kLocalBins = 256;                 // per warp; a block uses all its warps' bins
+constexpr int kLocalBlockBins = kLocalBins * kWarps;
+constexpr int kStage = 64;                      // listed vertices a warp holds back to append 32 at a time
+
+struct LocalCtl {
+  unsigned bar_count, bar_gen;
+  int pad[30];
+  int n[3][32];   // [counter set][class 0..2]: listed vertices
+  int all[32];    // [0..1] vertices of class 1, 2; [2] vertices placed; [3] largest core number
+};
+
+struct LocalArgs {
+  int64_t n;
+  int cap;  // sqrt(entries)
+  const int64_t *rp;
+  const int32_t *ci;
+  int32_t *h, *old, *stamp;  // h becomes the core numbers; old: the value before the last evaluation, then the support counts
+  int32_t *order, *pos;
+  int32_t *list[2][3], *all[2];  // listed vertices by row class; all vertices of classes 1 and 2
+  int32_t *start, *taken;        // per core number: first position, positions taken
+  LocalCtl *ctl;
+  int32_t *maxdeg, *maxcore, *done;
+  int32_t *err;
+  long long spin;
+};
+
+struct LocalShared {
+  int bins[kLocalBlockBins];
+  int stage[kWarps][kStage];
+  int cnt[3], err;
+  int red[4];
+};
+
+__device__ __forceinline__ int row_class(int64_t len) { return len <= 32 ? 0 : (len <= kLocalWarpRow ? 1 : 2); }
+
+// Short rows a warp takes at a time (four are read at once): as few as keep
+// every warp busy.
+__device__ __forceinline__ int short_batch(int64_t n0, int64_t nwarps) {
+  return (int)min((int64_t)32, max((int64_t)4, (n0 / nwarps + 4) & ~(int64_t)3));
+}
+
+// Grid barrier; afterwards S.cnt holds the three list lengths of `src`.
+// False: the error word is set.
+__device__ bool local_barrier(const LocalArgs &a, LocalShared &S, const int *src) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned g0 = *(volatile unsigned *)&a.ctl->bar_gen;
+    __threadfence();
+    if (atomicAdd(&a.ctl->bar_count, 1u) == gridDim.x - 1) {
+      *(volatile unsigned *)&a.ctl->bar_count = 0;
+      __threadfence();
+      atomicAdd(&a.ctl->bar_gen, 1u);
+    } else {
+      long long it = 0;
+      while (*(volatile unsigned *)&a.ctl->bar_gen == g0) {
+        if (++it > a.spin) {
+          atomicExch(a.err, kDevTimeout);
+          break;
+        }
+        __nanosleep(16);
+      }
+    }
+    __threadfence();
+    if (src) {
+      S.cnt[0] = __ldcg(src);
+      S.cnt[1] = __ldcg(src + 1);
+      S.cnt[2] = __ldcg(src + 2);
+    }
+    S.err = *(volatile int32_t *)a.err;
+  }
+  __syncthreads();
+  return S.err == 0;
+}
+
+// Append the lanes' vertices (has, u) to the lists of buffer b (counter set t)
+// by row class; with PLACE they also take their positions in the order.  All
+// lanes.
+template <bool PLACE>
+__device__ __forceinline__ void local_append(const LocalArgs &a, bool has, int u, int b, int t) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const int c = has ? row_class(a.rp[u + 1] - a.rp[u]) : -1;
+  unsigned m[3];
+#pragma unroll
+  for (int q = 0; q < 3; q++) m[q] = __ballot_sync(0xffffffffu, c == q);
+  int at = 0;
+  if (lane < 3) {  // the three classes' places at once
+    const int k = __popc(lane == 0 ? m[0] : lane == 1 ? m[1] : m[2]);
+    if (k) at = atomicAdd(&a.ctl->n[t][lane], k);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    const int base = __shfl_sync(0xffffffffu, at, q);
+    if (c == q) a.list[b][q][base + __popc(m[q] & lt)] = u;
+  }
+  if (PLACE) {
+    const int k = has ? a.h[u] : -1;
+    const unsigned peers = __match_any_sync(0xffffffffu, k);
+    const int first = __ffs(peers) - 1;
+    int to = 0;
+    if (has && lane == first) to = a.start[k] + atomicAdd(a.taken + k, __popc(peers));
+    to = __shfl_sync(0xffffffffu, to, first);
+    if (has) {
+      const int p = to + __popc(peers & lt);
+      a.order[p] = u;
+      a.pos[u] = p;
+    }
+    const unsigned any = __ballot_sync(0xffffffffu, has);
+    if (lane == 0 && any) atomicAdd(&a.ctl->all[2], __popc(any));
+  }
+}
+
+// Hold the lanes' vertices back until there are 32 to append.
+template <bool PLACE>
+__device__ __forceinline__ void local_stage(const LocalArgs &a, int *buf, int &held, bool has, int u, int b, int t) {
+  const int lane = threadIdx.x & 31;
+  const unsigned m = __ballot_sync(0xffffffffu, has);
+  if (!m) return;
+  if (has) buf[held + __popc(m & ((1u << lane) - 1u))] = u;
+  held += __popc(m);
+  __syncwarp();
+  if (held >= 32) {
+    local_append<PLACE>(a, true, buf[lane], b, t);
+    held -= 32;
+    const int x = lane < held ? buf[32 + lane] : 0;
+    __syncwarp();
+    if (lane < held) buf[lane] = x;
+    __syncwarp();
+  }
+}
+template <bool PLACE>
+__device__ __forceinline__ void local_stage_end(const LocalArgs &a, int *buf, int &held, int b, int t) {
+  const int lane = threadIdx.x & 31;
+  if (held) local_append<PLACE>(a, lane < held, lane < held ? buf[lane] : 0, b, t);
+  held = 0;
+  __syncwarp();
+}
+
+// Smallest i in [0, bins) with c + bin[0] + .. + bin[i] >= h - 1 - i (the new
+// value is h - 1 - i); -1 if none.  A warp, 32 bins
+// at a time: values seldom fall far, so the first group mostly has it.
+__device__ __forceinline__ int window_find(const int *bin, int bins, int h, int c) {
+  const int lane = threadIdx.x & 31;
+  for (int g = 0; g < bins; g += 32) {
+    int incl = bin[g + lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, c + incl >= h - 1 - (g + lane));
+    if (hit) return g + __ffs(hit) - 1;
+    c += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  return -1;
+}
+
+// New value of a row of 33..kLocalWarpRow entries whose vertex holds h.  The
+// values may fall while they are read: a pass counts every entry once (at or
+// above the window, or in it), so a value that is too high counts on a
+// neighbour that falls below it in this step and will list the vertex again.
+__device__ __forceinline__ int eval_warp(const LocalArgs &a, int64_t e0, int len, int h, int *bin) {
+  const int lane = threadIdx.x & 31;
+  int top = h;  // window: values top - 1 .. top - kLocalBins
+  for (;;) {
+    __syncwarp();
+    for (int i = lane; i < kLocalBins; i += 32) bin[i] = 0;
+    __syncwarp();
+    int mine = 0;
+    for (int b = 0; b < len; b += 32 * 8) {
+      int x[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int e = b + 32 * q + lane;
+        x[q] = e < len ? a.ci[e0 + e] : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; q++) x[q] = x[q] >= 0 ? a.h[x[q]] : INT_MIN;
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        if (x[q] >= top) mine++;
+        else if (x[q] >= top - kLocalBins) atomicAdd(&bin[top - 1 - x[q]], 1);
+      }
+    }
+    __syncwarp();
+    const int c = dev::warp_sum(mine);
+    if (top == h && c >= h) return h;
+    const int i = window_find(bin, kLocalBins, top, c);
+    if (i >= 0) return top - 1 - i;
+    top -= kLocalBins;
+  }
+}
+
+// The same by a block (all threads), for longer rows.
+__device__ int eval_block(const LocalArgs &a, LocalShared &S, int64_t e0, int64_t len, int h) {
+  const int lane = threadIdx.x & 31;
+  int top = h;
+  for (;;) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < kLocalBlockBins; i += kThreads) S.bins[i] = 0;
+    if (threadIdx.x == 0) S.red[0] = 0;
+    __syncthreads();
+    int mine = 0;
+    for (int64_t b = 0; b < len; b += kThreads * 8) {
+      int x[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int64_t e = b + kThreads * q + threadIdx.x;
+        x[q] = e < len ? a.ci[e0 + e] : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; q++) x[q] = x[q] >= 0 ? a.h[x[q]] : INT_MIN;
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        if (x[q] >= top) mine++;
+        else if (x[q] >= top - kLocalBlockBins) atomicAdd(&S.bins[top - 1 - x[q]], 1);
+      }
+    }
+    mine = dev::warp_sum(mine);
+    if (lane == 0 && mine) atomicAdd(&S.red[0], mine);
+    __syncthreads();
+    const int c = S.red[0];
+    if (top == h && c >= h) return h;
+    if (threadIdx.x < 32) {
+      const int i = window_find(S.bins, kLocalBlockBins, top, c);
+      if (lane == 0) S.red[1] = i;
+    }
+    __syncthreads();
+    if (S.red[1] >= 0) return top - 1 - S.red[1];
+    top -= kLocalBlockBins;
+  }
+}
+
+// Neighbour u of a vertex whose value fell from `was` to `now`: true when u
+// counted on it and has to be evaluated (once per step: stamp).
+__device__ __forceinline__ bool lost_support(const LocalArgs &a, int u, int now, int was, int step) {
+  if (u < 0) return false;
+  const int x = a.h[u];
+  if (x <= now || x > was) return false;
+  if (__ldcg(a.stamp + u) == step) return false;
+  return atomicExch(a.stamp + u, step) != step;
+}
+
+// Neighbour u of a vertex of core number k that left: true when u leaves in
+// the next round through it.
+__device__ __forceinline__ bool leaves_next(const LocalArgs &a, int u, int k) {
+  if (u < 0 || a.h[u] != k) return false;
+  if (__ldcg(a.old + u) <= k) return false;
+  return atomicSub(a.old + u, 1) == k + 1;
+}
+
+// The rows of the listed vertices, every neighbour tested; those that pass go
+// to the lists of buffer b.  Values (ORDER false): of the vertices whose value
+// fell in this step; order: of all.  When few rows are listed, a row is split
+// over several warps (blocks).
+template <bool ORDER>
+__device__ __forceinline__ void local_walk(const LocalArgs &a, const int32_t *l0, const int32_t *l1, const int32_t *l2,
+                                           int64_t n0, int64_t n1, int64_t n2, int step, int *buf, int b, int t) {
+  const int lane = threadIdx.x & 31;
+  const int64_t gwarp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const int64_t nwarps = (int64_t)gridDim.x * kWarps;
+  int held = 0;
+  auto test = [&](int u, int p, int was) { return ORDER ? leaves_next(a, u, p) : lost_support(a, u, p, was, step); };
+  auto row = [&](int64_t e0, int64_t e1, int at, int stride, int p, int was) {
+    for (int64_t c = e0; c < e1; c += 8 * (int64_t)stride) {
+      int u[8];
+      unsigned hit = 0;
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int64_t e = c + (int64_t)stride * q + at;
+        u[q] = e < e1 ? a.ci[e] : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; q++) hit |= test(u[q], p, was) ? 1u << q : 0u;
+#pragma unroll
+      for (int q = 0; q < 8; q++) local_stage<ORDER>(a, buf, held, (hit >> q) & 1u, u[q], b, t);
+    }
+  };
+  const int s2 = n2 > 0 ? (int)max((int64_t)1, (int64_t)gridDim.x / n2) : 1;
+  for (int64_t i = blockIdx.x; i < n2 * s2; i += gridDim.x) {
+    const int v = l2[i / s2], p = a.h[v], was = ORDER ? 0 : __ldcg(a.old + v);
+    if (ORDER || p < was) row(a.rp[v], a.rp[v + 1], (int)(i % s2) * kThreads + threadIdx.x, s2 * kThreads, p, was);
+  }
+  const int s1 = n1 > 0 ? (int)max((int64_t)1, min((int64_t)16, nwarps / n1)) : 1;
+  for (int64_t i = gwarp; i < n1 * s1; i += nwarps) {
+    const int v = l1[i / s1], p = a.h[v], was = ORDER ? 0 : __ldcg(a.old + v);
+    if (ORDER || p < was) row(a.rp[v], a.rp[v + 1], (int)(i % s1) * 32 + lane, s1 * 32, p, was);
+  }
+  const int per = short_batch(n0, nwarps);
+  for (int64_t c = gwarp * per; c < n0; c += nwarps * per) {
+    const int64_t i = c + lane;
+    int v = -1, len = 0, p = 0, was = 0;
+    int64_t e0 = 0;
+    if (lane < per && i < n0) {
+      v = l0 ? l0[i] : (int)i;
+      e0 = a.rp[v];
+      const int64_t d = a.rp[v + 1] - e0;
+      len = d <= 32 ? (int)d : 0;
+      if (len) {
+        p = a.h[v];
+        if (!ORDER) was = __ldcg(a.old + v);
+      }
+    }
+    unsigned m = __ballot_sync(0xffffffffu, len > 0 && (ORDER || p < was));
+    while (m) {
+      int u[4];
+      bool hit[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int j = m ? __ffs(m) - 1 : -1;
+        m &= m - 1;
+        const int64_t e = __shfl_sync(0xffffffffu, e0, j & 31);
+        const int L = __shfl_sync(0xffffffffu, len, j & 31);
+        const int pj = __shfl_sync(0xffffffffu, p, j & 31), wj = __shfl_sync(0xffffffffu, was, j & 31);
+        u[q] = (j >= 0 && lane < L) ? a.ci[e + lane] : -1;
+        hit[q] = test(u[q], pj, wj);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; q++) local_stage<ORDER>(a, buf, held, hit[q], u[q], b, t);
+    }
+  }
+  local_stage_end<ORDER>(a, buf, held, b, t);
+}
+
+__global__ void __launch_bounds__(kThreads, 1) kcore_local_kernel(LocalArgs a) {
+  __shared__ LocalShared S;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int64_t gwarp = (int64_t)wib * gridDim.x + blockIdx.x;  // neighbouring items go to different blocks
+  const int64_t nwarps = (int64_t)gridDim.x * kWarps;
+  const unsigned lt = (1u << lane) - 1u;
+  const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
+  int *bin = S.bins + wib * kLocalBins, *buf = S.stage[wib];
+  const int64_t n = a.n;
+
+  // ---- bounds, and the vertices of longer rows
+  int top = 0;
+  for (int64_t b = gwarp * 32; b < n; b += nwarps * 32) {
+    const int64_t v = b + lane;
+    int d = 0;
+    if (v < n) {
+      d = (int)(a.rp[v + 1] - a.rp[v]);
+      const int x = min(d, a.cap);
+      a.h[v] = x;
+      a.stamp[v] = 0;
+      top = max(top, d);
+    }
+#pragma unroll
+    for (int q = 1; q < 3; q++) {
+      const bool in = v < n && row_class(d) == q;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (!m) continue;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&a.ctl->all[q - 1], __popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (in) a.all[q - 1][at + __popc(m & lt)] = (int)v;
+    }
+  }
+  top = dev::warp_max(top);
+  if (lane == 0) atomicMax(a.maxdeg, top);
+  if (!local_barrier(a, S, nullptr)) return;
+  const int all1 = __ldcg(&a.ctl->all[0]), all2 = __ldcg(&a.ctl->all[1]);
+
+  // ---- values
+  int64_t n0 = n, n1 = all1, n2 = all2;
+  const int32_t *l0 = nullptr, *l1 = a.all[0], *l2 = a.all[1];
+  int step = 0;
+  for (;;) {
+    const int nxt = (step + 1) & 1;
+    step++;
+    if (leader) a.ctl->n[nxt][0] = a.ctl->n[nxt][1] = a.ctl->n[nxt][2] = 0;
+    // evaluate: long rows first
+    for (int64_t i = blockIdx.x; i < n2; i += gridDim.x) {
+      const int v = l2[i];
+      const int64_t e0 = a.rp[v];
+      const int h = __ldcg(a.h + v);
+      const int x = eval_block(a, S, e0, a.rp[v + 1] - e0, h);
+      if (threadIdx.x == 0) {
+        a.old[v] = h;
+        if (x < h) a.h[v] = x;
+      }
+    }
+    __syncthreads();
+    for (int64_t i = gwarp; i < n1; i += nwarps) {
+      const int v = l1[i];
+      const int64_t e0 = a.rp[v];
+      const int h = __ldcg(a.h + v);
+      const int x = eval_warp(a, e0, (int)(a.rp[v + 1] - e0), h, bin);
+      if (lane == 0) {
+        a.old[v] = h;
+        if (x < h) a.h[v] = x;
+      }
+    }
+    const int per = short_batch(n0, nwarps);
+    for (int64_t b = gwarp * per; b < n0; b += nwarps * per) {
+      const int64_t i = b + lane;
+      int v = -1, len = 0, h = 0;
+      int64_t e0 = 0;
+      if (lane < per && i < n0) {
+        v = l0 ? l0[i] : (int)i;
+        e0 = a.rp[v];
+        const int64_t d = a.rp[v + 1] - e0;
+        len = d <= 32 ? (int)d : 0;
+        if (len) h = __ldcg(a.h + v);
+      }
+      int nh = h;
+      unsigned m = __ballot_sync(0xffffffffu, len > 0);
+      while (m) {
+        int j[4], x[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          j[q] = m ? __ffs(m) - 1 : -1;
+          m &= m - 1;
+          const int64_t e = __shfl_sync(0xffffffffu, e0, j[q] & 31);
+          const int L = __shfl_sync(0xffffffffu, len, j[q] & 31);
+          x[q] = (j[q] >= 0 && lane < L) ? a.ci[e + lane] : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) x[q] = x[q] >= 0 ? a.h[x[q]] : INT_MIN;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          if (j[q] < 0) break;
+          int k = __shfl_sync(0xffffffffu, h, j[q]);
+          while (__popc(__ballot_sync(0xffffffffu, x[q] >= k)) < k) k--;
+          if (lane == j[q]) nh = k;
+        }
+      }
+      if (len) {
+        a.old[v] = h;
+        if (nh < h) a.h[v] = nh;
+      }
+    }
+    if (!local_barrier(a, S, nullptr)) return;
+    // push: the lowered vertices list the neighbours that counted on them
+    local_walk<false>(a, l0, l1, l2, n0, n1, n2, step, buf, nxt, nxt);
+    if (!local_barrier(a, S, a.ctl->n[nxt])) return;
+    n0 = S.cnt[0];
+    n1 = S.cnt[1];
+    n2 = S.cnt[2];
+    l0 = a.list[nxt][0];
+    l1 = a.list[nxt][1];
+    l2 = a.list[nxt][2];
+    if (n0 + n1 + n2 == 0) break;
+    if (step >= kLocalSteps) return;  // done stays 0: left to the peel
+  }
+
+  // ---- order.  Supports within K's own core and the shell sizes (a.taken).
+  if (leader) {
+    for (int t = 0; t < 3; t++) a.ctl->n[t][0] = a.ctl->n[t][1] = a.ctl->n[t][2] = 0;
+  }
+  __syncthreads();
+  for (int64_t i = blockIdx.x; i < all2; i += gridDim.x) {
+    const int v = a.all[1][i];
+    const int k = __ldcg(a.h + v);
+    const int64_t e0 = a.rp[v], e1 = a.rp[v + 1];
+    __syncthreads();
+    if (threadIdx.x == 0) S.red[0] = 0;
+    __syncthreads();
+    int c = 0;
+#pragma unroll 4
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += kThreads) c += a.h[a.ci[e]] >= k ? 1 : 0;
+    c = dev::warp_sum(c);
+    if (lane == 0 && c) atomicAdd(&S.red[0], c);
+    __syncthreads();
+    if (threadIdx.x == 0) a.old[v] = S.red[0];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kLocalBlockBins; i += kThreads) S.bins[i] = 0;
+  __syncthreads();
+  for (int64_t i = gwarp; i < all1; i += nwarps) {
+    const int v = a.all[0][i];
+    const int k = __ldcg(a.h + v);
+    const int64_t e0 = a.rp[v], e1 = a.rp[v + 1];
+    int c = 0;
+#pragma unroll 4
+    for (int64_t e = e0 + lane; e < e1; e += 32) c += a.h[a.ci[e]] >= k ? 1 : 0;
+    c = dev::warp_sum(c);
+    if (lane == 0) a.old[v] = c;
+  }
+  int kmax = 0;
+  for (int64_t b = gwarp * 32; b < n; b += nwarps * 32) {
+    const int64_t v = b + lane;
+    int len = 0, k = 0, cnt = 0;
+    int64_t e0 = 0;
+    if (v < n) {
+      e0 = a.rp[v];
+      const int64_t d = a.rp[v + 1] - e0;
+      len = d <= 32 ? (int)d : -1;
+      k = __ldcg(a.h + v);
+      kmax = max(kmax, k);
+      if (k < kLocalBlockBins) atomicAdd(&S.bins[k], 1);
+      else atomicAdd(a.taken + k, 1);
+    }
+    unsigned m = __ballot_sync(0xffffffffu, len > 0);
+    while (m) {
+      int j[4], x[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        j[q] = m ? __ffs(m) - 1 : -1;
+        m &= m - 1;
+        const int64_t e = __shfl_sync(0xffffffffu, e0, j[q] & 31);
+        const int L = __shfl_sync(0xffffffffu, len, j[q] & 31);
+        x[q] = (j[q] >= 0 && lane < L) ? a.ci[e + lane] : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; q++) x[q] = x[q] >= 0 ? a.h[x[q]] : INT_MIN;
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        if (j[q] < 0) break;
+        const int kk = __shfl_sync(0xffffffffu, k, j[q]);
+        const int c = __popc(__ballot_sync(0xffffffffu, x[q] >= kk));
+        if (lane == j[q]) cnt = c;
+      }
+    }
+    if (len >= 0 && v < n) a.old[v] = cnt;
+  }
+  kmax = dev::warp_max(kmax);
+  if (lane == 0) atomicMax(&a.ctl->all[3], kmax);
+  __syncthreads();
+  for (int i = threadIdx.x; i < kLocalBlockBins; i += kThreads)
+    if (S.bins[i]) atomicAdd(a.taken + i, S.bins[i]);
+  if (!local_barrier(a, S, nullptr)) return;
+  kmax = __ldcg(&a.ctl->all[3]);
+  if (blockIdx.x == 0) {  // first positions; a.taken restarts at 0
+    int carry = 0;
+    for (int b = 0; b <= kmax; b += kThreads) {
+      const int k = b + threadIdx.x;
+      const int x = k <= kmax ? __ldcg(a.taken + k) : 0;
+      int incl = x;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      __syncthreads();
+      if (lane == 31) S.bins[wib] = incl;
+      __syncthreads();
+      int before = 0, tot = 0;
+      for (int w = 0; w < kWarps; w++) {
+        if (w < wib) before += S.bins[w];
+        tot += S.bins[w];
+      }
+      if (k <= kmax) {
+        a.start[k] = carry + before + incl - x;
+        a.taken[k] = 0;
+      }
+      carry += tot;
+    }
+  }
+  if (!local_barrier(a, S, nullptr)) return;
+  for (int64_t b = gwarp * 32; b < n; b += nwarps * 32) {
+    const int64_t v = b + lane;
+    bool has = false;
+    if (v < n) has = __ldcg(a.old + v) <= a.h[v];
+    if (__any_sync(0xffffffffu, has)) local_append<true>(a, has, (int)v, 0, 0);
+  }
+  if (!local_barrier(a, S, a.ctl->n[0])) return;
+  for (int r = 0;; r++) {
+    const int cur = r & 1, nxt = cur ^ 1;
+    n0 = S.cnt[0];
+    n1 = S.cnt[1];
+    n2 = S.cnt[2];
+    if (n0 + n1 + n2 == 0) break;
+    if (r >= kLocalSteps) return;
+    // the counters of round r - 1, free since the last barrier and first used
+    // again after the next one
+    if (leader) a.ctl->n[(r + 2) % 3][0] = a.ctl->n[(r + 2) % 3][1] = a.ctl->n[(r + 2) % 3][2] = 0;
+    local_walk<true>(a, a.list[cur][0], a.list[cur][1], a.list[cur][2], n0, n1, n2, 0, buf, nxt, (r + 1) % 3);
+    if (!local_barrier(a, S, a.ctl->n[(r + 1) % 3])) return;
+  }
+  if (leader) {
+    *a.maxcore = kmax;
+    if (__ldcg(&a.ctl->all[2]) == (int)n) *a.done = 1;
   }
 }
 
@@ -671,6 +1290,59 @@ __global__ void batch_pos_kernel(int64_t n, const int32_t *__restrict__ order, i
 
 }  // namespace
 
+// Enqueues kcore_local_kernel; *out: three device words (done, largest
+// degree, K(G)).
+static int launch_local(mc_graph *g, long long spin_limit, const int32_t **out) {
+  const int64_t n = g->n;
+  LocalArgs a{};
+  a.n = n;
+  a.cap = (int)std::sqrt((double)g->nnz) + 1;
+  a.rp = g->row_ptr;
+  a.ci = g->col_idx;
+  a.h = g->core;
+  a.order = g->order;
+  a.pos = g->pos;
+  a.err = g->err;
+  a.spin = spin_limit;
+  const int64_t c1 = std::min<int64_t>(n, g->nnz / 33 + 1), c2 = std::min<int64_t>(n, g->nnz / kLocalWarpRow + 1);
+  void *p;
+  MC_TRY(ws_get(g, "kl.v", (size_t)(4 * n + 3 * (c1 + c2) + 2 * (a.cap + 2)) * sizeof(int32_t), &p));
+  int32_t *w = (int32_t *)p;
+  auto take = [&](int64_t k) {
+    int32_t *r = w;
+    w += k;
+    return r;
+  };
+  a.old = take(n);
+  a.stamp = take(n);
+  for (int b = 0; b < 2; b++) {
+    a.list[b][0] = take(n);
+    a.list[b][1] = take(c1);
+    a.list[b][2] = take(c2);
+  }
+  a.all[0] = take(c1);
+  a.all[1] = take(c2);
+  a.start = take(a.cap + 2);
+  a.taken = take(a.cap + 2);
+  MC_CUDA_TRY(cudaMemsetAsync(a.taken, 0, (size_t)(a.cap + 2) * sizeof(int32_t), g->stream));
+  MC_TRY(ws_get(g, "kl.ctl", sizeof(LocalCtl) + 64, &p));
+  MC_CUDA_TRY(cudaMemsetAsync(p, 0, sizeof(LocalCtl) + 64, g->stream));
+  a.ctl = (LocalCtl *)p;
+  a.done = (int32_t *)((char *)p + sizeof(LocalCtl));
+  a.maxdeg = a.done + 1;
+  a.maxcore = a.done + 2;
+  *out = a.done;
+  int per_sm = 0;
+  MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kcore_local_kernel, kThreads, 0));
+  if (per_sm < 1) return MC_ERR_CUDA;
+  const int blocks = (int)std::min<int64_t>(g->sm_count, std::max<int64_t>(1, (n + g->nnz / 2 + kThreads - 1) / kThreads));
+  void *args[] = {&a};
+  MC_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)kcore_local_kernel, dim3(blocks), dim3(kThreads), args, 0,
+                                          g->stream));
+  g_launches++;
+  return MC_OK;
+}
+
 int launch_core_numbers(mc_graph *g, long long spin_limit) {
   const int64_t n = g->n;
   if (n == 0) {
@@ -705,6 +1377,25 @@ int launch_core_numbers(mc_graph *g, long long spin_limit) {
     g->cores_valid = true;
     return MC_OK;
   }
+  // mid-size graphs: all levels at once; the peel below is then a fallback,
+  // skipped on the device in a captured solve and not launched otherwise
+  const int32_t *skip = nullptr;
+  if (g->nnz <= kLocalMaxNnz) {
+    MC_TRY(launch_local(g, spin_limit, &skip));
+    if (!g->capturing) {
+      int32_t *host = (int32_t *)g->h_small;
+      MC_CUDA_TRY(cudaMemcpyAsync(host, skip, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, g->stream));
+      MC_CUDA_TRY(cudaStreamSynchronize(g->stream));
+      MC_TRY(check_device_error(g));
+      if (host[0]) {
+        g->max_degree = host[1];
+        g->max_core = host[2];
+        g->cores_valid = true;
+        return MC_OK;
+      }
+      skip = nullptr;
+    }
+  }
   MC_TRY(ws_get(g, "kc.deg", n * sizeof(int32_t), &p));
   int32_t *deg = (int32_t *)p;
   MC_TRY(ws_get(g, "kc.live", 2 * n * sizeof(int32_t) + 64, &p));
@@ -719,7 +1410,7 @@ int launch_core_numbers(mc_graph *g, long long spin_limit) {
   MC_CUDA_TRY(cudaMemsetAsync(wq, 0xff, wcap * sizeof(long long), g->stream));
 
   int ib = (int)std::min<int64_t>((n + 255) / 256, (int64_t)g->sm_count * 8);
-  degree_init_kernel<<<ib, 256, 0, g->stream>>>(n, g->row_ptr, deg, g->core, maxdeg);
+  degree_init_kernel<<<ib, 256, 0, g->stream>>>(n, g->row_ptr, deg, g->core, maxdeg, skip);
   g_launches++;
   MC_CUDA_TRY(cudaGetLastError());
 
@@ -739,11 +1430,11 @@ int launch_core_numbers(mc_graph *g, long long spin_limit) {
   long long sl = spin_limit;
   int nocheck = n <= kNoCheckMaxN ? 1 : 0;
   void *args[] = {&n_arg, (void *)&rp, (void *)&ci, &deg, &core, &order, &live0, &live1, &wq, &ctl, &err, &sl,
-                  &nocheck};
+                  &nocheck, (void *)&skip};
   MC_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)kcore_peel_kernel, dim3(blocks), dim3(kThreads), args, pool,
                                           g->stream));
   g_launches++;
-  peel_pos_kernel<<<ib, 256, 0, g->stream>>>(n, g->order, g->pos, g->core, maxdeg + 1, g->err);
+  peel_pos_kernel<<<ib, 256, 0, g->stream>>>(n, g->order, g->pos, g->core, maxdeg + 1, g->err, skip);
   g_launches++;
   MC_CUDA_TRY(cudaGetLastError());
   if (g->capturing) {  // K(G) and the degree bound are kept from the direct solve before capture
@@ -876,7 +1567,7 @@ extern "C" int mc_core_numbers_noalloc(int64_t n, const int64_t *row_ptr, const 
   if (h_bad) return MC_ERR_INVALID_GRAPH;
 
   const int ib = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
-  degree_init_kernel<<<ib, 256, 0, s>>>(n, row_ptr, deg, core_out, maxdeg);
+  degree_init_kernel<<<ib, 256, 0, s>>>(n, row_ptr, deg, core_out, maxdeg, nullptr);
   g_launches++;
   MC_CUDA_TRY(cudaGetLastError());
   int per_sm = 0;
@@ -891,12 +1582,13 @@ extern "C" int mc_core_numbers_noalloc(int64_t n, const int64_t *row_ptr, const 
   int64_t n_arg = n;
   long long sl = kDefaultSpinLimit;
   int nocheck = n <= kNoCheckMaxN ? 1 : 0;
+  const int32_t *skip = nullptr;
   void *args[] = {&n_arg, (void *)&row_ptr, (void *)&col_idx, &deg, &core_out, &order, &live0, &live1, &wq, &ctl,
-                  &err, &sl, &nocheck};
+                  &err, &sl, &nocheck, (void *)&skip};
   MC_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)kcore_peel_kernel, dim3(blocks), dim3(kThreads), args, pool,
                                           s));
   g_launches++;
-  peel_pos_kernel<<<ib, 256, 0, s>>>(n, order, pos, core_out, maxdeg + 1, err);
+  peel_pos_kernel<<<ib, 256, 0, s>>>(n, order, pos, core_out, maxdeg + 1, err, nullptr);
   g_launches++;
   MC_CUDA_TRY(cudaGetLastError());
   int32_t host[3] = {0, 0, 0};

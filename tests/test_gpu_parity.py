@@ -122,6 +122,36 @@ def test_peel_block_lists_overflow_and_long_cascades(mc):
         h.close()
 
 
+def _hubs(n, hubs, seed):
+    """Hubs 0..len(hubs)-1 of the given degrees over a sparse random graph."""
+    rng = np.random.default_rng(seed)
+    g = gg.erdos_renyi(n, 6.0 / n, seed=seed)
+    src = [np.repeat(np.arange(n), np.diff(g.row_ptr))] + [np.full(d, i) for i, d in enumerate(hubs)]
+    dst = [g.col_idx] + [len(hubs) + rng.choice(n - len(hubs), size=d, replace=False) for d in hubs]
+    return gg.from_edges(n, np.concatenate(src), np.concatenate(dst), "hubs%s" % (tuple(hubs),))
+
+
+@pytest.mark.parametrize("g", [
+    gg.star(33), gg.star(34), gg.star(2049), gg.star(2050), gg.star(20000),
+    gg.complete(33), gg.complete(34), gg.complete(300), gg.complete(2050), gg.path(300), gg.path(3000), gg.cycle(4097),
+    gg.complete_bipartite(300, 5000), gg.complete_bipartite(3000, 3100), gg.disjoint_cliques([2, 33, 34, 257, 600]),
+    _hubs(6000, [31, 32, 33, 2047, 2048, 2049, 5000], 3), _hubs(40000, [39000, 20000, 9000, 300] + [2100] * 40, 4),
+    gg.turan(700, 7), gg.rmat(13, 24, planted=60, seed=9), gg.rmat(18, 24, planted=60, seed=9)], ids=lambda g: g.name)
+def test_core_numbers_by_row_length(mc, g):
+    """Rows on both sides of every class of the core-number kernel (32, 2,048
+    entries), values that fall far in one step (a star's hub, hubs over a
+    sparse graph), one shell for all vertices, and cascades below and above
+    the step limit: core numbers as the oracle's, the order a degeneracy
+    order, whatever the timing of the concurrent updates (several runs)."""
+    ref = oracle.core_numbers(g)
+    for _ in range(6):
+        h = load(mc, g, flags=0)
+        core, kmax = mc.mc_core_numbers(h)
+        assert np.array_equal(core, ref) and kmax == int(ref.max())
+        assert _is_degeneracy_order(g, mc.mc_peel_order(h).copy(), core)
+        h.close()
+
+
 @pytest.mark.parametrize("g", small_graphs() + medium_graphs(), ids=lambda g: g.name)
 def test_max_clique_matches_oracle(mc, g):
     h = load(mc, g)
