@@ -28,7 +28,7 @@
 // Launches: a warm-up launch grows the first 256 start vertices (the seeds
 // and the largest core numbers, whose candidate sets are whole neighbourhoods
 // before any clique is known) with one 512-thread block each, two blocks per
-// SM so that all 256 run in one wave; the main launch runs 32
+// SM so that all 256 run in one wave; the main launch runs 40
 // warps per SM with candidate buffers sharing 2 GiB; start vertices with more
 // candidates than a buffer holds go to a last launch with full-degree
 // buffers.  Every growth, by a block or a warp, yields the same clique.
@@ -44,6 +44,7 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kHT = 256;  // threads per block
+constexpr int kHW = 40;   // warps per SM of the main launch
 constexpr int64_t kSmallCap = 4096;  // least candidate entries per warp in the first launch
 constexpr int64_t kWarm = 256;       // start vertices of the warm-up launch
 
@@ -51,6 +52,7 @@ struct HA {
   int64_t n;
   const int64_t *rp;
   const int32_t *ci, *core, *order, *gid;
+  const unsigned long long *kd;  // core number (high word) and degree per vertex
   unsigned long long *ctr;  // [0] start vertices grown, [1] adjacency tests, [2] row entries read
   const int64_t *voff;
   int32_t *best, *lock, *wit, *err;
@@ -81,6 +83,10 @@ struct HA {
   // positions of the visiting order (after the seeds) grown by an earlier
   // launch of the same solve: position i >= nseeds maps to i - nseeds + skip
   int64_t skip;
+  // the first ntop positions of the visiting order (after the seeds), sorted
+  const int32_t *top;
+  int64_t ntop;
+  int falling;  // the visiting order's core numbers fall (one graph, the library's own order)
 };
 
 struct Key {
@@ -122,53 +128,87 @@ __device__ __forceinline__ bool in_row(const HA &a, int x, int y) {
   return lo < a.rp[x + 1] && a.ci[lo] == y;
 }
 
-// Greedy clique from v (all lanes).  thr: candidate core threshold; stop_at:
-// stop once |C| + |cand| < stop_at (cannot reach it).  by_score: the next
-// member is the candidate of highest learned score instead of Algorithm 1's
-// largest core number.  Writes the clique to cl[0..size) and returns its
-// size, or -1 if the candidates do not fit in cap entries (nothing is grown
-// then).
-__device__ int grow(const HA &a, int v, int thr, int stop_at, int32_t *cand, int32_t *cl, int64_t cap,
-                    bool by_score = false, int g = 0) {
+// Algorithm 1's order as one word pair: core number and degree, from kd.
+__global__ void key_kernel(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ core,
+                           unsigned long long *__restrict__ kd) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    kd[v] = ((unsigned long long)(unsigned)core[v] << 32) | (unsigned)(rp[v + 1] - rp[v]);
+}
+__device__ __forceinline__ Key key_at(const HA &a, int u, bool by_score) {
+  if (by_score) return key_of_scored(a, u);
+  const unsigned long long x = __ldg(a.kd + u);
+  return Key{(int)(x >> 32), (int)(x & 0xffffffffu), u};
+}
+// The warp's best key, three reductions instead of a shuffle tree.
+__device__ __forceinline__ int warp_best_id(const Key &x) {
+  const int k = __reduce_max_sync(FULL, x.k);
+  const int d = __reduce_max_sync(FULL, x.k == k ? x.d : INT_MIN);
+  return __reduce_min_sync(FULL, (x.k == k && x.d == d) ? x.id : INT_MAX);
+}
+
+// A warp's shared memory: a row and a candidate list of at most kNear entries.
+constexpr int kNear = 256;
+struct NearSmem {
+  int32_t row[kNear], cand[kNear];
+};
+struct GrowCount {
+  unsigned long long grows = 0, tests = 0, rows = 0;  // counted by lane 0
+};
+
+// Greedy clique from v (all lanes), whose row is [e0, e1).  thr: candidate
+// core threshold; stop_at: stop once |C| + |cand| < stop_at (cannot reach it).
+// by_score: the next member is the candidate of highest learned score instead
+// of Algorithm 1's largest core number.  Writes the clique to cl[0..size) and
+// returns its size, or -1 if the candidates do not fit in cap entries (nothing
+// is grown then).  Rows and candidate lists of at most kNear entries are held
+// in the warp's shared memory: membership is then a binary search of the
+// staged row, every candidate at once, instead of dependent loads from L2.
+__device__ int grow(const HA &a, int v, int64_t e0, int64_t e1, int thr, int stop_at, int32_t *cand, int32_t *cl,
+                    int64_t cap, NearSmem &N, GrowCount &ct, bool by_score = false, int g = 0) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const Key none{INT_MIN, INT_MIN, INT_MAX};
   int cnt = 0;
   Key bk = none;
-  const int64_t e0 = a.rp[v], e1 = a.rp[v + 1];
+  __syncwarp();
+  if (e1 - e0 <= kNear) {
+    cand = N.cand;
+    cap = kNear;
+  }
   for (int64_t eb = e0; eb < e1; eb += 32) {
     int64_t e = eb + lane;
     int u = -1;
     bool ok = false;
+    Key k = none;
     if (e < e1) {
       u = a.ci[e];
-      ok = a.core[u] >= thr;
+      k = key_at(a, u, by_score);
+      ok = (by_score ? k.d : k.k) >= thr;  // the core number either way
     }
     unsigned m = __ballot_sync(FULL, ok);
     if (ok) {
       const int at = cnt + __popc(m & lt);
       if (at < cap) cand[at] = u;
-      Key k = by_score ? key_of_scored(a, u) : key_of(a, u);
       if (better(k, bk)) bk = k;
     }
     cnt += __popc(m);
   }
   if (cnt > cap) return -1;
-  if (lane == 0) {
-    atomicAdd(a.ctr + 0, 1ull);
-    atomicAdd(a.ctr + 2, (unsigned long long)(e1 - e0));
-  }
-  bk = warp_best(bk);
+  ct.grows++;
+  ct.rows += (unsigned long long)(e1 - e0);
   int size = 1;
   if (lane == 0) cl[0] = v;
   for (;;) {
     // the shared best rises while this clique grows: re-read it every step
     // (mode 0: prune candidates below it and stop when C plus candidates
     // cannot beat it; mode 1: stop when they cannot reach its size)
+    if (cnt == 0 || size + cnt < stop_at) break;
     int cur = 0;
     if (lane == 0)
       cur = a.mode == 0 ? *(volatile int32_t *)(a.best + g)
                         : (int)(*(volatile unsigned long long *)(a.detkey + g) >> 32);
+    const int w = warp_best_id(bk);
+    const int64_t r0 = a.rp[w], r1 = a.rp[w + 1];
     cur = __shfl_sync(FULL, cur, 0);
     if (a.mode == 0) {
       thr = max(thr, cur);
@@ -176,28 +216,38 @@ __device__ int grow(const HA &a, int v, int thr, int stop_at, int32_t *cand, int
     } else {
       stop_at = max(stop_at, cur);
     }
-    if (cnt == 0 || size + cnt < stop_at) break;
-    const int w = bk.id;
+    if (size + cnt < stop_at) break;
     if (lane == 0) cl[size] = w;
     size++;
     __syncwarp();
     // keep the candidates adjacent to w (in-place compaction, reads ahead of
-    // writes).  Few candidates against a long row: binary search per
-    // candidate; otherwise a warp-cooperative merge of the two sorted lists.
+    // writes).  A short row is staged and searched there; otherwise few
+    // candidates against a long row: binary search per candidate; else a
+    // warp-cooperative merge of the two sorted lists.
     int out = 0;
     Key nb = none;
-    const int64_t r0 = a.rp[w], r1 = a.rp[w + 1];
-    const bool merge = (int64_t)cnt * 16 >= (r1 - r0);
-    if (lane == 0) {
-      atomicAdd(a.ctr + 1, (unsigned long long)cnt);
-      if (merge) atomicAdd(a.ctr + 2, (unsigned long long)(r1 - r0));
+    const int rl = (int)min(r1 - r0, (int64_t)kNear + 1);
+    const bool near = rl <= kNear;
+    const bool merge = !near && (int64_t)cnt * 16 >= (r1 - r0);
+    ct.tests += (unsigned long long)cnt;
+    if (near || merge) ct.rows += (unsigned long long)(r1 - r0);
+    int top = 1;
+    if (near) {
+      for (int i = lane; i < rl; i += 32) N.row[i] = a.ci[r0 + i];
+      while (top < rl) top <<= 1;
+      __syncwarp();
     }
     int64_t pos = r0;
     for (int base = 0; base < cnt; base += 32) {
       const int i = base + lane;
       const int x = (i < cnt) ? cand[i] : INT_MAX;
       bool keep = false;
-      if (!merge) {
+      if (near) {
+        int lo = 0;  // entries below x
+        for (int st = top; st > 0; st >>= 1)
+          if (lo + st <= rl && N.row[lo + st - 1] < x) lo += st;
+        keep = i < cnt && x != w && lo < rl && N.row[lo] == x;
+      } else if (!merge) {
         keep = i < cnt && x != w && in_row(a, w, x);
       } else {
         const int last = min(31, cnt - 1 - base);
@@ -227,19 +277,22 @@ __device__ int grow(const HA &a, int v, int thr, int stop_at, int32_t *cand, int
         pos = wp;
         keep = keep && i < cnt && x != w;
       }
-      if (keep && thr > 0) keep = a.core[x] >= thr;
+      Key k = none;
+      if (keep) {
+        k = key_at(a, x, by_score);
+        keep = thr <= 0 || (by_score ? k.d : k.k) >= thr;
+      }
       unsigned m = __ballot_sync(FULL, keep);
       __syncwarp();
       if (keep) {
         cand[out + __popc(m & lt)] = x;
-        Key k = by_score ? key_of_scored(a, x) : key_of(a, x);
         if (better(k, nb)) nb = k;
       }
       out += __popc(m);
       __syncwarp();
     }
     cnt = out;
-    bk = warp_best(nb);
+    bk = nb;
   }
   __syncwarp();
   return size;
@@ -261,9 +314,47 @@ __device__ __forceinline__ bool pick_vertex(const HA &a, int64_t i, int *v) {
   } else {
     const int64_t r = i - a.nseeds + a.skip;
     if (r >= a.n) return false;
-    *v = a.order[a.n - 1 - r];
+    *v = r < a.ntop ? a.top[r] : a.order[a.n - 1 - r];
   }
   return true;
+}
+
+// The front of the visiting order by core number, then degree (Algorithm 1's
+// own tie-break): the hubs of the densest shell, whose candidate sets hold
+// thousands of vertices, are then among the warm-up's whole-block growths
+// wherever the order has put them in their shell.  Without it a hub left to
+// one warp of the main launch held it for 5 ms (R-MAT scale 20, launch 3.6 ms
+// otherwise).  One block, 4,096 keys in shared memory.
+constexpr int kTop = 4096;
+constexpr int32_t kTopDegree = 8192;  // largest degree above which it is sorted (the sort takes 60 us)
+__global__ void __launch_bounds__(1024) top_kernel(int64_t n, int ntop, const int32_t *__restrict__ order,
+                                                   const int32_t *__restrict__ core, const int64_t *__restrict__ rp,
+                                                   int32_t *__restrict__ top) {
+  __shared__ unsigned long long key[kTop];
+  for (int i = threadIdx.x; i < kTop; i += 1024) {
+    unsigned long long k = 0;
+    if (i < ntop) {
+      const int v = order[n - 1 - i];
+      // core numbers are below 2^17 (n below 2^31 entries square), degrees below 2^31
+      k = ((unsigned long long)core[v] << 44) | ((unsigned long long)(rp[v + 1] - rp[v]) << 12) |
+          (unsigned)(kTop - 1 - i);
+    }
+    key[i] = k;
+  }
+  __syncthreads();
+  for (int k = 2; k <= kTop; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int t = threadIdx.x; t < kTop / 2; t += 1024) {
+        const int i = 2 * t - (t & (j - 1)), l = i | j;
+        const unsigned long long x = key[i], y = key[l];
+        if ((x < y) == ((i & k) == 0)) {
+          key[i] = y;
+          key[l] = x;
+        }
+      }
+      __syncthreads();
+    }
+  for (int i = threadIdx.x; i < ntop; i += 1024) top[i] = order[n - 1 - (kTop - 1 - (int)(key[i] & (kTop - 1)))];
 }
 
 constexpr int kWT = 512;       // threads of a warm-up block (two per SM: all 256 starts in one wave)
@@ -472,59 +563,94 @@ __global__ void __launch_bounds__(kWT, 2) heuristic_warm_kernel(HA a) {
   }
 }
 
-__global__ void __launch_bounds__(kHT) heuristic_kernel(HA a) {
+// Bound by the latency of dependent L2 reads (30 of 37 stall cycles per issue
+// before).  One 64-bit word per candidate gives its whole key, the start
+// vertices' words are read 32 at a time, short rows are searched in shared
+// memory, and the work counters stay in registers (as three atomics per growth
+// on one line they were most of the batches' time).  4 M start vertices of a
+// 2,000-graph batch: 13.5 to 3.2 ms; R-MAT scale 22, 35,500 growths: 12.0 to
+// 9.2 ms; Chung-Lu 1.5 M vertices: 1.2 to 0.27 ms.
+// A warp takes `take` positions of the visiting order at a time and reads
+// their vertices' words at once, one lane each: one near the front, where a
+// growth is long and raises the maximum for the others, up to 32 far back,
+// where most are skipped.  In a graph's own order the core numbers fall, so
+// the first vertex below the maximum ends the launch for this warp.
+__global__ void __launch_bounds__(kHT, 5) heuristic_kernel(HA a) {
+  __shared__ NearSmem near[kHT / 32];
+  NearSmem &N = near[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int32_t *cand = a.cand + gw * a.cand_stride;
   int32_t *cl = a.cl + gw * a.cl_stride;
   const int64_t total = a.list ? (int64_t)*a.nlist : a.limit;
-  for (;;) {
-    int64_t i = 0;
-    if (lane == 0) i = *(volatile int32_t *)a.err ? total : a.begin + atomicAdd(a.next, 1);
-    i = __shfl_sync(FULL, (long long)i, 0);
-    if (i >= total) break;
-    int v = 0;
-    if (!pick_vertex(a, i, &v)) continue;
-    const int g = a.gid ? a.gid[v] : 0;
-    const int kv = a.core[v];
-    if (a.mode == 0) {
-      int mx = 0;
-      if (lane == 0) mx = *(volatile int32_t *)(a.best + g);
-      mx = __shfl_sync(FULL, mx, 0);
-      if (kv < mx) continue;
-      const bool seeded = !a.list && i < a.nseeds && a.score;
-      int size = grow(a, v, mx, mx + 1, cand, cl, a.cap, seeded, g);
-      if (size < 0) {
-        if (lane == 0) a.defer[atomicAdd(a.ndefer, 1ull)] = v;
-        continue;
+  const bool falling = a.falling && a.mode == 0 && !a.list;
+  GrowCount ct;
+  int take = 1;
+  bool end = false;
+  while (!end) {
+    int64_t i0 = 0;
+    if (lane == 0) i0 = *(volatile int32_t *)a.err ? total : a.begin + atomicAdd(a.next, take);
+    i0 = __shfl_sync(FULL, (long long)i0, 0);
+    if (i0 >= total) break;
+    const int64_t i = i0 + lane;
+    int v = 0, g = 0, best = 0;
+    int64_t e0 = 0, e1 = 0;
+    bool ok = lane < take && i < total && pick_vertex(a, i, &v);
+    if (ok) {
+      g = a.gid ? a.gid[v] : 0;
+      const int kv = a.core[v];
+      e0 = a.rp[v];
+      e1 = a.rp[v + 1];
+      if (a.mode == 0) {
+        best = *(volatile int32_t *)(a.best + g);
+        ok = kv >= best;
+        if (!ok && falling && i >= a.nseeds) end = true;
+      } else {
+        best = (int)(*(volatile unsigned long long *)(a.detkey + g) >> 32);
+        ok = kv + 1 >= best;
       }
-      if (size > mx) {
-        dev::raise_incumbent(a.best, a.lock, a.wit, a.voff, g, size, a.err, a.spin, [&](int ln, int32_t *base) {
-          for (int t = ln; t < size; t += 32) base[t] = cl[t];
-        });
-      }
-    } else {
-      unsigned long long cur = 0;
-      if (lane == 0) cur = *(volatile unsigned long long *)(a.detkey + g);
-      cur = __shfl_sync(FULL, cur, 0);
-      int bsz = (int)(cur >> 32);
-      if (kv + 1 < bsz) continue;
-      const bool seeded = !a.list && i < a.nseeds && a.score;
-      int size = grow(a, v, 0, bsz, cand, cl, a.cap, seeded, g);
-      if (size < 0) {
-        if (lane == 0) a.defer[atomicAdd(a.ndefer, 1ull)] = v;
-        continue;
-      }
-      // key: size, then seeded growth, then the smaller start vertex
-      unsigned long long key = ((unsigned long long)size << 32) | ((seeded ? 1ull : 0ull) << 31) |
-                               (unsigned)(0x7fffffff - v);
-      if (lane == 0 && key > cur) atomicMax(a.detkey + g, key);
     }
+    end = __any_sync(FULL, end);
+    unsigned todo = __ballot_sync(FULL, ok);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int vs = __shfl_sync(FULL, v, src), gs = __shfl_sync(FULL, g, src), bs = __shfl_sync(FULL, best, src);
+      const int64_t f0 = __shfl_sync(FULL, e0, src), f1 = __shfl_sync(FULL, e1, src);
+      const bool seeded = !a.list && i0 + src < a.nseeds && a.score;
+      const int size = a.mode == 0 ? grow(a, vs, f0, f1, bs, bs + 1, cand, cl, a.cap, N, ct, seeded, gs)
+                                   : grow(a, vs, f0, f1, 0, bs, cand, cl, a.cap, N, ct, seeded, gs);
+      if (size < 0) {
+        if (lane == 0) a.defer[atomicAdd(a.ndefer, 1ull)] = vs;
+        continue;
+      }
+      if (a.mode == 0) {
+        if (size > bs) {
+          dev::raise_incumbent(a.best, a.lock, a.wit, a.voff, gs, size, a.err, a.spin, [&](int ln, int32_t *base) {
+            for (int t = ln; t < size; t += 32) base[t] = cl[t];
+          });
+        }
+      } else if (size >= bs) {
+        // key: size, then seeded growth, then the smaller start vertex
+        const unsigned long long key = ((unsigned long long)size << 32) | ((seeded ? 1ull : 0ull) << 31) |
+                                       (unsigned)(0x7fffffff - vs);
+        if (lane == 0) atomicMax(a.detkey + gs, key);
+      }
+    }
+    if (!a.list) take = (int)min((int64_t)32, 1 + i0 / (4 * nw));
+  }
+  if (lane == 0) {
+    atomicAdd(a.ctr + 0, ct.grows);
+    atomicAdd(a.ctr + 1, ct.tests);
+    atomicAdd(a.ctr + 2, ct.rows);
   }
 }
 
 // mode 1: regrow each graph's winning start vertex and publish it
-__global__ void heuristic_finalize_kernel(HA a, int32_t ngraphs) {
+__global__ void __launch_bounds__(kHT) heuristic_finalize_kernel(HA a, int32_t ngraphs) {
+  __shared__ NearSmem near[kHT / 32];
+  GrowCount ct;
   const int lane = threadIdx.x & 31;
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -536,7 +662,8 @@ __global__ void heuristic_finalize_kernel(HA a, int32_t ngraphs) {
     if (size == 0) continue;
     const bool seeded = ((key >> 31) & 1ull) != 0;
     int v = 0x7fffffff - (int)(key & 0x7fffffffu);
-    int s2 = grow(a, v, 0, 0, cand, cl, a.cap, seeded && a.score, (int)g);
+    int s2 = grow(a, v, a.rp[v], a.rp[v + 1], 0, 0, cand, cl, a.cap, near[threadIdx.x >> 5], ct, seeded && a.score,
+                  (int)g);
     if (s2 != size) {
       if (lane == 0) atomicExch(a.err, kDevCheck);
       continue;
@@ -558,15 +685,15 @@ int launch_heuristic(mc_graph *g, int mode, long long spin_limit, const int32_t 
   if (g->n == 0) return MC_OK;
   if (warm_only && mode != 0) return MC_ERR_ARG;  // the deterministic form needs every start vertex
   void *p;
-  // First launch: 32 warps per SM with candidate buffers that share 2 GiB;
+  // First launch: kHW warps per SM with candidate buffers that share 2 GiB;
   // start vertices with more candidates are deferred to a second launch with
   // buffers for the largest degree (as many warps as 2 GiB allows).
   const int64_t full = (int64_t)g->max_degree + 1;
   const int64_t budget = (int64_t)1 << 29;  // int32 entries (2 GiB)
-  const int64_t cap_s = std::min<int64_t>(full, std::max<int64_t>(kSmallCap, budget / ((int64_t)g->sm_count * 32)));
+  const int64_t cap_s = std::min<int64_t>(full, std::max<int64_t>(kSmallCap, budget / ((int64_t)g->sm_count * kHW)));
   const bool two = full > cap_s;
   const int64_t lstride = (int64_t)g->max_core + 2;
-  int64_t warps_s = std::min<int64_t>((int64_t)g->sm_count * 32, budget / cap_s);
+  int64_t warps_s = std::min<int64_t>((int64_t)g->sm_count * kHW, budget / cap_s);
   warps_s = std::max<int64_t>(32, std::min<int64_t>(warps_s, g->n + nseeds + 32));
   warps_s = (warps_s + 7) / 8 * 8;
   int64_t warps_b = std::max<int64_t>(32, std::min<int64_t>((int64_t)g->sm_count * 16, budget / full));
@@ -623,6 +750,15 @@ int launch_heuristic(mc_graph *g, int mode, long long spin_limit, const int32_t 
   a.max_graph_n = g->max_graph_n;
   a.interleave = (g->count > 1 && g->max_graph_n <= kBatchPeelCap) ? 1 : 0;
   a.skip = skip;
+  a.falling = g->count == 1 && !g->order_given ? 1 : 0;
+  if (a.falling && g->max_degree > kTopDegree) {
+    a.ntop = std::min<int64_t>(g->n, kTop);
+    MC_TRY(ws_get(g, "he.top", kTop * sizeof(int32_t), &p));
+    a.top = (const int32_t *)p;
+    top_kernel<<<1, 1024, 0, g->stream>>>(g->n, (int)a.ntop, g->order, g->core, g->row_ptr, (int32_t *)p);
+    g_launches++;
+    MC_CUDA_TRY(cudaGetLastError());
+  }
   const int64_t order_len = a.interleave ? (int64_t)g->count * g->max_graph_n : g->n;
   const int64_t total = std::max<int64_t>(order_len - skip, 0) + a.nseeds;
   // The warm-up part: the seeds, then the first positions of the visiting
@@ -644,6 +780,14 @@ int launch_heuristic(mc_graph *g, int mode, long long spin_limit, const int32_t 
   }
   a.cand_stride = cap_s;
   const int64_t main_end = warm_only ? warm_end : total;
+  if (warm < main_end || mode == 1) {
+    MC_TRY(ws_get(g, "he.kd", (size_t)g->n * 8, &p));
+    a.kd = (const unsigned long long *)p;
+    key_kernel<<<(int)std::min<int64_t>((g->n + 255) / 256, (int64_t)g->sm_count * 8), 256, 0, g->stream>>>(
+        g->n, g->row_ptr, g->core, (unsigned long long *)p);
+    g_launches++;
+    MC_CUDA_TRY(cudaGetLastError());
+  }
   if (warm < main_end) {
     a.begin = warm;
     a.limit = main_end;

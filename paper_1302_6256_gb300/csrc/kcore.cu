@@ -1345,6 +1345,7 @@ static int launch_local(mc_graph *g, long long spin_limit, const int32_t **out) 
 
 int launch_core_numbers(mc_graph *g, long long spin_limit) {
   const int64_t n = g->n;
+  g->order_given = false;
   if (n == 0) {
     g->max_core = 0;
     g->cores_valid = true;

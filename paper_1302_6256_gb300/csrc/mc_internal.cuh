@@ -157,6 +157,7 @@ struct mc_graph {
   int64_t max_graph_n = 0;  // largest graph of a batch
   // core numbers cache
   bool cores_valid = false;
+  bool order_given = false;  // order holds a caller's degeneracy order, not sorted by core number
   int32_t max_core = 0;
   int32_t heur0 = 0;  // heuristic clique size of graph 0 in the last solve
   unsigned long long *d_heur_ctr = nullptr;  // heuristic work counters of the last solve (device)

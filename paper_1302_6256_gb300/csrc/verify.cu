@@ -181,6 +181,7 @@ int launch_validate(mc_graph *g, int32_t *d_bad) {
 }
 
 int use_order(mc_graph *g, const int32_t *order) {
+  g->order_given = true;
   if (g->n == 0) return MC_OK;
   void *p;
   MC_TRY(ws_get(g, "ord.in", (size_t)g->n * 4 + 64, &p));

@@ -170,6 +170,28 @@ def test_heuristic_deterministic_bit_exact(mc, g):
     assert np.array_equal(H, ref)
 
 
+@pytest.mark.parametrize("g", [
+    gg.complete(255), gg.complete(257), gg.complete(258), gg.star(300), gg.erdos_renyi(700, 0.36, planted=20, seed=31),
+    gg.erdos_renyi(900, 0.4, planted=24, seed=32), _hubs(30000, [9000, 8500, 300, 257, 256, 255, 200, 31], 6),
+    gg.rmat(14, 16, planted=40, seed=33)], ids=lambda g: g.name)
+def test_heuristic_by_row_length(mc, g):
+    """Start vertices, rows and candidate lists on both sides of the length
+    that a warp holds in shared memory (256), and graphs whose front of the
+    visiting order is sorted (a degree above 8,192): the deterministic form
+    bit for bit as the oracle's, the shared-maximum form a clique no larger."""
+    h = load(mc, g, flags=0)
+    ref = oracle.heuristic_clique(g, mode=1)
+    H = mc.mc_heuristic_clique(h, mode=1)
+    assert np.array_equal(H, ref)
+    H0 = mc.mc_heuristic_clique(h, mode=0)
+    assert 1 <= len(H0) and oracle.is_clique(g, H0)
+    # a caller's degeneracy order need not have falling core numbers
+    order = mc.mc_peel_order(h).copy()
+    om, wit, st = mc.mc_max_clique(h, order=order, part_rank=0, part_count=1)
+    assert om >= len(ref) and oracle.is_clique(g, wit)
+    h.close()
+
+
 @pytest.mark.parametrize("g", medium_graphs()[:6], ids=lambda g: g.name)
 def test_heuristic_racy_is_valid(mc, g):
     h = load(mc, g)
