@@ -136,13 +136,15 @@ typedef struct {
   int32_t part_rank, part_count;
   /* Block-worker layout (an autotuner coordinate): 0 = (default) roots of at
    * most 512 candidates searched in a 512-bit-row layout at two blocks per
-   * SM, larger ones in the 1,024-bit-row layout at one block per SM; 1 =
+   * SM, larger ones in an 864-bit-row layout at two (where bit rows serve) or
+   * the 1,024-bit-row layout at one block per SM; 1 =
    * every block-class root in the 1,024-bit-row layout. */
   int32_t layout;
   /* 1 = neighbourhood builds look up P's members in a hash table only; 0 =
-   * (default) in a shared-memory bitmap of the root's later ranks when those
-   * fit (196,608 ranks), in the hash table otherwise (an autotuner
-   * coordinate). */
+   * (default) for one graph, block workers gather the matrix from bit rows of
+   * the last 40,960 ranks; other roots use a shared-memory bitmap of the
+   * root's later ranks when those fit (196,608 ranks), the hash table
+   * otherwise (an autotuner coordinate). */
   int32_t no_bitmap;
   /* Work-triggered re-pruning (the paper's periodic explicit rebuild,
    * Algorithm 2 line 9, triggered by progress instead of a clock): with
@@ -169,8 +171,9 @@ typedef struct {
   int64_t roots_branched;      /* roots that reached Branch */
   int64_t nodes;               /* Branch nodes expanded */
   int64_t donations;           /* subproblems handed to other warps (of a block, or by a task to the queue) */
-  int64_t neighbourhood_entries; /* later-neighbour row entries read to build the
-                                    roots' adjacency matrices (Fact 3's work) */
+  int64_t neighbourhood_entries; /* lookups made to build the roots' adjacency matrices
+                                    (Fact 3's work): later-neighbour row entries read, or
+                                    member pairs where bit rows serve */
   int64_t neighbourhood_entries_block; /* ... of which read by block workers */
   int64_t tasks;               /* subproblems published to the task queue */
   int64_t heuristic_grows;     /* start vertices grown by Algorithm 1 */

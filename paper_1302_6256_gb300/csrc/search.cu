@@ -7,10 +7,10 @@
 // and the search looks for a clique larger than omega containing u:
 //   1. |P| < omega                    -> return (degree bound, Fact 2 (3))
 //   2. bitset adjacency of G[P]       (the small-graph adjacency matrix of
-//      Section 4.4): each member's later-neighbour row is probed against a
-//      hash table of P, which sets the lower triangle (a later neighbour has
-//      a smaller index in P); warp-ballot transposes of 32 x 32 tiles fill
-//      the upper triangle
+//      Section 4.4): gathered from bit rows of the top ranks, or each member's
+//      later-neighbour row probed against a bitmap or hash table of P; that
+//      sets the lower triangle (a later neighbour has a smaller index in P),
+//      and transposes of 32 x 32 tiles fill the upper triangle
 //   3. (omega-1)-core of G[P]: exactly the vertices with neighbourhood core
 //      number K_N >= |H| when u is counted (lines 15-18 of InitialBranch;
 //      the tight form of the test); fewer than omega left -> return
@@ -26,8 +26,9 @@
 // Workers, split by the out-degree of the root (an upper bound on |P|):
 //   warp class   |N+(u)| <= 128: one warp per root, matrix in shared memory;
 //   block class  |N+(u)| <= 1024: one block per root, matrix in shared
-//                memory; a 512-candidate layout at two blocks per SM first,
-//                then a 1,024-candidate launch for the roots it deferred; the
+//                memory; a 512-candidate and an 864-candidate layout at two
+//                blocks per SM first (the second for dense rows only), then a
+//                1,024-candidate launch for the roots they deferred; the
 //                block's 16 warps share the root's search tree through a
 //                shared-memory pool (a busy warp hands the shallowest untried
 //                branch to an idle one);
@@ -60,6 +61,8 @@ struct SA {
   const int32_t *roots;
   const int64_t *nroots;    // device: number of roots in this class
   const int64_t *np_count;  // device: vertices of the pruned graph
+  const uint32_t *dense;    // bit rows of the top ranks (null: none), see dense_rows_kernel
+  int32_t dense_cap, dense_stride;  // ranks covered, words per row
   int32_t use_bitmap;       // look members up in a bitmap of the later ranks when they fit
   int32_t *best, *lock, *wit;
   const int64_t *voff;
@@ -87,6 +90,8 @@ struct SA {
   int32_t *task_next;            // tickets taken by the task kernel's warps (runs ahead of ntasks by the waiting ones)
   int32_t *pending;              // tasks published and not yet finished
   int32_t *progress;             // heartbeat: bumped every 256 Branch nodes
+  uint32_t *sort;                // per-block room for a sorted matrix (roots searched in place; or null)
+  int64_t sort_stride;
   int32_t *overflow;             // roots too large for this launch's layout (or null)
   int64_t *noverflow;
   int32_t offer_nodes;           // Branch nodes of a task between two looks for waiting warps
@@ -106,7 +111,11 @@ constexpr size_t kCtrBytes = 96 * 8;       // counters and the queue's control w
 // 3.5 / 4.4 / 5.7 ms, 64 nodes 8 / 10 / 12 ms: rare offers leave warps idle,
 // frequent ones make tasks too small for their set-up (10-30 us).
 constexpr int kOfferNodes = 8;
-constexpr int kMidCap = 512;               // candidates of the two-blocks-per-SM block layout
+constexpr int kMidCap = 512;               // candidates of the two-blocks-per-SM block layout ...
+// ... and of the one that serves dense rows only, also two blocks per SM: 102
+// KB without the lookup structures.  At one block per SM (the 1,024 layout) its
+// 7,850 roots at R-MAT scale 22 took 9.0 ms, now 5.5.
+constexpr int kWideCap = 864;
 
 template <int WPL>
 struct Bits {
@@ -134,29 +143,21 @@ __device__ __forceinline__ int bcount(const Bits<WPL> &b) {
 }
 template <int WPL>
 __device__ __forceinline__ int blowest(const Bits<WPL> &b) {
+  // one reduction: shorter than ballot, shuffle and two find-first-sets
+  int v = INT_MAX;
 #pragma unroll
-  for (int k = 0; k < WPL; k++) {
-    unsigned m = __ballot_sync(FULL, b.w[k] != 0);
-    if (m) {
-      int l = __ffs(m) - 1;
-      uint32_t x = __shfl_sync(FULL, b.w[k], l);
-      return ((k * 32 + l) << 5) + __ffs(x) - 1;
-    }
-  }
-  return -1;
+  for (int k = WPL - 1; k >= 0; k--)
+    if (b.w[k]) v = ((k * 32 + (int)(threadIdx.x & 31)) << 5) + __ffs(b.w[k]) - 1;
+  v = __reduce_min_sync(FULL, v);
+  return v == INT_MAX ? -1 : v;
 }
 template <int WPL>
 __device__ __forceinline__ int bhighest(const Bits<WPL> &b) {
+  int v = -1;
 #pragma unroll
-  for (int k = WPL - 1; k >= 0; k--) {
-    unsigned m = __ballot_sync(FULL, b.w[k] != 0);
-    if (m) {
-      int l = 31 - __clz(m);
-      uint32_t x = __shfl_sync(FULL, b.w[k], l);
-      return ((k * 32 + l) << 5) + 31 - __clz(x);
-    }
-  }
-  return -1;
+  for (int k = 0; k < WPL; k++)
+    if (b.w[k]) v = ((k * 32 + (int)(threadIdx.x & 31)) << 5) + 31 - __clz(b.w[k]);
+  return __reduce_max_sync(FULL, v);
 }
 template <int WPL>
 __device__ __forceinline__ void bclear(Bits<WPL> &b, int v) {
@@ -404,29 +405,6 @@ __device__ int reserve_record(const SA &a, const Root &r, int Ws, long long *off
   return rec;
 }
 
-// Copy a root's matrix and P list to its arena room and write its record,
-// over the 32 lanes of a warp.
-__device__ void write_record(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, int rec, long long off) {
-  const int lane = threadIdx.x & 31;
-  uint32_t *dm = a.arena + off;
-  for (int i = lane; i < r.p * Ws; i += 32) dm[i] = A[i];
-  int *dp = (int *)(dm + (int64_t)r.p * Ws);
-  for (int i = lane; i < r.p; i += 32) dp[i] = r.Pidx[i];
-  if (lane == 0) {
-    RootRec rr;
-    rr.u = r.u;
-    rr.g = r.g;
-    rr.p = r.p;
-    rr.W = W;
-    rr.Ws = Ws;
-    rr.pad = 0;
-    rr.off = off;
-    a.recs[rec] = rr;
-  }
-  __syncwarp();
-  __threadfence();
-}
-
 // Write the task at queue position t (clique size cs counting u, 0 =
 // empty; clique bits C; candidates P) and mark its slot written.  Position
 // t uses slot t mod task_cap in lap t / task_cap: the slot's word counts
@@ -484,28 +462,6 @@ __device__ void emit_task(const SA &a, const Root &r, const uint32_t *A, int Ws,
   Bits<1> Cx = Cl;
   bset(Cx, x);
   write_task(a, t, rec, cs, Cx, TP);
-}
-
-// The whole search of a root as one task (clique {u}, candidates P): its
-// matrix and P list go to the arena once.  False, publishing nothing, without
-// room for the record or in the queue.  Warp-collective.
-__device__ bool publish_root(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, const Bits<1> &P) {
-  const int lane = threadIdx.x & 31;
-  int rec = -1, t = -1;
-  long long off = 0;
-  if (lane == 0) {
-    rec = reserve_record(a, r, Ws, &off);
-    if (rec >= 0) t = reserve_tasks(a, 1, a.spin);
-  }
-  rec = __shfl_sync(FULL, rec, 0);
-  off = __shfl_sync(FULL, off, 0);
-  t = __shfl_sync(FULL, t, 0);
-  if (t < 0) return false;
-  write_record(a, r, A, Ws, W, rec, off);
-  Bits<1> C;
-  bzero(C);
-  write_task(a, t, rec, 1, C, P);
-  return true;
 }
 
 // Depth-first Branch from one level (csize0 = |C| including the root u).
@@ -810,6 +766,161 @@ __device__ void symmetrize(uint32_t *A, int Ws, int W, int p, int wid, int nw) {
   }
 }
 
+// Arena room, record and queue position (*t_out, -1: none) of a root of m
+// candidates; the record, or -1.  One thread.
+__device__ int open_record(const SA &a, const Root &r, int m, int *t_out) {
+  const Root rm{r.u, r.g, r.Pidx, m};
+  const int Wsm = ((m + 31) >> 5) | 1;
+  long long off = 0;
+  *t_out = -1;
+  const int rec = reserve_record(a, rm, Wsm, &off);
+  if (rec < 0) return -1;
+  *t_out = reserve_tasks(a, 1, a.spin);
+  RootRec rr;
+  rr.u = r.u;
+  rr.g = r.g;
+  rr.p = m;
+  rr.W = (m + 31) >> 5;
+  rr.Ws = Wsm;
+  rr.pad = 0;
+  rr.off = off;
+  a.recs[rec] = rr;
+  return rec;
+}
+__device__ __forceinline__ uint32_t first_bits(int m) {  // this lane's word of the set {0 .. m-1}
+  const int lane = threadIdx.x & 31;
+  return m >= 32 * (lane + 1) ? FULL : (m > 32 * lane ? (1u << (m - 32 * lane)) - 1u : 0u);
+}
+// Row i of a matrix in another order (word w: a ballot over new positions 32w
+// .. 32w+31); keys hold the complement of the old index in their low half.
+__device__ __forceinline__ uint32_t permuted_row(const uint32_t *A, int Ws, const uint32_t *keys, int m, int i) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t *row = A + (int64_t)(0xffff - (int)(keys[i] & 0xffffu)) * Ws;
+  uint32_t mine = 0;
+  for (int w = 0; w < (m + 31) >> 5; w++) {
+    const int j = 32 * w + lane;
+    const int at = j < m ? 0xffff - (int)(keys[j] & 0xffffu) : 0;
+    const unsigned word = __ballot_sync(FULL, j < m && ((row[at >> 5] >> (at & 31)) & 1u));
+    if (lane == w) mine = word;
+  }
+  return mine;
+}
+
+// A warp's root (at most kWarpCap candidates, those left by the core test in
+// al) as a task: its candidates in minimum-width order (see width_keys), its
+// matrix and P list copied to the arena once.  keys: kWarpCap words.  False,
+// publishing nothing, without room for the record or in the queue.
+__device__ bool publish_warp(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, const uint32_t *al,
+                             uint32_t *keys) {
+  const int lane = threadIdx.x & 31;
+  int deg[4], m = 0;
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    const int i = 32 * q + lane;
+    deg[q] = INT_MAX;
+    keys[i] = 0;
+    if (q >= W) continue;
+    m += __popc(al[q]);
+    if (i < r.p && ((al[q] >> lane) & 1u)) {
+      deg[q] = 0;
+      for (int w = 0; w < W; w++) deg[q] += __popc(A[i * Ws + w] & al[w]);
+    }
+  }
+  int left = m;
+  for (uint32_t step = 1; left > 0; step++) {
+    const int lo = __reduce_min_sync(FULL, min(min(deg[0], deg[1]), min(deg[2], deg[3])));
+    unsigned out[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      out[q] = __ballot_sync(FULL, deg[q] == lo);
+      if (deg[q] == lo) {
+        keys[32 * q + lane] = (step << 16) | (uint32_t)(0xffff - (32 * q + lane));
+        deg[q] = INT_MAX;
+      }
+      left -= __popc(out[q]);
+    }
+#pragma unroll
+    for (int w = 0; w < 4; w++)
+      if (out[w]) {
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if (deg[q] != INT_MAX) deg[q] -= __popc(A[(32 * q + lane) * Ws + w] & out[w]);
+      }
+  }
+  __syncwarp();
+  int rec = -1, t = -1;
+  if (lane == 0) rec = open_record(a, r, m, &t);
+  rec = __shfl_sync(FULL, rec, 0);
+  t = __shfl_sync(FULL, t, 0);
+  if (t < 0) return false;
+  bitonic_desc<false>((int *)keys, kWarpCap, lane, 32);
+  uint32_t *dm = a.arena + __shfl_sync(FULL, lane == 0 ? a.recs[rec].off : 0ll, 0);
+  const int Wsm = ((m + 31) >> 5) | 1;
+  for (int i = 0; i < m; i++) {
+    const uint32_t x = permuted_row(A, Ws, keys, m, i);
+    if (lane < Wsm) dm[i * Wsm + lane] = x;
+  }
+  int *dp = (int *)(dm + m * Wsm);
+  for (int i = lane; i < m; i += 32) dp[i] = r.Pidx[0xffff - (int)(keys[i] & 0xffffu)];
+  __syncwarp();
+  __threadfence();
+  Bits<1> C, P;
+  bzero(C);
+  P.w[0] = first_bits(m);
+  write_task(a, t, rec, 1, C, P);
+  return true;
+}
+
+// ------------------------------------------------------------- dense rows ---
+//
+// The adjacency of the top ranks as a bit matrix: row r holds r's later
+// neighbours, for the last dense_cap ranks of the pruned graph (all of it at
+// R-MAT scale 22: 35,500 vertices, 2.9% of the pairs, 79 MB used of the upper
+// triangle, in L2).  A root's matrix is then gathered from it, 32 members per
+// load and ballot, where the row lists took a lookup per entry (9.5 G per
+// solve) and an atomic per member.  It is bound by L2: nearly every sector of
+// a row's later part holds a member, 30-40 GB per solve.  The builder takes
+// 0.1 ms, the block kernels 11.7 ms at scale 22 (24.4 before), 5.4 at scale 21
+// (8.5), 2.6 at scale 20 (3.5).  Words before a row's own are not written and
+// not read.  The cap bounds the room to 210 MB; roots below the covered ranks
+// use the row lists.
+constexpr int64_t kDenseCap = 40960;
+constexpr int kDW = 8;  // warps per block of the builder
+
+__host__ __device__ __forceinline__ int64_t dense_base(int64_t np, int64_t cap) { return np > cap ? np - cap : 0; }
+
+__global__ void __launch_bounds__(kDW * 32) dense_rows_kernel(const int64_t *__restrict__ d_np,
+                                                              const int64_t *__restrict__ orow,
+                                                              const int32_t *__restrict__ ocol, int32_t cap,
+                                                              int32_t stride, uint32_t *__restrict__ dense) {
+  extern __shared__ uint32_t drow[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  uint32_t *row = drow + (size_t)wib * stride;
+  const int64_t np = *d_np, base = dense_base(np, cap);
+  const int words = (int)((np - base + 31) >> 5);
+  for (int64_t r = base + (int64_t)blockIdx.x * kDW + wib; r < np; r += (int64_t)gridDim.x * kDW) {
+    const int w0 = (int)((r - base) >> 5);
+    for (int w = w0 + lane; w < words; w += 32) row[w] = 0;
+    __syncwarp();
+    const int64_t e0 = orow[r];
+    const int4 *q = reinterpret_cast<const int4 *>(ocol + e0);
+    const int nq = (int)((orow[r + 1] - e0) >> 2);
+    for (int i = lane; i < nq; i += 32) {
+      const int4 y = __ldg(q + i);
+      const int ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int c = (int)(ys[j] - base);
+        if (ys[j] >= 0) atomicOr(&row[c >> 5], 1u << (c & 31));
+      }
+    }
+    __syncwarp();
+    uint32_t *out = dense + (r - base) * stride;
+    for (int w = w0 + lane; w < words; w += 32) out[w] = row[w];
+    __syncwarp();
+  }
+}
+
 // ------------------------------------------------------------ warp class ---
 
 struct WarpSmem {
@@ -903,7 +1014,7 @@ __global__ void __launch_bounds__(kSW * 32) search_warp_kernel(SA a) {
     Bits<1> C;
     bzero(C);
     Root r{u, g, S.Pidx, p};
-    if (a.tasks && publish_root(a, r, S.A, Ws, W, al)) continue;
+    if (a.tasks && publish_warp(a, r, S.A, Ws, W, S.al, (uint32_t *)S.hk)) continue;
     dfs<1, true>(a, r, S.A, Ws, W, stk, 1, al, B, C, om, (Pool<1> *)nullptr, nodes, don);
   }
   if (lane == 0) {
@@ -915,91 +1026,216 @@ __global__ void __launch_bounds__(kSW * 32) search_warp_kernel(SA a) {
 
 // ----------------------------------------------------------- block class ---
 
-template <int WPL, bool SM, int PC = 1024 * WPL>
+// DENSE: roots of the dense rows only, so neither the hash table (its place
+// holds sort keys) nor the bitmap is needed.
+template <int WPL, bool SM, int PC = 1024 * WPL, bool DENSE = false>
 struct BlockLayout {
   static constexpr int PCAP = PC;
-  static constexpr int HCAP = 4 * PCAP;  // load factor 1/4: short probes
+  static constexpr int HCAP = DENSE ? 1024 : 4 * PCAP;  // load factor 1/4: short probes
   static constexpr int WMAX = 32 * WPL;                 // alive / removal words (one per lane)
   static constexpr int WSMAX = ((PCAP + 31) / 32) | 1;  // largest matrix row stride, W | 1
   // bytes: Pidx, hk, hv, alive/rm words, pool, control, matrix
   static constexpr size_t off_P = 0;
   static constexpr size_t off_hk = off_P + PCAP * 4;
   static constexpr size_t off_hv = off_hk + HCAP * 4;
-  static constexpr size_t off_al = off_hv + HCAP * 2;
+  static constexpr size_t off_al = off_hv + (DENSE ? 0 : HCAP * 2);
   static constexpr size_t off_rm = off_al + WMAX * 4;
   static constexpr size_t off_pool = off_rm + WMAX * 4;
   static constexpr size_t off_ctl = off_pool + ((sizeof(Pool<WPL>) + 15) / 16) * 16;
   static constexpr size_t off_bm = off_ctl + 64;                        // kBitmapWords words
-  static constexpr size_t off_pre = off_bm + (size_t)kBitmapWords * 4;  // kBitmapWords uint16
-  static constexpr size_t off_A = off_pre + (size_t)kBitmapWords * 2;
+  static constexpr size_t off_pre = off_bm + (DENSE ? 0 : (size_t)kBitmapWords * 4);  // kBitmapWords uint16
+  static constexpr size_t off_A = off_pre + (DENSE ? 0 : (size_t)kBitmapWords * 2);
   static constexpr size_t bytes = off_A + (SM ? (size_t)PCAP * WSMAX * 4 : 0);
 };
 
-// A block's root as a task: the candidates left by the core test, sorted by
-// decreasing degree among them, with their adjacency in that order (the
-// colouring of the task's upper levels takes the densest first too).  All
-// threads; keys: room for the next power of two above p, ctl: two words.
-// False, publishing nothing, without room.
-__device__ bool publish_sorted(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, const uint32_t *al,
-                               uint32_t *keys, int *ctl) {
+// P = {w in N+(u) : K(w) >= om} from u's dense row, in decreasing rank, into
+// Pidx; returns its size, or more than cap (nothing usable written) when u has
+// more later neighbours than that.  scan: kBW + 1 words, cnt: one word.  All
+// threads.
+__device__ int dense_P(const SA &a, int u, int om, int64_t base, int64_t np, int *Pidx, int cap, uint32_t *scan) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const uint32_t *row = a.dense + (u - base) * a.dense_stride;
+  const int w0 = (int)((u - base) >> 5), words = (int)((np - base + 31) >> 5);
+  const int last = words - 1;
+  // words from the last one down, kBT at a time
+  int total = 0;
+  for (int k0 = 0; k0 <= last - w0; k0 += kBT) {
+    const int w = last - (k0 + tid);
+    uint32_t x = 0;
+    if (w >= w0) {
+      x = __ldg(row + w);
+      if (w == w0) x &= ~((2u << ((u - (int)base) & 31)) - 1u);  // later ranks only
+    }
+    const int c = __popc(x);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += y;
+    }
+    __syncthreads();
+    if (lane == 31) scan[wid] = (uint32_t)incl;
+    __syncthreads();
+    int at = total + incl - c, all = 0;
+    for (int i = 0; i < kBW; i++) {
+      if (i < wid) at += (int)scan[i];
+      all += (int)scan[i];
+    }
+    for (; x; at++) {
+      const int b = 31 - __clz(x);
+      x ^= 1u << b;
+      if (at < cap) Pidx[at] = (int)base + 32 * w + b;
+    }
+    total += all;
+  }
+  __syncthreads();
+  if (total > cap) return total;
+  // drop the members whose core number omega has passed (none, unless omega
+  // rose since the pruning)
+  bool low = false;
+  for (int i = tid; i < total; i += kBT) low |= __ldg(a.ocore + Pidx[i]) < om;
+  if (!__syncthreads_or(low)) return total;
+  int kept = 0;
+  for (int i0 = 0; i0 < total; i0 += kBT) {
+    const int i = i0 + tid, y = i < total ? Pidx[i] : 0;
+    const bool keep = i < total && __ldg(a.ocore + y) >= om;
+    const unsigned m = __ballot_sync(FULL, keep);
+    __syncthreads();
+    if (lane == 0) scan[wid] = (uint32_t)__popc(m);
+    __syncthreads();
+    int at = kept + __popc(m & ((1u << lane) - 1u)), all = 0;
+    for (int k = 0; k < kBW; k++) {
+      if (k < wid) at += (int)scan[k];
+      all += (int)scan[k];
+    }
+    if (keep) Pidx[at] = y;
+    kept += all;
+  }
+  __syncthreads();
+  return kept;
+}
+
+// Lower triangle of G[P] from the dense rows: word w of row i is a ballot over
+// members 32w .. 32w+31 (later ranks than member i for indices below i).  Rows
+// go to warps as they free up, the longest first; eight words in flight.
+__device__ __forceinline__ void dense_build(const SA &a, const int *Pidx, int p, int64_t base, uint32_t *A, int Ws,
+                                            int W, int *dyn, unsigned long long *count) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long words = 0;
+  for (;;) {
+    int i = 0;
+    if (lane == 0) i = p - 1 - atomicAdd(dyn, 1);
+    i = __shfl_sync(FULL, i, 0);
+    if (i < 0) break;
+    const uint32_t *row = a.dense + (int64_t)(Pidx[i] - base) * a.dense_stride;
+    const int nw = (i + 31) >> 5;  // words with an index below i
+    uint32_t mine = 0;
+    for (int w0 = 0; w0 < nw; w0 += 8) {
+      uint32_t x[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int j = 32 * (w0 + q) + lane;
+        const int c = j < i ? Pidx[j] - (int)base : -1;
+        x[q] = c >= 0 ? __ldg(row + (c >> 5)) >> (c & 31) : 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const unsigned m = __ballot_sync(FULL, x[q] & 1u);
+        if (lane == w0 + q) mine = m;
+      }
+    }
+    if (lane < W) A[i * Ws + lane] = mine;
+    words += (unsigned long long)i;
+  }
+  if (lane == 0 && words) atomicAdd(count, words);
+}
+
+// The candidates left by the core test (bits al) in minimum-width order: those
+// of smallest degree among the remaining ones leave step by step (all of them
+// at once), and later ones come first (ties: smaller index).  keys[0..m) =
+// step and complement of the index, sorted; returns m.  keys: room for the
+// next power of two above p; gone: one word per 32 candidates.  All threads.
+__device__ int width_keys(const uint32_t *A, int p, int Ws, int W, const uint32_t *al, uint32_t *keys, uint32_t *gone) {
+  __shared__ int s_min;
+  const int tid = threadIdx.x, lane = tid & 31;
   int np2 = 32;
-  while (np2 < r.p) np2 <<= 1;
+  while (np2 < p) np2 <<= 1;
   int m = 0;
   for (int w = 0; w < W; w++) m += __popc(al[w]);
-  for (int i = tid; i < np2; i += kBT) {
-    uint32_t key = 0;
-    if (i < r.p && ((al[i >> 5] >> (i & 31)) & 1u)) {
-      int deg = 0;
-      for (int w = 0; w < W; w++) deg += __popc(A[i * Ws + w] & al[w]);
-      key = ((uint32_t)(deg + 1) << 16) | (uint32_t)(0xffff - i);
+  int deg[2];  // candidates tid and tid + kBT; INT_MAX: not (or no longer) there
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    const int i = tid + q * kBT;
+    deg[q] = INT_MAX;
+    if (i < p && ((al[i >> 5] >> (i & 31)) & 1u)) {
+      deg[q] = 0;
+      for (int w = 0; w < W; w++) deg[q] += __popc(A[i * Ws + w] & al[w]);
     }
-    keys[i] = key;
+    if (i < np2) keys[i] = 0;
   }
-  const int Wm = (m + 31) >> 5, Wsm = Wm | 1;
-  if (tid == 0) {
-    const Root rm{r.u, r.g, r.Pidx, m};
-    long long off = 0;
-    int t = -1;
-    const int rec = reserve_record(a, rm, Wsm, &off);
-    if (rec >= 0) t = reserve_tasks(a, 1, a.spin);
-    ctl[0] = t;
-    ctl[1] = rec;
-    if (t >= 0) {
-      RootRec rr;
-      rr.u = r.u;
-      rr.g = r.g;
-      rr.p = m;
-      rr.W = Wm;
-      rr.Ws = Wsm;
-      rr.pad = 0;
-      rr.off = off;
-      a.recs[rec] = rr;
+  int left = m;
+  for (uint32_t step = 1; left > 0; step++) {
+    __syncthreads();
+    if (tid == 0) s_min = INT_MAX;
+    __syncthreads();
+    const int mine = __reduce_min_sync(FULL, min(deg[0], deg[1]));
+    if (lane == 0 && mine != INT_MAX) atomicMin(&s_min, mine);
+    __syncthreads();
+    const int lo = s_min;
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+      const int i = tid + q * kBT;
+      const unsigned out = __ballot_sync(FULL, deg[q] == lo);
+      if (deg[q] == lo) {
+        keys[i] = (step << 16) | (uint32_t)(0xffff - i);
+        deg[q] = INT_MAX;
+      }
+      if (lane == 0 && (i >> 5) < W) gone[i >> 5] = out;
+    }
+    __syncthreads();
+    for (int w = 0; w < W; w++) {
+      const uint32_t x = gone[w];
+      if (!x) continue;
+      left -= __popc(x);
+#pragma unroll
+      for (int q = 0; q < 2; q++)
+        if (deg[q] != INT_MAX) deg[q] -= __popc(A[(tid + q * kBT) * Ws + w] & x);
     }
   }
+  __syncthreads();
+  bitonic_desc<true>((int *)keys, np2, tid, kBT);
+  return m;
+}
+
+// Their matrix and P list in that order, to global memory: dm (m rows of Wsm
+// words), dp.  All threads.
+__device__ void permute_rows(const uint32_t *A, int Ws, const int *Pidx, const uint32_t *keys, int m, uint32_t *dm,
+                             int Wsm, int *dp) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int i = wid; i < m; i += kBW) {
+    const uint32_t x = permuted_row(A, Ws, keys, m, i);
+    if (lane < Wsm) dm[(int64_t)i * Wsm + lane] = x;
+  }
+  for (int i = tid; i < m; i += kBT) dp[i] = Pidx[0xffff - (int)(keys[i] & 0xffffu)];
+}
+
+// A block's root as a task, sorted as above (the colouring of the task's upper
+// levels takes the densest first too).  ctl: two words.  False, publishing
+// nothing, without room.  All threads.
+__device__ bool publish_sorted(const SA &a, const Root &r, const uint32_t *A, int Ws, const uint32_t *keys, int m,
+                               int *ctl) {
+  const int Wsm = ((m + 31) >> 5) | 1;
+  if (threadIdx.x == 0) ctl[1] = open_record(a, r, m, &ctl[0]);
   __syncthreads();
   if (ctl[0] < 0) return false;
-  bitonic_desc<true>((int *)keys, np2, tid, kBT);
   uint32_t *dm = a.arena + a.recs[ctl[1]].off;
-  int *dp = (int *)(dm + (int64_t)m * Wsm);
-  for (int i = wid; i < m; i += kBW) {
-    const uint32_t *row = A + (int64_t)(0xffff - (int)(keys[i] & 0xffffu)) * Ws;
-    uint32_t mine = 0;
-    for (int w = 0; w < Wm; w++) {
-      const int j = 32 * w + lane;
-      const int at = j < m ? 0xffff - (int)(keys[j] & 0xffffu) : 0;
-      const unsigned word = __ballot_sync(FULL, j < m && ((row[at >> 5] >> (at & 31)) & 1u));
-      if (lane == w) mine = word;
-    }
-    if (lane < Wm) dm[(int64_t)i * Wsm + lane] = mine;
-  }
-  for (int i = tid; i < m; i += kBT) dp[i] = r.Pidx[0xffff - (int)(keys[i] & 0xffffu)];
+  permute_rows(A, Ws, r.Pidx, keys, m, dm, Wsm, (int *)(dm + (int64_t)m * Wsm));
   __threadfence();
   __syncthreads();
-  if (wid == 0) {
+  if (threadIdx.x < 32) {
     Bits<1> C, P;
     bzero(C);
-    P.w[0] = m >= 32 * (lane + 1) ? FULL : (m > 32 * lane ? (1u << (m - 32 * lane)) - 1u : 0u);
+    P.w[0] = first_bits(m);
     write_task(a, ctl[0], ctl[1], 1, C, P);
   }
   return true;
@@ -1086,9 +1322,9 @@ __device__ void block_search(const SA &a, const Root &r, const uint32_t *A, int 
 // PC: candidate capacity of the shared-memory layout.  The kMidCap layout
 // fits two blocks per SM; its roots with more candidates go to the overflow
 // list, which the 1,024-candidate launch then searches.
-template <int WPL, bool SM, int PC>
-__global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_block_kernel(SA a) {
-  using L = BlockLayout<WPL, SM, PC>;
+template <int WPL, bool SM, int PC, bool DENSE = false>
+__global__ void __launch_bounds__(kBT, (SM && (PC <= kMidCap || DENSE)) ? 2 : 1) search_block_kernel(SA a) {
+  using L = BlockLayout<WPL, SM, PC, DENSE>;
   extern __shared__ __align__(16) unsigned char smem[];
   int *Pidx = (int *)(smem + L::off_P);
   int *hk = (int *)(smem + L::off_hk);
@@ -1106,7 +1342,8 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
   const int hmask = L::HCAP - 1;
   const int64_t nroots = *a.nroots;
   const int64_t npr = *a.np_count;
-  for (int i = tid; i < kBitmapWords; i += kBT) bm[i] = 0u;  // each root clears the bits it set
+  if (!DENSE)
+    for (int i = tid; i < kBitmapWords; i += kBT) bm[i] = 0u;  // each root clears the bits it set
 
   for (;;) {
     __syncthreads();
@@ -1125,17 +1362,29 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
     __syncthreads();
     int om = ctl[1];
     if (a.ocore[u] < om) continue;
-    // the later ranks (u, n') fit the bitmap: member lookups by bitmap,
-    // otherwise by hash table
+    // u among the dense rows: its candidates and their matrix from those;
+    // else by member lookups, in a bitmap when the later ranks (u, n') fit it,
+    // otherwise in a hash table
+    const int64_t dbase = dense_base(npr, a.dense_cap);
+    const bool dense = SM && a.dense && u >= dbase;
+    if (DENSE && !dense) {  // to the launch with the lookup structures
+      if (tid == 0) a.overflow[atomicAdd((unsigned long long *)a.noverflow, 1ull)] = u;
+      continue;
+    }
     const int base = u + 1;
-    const bool use_bm = a.use_bitmap && ((npr - base + 31) >> 5) <= kBitmapWords;
-    if (!use_bm)
-      for (int i = tid; i < L::HCAP; i += kBT) hk[i] = -1;
-    for (int i = tid; i < L::PCAP; i += kBT) Pidx[i] = INT_MIN;
-    __syncthreads();
-    load_P(a, u, om, Pidx, L::PCAP, &ctl[2], tid, kBT);
-    __syncthreads();
-    const int p = ctl[2];
+    const bool use_bm = !dense && a.use_bitmap && ((npr - base + 31) >> 5) <= kBitmapWords;
+    int p;
+    if (dense) {
+      p = dense_P(a, u, om, dbase, npr, Pidx, L::PCAP, rm);
+    } else {
+      if (!use_bm)
+        for (int i = tid; i < L::HCAP; i += kBT) hk[i] = -1;
+      for (int i = tid; i < L::PCAP; i += kBT) Pidx[i] = INT_MIN;
+      __syncthreads();
+      load_P(a, u, om, Pidx, L::PCAP, &ctl[2], tid, kBT);
+      __syncthreads();
+      p = ctl[2];
+    }
     if (p > L::PCAP) {
       if (a.overflow) {
         if (tid == 0) a.overflow[atomicAdd((unsigned long long *)a.noverflow, 1ull)] = u;
@@ -1146,7 +1395,8 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
     }
     if (p < om || p == 0) continue;
     const int wwin = (int)((npr - base + 31) >> 5);
-    if (use_bm) {
+    if (dense) {
+    } else if (use_bm) {
       // P in any order: its bits, the prefix counts, and then every member
       // moves to its index in decreasing-rank order, which the counts give
       // (the hash table's space, unused on this path, holds the list)
@@ -1189,10 +1439,13 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
       for (int i = tid; i < p; i += kBT) hash_insert(hk, hv, hmask, Pidx[i], i);
     }
     const int W = (p + 31) >> 5, Ws = W | 1;
-    for (int64_t i = tid; i < (int64_t)p * Ws; i += kBT) A[i] = 0;
+    if (!dense)
+      for (int64_t i = tid; i < (int64_t)p * Ws; i += kBT) A[i] = 0;
     if (!SM) __threadfence();
     __syncthreads();
-    if (use_bm)
+    if (dense)
+      dense_build(a, Pidx, p, dbase, A, Ws, W, &ctl[6], a.counters + 5);
+    else if (use_bm)
       build_rows(a, Pidx, p, BitmapLookup{bm, pre, base, p}, A, Ws, wid, kBW, a.counters + 5, &ctl[6]);
     else
       build_rows(a, Pidx, p, HashLookup{hk, hv, hmask}, A, Ws, wid, kBW, a.counters + 5, &ctl[6]);
@@ -1262,11 +1515,37 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
     }
     __syncthreads();
     if (!ctl[4]) continue;
+    int Wr = W, Wsr = Ws;  // row words and stride of the searched matrix
     if constexpr (WPL == 1 && SM) {
-      // (the hash table's space is free: the matrix is built)
-      if (a.tasks && publish_sorted(a, r, A, Ws, W, al, (uint32_t *)hk, ctl + 8)) continue;
+      // in minimum-width order (in the hash table's space: the matrix is
+      // built); a task, or searched here: the matrix goes through global
+      // memory, and the colouring test is taken again in the new order.  In
+      // rank order the search in place took 1 to 10 s on 2 of 3 R-MAT scale-20
+      // graphs (5.7 and 9.4 ms sorted), 10-14 ms at scale 21 (9)
+      const int m = width_keys(A, p, Ws, W, al, (uint32_t *)hk, rm);
+      if (a.tasks && publish_sorted(a, r, A, Ws, (uint32_t *)hk, m, ctl + 8)) continue;
+      if (a.sort) {
+        uint32_t *dm = a.sort + (int64_t)blockIdx.x * a.sort_stride;
+        Wr = (m + 31) >> 5;
+        Wsr = Wr | 1;
+        int *dp = (int *)(dm + (int64_t)m * Wsr);
+        permute_rows(A, Ws, Pidx, (uint32_t *)hk, m, dm, Wsr, dp);
+        __syncthreads();
+        for (int i = tid; i < m * Wsr; i += kBT) A[i] = dm[i];
+        for (int i = tid; i < m; i += kBT) Pidx[i] = dp[i];
+        __syncthreads();
+        r.p = m;
+        if (wid == 0) {
+          P.w[0] = first_bits(m);
+          color_ise<WPL, SM>(A, Wsr, Wr, P, om - 1, B);
+          have = bany(B);
+          if (lane == 0) ctl[4] = have ? 1 : 0;
+        }
+        __syncthreads();
+        if (!ctl[4]) continue;
+      }
     }
-    block_search<WPL, SM>(a, r, A, Ws, W, stk, pool, have, P, B, C, cs, wat, nodes, don);
+    block_search<WPL, SM>(a, r, A, Wsr, Wr, stk, pool, have, P, B, C, cs, wat, nodes, don);
     __syncthreads();
   }
   if (lane == 0) {
@@ -1288,8 +1567,8 @@ __global__ void __launch_bounds__(kBT, (SM && PC <= kMidCap) ? 2 : 1) search_blo
 // chain from vertex to vertex.  Against whole blocks per task with a bit
 // matrix of up to 1,024 candidates, the candidates in rank order and one set
 // word per lane: 13 us per Branch node before, 7 us now, and 5 to 30 times
-// fewer nodes, since the candidates are sorted by their degree in the
-// subproblem.  R-MAT scale 18, edge factor 12: search 83-330 ms before (it
+// fewer nodes, since a root's candidates are in the minimum-width order of its
+// neighbourhood.  R-MAT scale 18, edge factor 12: search 83-330 ms before (it
 // depends on when the larger cliques are found), 4.2-4.6 ms now; scale 15,
 // edge factor 16: 60-104 ms before, 1.3 ms now.
 // Subproblems above 256 candidates are searched depth first by the warp on the
@@ -1686,15 +1965,14 @@ __device__ void compact_matrix(const TaskCtx &T, TaskSmem &S, int m) {
 // Candidates that can be in a clique larger than omega with T's clique: omega
 // + 1 - cs of them are needed, each with at least omega - cs neighbours among
 // them; the others are dropped until none is.  Returns how many are left (0:
-// decided; a maximal clique {u} + C larger than omega was raised).  Their sort
-// keys (degree, then smaller position) are left in S.A + 1024.
+// decided; a maximal clique {u} + C larger than omega was raised).  Their
+// positions are left in S.A.
 __device__ int prune_candidates(const SA &a, const TaskCtx &T, Bits<1> &P, TaskSmem &S) {
   const int lane = threadIdx.x & 31;
   const int om = read_best(a.best, T.g);
-  // the candidates' list and keys use the matrix's space, which is not built
-  // yet; lane i takes every 32nd candidate
+  // the candidates' list uses the matrix's space, which is not built yet; lane
+  // i takes every 32nd candidate
   int *lst = (int *)S.A;
-  uint32_t *key = S.A + 1024;
   for (;;) {
     const int cnt = __popc(P.w[0]);
     int incl = cnt;
@@ -1723,7 +2001,6 @@ __device__ int prune_candidates(const SA &a, const TaskCtx &T, Bits<1> &P, TaskS
 #pragma unroll 4
       for (int w = 0; w < T.W; w++) deg += __popc(__ldcg(row + w) & S.bits[w]);
       if (deg < om - T.cs) atomicOr(&S.drop[pos >> 5], 1u << (pos & 31));
-      key[i] = ((uint32_t)(deg + 1) << 16) | (uint32_t)(0xffff - pos);
     }
     __syncwarp();
     const uint32_t dr = S.drop[lane];
@@ -1733,19 +2010,14 @@ __device__ int prune_candidates(const SA &a, const TaskCtx &T, Bits<1> &P, TaskS
 }
 
 // Search T's clique with its m pruned candidates (at most kTM) on a compact
-// matrix, the members by decreasing degree among the candidates: the
-// colouring takes the densest first, the branching the sparsest.
+// matrix, in the order of the record's positions (the root's minimum-width
+// order): the colouring takes the densest first, the branching the sparsest.
 __device__ __forceinline__ void search_compact(const SA &a, const TaskCtx &T, int m, TaskSmem &S, uint32_t *stk,
                                                unsigned long long &nodes, unsigned long long &don) {
   const int lane = threadIdx.x & 31;
-  uint32_t *key = S.A + 1024;
-  int np2 = 32;
-  while (np2 < m) np2 <<= 1;
-  for (int i = m + lane; i < np2; i += 32) key[i] = 0;
-  __syncwarp();
-  bitonic_desc<false>((int *)key, np2, lane, 32);  // keys below 2^27: the signed order is the same
-  for (int i = lane; i < m; i += 32) S.mem[i] = 0xffff - (int)(key[i] & 0xffffu);
-  __syncwarp();  // the keys are read before the matrix takes their place
+  const int *lst = (const int *)S.A;
+  for (int i = lane; i < m; i += 32) S.mem[i] = lst[i];
+  __syncwarp();  // the list is read before the matrix takes its place
   if (m <= 128) {
     compact_matrix<4>(T, S, m);
     task_dfs<4>(a, T, S, stk, m, nodes, don);
@@ -1927,8 +2199,9 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   void *p;
   MC_TRY(ws_get(g, "se.ctr", kCtrBytes, &p));
   // [0..5] colored, branched, nodes, donations, row entries read by warp
-  // workers, by block workers; [8..9] four root queue heads; [10] arena
-  // words used; [11] records; [14] roots left to the 1,024-candidate launch;
+  // workers, by block workers; [8..9] four root queue heads, [12] a fifth;
+  // [10] arena words used; [11] records; [14], [15] roots left to the wider
+  // launches;
   // the queue's hot words on 128-byte lines of their own: [32] tasks, [48]
   // tickets, [64] unfinished tasks, [80] heartbeat
   unsigned long long *ctr = (unsigned long long *)p;
@@ -2020,9 +2293,34 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
     stk_t = (uint32_t *)p;
   }
 
+  if (no_split && kbound > wmax) {
+    const int cap = std::min(kbound, 1024);
+    a.sort_stride = (int64_t)cap * (((cap + 31) / 32) | 1) + cap;
+    const int blocks = std::max({blocks_b, blocks_m, g->sm_count * 2});
+    MC_TRY(ws_get(g, "se.sort", (size_t)blocks * a.sort_stride * 4, &p));
+    a.sort = (uint32_t *)p;
+  }
+  // one graph's block workers gather their matrices from dense rows; the
+  // builder's time counts with theirs
+  const bool dense = g->count == 1 && !no_bitmap && kbound > wmax;
+  if (dense) {
+    a.dense_cap = (int32_t)std::min<int64_t>(kDenseCap, (g->n + 31) & ~(int64_t)31);
+    a.dense_stride = a.dense_cap / 32;
+    MC_TRY(ws_get(g, "se.dense", (size_t)a.dense_cap * a.dense_stride * 4, &p));
+    a.dense = (const uint32_t *)p;
+  }
+
   // block class first (largest trees), then big, then warp class, then the
   // tasks the first and last of these published; events 8-12 time each
   MC_TRY(record_event(g, 8));
+  if (dense) {
+    const size_t smem = (size_t)kDW * a.dense_stride * 4;
+    MC_CUDA_TRY(cudaFuncSetAttribute(dense_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    dense_rows_kernel<<<(int)std::min<int64_t>((int64_t)g->sm_count * 4, (g->n + kDW - 1) / kDW), kDW * 32, smem,
+                        g->stream>>>(pg.d_counts, pg.orow, pg.ocol, a.dense_cap, a.dense_stride, (uint32_t *)a.dense);
+    g_launches++;
+    MC_CUDA_TRY(cudaGetLastError());
+  }
   if (kbound > wmax) {
     a.gmat = nullptr;
     a.roots = pg.roots_block;
@@ -2051,6 +2349,29 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
       if (kbound > kMidCap) {
         a.roots = a.overflow;
         a.nroots = a.noverflow;
+        if (dense) {
+          // roots of up to kWideCap candidates on the dense rows: without the
+          // lookup structures two blocks fit an SM
+          using LW = BlockLayout<1, true, kWideCap, true>;
+          int per_sm_w = 0;
+          MC_CUDA_TRY(cudaFuncSetAttribute(search_block_kernel<1, true, kWideCap, true>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LW::bytes));
+          MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+              &per_sm_w, search_block_kernel<1, true, kWideCap, true>, kBT, LW::bytes));
+          const int blocks_w = (int)std::min<int64_t>((int64_t)g->sm_count * std::max(per_sm_w, 1), small_cap);
+          MC_TRY(ws_get(g, "se.ovf2", (size_t)std::max<int64_t>(g->n, 1) * 4, &p));
+          a.overflow = (int32_t *)p;
+          a.noverflow = (int64_t *)(ctr + 15);
+          a.next = (int32_t *)(ctr + 12);
+          MC_TRY(ws_get(g, "se.stk_x", (size_t)blocks_w * kBW * stride_b * 4, &p));
+          a.stack = (uint32_t *)p;
+          a.stack_stride = stride_b;
+          search_block_kernel<1, true, kWideCap, true><<<blocks_w, kBT, LW::bytes, g->stream>>>(a);
+          g_launches++;
+          MC_CUDA_TRY(cudaGetLastError());
+          a.roots = a.overflow;
+          a.nroots = a.noverflow;
+        }
         a.next = next + 3;
         a.overflow = nullptr;
         a.noverflow = nullptr;

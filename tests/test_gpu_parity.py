@@ -254,6 +254,28 @@ def test_task_sizes_keep_omega(mc, n, p, planted):
         assert st["tasks"] > 0 or st["roots_branched"] == 0
 
 
+@pytest.mark.parametrize("n,p,planted", [(33, 0.95, 12), (64, 0.9, 14), (700, 0.4, 12), (1100, 0.55, 16),
+                                         (1500, 0.55, 18), (1760, 0.58, 20), (2300, 0.5, 18)])
+def test_dense_rows_match_lookups(mc, n, p, planted):
+    """Block workers on bit rows of the top ranks against the hash-table
+    build: the same roots survive the neighbourhood-core and colouring tests
+    (both orders of the same graph, one worker class), at candidate counts in
+    every layout (512, 864, 1,024) and just around words and tiles.  A planted
+    clique of over twice G(n, p)'s own keeps the trees short; omega is the
+    planted size."""
+    k = min(3 * planted, n - 5)
+    g = gg.relabel(gg.erdos_renyi(n, p, planted=k, seed=n), 7)
+    h = load(mc, g, flags=0)
+    order = mc.mc_peel_order(h).copy()
+    out = []
+    for opts in (dict(), dict(no_bitmap=True), dict(layout=1), dict(no_split=True)):
+        om, wit, st = mc.mc_max_clique(h, warp_max=1, order=order, **opts)
+        assert oracle.is_clique(g, wit) and om >= k
+        out.append((om, st["roots"], st["pruned_n"], st["heuristic_size"]))
+    assert len(set(out)) == 1, out
+    h.close()
+
+
 def test_host_pointers_and_repeat_calls(mc):
     g = gg.chung_lu(5000, 2.4, 10.0, 500.0, planted=14, seed=21)
     h = load(mc, g, device=False)
