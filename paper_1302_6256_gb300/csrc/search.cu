@@ -664,13 +664,13 @@ __device__ __forceinline__ void load_P(const SA &a, int u, int om, int *Pidx, in
 // that is in P (index j) sets bits (i, j) and (j, i).  The lanes of a warp
 // form four groups of eight, each walking a different member's row, with two
 // int4 loads per lane in flight, so a warp keeps eight rows' loads in the
-// memory system instead of one.
+// memory system instead of one.  scanned: the row entries a lane's group read
+// (Fact 3's work) are added by the group's first lane.
 template <class Lookup>
 __device__ __forceinline__ void build_rows(const SA &a, const int *Pidx, int p, const Lookup &find, uint32_t *A, int Ws,
-                                           int wid, int nw, unsigned long long *count, int *dyn = nullptr) {
+                                           int wid, int nw, unsigned long long &scanned, int *dyn = nullptr) {
   const int lane = threadIdx.x & 31;
   const int grp = lane >> 3, gl = lane & 7;
-  unsigned long long scanned = 0;
   // groups of 4 rows: statically wid, wid + nw, ...; or, with a shared
   // counter (dyn, zero before the call), taken by each warp as it frees up,
   // so rows of uneven length do not leave warps waiting at the next barrier
@@ -717,10 +717,6 @@ __device__ __forceinline__ void build_rows(const SA &a, const int *Pidx, int p, 
       i0 += nw * 4;
     }
   }
-  // row entries scanned (Fact 3's work), one atomic per warp
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) scanned += __shfl_xor_sync(FULL, scanned, o);
-  if (lane == 0 && scanned) atomicAdd(count, scanned);
 }
 
 // 32 x 32 bit transpose across a warp: lane r holds row r (bit c = column
@@ -932,15 +928,80 @@ struct WarpSmem {
   int cnt;
 };
 
-__global__ void __launch_bounds__(kSW * 32) search_warp_kernel(SA a) {
+// An upper bound of the edges of G[P] by one warp: the members' later-neighbour
+// entries whose hash bit is set in a 2,048-bit filter of P (bits: 64 words).
+// Eight lanes per row, four rows at a time, the next rows' offsets on their way.
+__device__ __forceinline__ int edges_upto(const SA &a, const int *Pidx, int p, uint32_t *bits,
+                                          unsigned long long &scanned) {
+  const int lane = threadIdx.x & 31, grp = lane >> 3, gl = lane & 7;
+  auto slot = [](int y) { return (unsigned)((unsigned)y * 2654435761u) >> 21; };
+  bits[lane] = 0;
+  bits[lane + 32] = 0;
+  __syncwarp();
+  for (int i = lane; i < p; i += 32) {
+    const unsigned h = slot(Pidx[i]);
+    atomicOr(&bits[h >> 5], 1u << (h & 31));
+  }
+  __syncwarp();
+  int hits = 0;
+  int64_t e0 = 0, e1 = 0;
+  if (grp < p) {
+    const int x = Pidx[grp];
+    e0 = a.orow[x];
+    e1 = a.orow[x + 1];
+  }
+  for (int i0 = 0; i0 < p; i0 += 4) {
+    const int64_t c0 = e0;
+    const int nq = (int)((e1 - e0) >> 2);
+    e0 = e1 = 0;
+    if (i0 + 4 + grp < p) {
+      const int x = Pidx[i0 + 4 + grp];
+      e0 = a.orow[x];
+      e1 = a.orow[x + 1];
+    }
+    if (gl == 0) scanned += 4ull * (unsigned long long)nq;
+    const int4 *row = reinterpret_cast<const int4 *>(a.ocol + c0);
+    for (int q = gl; q < nq; q += 8) {
+      const int4 y = __ldg(row + q);
+      const int ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const unsigned h = slot(ys[j]);
+        hits += (ys[j] >= 0 && ((bits[h >> 5] >> (h & 31)) & 1u)) ? 1 : 0;
+      }
+    }
+  }
+  __syncwarp();
+  return dev::warp_sum(hits);
+}
+
+// Branching roots leave the kernel's registers to the others: their part is
+// kept out of line.
+__device__ __noinline__ void branch_warp_root(const SA &a, const Root &r, uint32_t *A, int Ws, int W,
+                                              const uint32_t *al, uint32_t *keys, uint32_t *stk, int om,
+                                              unsigned long long *nodes) {
+  if (a.tasks && publish_warp(a, r, A, Ws, W, al, keys)) return;
+  const int lane = threadIdx.x & 31;
+  Bits<1> P, B, C;
+  P.w[0] = (lane < 4) ? al[lane] : 0u;
+  bzero(C);
+  unsigned long long n = 0, don = 0;
+  color_ise<1, true>(A, Ws, W, P, om - 1, B);
+  dfs<1, true>(a, r, A, Ws, W, stk, 1, P, B, C, om, (Pool<1> *)nullptr, n, don);
+  *nodes += n;
+}
+
+__global__ void __launch_bounds__(kSW * 32, 6) search_warp_kernel(SA a) {
   __shared__ WarpSmem sm[kSW];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   WarpSmem &S = sm[wib];
   const int64_t gw = (int64_t)blockIdx.x * kSW + wib;
   uint32_t *stk = a.stack + gw * a.stack_stride;
-  unsigned long long colored = 0, branched = 0, nodes = 0, don = 0;
+  unsigned long long colored = 0, branched = 0, nodes = 0, scanned = 0;
+  int probe = 0;
   const int hmask = 2 * kWarpCap - 1;
   const int64_t nroots = *a.nroots;
+  int score = nroots > 4 * (int64_t)gridDim.x * kSW ? 0 : -8;  // of the edge test below
   for (;;) {
     __syncwarp();
     int idx = 0;
@@ -952,8 +1013,6 @@ __global__ void __launch_bounds__(kSW * 32) search_warp_kernel(SA a) {
     int om = read_best(a.best, g);
     if (a.ocore[u] < om) continue;
     if (lane == 0) S.cnt = 0;
-    for (int i = lane; i < 2 * kWarpCap; i += 32) S.hk[i] = -1;
-    for (int i = lane; i < kWarpCap; i += 32) S.Pidx[i] = INT_MIN;
     __syncwarp();
     load_P(a, u, om, S.Pidx, kWarpCap, &S.cnt, lane, 32);
     __syncwarp();
@@ -963,14 +1022,30 @@ __global__ void __launch_bounds__(kSW * 32) search_warp_kernel(SA a) {
       break;
     }
     if (p < om || p == 0) continue;
+    // a larger clique needs om (om - 1) / 2 edges among the candidates: while
+    // that decides most roots (sparse graphs), it is tested before the matrix
+    // is built.  2.2 M roots of a 2,000-graph batch: 7.2 to 3.0 ms (3,100
+    // instructions per root before); with a few roots per warp only, the test
+    // costs more than it can learn (R-MAT scale 15: 0.21 to 0.27 ms)
+    if (score >= 0 || (++probe & 31) == 0) {
+      const int e = edges_upto(a, S.Pidx, p, S.A, scanned);
+      if (2 * e < om * (om - 1)) {
+        score = min(score + 1, 8);
+        continue;
+      }
+      score = max(score - 2, -8);
+    }
     int np2 = 32;
     while (np2 < p) np2 <<= 1;
+    for (int i = lane; i < 2 * kWarpCap; i += 32) S.hk[i] = -1;
+    for (int i = p + lane; i < np2; i += 32) S.Pidx[i] = INT_MIN;
+    __syncwarp();
     bitonic_desc<false>(S.Pidx, np2, lane, 32);
     for (int i = lane; i < p; i += 32) hash_insert(S.hk, S.hv, hmask, S.Pidx[i], i);
     const int W = (p + 31) >> 5, Ws = W | 1;
     for (int i = lane; i < p * Ws; i += 32) S.A[i] = 0;
     __syncwarp();
-    build_rows(a, S.Pidx, p, HashLookup{S.hk, S.hv, hmask}, S.A, Ws, 0, 1, a.counters + 4);
+    build_rows(a, S.Pidx, p, HashLookup{S.hk, S.hv, hmask}, S.A, Ws, 0, 1, scanned);
     __syncwarp();
     symmetrize<true>(S.A, Ws, W, p, 0, 1);
     __syncwarp();
@@ -1011,17 +1086,15 @@ __global__ void __launch_bounds__(kSW * 32) search_warp_kernel(SA a) {
     color_ise<1, true>(S.A, Ws, W, al, om - 1, B);
     if (!bany(B)) continue;
     branched++;
-    Bits<1> C;
-    bzero(C);
-    Root r{u, g, S.Pidx, p};
-    if (a.tasks && publish_warp(a, r, S.A, Ws, W, S.al, (uint32_t *)S.hk)) continue;
-    dfs<1, true>(a, r, S.A, Ws, W, stk, 1, al, B, C, om, (Pool<1> *)nullptr, nodes, don);
+    const Root r{u, g, S.Pidx, p};
+    branch_warp_root(a, r, S.A, Ws, W, S.al, (uint32_t *)S.hk, stk, om, &nodes);
   }
   if (lane == 0) {
     atomicAdd(a.counters + 0, colored);
     atomicAdd(a.counters + 1, branched);
     atomicAdd(a.counters + 2, nodes);
   }
+  if ((lane & 7) == 0 && scanned) atomicAdd(a.counters + 4, scanned);
 }
 
 // ----------------------------------------------------------- block class ---
@@ -1119,9 +1192,8 @@ __device__ int dense_P(const SA &a, int u, int om, int64_t base, int64_t np, int
 // members 32w .. 32w+31 (later ranks than member i for indices below i).  Rows
 // go to warps as they free up, the longest first; eight words in flight.
 __device__ __forceinline__ void dense_build(const SA &a, const int *Pidx, int p, int64_t base, uint32_t *A, int Ws,
-                                            int W, int *dyn, unsigned long long *count) {
+                                            int W, int *dyn, unsigned long long &scanned) {
   const int lane = threadIdx.x & 31;
-  unsigned long long words = 0;
   for (;;) {
     int i = 0;
     if (lane == 0) i = p - 1 - atomicAdd(dyn, 1);
@@ -1145,9 +1217,8 @@ __device__ __forceinline__ void dense_build(const SA &a, const int *Pidx, int p,
       }
     }
     if (lane < W) A[i * Ws + lane] = mine;
-    words += (unsigned long long)i;
+    if (lane == 0) scanned += (unsigned long long)i;
   }
-  if (lane == 0 && words) atomicAdd(count, words);
 }
 
 // The candidates left by the core test (bits al) in minimum-width order: those
@@ -1338,7 +1409,7 @@ __global__ void __launch_bounds__(kBT, (SM && (PC <= kMidCap || DENSE)) ? 2 : 1)
   uint16_t *pre = (uint16_t *)(smem + L::off_pre);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   uint32_t *stk = a.stack + ((int64_t)blockIdx.x * kBW + wid) * a.stack_stride;
-  unsigned long long colored = 0, branched = 0, nodes = 0, don = 0;
+  unsigned long long colored = 0, branched = 0, nodes = 0, don = 0, scanned = 0;
   const int hmask = L::HCAP - 1;
   const int64_t nroots = *a.nroots;
   const int64_t npr = *a.np_count;
@@ -1444,11 +1515,11 @@ __global__ void __launch_bounds__(kBT, (SM && (PC <= kMidCap || DENSE)) ? 2 : 1)
     if (!SM) __threadfence();
     __syncthreads();
     if (dense)
-      dense_build(a, Pidx, p, dbase, A, Ws, W, &ctl[6], a.counters + 5);
+      dense_build(a, Pidx, p, dbase, A, Ws, W, &ctl[6], scanned);
     else if (use_bm)
-      build_rows(a, Pidx, p, BitmapLookup{bm, pre, base, p}, A, Ws, wid, kBW, a.counters + 5, &ctl[6]);
+      build_rows(a, Pidx, p, BitmapLookup{bm, pre, base, p}, A, Ws, wid, kBW, scanned, &ctl[6]);
     else
-      build_rows(a, Pidx, p, HashLookup{hk, hv, hmask}, A, Ws, wid, kBW, a.counters + 5, &ctl[6]);
+      build_rows(a, Pidx, p, HashLookup{hk, hv, hmask}, A, Ws, wid, kBW, scanned, &ctl[6]);
     if (!SM) __threadfence();
     __syncthreads();
     if (use_bm)
@@ -1554,6 +1625,7 @@ __global__ void __launch_bounds__(kBT, (SM && (PC <= kMidCap || DENSE)) ? 2 : 1)
     atomicAdd(a.counters + 2, nodes);
     atomicAdd(a.counters + 3, don);
   }
+  if ((lane & 7) == 0 && scanned) atomicAdd(a.counters + 5, scanned);
 }
 
 
