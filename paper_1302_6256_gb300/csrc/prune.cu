@@ -107,8 +107,17 @@ struct PosG {
   __device__ void operator()(int64_t c, int64_t excl, int64_t) const { cpos[c] = excl; }
 };
 
+// Chunks a warp takes at a time: their words are read at once, a lane each,
+// and four chunks' entries are in flight together (short rows otherwise leave
+// a warp waiting on one chain of five dependent reads per row).  The pruning of
+// a 2,000-graph batch (4 M rows of 36 entries): 2.5 to 1.15 ms; R-MAT scale 22
+// (100,000 chunks of long rows): 0.82 ms either way.
+__device__ __forceinline__ int chunk_batch(int64_t nch, int64_t nw) {
+  return (int)min((int64_t)32, max((int64_t)1, nch / (2 * nw)));
+}
+
 // kept entries (later neighbours) per chunk, summed into the row's
-// out-degree; one warp per chunk
+// out-degree
 __global__ void outdeg_chunk_kernel(const int64_t *__restrict__ d_np, const int64_t *__restrict__ coff,
                                     const int32_t *__restrict__ crow, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
                                     const int32_t *__restrict__ oold, const int32_t *__restrict__ nid,
@@ -118,20 +127,57 @@ __global__ void outdeg_chunk_kernel(const int64_t *__restrict__ d_np, const int6
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t np = *d_np, nch = coff[np];
+  const int per = chunk_batch(nch, nw);
   unsigned long long rows = 0;
-  for (int64_t c = w0; c < nch; c += nw) {
-    const int64_t j = crow[c];
-    const int v = oold[j];
-    const int64_t e0 = rp[v] + (c - coff[j]) * kRowChunk, e1 = min(rp[v + 1], e0 + kRowChunk);
-    int k = 0;
-    for (int64_t e = e0 + lane; e < e1; e += 32) k += (nid[ci[e]] > (int32_t)j) ? 1 : 0;
-    k = dev::warp_sum(k);
-    if (lane == 0) {
-      ccnt[c] = k;
-      if (k) atomicAdd(odeg + j, k);
+  for (int64_t c0 = w0 * per; c0 < nch; c0 += nw * per) {
+    const int64_t c = c0 + lane;
+    const bool in = lane < per && c < nch;
+    int j = 0, len = 0, kept = 0;
+    int64_t e0 = 0;
+    bool only = false;  // the row's only chunk
+    if (in) {
+      j = crow[c];
+      const int v = oold[j];
+      const int64_t f = coff[j];
+      only = coff[j + 1] - f == 1;
+      e0 = rp[v] + (c - f) * kRowChunk;
+      len = (int)(min(rp[v + 1], e0 + kRowChunk) - e0);
+      rows += (unsigned long long)len;
     }
-    rows += (unsigned long long)(e1 - e0);
+    const int cnt = (int)min((int64_t)per, nch - c0);
+    for (int s0 = 0; s0 < cnt; s0 += 4) {
+      int64_t e[4];
+      int L[4], jj[4], k[4], most = 0;
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int src = (s0 + q) & 31;
+        e[q] = __shfl_sync(0xffffffffu, e0, src);
+        L[q] = __shfl_sync(0xffffffffu, len, src);
+        jj[q] = __shfl_sync(0xffffffffu, j, src);
+        if (s0 + q >= cnt) L[q] = 0;
+        k[q] = 0;
+        most = max(most, L[q]);
+      }
+      for (int b = lane; b - lane < most; b += 32) {
+        int y[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) y[q] = b < L[q] ? ci[e[q] + b] : -1;
+#pragma unroll
+        for (int q = 0; q < 4; q++) k[q] += (y[q] >= 0 && nid[y[q]] > jj[q]) ? 1 : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int t = dev::warp_sum(k[q]);
+        if (lane == s0 + q) kept = t;
+      }
+    }
+    if (in) {
+      ccnt[c] = kept;
+      if (only) odeg[j] = kept;
+      else if (kept) atomicAdd(odeg + j, kept);
+    }
   }
+  for (int o = 16; o > 0; o >>= 1) rows += __shfl_xor_sync(0xffffffffu, rows, o);
   if (lane == 0 && rows) atomicAdd(scanned, rows);
 }
 
@@ -155,9 +201,8 @@ struct RowG {
   __device__ void operator()(int64_t j, int64_t excl, int64_t) const { orow[j] = excl; }
 };
 
-// the oriented rows, one warp per chunk: a chunk's kept entries go after
-// those of the row's earlier chunks (row order kept), and the row's last
-// chunk writes its padding
+// the oriented rows: a chunk's kept entries go after those of the row's
+// earlier chunks (row order kept), and the row's last chunk writes its padding
 __global__ void fill_chunk_kernel(const int64_t *__restrict__ d_np, const int64_t *__restrict__ coff,
                                   const int32_t *__restrict__ crow, const int64_t *__restrict__ cpos,
                                   const int64_t *__restrict__ rp,
@@ -169,22 +214,51 @@ __global__ void fill_chunk_kernel(const int64_t *__restrict__ d_np, const int64_
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t np = *d_np, nch = coff[np];
-  for (int64_t c = w0; c < nch; c += nw) {
-    const int64_t j = crow[c];
-    const int v = oold[j];
-    const int64_t e0 = rp[v] + (c - coff[j]) * kRowChunk, e1 = min(rp[v + 1], e0 + kRowChunk);
-    int64_t out = orow[j] + (cpos[c] - cpos[coff[j]]);
-    for (int64_t eb = e0; eb < e1; eb += 32) {
-      const int64_t e = eb + lane;
-      const int y = (e < e1) ? nid[ci[e]] : -1;
-      const bool k = y > (int32_t)j;
-      const unsigned m = __ballot_sync(0xffffffffu, k);
-      if (k) ocol[out + __popc(m & lt)] = y;
-      out += __popc(m);
+  const int per = chunk_batch(nch, nw);
+  for (int64_t c0 = w0 * per; c0 < nch; c0 += nw * per) {
+    const int64_t c = c0 + lane;
+    int j = 0, len = 0;
+    int64_t e0 = 0, out = 0;
+    if (lane < per && c < nch) {
+      j = crow[c];
+      const int v = oold[j];
+      const int64_t f = coff[j], o0 = orow[j];
+      e0 = rp[v] + (c - f) * kRowChunk;
+      len = (int)(min(rp[v + 1], e0 + kRowChunk) - e0);
+      out = o0 + (cpos[c] - cpos[f]);
+      if (c == coff[j + 1] - 1) {
+        const int d = odeg[j], padded = (d + 3) & ~3;
+        for (int t = d; t < padded; t++) ocol[o0 + t] = -1;
+      }
     }
-    if (c == coff[j + 1] - 1) {
-      const int padded = (odeg[j] + 3) & ~3;
-      for (int t = odeg[j] + lane; t < padded; t += 32) ocol[orow[j] + t] = -1;
+    const int cnt = (int)min((int64_t)per, nch - c0);
+    for (int s0 = 0; s0 < cnt; s0 += 4) {
+      int64_t e[4], to[4];
+      int L[4], jj[4], most = 0;
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int src = (s0 + q) & 31;
+        e[q] = __shfl_sync(0xffffffffu, e0, src);
+        to[q] = __shfl_sync(0xffffffffu, out, src);
+        L[q] = __shfl_sync(0xffffffffu, len, src);
+        jj[q] = __shfl_sync(0xffffffffu, j, src);
+        if (s0 + q >= cnt) L[q] = 0;
+        most = max(most, L[q]);
+      }
+      for (int b = lane; b - lane < most; b += 32) {
+        int y[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) y[q] = b < L[q] ? ci[e[q] + b] : -1;
+#pragma unroll
+        for (int q = 0; q < 4; q++) y[q] = y[q] >= 0 ? nid[y[q]] : -1;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const bool k = y[q] > jj[q];
+          const unsigned m = __ballot_sync(0xffffffffu, k);
+          if (k) ocol[to[q] + __popc(m & lt)] = y[q];
+          to[q] += __popc(m);
+        }
+      }
     }
   }
 }
