@@ -134,6 +134,17 @@ __global__ void trivial_kernel(int32_t count, const int64_t *voff, int64_t n, in
   }
 }
 
+// the witnesses of a batch, one after the other, in each graph's own ids: a
+// warp per graph
+__global__ void pack_witness_kernel(int32_t count, const int64_t *voff, const int64_t *off, const int32_t *wit,
+                                    int32_t *out) {
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < count; g += nw) {
+    const int64_t v0 = voff[g], o0 = off[g], k = off[g + 1] - o0;
+    for (int64_t t = threadIdx.x & 31; t < k; t += 32) out[o0 + t] = wit[v0 + t] - (int32_t)v0;
+  }
+}
+
 static void free_graph(mc_graph *g) {
   if (!g) return;
   if (g->stream) cudaStreamSynchronize(g->stream);
@@ -816,14 +827,22 @@ int mc_max_clique_batch(mc_graph *g, const mc_options *opt, int32_t *omegas_out,
   st->omega = mx;
   if (off[g->count] > capacity) return MC_ERR_BUFFER;
   if (off[g->count] > 0 && !witness_out) return MC_ERR_ARG;
-  // gather all witnesses on the host in one copy of the witness area
-  std::vector<int32_t> all(std::max<int64_t>(g->n, 1));
-  if (g->n > 0) MC_CUDA_TRY(cudaMemcpy(all.data(), g->wit, g->n * 4, cudaMemcpyDeviceToHost));
+  // packed on the device, one copy of their sizes' sum, sorted on the host
   std::vector<int32_t> outv(std::max<int64_t>(off[g->count], 1));
-  for (int32_t i = 0; i < g->count; i++) {
-    int64_t b = g->h_voff[i];
-    for (int32_t t = 0; t < om[i]; t++) outv[off[i] + t] = all[b + t] - (int32_t)b;
-    std::sort(outv.begin() + off[i], outv.begin() + off[i] + om[i]);
+  if (off[g->count] > 0) {
+    void *p;
+    MC_TRY(ws_get(g, "cp.woff", (size_t)(g->count + 1) * 8, &p));
+    int64_t *d_off = (int64_t *)p;
+    MC_TRY(ws_get(g, "cp.wout", (size_t)off[g->count] * 4, &p));
+    int32_t *d_out = (int32_t *)p;
+    MC_CUDA_TRY(cudaMemcpyAsync(d_off, off.data(), (size_t)(g->count + 1) * 8, cudaMemcpyHostToDevice, g->stream));
+    pack_witness_kernel<<<std::max(1, std::min(g->count / 8 + 1, 4096)), 256, 0, g->stream>>>(g->count, g->voff, d_off,
+                                                                                             g->wit, d_out);
+    g_launches++;
+    MC_CUDA_TRY(cudaGetLastError());
+    MC_CUDA_TRY(cudaMemcpyAsync(outv.data(), d_out, (size_t)off[g->count] * 4, cudaMemcpyDeviceToHost, g->stream));
+    MC_CUDA_TRY(cudaStreamSynchronize(g->stream));
+    for (int32_t i = 0; i < g->count; i++) std::sort(outv.begin() + off[i], outv.begin() + off[i + 1]);
   }
   if (off[g->count] > 0)
     MC_CUDA_TRY(cudaMemcpy(witness_out, outv.data(), off[g->count] * 4, cudaMemcpyDefault));
