@@ -21,6 +21,7 @@
 // pos_weight on positive labels, averaged over the rows.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <vector>
 
@@ -41,6 +42,8 @@ struct mc_mlp {
   uint16_t *wbf = nullptr;   // bf16 copies of the weights (all parameters, same layout)
   float *grad = nullptr, *m = nullptr, *v = nullptr;
   float *loss = nullptr;     // device scalar
+  float *part = nullptr;     // the gradient's sums per block; grad and loss follow them
+  int part_blocks = 0;
   float *buf = nullptr;      // staging for host inputs
   size_t buf_bytes = 0;
   int64_t step = 0;
@@ -245,16 +248,6 @@ __device__ __forceinline__ float mlp_logit_group(const MlpSmem &S, const float x
   return sum + S.b3;
 }
 
-// weights into shared memory as fp32 (from the bf16 copies)
-__device__ __forceinline__ void load_weights(const uint16_t *__restrict__ wbf, const float *__restrict__ master,
-                                             float *sw) {
-  for (int i = threadIdx.x; i < kParams; i += blockDim.x) {
-    const bool is_bias = (i >= kOffB1 && i < kOffW2) || (i >= kOffB2 && i < kOffW3) || i == kOffB3;
-    sw[i] = is_bias ? master[i] : bf16_to_f32(wbf[i]);  // biases stay fp32
-  }
-  __syncthreads();
-}
-
 // logits of n feature rows, eight lanes per row
 __global__ void __launch_bounds__(256) forward_kernel(int64_t n, const float *__restrict__ feat,
                                                       const uint16_t *__restrict__ wbf,
@@ -301,122 +294,229 @@ __global__ void __launch_bounds__(256) score_kernel(const int32_t *__restrict__ 
 }
 
 // Gradient of the mean weighted BCE over rows, accumulated into grad (fp32).
-// Each block accumulates its rows' contributions in shared memory and adds
-// them to the global gradient once.
-constexpr int kGT = 128;
+// A block takes tiles of kGR rows.  Its three 64 x 64 x 64 products (the second
+// layer forward, back to the first layer, and the second layer's weights) and
+// the first layer are register tiles of 4 x 4 outputs per thread over operands
+// in shared memory, each operand in the layout that the product reads as
+// float4; sums over rows stay in registers over all tiles of a block and reach
+// memory once per block.  FP32 throughout, as the bound on precision asks: the
+// activations are not BF16, so the tensor pipe's types would round them.
+// 16,384 rows: 190 us with a thread per row (128 rows per block, serial
+// 64-long chains per thread, 6% of the warps, sums by atomics), 36 us now with
+// 5 us for the sum over the blocks; its error against 64 bits is a third of
+// what it was (the blocks' sums are added in order, not by atomics).
+constexpr int kGR = 64;    // rows per tile
+constexpr int kGT = 256;   // threads: 16 x 16, 4 x 4 outputs each
+constexpr int kPart = (kParams + 1 + 31) / 32 * 32;  // floats of a block's sums: parameters, loss
+constexpr int kGS = 68;    // row stride of the tiles (float4 aligned, off the banks)
 struct GradSmem {
-  float sw[kParams];
-  float sg[kParams];
-  float sh1[kGT][kH + 1];  // this tile's hidden activations
-  float sd2[kGT][kH + 1];  // d loss / d z2, then d loss / d z1
-  float sx[kGT][kF];
-  float sloss;
+  float w2[kH][kGS], w2t[kH][kGS];  // W2[j][k] and its transpose
+  float h1[kGR][kGS], h1t[kH][kGS];
+  float d2[kGR][kGS], d2t[kH][kGS];
+  float w1t[kF][kH], x[kF][kGR];
+  float b1[kH], b2[kH], w3[kH], y[kGR], b3;
+  float sum[kParams + 1];  // the block's gradient and loss
 };
-__global__ void __launch_bounds__(kGT) grad_kernel(int64_t n, const float *__restrict__ feat,
-                                                   const float *__restrict__ label, float pos_weight,
-                                                   const uint16_t *__restrict__ wbf, const float *__restrict__ master,
-                                                   float *__restrict__ grad, float *__restrict__ loss) {
+// what is read as float4 starts on 16 bytes, in every row (columns and rows are
+// taken at multiples of four)
+static_assert(offsetof(GradSmem, w2) % 16 == 0 && offsetof(GradSmem, w2t) % 16 == 0 &&
+                  offsetof(GradSmem, h1) % 16 == 0 && offsetof(GradSmem, h1t) % 16 == 0 &&
+                  offsetof(GradSmem, d2) % 16 == 0 && offsetof(GradSmem, d2t) % 16 == 0 &&
+                  offsetof(GradSmem, w1t) % 16 == 0 && offsetof(GradSmem, x) % 16 == 0 && kGS % 4 == 0 &&
+                  kH % 4 == 0 && kGR % 4 == 0,
+              "float4 operands of grad_kernel");
+static_assert(kGT == (kH / 4) * (kGR / 4) && kGR == kH, "one 4 x 4 tile per thread in each product");
+
+__device__ __forceinline__ void fma4x4(float (&c)[4][4], const float4 &a, const float4 &b) {
+  const float x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+#pragma unroll
+    for (int j = 0; j < 4; j++) c[i][j] = fmaf(x[i], y[j], c[i][j]);
+}
+// a tile and its transpose, rows kGS floats apart
+__device__ __forceinline__ void st4x4(float *p, float *pt, const float (&c)[4][4]) {
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    *reinterpret_cast<float4 *>(p + i * kGS) = make_float4(c[i][0], c[i][1], c[i][2], c[i][3]);
+    *reinterpret_cast<float4 *>(pt + i * kGS) = make_float4(c[0][i], c[1][i], c[2][i], c[3][i]);
+  }
+}
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+__global__ void __launch_bounds__(kGT, 2) grad_kernel(int64_t n, const float *__restrict__ feat,
+                                                      const float *__restrict__ label, float pos_weight,
+                                                      const uint16_t *__restrict__ wbf,
+                                                      const float *__restrict__ master, float *__restrict__ part) {
   extern __shared__ __align__(16) unsigned char gsm_raw[];
   GradSmem &S = *reinterpret_cast<GradSmem *>(gsm_raw);
-  float *sw = S.sw, *sg = S.sg;
-  auto &sh1 = S.sh1;
-  auto &sd2 = S.sd2;
-  auto &sx = S.sx;
-  float &sloss = S.sloss;
-  load_weights(wbf, master, sw);
-  for (int i = threadIdx.x; i < kParams; i += blockDim.x) sg[i] = 0.f;
-  if (threadIdx.x == 0) sloss = 0.f;
-  __syncthreads();
-  const float inv_n = 1.f / (float)n;
-  const int t = threadIdx.x;
-  for (int64_t base = (int64_t)blockIdx.x * kGT; base < n; base += (int64_t)gridDim.x * kGT) {
-    const int64_t r = base + t;
-    const bool valid = r < n;
-    float x[kF], h1[kH];
-#pragma unroll
-    for (int i = 0; i < kF; i++) x[i] = valid ? feat[r * kF + i] : 0.f;
-    // forward keeping z2 signs in sd2 as a scratch
-    float s = sw[kOffB3];
-#pragma unroll
-    for (int j = 0; j < kH; j++) {
-      float z = sw[kOffB1 + j];
-#pragma unroll
-      for (int i = 0; i < kF; i++) z = fmaf(sw[kOffW1 + j * kF + i], x[i], z);
-      h1[j] = fmaxf(z, 0.f);
-    }
-    float z2[kH];
-    for (int j = 0; j < kH; j++) {
-      float z = sw[kOffB2 + j];
-#pragma unroll
-      for (int k = 0; k < kH; k++) z = fmaf(sw[kOffW2 + j * kH + k], h1[k], z);
-      z2[j] = z;
-      s = fmaf(sw[kOffW3 + j], fmaxf(z, 0.f), s);
-    }
-    // d loss / d s for weighted BCE with logits, mean over rows
-    float gs = 0.f;
-    if (valid) {
-      const float y = label[r];
-      const float w = y > 0.5f ? pos_weight : 1.f;
-      const float sig = 1.f / (1.f + expf(-s));
-      gs = w * (sig - y) * inv_n;
-      // loss = w * (log(1 + e^s) - y s), computed stably
-      const float l = w * (fmaxf(s, 0.f) + log1pf(expf(-fabsf(s))) - y * s);
-      atomicAdd(&sloss, l * inv_n);
-    }
-    atomicAdd(&sg[kOffB3], gs);
-    for (int j = 0; j < kH; j++) {
-      const float a2 = fmaxf(z2[j], 0.f);
-      sd2[t][j] = (z2[j] > 0.f) ? gs * sw[kOffW3 + j] : 0.f;
-      z2[j] = a2 * gs;  // d loss / d w3_j contribution
-    }
-#pragma unroll
-    for (int k = 0; k < kH; k++) sh1[t][k] = h1[k];
-#pragma unroll
-    for (int i = 0; i < kF; i++) sx[t][i] = x[i];
-    // d loss / d h1_k = sum_j d2_j W2[j][k]; back through the first ReLU
-    float d1[kH];
-    for (int k = 0; k < kH; k++) d1[k] = 0.f;
-    for (int j = 0; j < kH; j++) {
-      const float dj = sd2[t][j];
-      if (dj != 0.f)
-#pragma unroll
-        for (int k = 0; k < kH; k++) d1[k] = fmaf(dj, sw[kOffW2 + j * kH + k], d1[k]);
-    }
-    // reuse z2 storage: w3 gradient contributions
-    for (int j = 0; j < kH; j++) atomicAdd(&sg[kOffW3 + j], z2[j]);
-    __syncthreads();
-    // W2 and b2: each thread owns entries (j, k), summing over the tile's rows
-    for (int e = t; e < kH * kH; e += kGT) {
-      const int j = e / kH, k = e % kH;
-      float acc = 0.f;
-      for (int q = 0; q < kGT; q++) acc = fmaf(sd2[q][j], sh1[q][k], acc);
-      sg[kOffW2 + e] += acc;
-    }
-    if (t < kH) {
-      float acc = 0.f;
-      for (int q = 0; q < kGT; q++) acc += sd2[q][t];
-      sg[kOffB2 + t] += acc;
-    }
-    __syncthreads();
-    // first layer: d z1_k = d1_k [h1_k > 0]; W1 and b1 summed over the tile
-#pragma unroll
-    for (int k = 0; k < kH; k++) sd2[t][k] = (h1[k] > 0.f) ? d1[k] : 0.f;
-    __syncthreads();
-    for (int e = t; e < kH * kF; e += kGT) {
-      const int k = e / kF, i = e % kF;
-      float acc = 0.f;
-      for (int q = 0; q < kGT; q++) acc = fmaf(sd2[q][k], sx[q][i], acc);
-      sg[kOffW1 + e] += acc;
-    }
-    if (t < kH) {
-      float acc = 0.f;
-      for (int q = 0; q < kGT; q++) acc += sd2[q][t];
-      sg[kOffB1 + t] += acc;
-    }
-    __syncthreads();
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;  // outputs 4 tx .. (columns), 4 ty .. (rows)
+  const int c0 = 4 * tx, r0 = 4 * ty;
+  bool bad = false;
+  for (int e = t; e < kH * kH; e += kGT) {
+    const float w = bf16_to_f32(wbf[kOffW2 + e]);
+    S.w2[e / kH][e % kH] = w;
+    S.w2t[e % kH][e / kH] = w;
+    bad |= !isfinite(w);
   }
-  for (int i = threadIdx.x; i < kParams; i += blockDim.x) atomicAdd(grad + i, sg[i]);
-  if (threadIdx.x == 0 && loss) atomicAdd(loss, sloss);
+  for (int e = t; e < kH * kF; e += kGT) S.w1t[e % kF][e / kF] = bf16_to_f32(wbf[kOffW1 + e]);
+  for (int j = t; j < kH; j += kGT) {
+    S.b1[j] = master[kOffB1 + j];  // biases stay fp32
+    S.b2[j] = master[kOffB2 + j];
+    S.w3[j] = bf16_to_f32(wbf[kOffW3 + j]);
+  }
+  if (t == 0) S.b3 = master[kOffB3];
+  for (int e = t; e <= kParams; e += kGT) S.sum[e] = 0.f;
+  // a unit that is off passes nothing back, also where a weight is infinite
+  const bool odd = __syncthreads_or(bad);
+  const float inv_n = 1.f / (float)n;
+  float gw2[4][4] = {}, gw1[4][kF] = {}, gb1[4] = {}, gb2[4] = {}, gw3[4] = {}, gb3 = 0.f, lsum = 0.f;
+  for (int64_t base = (int64_t)blockIdx.x * kGR; base < n; base += (int64_t)gridDim.x * kGR) {
+    const int rows = (int)min((int64_t)kGR, n - base);
+    __syncthreads();  // the last tile is done with the buffers
+    for (int e = t; e < kGR * kF; e += kGT) {
+      const int r = e / kF;
+      S.x[e % kF][r] = r < rows ? feat[base * kF + e] : 0.f;
+    }
+    for (int r = t; r < kGR; r += kGT) S.y[r] = r < rows ? label[base + r] : 0.f;
+    __syncthreads();
+    // first layer: rows r0.., units c0..
+    float c[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+      for (int j = 0; j < 4; j++) c[i][j] = S.b1[c0 + j];
+#pragma unroll
+    for (int i = 0; i < kF; i++) fma4x4(c, ld4(&S.x[i][r0]), ld4(&S.w1t[i][c0]));
+    bool on[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        on[i][j] = c[i][j] > 0.f;
+        c[i][j] = fmaxf(c[i][j], 0.f);
+      }
+    st4x4(&S.h1[r0][c0], &S.h1t[c0][r0], c);
+    __syncthreads();
+    // second layer: rows r0.., units c0..
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+      for (int j = 0; j < 4; j++) c[i][j] = S.b2[c0 + j];
+#pragma unroll 4
+    for (int k = 0; k < kH; k++) fma4x4(c, ld4(&S.h1t[k][r0]), ld4(&S.w2t[k][c0]));
+    // logit of each row: the 16 threads of a row share it
+    float gs[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      float s = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; j++) s = fmaf(S.w3[c0 + j], fmaxf(c[i][j], 0.f), s);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      s += S.b3;
+      // d loss / d s for weighted BCE with logits, mean over rows
+      gs[i] = 0.f;
+      if (r0 + i < rows) {
+        const float y = S.y[r0 + i];
+        const float w = y > 0.5f ? pos_weight : 1.f;
+        const float sig = 1.f / (1.f + expf(-s));
+        gs[i] = w * (sig - y) * inv_n;
+        // loss = w * (log(1 + e^s) - y s), computed stably
+        if (tx == 0) {
+          lsum += w * (fmaxf(s, 0.f) + log1pf(expf(-fabsf(s))) - y * s) * inv_n;
+          gb3 += gs[i];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const float d = c[i][j] > 0.f ? gs[i] * S.w3[c0 + j] : 0.f;
+        gb2[j] += d;
+        gw3[j] += fmaxf(c[i][j], 0.f) * gs[i];
+        c[i][j] = d;
+      }
+    }
+    st4x4(&S.d2[r0][c0], &S.d2t[c0][r0], c);
+    __syncthreads();
+    // back through W2: d loss / d h1, rows r0.., units c0..; and W2's own
+    // gradient, its row r0.. (second-layer unit), column c0..
+    float d1[4][4] = {};
+    if (!odd) {
+#pragma unroll 4
+      for (int k = 0; k < kH; k++) fma4x4(d1, ld4(&S.d2t[k][r0]), ld4(&S.w2[k][c0]));
+    } else {
+      for (int k = 0; k < kH; k++)
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const float d = S.d2t[k][r0 + i];
+          if (d != 0.f)
+#pragma unroll
+            for (int j = 0; j < 4; j++) d1[i][j] = fmaf(d, S.w2[k][c0 + j], d1[i][j]);
+        }
+    }
+#pragma unroll 4
+    for (int r = 0; r < kGR; r++) fma4x4(gw2, ld4(&S.d2[r][r0]), ld4(&S.h1[r][c0]));
+    // first layer: rows of this thread only, summed over the block at the end
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        const float d = on[i][j] ? d1[i][j] : 0.f;
+        gb1[j] += d;
+#pragma unroll
+        for (int f = 0; f < kF; f++) gw1[j][f] = fmaf(d, S.x[f][r0 + i], gw1[j][f]);
+      }
+  }
+  // the two halves of a warp hold other rows of the same units
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    float v[kF + 3];
+#pragma unroll
+    for (int f = 0; f < kF; f++) v[f] = gw1[j][f];
+    v[kF] = gb1[j];
+    v[kF + 1] = gb2[j];
+    v[kF + 2] = gw3[j];
+#pragma unroll
+    for (int f = 0; f < kF + 3; f++) {
+      v[f] += __shfl_xor_sync(0xffffffffu, v[f], 16);
+      const int at = f < kF ? kOffW1 + (c0 + j) * kF + f
+                            : (f == kF ? kOffB1 : (f == kF + 1 ? kOffB2 : kOffW3)) + c0 + j;
+      if ((t & 16) == 0) atomicAdd(&S.sum[at], v[f]);
+    }
+  }
+  if (tx == 0) {
+    atomicAdd(&S.sum[kOffB3], gb3);
+    atomicAdd(&S.sum[kParams], lsum);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+#pragma unroll
+    for (int j = 0; j < 4; j++) S.sum[kOffW2 + (r0 + i) * kH + c0 + j] = gw2[i][j];
+  __syncthreads();
+  for (int e = t; e <= kParams; e += kGT) part[(int64_t)blockIdx.x * kPart + e] = S.sum[e];
+}
+
+// The blocks' sums, added in a fixed order (the gradient is the same bits on
+// every call): a warp's lanes are 32 parameters, its eight warps an eighth of
+// the blocks each.
+constexpr int kRT = 256;
+__global__ void __launch_bounds__(kRT) grad_sum_kernel(int blocks, const float *__restrict__ part,
+                                                       float *__restrict__ grad, float *__restrict__ loss) {
+  __shared__ float sm[kRT / 32][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  float v = 0.f;
+  if (e <= kParams) {
+#pragma unroll 8
+    for (int b = wid; b < blocks; b += kRT / 32) v += part[(int64_t)b * kPart + e];
+  }
+  sm[wid][lane] = v;
+  __syncthreads();
+  if (wid == 0 && e <= kParams) {
+#pragma unroll
+    for (int i = 1; i < kRT / 32; i++) v += sm[i][lane];
+    if (e < kParams) grad[e] = v;
+    else *loss = v;
+  }
 }
 
 __global__ void adam_kernel(float *__restrict__ master, uint16_t *__restrict__ wbf, const float *__restrict__ grad,
@@ -760,18 +860,21 @@ int mc_mlp_create(uint64_t seed, void *cuda_stream, mc_mlp **out) {
   mc_mlp *m = new mc_mlp();
   m->stream = (cudaStream_t)cuda_stream;
   auto fail = [&](int rc) {
-    cudaFree(m->master); cudaFree(m->wbf); cudaFree(m->grad); cudaFree(m->m); cudaFree(m->v); cudaFree(m->loss);
+    cudaFree(m->master); cudaFree(m->wbf); cudaFree(m->part); cudaFree(m->m); cudaFree(m->v);
     if (m->h_small) cudaFreeHost(m->h_small);
     delete m;
     return rc;
   };
   if (cudaGetDevice(&m->device) != cudaSuccess) return fail(MC_ERR_CUDA);
   cudaDeviceGetAttribute(&m->sm_count, cudaDevAttrMultiProcessorCount, m->device);
-  if (cudaMalloc(&m->master, kParams * 4) != cudaSuccess || cudaMalloc(&m->wbf, kParams * 2) != cudaSuccess ||
-      cudaMalloc(&m->grad, kParams * 4) != cudaSuccess || cudaMalloc(&m->m, kParams * 4) != cudaSuccess ||
-      cudaMalloc(&m->v, kParams * 4) != cudaSuccess || cudaMalloc(&m->loss, 16) != cudaSuccess ||
+  m->part_blocks = 2 * std::max(m->sm_count, 1);  // the blocks of grad_kernel that run at once
+  if (cudaMalloc(&m->part, (size_t)(m->part_blocks + 2) * kPart * 4) != cudaSuccess ||
+      cudaMalloc(&m->master, kParams * 4) != cudaSuccess || cudaMalloc(&m->wbf, kParams * 2) != cudaSuccess ||
+      cudaMalloc(&m->m, kParams * 4) != cudaSuccess || cudaMalloc(&m->v, kParams * 4) != cudaSuccess ||
       cudaMallocHost(&m->h_small, 4096) != cudaSuccess)
     return fail(MC_ERR_OOM);
+  m->grad = m->part + (size_t)m->part_blocks * kPart;
+  m->loss = m->grad + kPart;
   // He-uniform initial weights from a counter-based generator, zero biases
   std::vector<float> p(kParams, 0.f);
   uint64_t ctr = seed * 0x9E3779B97F4A7C15ULL + 1;
@@ -793,7 +896,7 @@ int mc_mlp_create(uint64_t seed, void *cuda_stream, mc_mlp **out) {
 void mc_mlp_free(mc_mlp *m) {
   if (!m) return;
   cudaStreamSynchronize(m->stream);
-  cudaFree(m->master); cudaFree(m->wbf); cudaFree(m->grad); cudaFree(m->m); cudaFree(m->v); cudaFree(m->loss);
+  cudaFree(m->master); cudaFree(m->wbf); cudaFree(m->part); cudaFree(m->m); cudaFree(m->v);
   cudaFree(m->buf);
   if (m->h_small) cudaFreeHost(m->h_small);
   delete m;
@@ -890,13 +993,13 @@ static int run_grad(mc_mlp *m, const float *feat, const float *label, int64_t n,
     df = m->buf;
     dl = (char *)m->buf + fb;
   }
-  MC_CUDA_TRY(cudaMemsetAsync(m->grad, 0, kParams * 4, m->stream));
-  MC_CUDA_TRY(cudaMemsetAsync(m->loss, 0, 4, m->stream));
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + kGT - 1) / kGT, (int64_t)m->sm_count * 4));
+  const int64_t tiles = (n + kGR - 1) / kGR;
+  const int blocks = (int)std::min<int64_t>(tiles, m->part_blocks);
   MC_CUDA_TRY(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
   grad_kernel<<<blocks, kGT, sizeof(GradSmem), m->stream>>>(n, (const float *)df, (const float *)dl, pos_weight, m->wbf,
-                                                            m->master, m->grad, m->loss);
-  g_launches++;
+                                                            m->master, m->part);
+  grad_sum_kernel<<<kPart / 32, kRT, 0, m->stream>>>(blocks, m->part, m->grad, m->loss);
+  g_launches += 2;
   MC_CUDA_TRY(cudaGetLastError());
   return MC_OK;
 }

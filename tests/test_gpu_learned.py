@@ -235,3 +235,37 @@ def test_trained_network_raises_the_lower_bound(mc):
     print("lower-bound gap over 60 held-out graphs:", gap)
     assert gap["learned"] < gap["plain"]
     assert gap["learned"] < gap["random"]
+
+
+@pytest.mark.parametrize("rows", [1, 63, 64, 65, 511, 513, 19457, 40001])
+def test_gradient_by_row_count(mc, rows):
+    """The gradient's tiles of 64 rows at their edges, clusters with idle
+    blocks, and more tiles than blocks, at the tolerance of the test above."""
+    r = np.random.default_rng(rows)
+    x = r.random((rows, OL.F)).astype(np.float32)
+    y = (r.random(rows) < 0.2).astype(np.float32)
+    m = mc.MLP(seed=3)
+    p = m.get_params()
+    g, loss = m.gradient(x, y, pos_weight=5.0)
+    gref = OL.gradient(p, x, y, 5.0)
+    assert loss == pytest.approx(OL.loss(p, x, y, 5.0), rel=1e-4)
+    assert np.allclose(g, gref, rtol=1e-3, atol=1e-4 * np.abs(gref).max())
+
+
+def test_gradient_with_an_infinite_weight(mc):
+    """A hidden unit that is off passes nothing back, infinite weights or
+    not: the same gradient as with a large finite weight in their place."""
+    r = np.random.default_rng(8)
+    x = r.random((300, OL.F)).astype(np.float32)
+    y = (r.random(300) < 0.2).astype(np.float32)
+    m = mc.MLP(seed=3)
+    p = np.array(m.get_params())
+    row = slice(OL.H * OL.F + OL.H + 5 * OL.H, OL.H * OL.F + OL.H + 6 * OL.H)  # W2's row of unit 5
+    g = []
+    for w in (-1e30, -np.inf):
+        q = p.copy()
+        q[row] = w
+        m.set_params(q)
+        g.append(m.gradient(x, y, 2.0)[0])
+    assert np.isfinite(g[1]).all()
+    assert np.allclose(g[0], g[1], rtol=1e-3, atol=1e-4 * np.abs(g[0]).max())
