@@ -11,10 +11,10 @@
 //   f2 = t / 28, t = edges among Q          increasing id (a bound on a
 //                                           clique through v inside Q + v)
 //   f4 = c / max(d, 1)                 f5 = log1p(c) / log1p(Dmax)
-// Eight lanes per vertex, four vertices per warp in flight: a pass over the
-// row (c and Q), the 28 pairs of Q each found by binary search in the
-// shorter of the two rows, the colouring with one colour class per lane,
-// and the network with eight hidden units per lane.
+// A pass over the row gives c and Q (eight lanes, a warp or a block by its
+// length), then eight lanes per vertex find the 28 pairs of Q by binary search
+// in the shorter of the two rows and colour, one colour class per lane; fused
+// with the network, it has eight hidden units per lane.
 //
 // Parameters, flat fp32 (4673): W1[64][6], b1[64], W2[64][64], b2[64],
 // w3[64], b3.  Loss: binary cross-entropy on the logit s with weight
@@ -75,80 +75,110 @@ __device__ __forceinline__ unsigned group_ballot(unsigned gm, bool x, int grp) {
   return (__ballot_sync(gm, x) >> (grp * 8)) & 0xFFu;
 }
 
-__device__ __forceinline__ bool in_row(const int64_t *__restrict__ rp, const int32_t *__restrict__ ci, int x, int y) {
-  int64_t lo = rp[x], hi = rp[x + 1];
-  const int64_t end = hi;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (ci[mid] < y) lo = mid + 1; else hi = mid;
+// Row lengths up to which a group of 8 lanes, a whole warp or (above) a block
+// counts a vertex's row; entries that a lane has in flight.  With 8 lanes for
+// every row the hubs' rows were the tail (R-MAT scale 18: 1.44 ms with 35% of
+// the warps, 9 of 32 lanes active; 0.21 ms now).
+constexpr int64_t kGroupRow = 256, kWarpRow = 4096;
+constexpr int kRowFly = 4;
+
+// Number of u in ci[e0, e1) with core[u] >= kv, counted by LANES lanes (gl =
+// the lane's place among them, shift = their first lane, gm = their mask); the
+// first kQ of them go to qs.
+template <int LANES>
+__device__ int count_row(const int32_t *__restrict__ ci, const int32_t *__restrict__ core, int kv, int64_t e0,
+                         int64_t e1, unsigned gm, int shift, int gl, int *qs) {
+  constexpr unsigned all = LANES == 32 ? 0xffffffffu : (1u << (LANES & 31)) - 1u;
+  const unsigned below = (1u << gl) - 1u;
+  int c = 0;
+  for (int64_t eb = e0; eb < e1; eb += LANES * kRowFly) {
+    int u[kRowFly];
+    bool ok[kRowFly];
+#pragma unroll
+    for (int i = 0; i < kRowFly; i++) {
+      const int64_t e = eb + i * LANES + gl;
+      u[i] = e < e1 ? ci[e] : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < kRowFly; i++) ok[i] = u[i] >= 0 && core[u[i]] >= kv;
+#pragma unroll
+    for (int i = 0; i < kRowFly; i++) {
+      const unsigned m = (__ballot_sync(gm, ok[i]) >> shift) & all;
+      const int pos = c + __popc(m & below);
+      if (ok[i] && pos < kQ) qs[pos] = u[i];
+      c += __popc(m);
+    }
   }
-  return lo < end && ci[lo] == y;
+  return c;
 }
 
-// The six features of vertex v, computed by the 8 lanes of one group (all
-// 8 call with the same v; every lane of the group returns them).  qs: 8
-// ints of shared memory for this group.
-__device__ void vertex_features(const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                                const int32_t *__restrict__ core, float kmax, float ldmax, int64_t v, int *qs,
-                                float f[kF]) {
+// The six features of vertex v (row [e0, e1), core number kv) from its count c
+// and Q, by the 8 lanes of one group (every lane returns them).  The 28 pairs
+// of Q are four per lane -- member gl with the members gl + 1 .. gl + 4, around
+// -- and a lane's four binary searches run side by side.
+__device__ void vertex_features(const int64_t *__restrict__ rp, const int32_t *__restrict__ ci, float kmax,
+                                float ldmax, int64_t deg, int kv, int c, const int *qs, float f[kF]) {
   const int lane = threadIdx.x & 31, grp = lane >> 3, gl = lane & 7;
   const unsigned gm = 0xFFu << (grp * 8);
-  const unsigned below = (1u << gl) - 1u;
-  const int kv = core[v];
-  const int64_t e0 = rp[v], e1 = rp[v + 1];
-  int c = 0;
-  for (int64_t eb = e0; eb < e1; eb += 8) {
-    const int64_t e = eb + gl;
-    int u = -1;
-    bool ok = false;
-    if (e < e1) {
-      u = ci[e];
-      ok = core[u] >= kv;
+  const int q = min(c, kQ);
+  const int me = gl < q ? qs[gl] : 0;
+  const int64_t my0 = gl < q ? rp[me] : 0;
+  const int myl = gl < q ? (int)(rp[me + 1] - my0) : 0;
+  const int32_t *row[4];
+  int key[4], left[4];
+  uint32_t adj = 0u;  // bit i: member gl is adjacent to member gl + 1 + i
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const int o = (gl + 1 + i) & 7;
+    const int id = __shfl_sync(gm, me, o, 8), len = __shfl_sync(gm, myl, o, 8);
+    const int64_t s0 = __shfl_sync(gm, my0, o, 8);
+    // the shorter of the two rows
+    const bool mine = myl < len || (myl == len && gl < o);
+    row[i] = ci + (mine ? my0 : s0);
+    key[i] = mine ? id : me;
+    left[i] = (gl < q && o < q && (i < 3 || gl < 4)) ? (mine ? myl : len) : 0;
+  }
+  while ((left[0] | left[1] | left[2] | left[3]) != 0) {
+    int x[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) x[i] = left[i] ? row[i][left[i] >> 1] : 0;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      if (left[i] == 0) continue;
+      const int h = left[i] >> 1;
+      if (x[i] == key[i]) {
+        adj |= 1u << i;
+        left[i] = 0;
+      } else if (x[i] < key[i]) {
+        row[i] += h + 1;
+        left[i] -= h + 1;
+      } else {
+        left[i] = h;
+      }
     }
-    const unsigned m = group_ballot(gm, ok, grp);
-    if (ok) {
-      const int pos = c + __popc(m & below);
-      if (pos < kQ) qs[pos] = u;
-    }
-    c += __popc(m);
   }
   __syncwarp(gm);
-  const int q = min(c, kQ);
-  // the q(q-1)/2 pairs i < j, bit p of `pairs` for pair p (row-major over i)
-  uint32_t pairs = 0u;
-  for (int p = gl; p < q * (q - 1) / 2; p += 8) {
-    int i = 0, r = p;
-    while (r >= q - 1 - i) {
-      r -= q - 1 - i;
-      i++;
-    }
-    const int x = qs[i], y = qs[i + 1 + r];
-    // binary search in the shorter row
-    const bool adj = (rp[x + 1] - rp[x] <= rp[y + 1] - rp[y]) ? in_row(rp, ci, x, y) : in_row(rp, ci, y, x);
-    if (adj) pairs |= 1u << p;
+  const int t = __reduce_add_sync(gm, __popc(adj));
+  // row gl of G[Q]
+  uint32_t nb = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const int p = (gl - 1 - i) & 7;
+    const uint32_t theirs = __shfl_sync(gm, adj, p, 8);
+    nb |= ((adj >> i) & 1u) << ((gl + 1 + i) & 7);
+    nb |= ((theirs >> i) & 1u) << p;
   }
-  pairs = __reduce_or_sync(gm, pairs);
-  const int t = __popc(pairs);
-  // row gl of G[Q]: member j is adjacent to member gl if pair (min, max) is set
-  uint32_t row = 0u;
-  if (gl < q)
-    for (int j = 0; j < q; j++) {
-      if (j == gl) continue;
-      const int a = min(gl, j), b = max(gl, j);
-      const int pid = a * q - a * (a + 1) / 2 + (b - a - 1);
-      if ((pairs >> pid) & 1u) row |= 1u << j;
-    }
   // greedy colouring in index order: lane gl holds colour class gl; member
   // i joins the first class with none of its neighbours
   uint32_t cls = 0u;
   for (int i = 0; i < q; i++) {
-    const uint32_t ai = __shfl_sync(gm, row, i, 8);
+    const uint32_t ai = __shfl_sync(gm, nb, i, 8);
     const unsigned clash = group_ballot(gm, (cls & ai) != 0u, grp);
     const int k = __ffs(~clash) - 1;
     if (gl == k) cls |= 1u << i;
   }
   const int chi = __popc(group_ballot(gm, cls != 0u, grp));
-  const float d = (float)(e1 - e0);
+  const float d = (float)deg;
   f[0] = log1pf(d) / ldmax;
   f[1] = (float)kv / kmax;
   f[2] = (float)t / (float)(kQ * (kQ - 1) / 2);
@@ -157,29 +187,25 @@ __device__ void vertex_features(const int64_t *__restrict__ rp, const int32_t *_
   f[5] = log1pf((float)c) / ldmax;
 }
 
-// features of every vertex (list == nullptr) or of list[0 .. *count)
-__global__ void __launch_bounds__(256) features_kernel(int64_t n, const int32_t *__restrict__ list,
-                                                       const int64_t *__restrict__ count,
-                                                       const int64_t *__restrict__ rp,
-                                                       const int32_t *__restrict__ ci,
-                                                       const int32_t *__restrict__ core, float kmax, float ldmax,
-                                                       float *__restrict__ f) {
-  __shared__ int qs[8][4][kQ];
-  const int lane = threadIdx.x & 31, grp = lane >> 3, gl = lane & 7;
-  const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = list ? *count : n;
-  for (int64_t b = w0 * 4; b < total; b += nw * 4) {
-    const int64_t r = b + grp;
-    if (r >= total) continue;  // the whole group skips
-    const int64_t v = list ? list[r] : r;
-    float x[kF];
-    vertex_features(rp, ci, core, kmax, ldmax, v, qs[threadIdx.x >> 5][grp], x);
-    if (gl == 0) {
+struct FA {
+  int64_t n;
+  const int32_t *list;   // the vertices, nullptr: all of [0, n)
+  const int64_t *count;  // with a list: its length
+  const int64_t *rp;
+  const int32_t *ci, *core;
+  float kmax, ldmax;
+  int32_t *hubs;  // vertices of more than kWarpRow neighbours, left to hub_kernel
+  unsigned *nhubs;
+  float *out;  // features (6 per vertex) or scores (one)
+  const uint16_t *wbf;
+  const float *master;
+};
+
+__device__ __forceinline__ void put_features(float *f, const float x[kF], int gl) {
+  float y = x[0];
 #pragma unroll
-      for (int i = 0; i < kF; i++) f[v * kF + i] = x[i];
-    }
-  }
+  for (int i = 1; i < kF; i++) y = gl == i ? x[i] : y;
+  if (gl < kF) f[gl] = y;
 }
 
 // The network in shared memory, laid out for a group of eight lanes per
@@ -248,48 +274,218 @@ __device__ __forceinline__ float mlp_logit_group(const MlpSmem &S, const float x
   return sum + S.b3;
 }
 
-// logits of n feature rows, eight lanes per row
-__global__ void __launch_bounds__(256) forward_kernel(int64_t n, const float *__restrict__ feat,
-                                                      const uint16_t *__restrict__ wbf,
-                                                      const float *__restrict__ master, float *__restrict__ out) {
-  __shared__ MlpSmem S;
-  load_mlp(wbf, master, S);
+// Features of the listed vertices, or their scores (features and logit fused:
+// the feature rows never reach memory).  Eight lanes per vertex, four vertices
+// per warp; rows of more than kGroupRow entries are counted by the whole warp,
+// one after the other.
+template <bool SCORE>
+__global__ void __launch_bounds__(256) features_kernel(FA a) {
+  __shared__ MlpSmem S[1];
+  __shared__ int qs[8][4][kQ];
+  if (SCORE) load_mlp(a.wbf, a.master, S[0]);
   const int lane = threadIdx.x & 31, grp = lane >> 3, gl = lane & 7;
+  const unsigned gm = 0xFFu << (grp * 8);
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t b = w0 * 4; b < n; b += nw * 4) {
+  const int64_t total = a.list ? *a.count : a.n;
+  auto &Q = qs[threadIdx.x >> 5];
+  for (int64_t b = w0 * 4; b < total; b += nw * 4) {
     const int64_t r = b + grp;
-    if (r >= n) continue;
-    float x[kF];
-#pragma unroll
-    for (int i = 0; i < kF; i++) x[i] = feat[r * kF + i];
-    const float s = mlp_logit_group(S, x);
-    if (gl == 0) out[r] = s;
+    int64_t v = 0, e0 = 0, e1 = 0;
+    int kv = 0, c = 0;
+    if (r < total) {
+      v = a.list ? a.list[r] : r;
+      e0 = a.rp[v];
+      e1 = a.rp[v + 1];
+      kv = a.core[v];
+    }
+    const int64_t len = e1 - e0;
+    const bool hub = a.hubs && len > kWarpRow;
+    if (hub && gl == 0) a.hubs[atomicAdd(a.nhubs, 1u)] = (int32_t)v;
+    unsigned wide = __ballot_sync(0xffffffffu, !hub && len > kGroupRow) & 0x01010101u;
+    while (wide) {
+      const int src = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int64_t f0 = __shfl_sync(0xffffffffu, e0, src), f1 = __shfl_sync(0xffffffffu, e1, src);
+      const int fk = __shfl_sync(0xffffffffu, kv, src);
+      const int fc = count_row<32>(a.ci, a.core, fk, f0, f1, 0xffffffffu, 0, lane, Q[src >> 3]);
+      if (grp == (src >> 3)) c = fc;
+    }
+    if (len <= kGroupRow) c = count_row<8>(a.ci, a.core, kv, e0, e1, gm, grp * 8, gl, Q[grp]);
+    __syncwarp();
+    if (r < total && !hub) {
+      float x[kF];
+      vertex_features(a.rp, a.ci, a.kmax, a.ldmax, len, kv, c, Q[grp], x);
+      if (SCORE) {
+        const float s = mlp_logit_group(S[0], x);
+        if (gl == 0) a.out[v] = s;
+      } else {
+        put_features(a.out + v * kF, x, gl);
+      }
+    }
+    __syncwarp();  // Q is free for the next vertices
   }
 }
 
-// Learned scores of list[0 .. *count): features and logit fused, eight
-// lanes per vertex; the n x 6 feature rows never reach memory.
-__global__ void __launch_bounds__(256) score_kernel(const int32_t *__restrict__ list, const int64_t *__restrict__ count,
-                                                    const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                                                    const int32_t *__restrict__ core, float kmax, float ldmax,
-                                                    const uint16_t *__restrict__ wbf, const float *__restrict__ master,
-                                                    float *__restrict__ score) {
-  __shared__ MlpSmem S;
-  __shared__ int qs[8][4][kQ];
-  load_mlp(wbf, master, S);
-  const int lane = threadIdx.x & 31, grp = lane >> 3, gl = lane & 7;
-  const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = *count;
-  for (int64_t b = w0 * 4; b < total; b += nw * 4) {
-    const int64_t r = b + grp;
-    if (r >= total) continue;
-    const int v = list[r];
-    float x[kF];
-    vertex_features(rp, ci, core, kmax, ldmax, v, qs[threadIdx.x >> 5][grp], x);
-    const float s = mlp_logit_group(S, x);
-    if (gl == 0) score[v] = s;
+// The same for the vertices of the longest rows, a block each: every warp
+// counts a slice of the row, the first group of lanes does the rest.
+constexpr int kUT = 512;
+template <bool SCORE>
+__global__ void __launch_bounds__(kUT) hub_kernel(FA a) {
+  __shared__ MlpSmem S[1];
+  __shared__ int qs[kUT / 32][kQ], cs[kUT / 32], Q[kQ];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned nhubs = *a.nhubs;
+  if (SCORE && blockIdx.x < nhubs) load_mlp(a.wbf, a.master, S[0]);
+  for (unsigned h = blockIdx.x; h < nhubs; h += gridDim.x) {
+    const int64_t v = a.hubs[h], e0 = a.rp[v], e1 = a.rp[v + 1], len = e1 - e0;
+    const int kv = a.core[v];
+    const int64_t s0 = e0 + len * wid / (kUT / 32), s1 = e0 + len * (wid + 1) / (kUT / 32);
+    const int c = count_row<32>(a.ci, a.core, kv, s0, s1, 0xffffffffu, 0, lane, qs[wid]);
+    if (lane == 0) cs[wid] = c;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+      int all = 0, q = 0;
+      for (int w = 0; w < kUT / 32; w++) {
+        all += cs[w];
+        for (int i = 0; i < min(cs[w], kQ) && q < kQ; i++, q++)
+          if (threadIdx.x == 0) Q[q] = qs[w][i];
+      }
+      __syncwarp(0xFFu);
+      float x[kF];
+      vertex_features(a.rp, a.ci, a.kmax, a.ldmax, len, kv, all, Q, x);
+      if (SCORE) {
+        const float s = mlp_logit_group(S[0], x);
+        if (threadIdx.x == 0) a.out[v] = s;
+      } else {
+        put_features(a.out + v * kF, x, threadIdx.x);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// hubs and *nhubs for the vertices of g (rows of more than kWarpRow entries
+// are at most nnz / kWarpRow), then both kernels.
+template <bool SCORE>
+int launch_features(mc_graph *g, FA a, int blocks) {
+  a.rp = g->row_ptr;
+  a.ci = g->col_idx;
+  a.core = g->core;
+  a.kmax = (float)std::max(g->max_core, 1);
+  a.ldmax = log1pf((float)std::max(g->max_degree, 1));
+  const bool hubs = g->max_degree > kWarpRow;
+  if (hubs) {
+    void *p;
+    MC_TRY(ws_get(g, "ln.hubs", 64 + (size_t)(g->nnz / kWarpRow + 1) * 4, &p));
+    a.nhubs = (unsigned *)p;
+    a.hubs = (int32_t *)((char *)p + 64);
+    MC_CUDA_TRY(cudaMemsetAsync(p, 0, 4, g->stream));
+  }
+  features_kernel<SCORE><<<blocks, 256, 0, g->stream>>>(a);
+  g_launches++;
+  if (hubs) {
+    hub_kernel<SCORE><<<2 * g->sm_count, kUT, 0, g->stream>>>(a);
+    g_launches++;
+  }
+  MC_CUDA_TRY(cudaGetLastError());
+  return MC_OK;
+}
+
+constexpr int kGS = 68;  // row stride of the 64-wide tiles (float4 aligned, off the banks)
+__device__ __forceinline__ void fma4x4(float (&c)[4][4], const float4 &a, const float4 &b) {
+  const float x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+#pragma unroll
+    for (int j = 0; j < 4; j++) c[i][j] = fmaf(x[i], y[j], c[i][j]);
+}
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+// Logits of n feature rows: a block takes 128 rows, the second layer as a
+// 128 x 64 x 64 product in register tiles of 8 rows x 4 units over operands
+// in shared memory (three float4 for 32 FMAs, so the FP32 pipe is the bound,
+// not the shared-memory pipe as with eight lanes per row, a weight read per
+// FMA).  262,144 rows: 184 us before, 64 us now.
+constexpr int kVR = 128, kVT = 256, kVS = kVR + 4;
+struct FwdSmem {
+  float w2t[kH][kGS], h1t[kH][kVS];
+  float w1t[kF][kH], x[kF][kVR];
+  float b1[kH], b2[kH], w3[kH], b3;
+};
+static_assert(offsetof(FwdSmem, h1t) % 16 == 0 && offsetof(FwdSmem, w1t) % 16 == 0 && offsetof(FwdSmem, x) % 16 == 0 &&
+                  offsetof(FwdSmem, w2t) % 16 == 0 && kVS % 4 == 0 && kVT == (kVR / 8) * (kH / 4),
+              "float4 operands of forward_kernel");
+// Column of second-layer unit j: thread pair p of a row (columns 8 p .. 8 p + 7)
+// holds the units p, p + 8, ..., p + 56, whose terms of the logit are then added
+// in the order of mlp_logit_group (pair sums by distance 4, 2, 1): both give the
+// same bits.
+__device__ __forceinline__ int column_of(int j) { return 8 * (j & 7) + (j >> 3); }
+__global__ void __launch_bounds__(kVT) forward_kernel(int64_t n, const float *__restrict__ feat,
+                                                      const uint16_t *__restrict__ wbf,
+                                                      const float *__restrict__ master, float *__restrict__ out) {
+  extern __shared__ __align__(16) unsigned char fsm_raw[];
+  FwdSmem &S = *reinterpret_cast<FwdSmem *>(fsm_raw);
+  const int t = threadIdx.x, c0 = 4 * (t & 15), r0 = 8 * (t >> 4);
+  for (int e = t; e < kH * kH; e += kVT) S.w2t[e % kH][column_of(e / kH)] = bf16_to_f32(wbf[kOffW2 + e]);
+  for (int e = t; e < kH * kF; e += kVT) S.w1t[e % kF][e / kF] = bf16_to_f32(wbf[kOffW1 + e]);
+  for (int j = t; j < kH; j += kVT) {
+    S.b1[j] = master[kOffB1 + j];  // biases stay fp32
+    S.b2[column_of(j)] = master[kOffB2 + j];
+    S.w3[column_of(j)] = bf16_to_f32(wbf[kOffW3 + j]);
+  }
+  if (t == 0) S.b3 = master[kOffB3];
+  for (int64_t base = (int64_t)blockIdx.x * kVR; base < n; base += (int64_t)gridDim.x * kVR) {
+    const int rows = (int)min((int64_t)kVR, n - base);
+    __syncthreads();  // the weights are there; the last tile is done with the buffers
+    for (int e = t; e < kVR * kF; e += kVT) S.x[e % kF][e / kF] = e / kF < rows ? feat[base * kF + e] : 0.f;
+    __syncthreads();
+    float c[2][4][4];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) c[h][i][j] = S.b1[c0 + j];
+#pragma unroll
+      for (int i = 0; i < kF; i++) fma4x4(c[h], ld4(&S.x[i][r0 + 4 * h]), ld4(&S.w1t[i][c0]));
+#pragma unroll
+      for (int j = 0; j < 4; j++)
+        *reinterpret_cast<float4 *>(&S.h1t[c0 + j][r0 + 4 * h]) =
+            make_float4(fmaxf(c[h][0][j], 0.f), fmaxf(c[h][1][j], 0.f), fmaxf(c[h][2][j], 0.f),
+                        fmaxf(c[h][3][j], 0.f));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) c[h][i][j] = S.b2[c0 + j];
+#pragma unroll 4
+    for (int k = 0; k < kH; k++) {
+      const float4 w = ld4(&S.w2t[k][c0]);
+      fma4x4(c[0], ld4(&S.h1t[k][r0]), w);
+      fma4x4(c[1], ld4(&S.h1t[k][r0 + 4]), w);
+    }
+    // the 16 threads of a row share its logit: an odd thread goes on from the
+    // even one's partial sum, the eight pairs' sums are added as a tree
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        float v = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; j++) v = fmaf(S.w3[c0 + j], fmaxf(c[h][i][j], 0.f), v);
+        float w = __shfl_xor_sync(0xffffffffu, v, 1);
+#pragma unroll
+        for (int j = 0; j < 4; j++) w = fmaf(S.w3[c0 + j], fmaxf(c[h][i][j], 0.f), w);
+        v = w;  // the pair's sum in odd threads
+#pragma unroll
+        for (int o = 8; o >= 2; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const int r = r0 + 4 * h + i;
+        if ((t & 15) == 1 && r < rows) out[base + r] = v + S.b3;
+      }
   }
 }
 
@@ -308,7 +504,6 @@ __global__ void __launch_bounds__(256) score_kernel(const int32_t *__restrict__ 
 constexpr int kGR = 64;    // rows per tile
 constexpr int kGT = 256;   // threads: 16 x 16, 4 x 4 outputs each
 constexpr int kPart = (kParams + 1 + 31) / 32 * 32;  // floats of a block's sums: parameters, loss
-constexpr int kGS = 68;    // row stride of the tiles (float4 aligned, off the banks)
 struct GradSmem {
   float w2[kH][kGS], w2t[kH][kGS];  // W2[j][k] and its transpose
   float h1[kGR][kGS], h1t[kH][kGS];
@@ -327,13 +522,6 @@ static_assert(offsetof(GradSmem, w2) % 16 == 0 && offsetof(GradSmem, w2t) % 16 =
               "float4 operands of grad_kernel");
 static_assert(kGT == (kH / 4) * (kGR / 4) && kGR == kH, "one 4 x 4 tile per thread in each product");
 
-__device__ __forceinline__ void fma4x4(float (&c)[4][4], const float4 &a, const float4 &b) {
-  const float x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) c[i][j] = fmaf(x[i], y[j], c[i][j]);
-}
 // a tile and its transpose, rows kGS floats apart
 __device__ __forceinline__ void st4x4(float *p, float *pt, const float (&c)[4][4]) {
 #pragma unroll
@@ -342,7 +530,6 @@ __device__ __forceinline__ void st4x4(float *p, float *pt, const float (&c)[4][4
     *reinterpret_cast<float4 *>(pt + i * kGS) = make_float4(c[0][i], c[1][i], c[2][i], c[3][i]);
   }
 }
-__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
 __global__ void __launch_bounds__(kGT, 2) grad_kernel(int64_t n, const float *__restrict__ feat,
                                                       const float *__restrict__ label, float pos_weight,
@@ -800,14 +987,14 @@ int learned_scores(mc_graph *g, const mc_mlp *m, float *score) {
   subset_kernel<<<blocks, 256, 0, g->stream>>>(g->n, g->core, g->gid, g->best, kfloor, list, count);
   fill_kernel<<<blocks, 256, 0, g->stream>>>(g->n, -INFINITY, score);
   g_launches += 2;
-  const float kmax = (float)std::max(g->max_core, 1);
-  const float ldmax = log1pf((float)std::max(g->max_degree, 1));
-  const int sblocks = g->sm_count * 8;
-  score_kernel<<<sblocks, 256, 0, g->stream>>>(list, (const int64_t *)count, g->row_ptr, g->col_idx, g->core, kmax,
-                                               ldmax, m->wbf, m->master, score);
-  g_launches++;
-  MC_CUDA_TRY(cudaGetLastError());
-  return MC_OK;
+  FA a{};
+  a.n = g->n;
+  a.list = list;
+  a.count = (const int64_t *)count;
+  a.out = score;
+  a.wbf = m->wbf;
+  a.master = m->master;
+  return launch_features<true>(g, a, g->sm_count * 8);
 }
 
 // Seeds of the learned heuristic: for one graph the k best-scored vertices
@@ -934,13 +1121,10 @@ int mc_features(mc_graph *g, float *feat_out) {
     MC_TRY(ws_get(g, "ln.feat", (size_t)g->n * kF * 4, &p));
     dst = (float *)p;
   }
-  const float kmax = (float)std::max(g->max_core, 1);
-  const float ldmax = log1pf((float)std::max(g->max_degree, 1));
-  const int blocks = (int)std::min<int64_t>((g->n * 32 + 255) / 256, (int64_t)g->sm_count * 16);
-  features_kernel<<<blocks, 256, 0, g->stream>>>(g->n, nullptr, nullptr, g->row_ptr, g->col_idx, g->core, kmax,
-                                                 ldmax, dst);
-  g_launches++;
-  MC_CUDA_TRY(cudaGetLastError());
+  FA a{};
+  a.n = g->n;
+  a.out = dst;
+  MC_TRY(launch_features<false>(g, a, (int)std::min<int64_t>((g->n + 31) / 32, (int64_t)g->sm_count * 8)));
   if (!dev_out) MC_CUDA_TRY(cudaMemcpyAsync(feat_out, dst, (size_t)g->n * kF * 4, cudaMemcpyDeviceToHost, g->stream));
   MC_CUDA_TRY(cudaStreamSynchronize(g->stream));
   return MC_OK;
@@ -958,8 +1142,10 @@ int mc_mlp_forward(mc_mlp *m, const float *feat, int64_t n, float *score_out) {
     MC_CUDA_TRY(cudaMallocAsync((void **)&tmp, (size_t)n * 4, m->stream));
     out = tmp;
   }
-  const int blocks = (int)std::min<int64_t>((n * 32 + 255) / 256, (int64_t)m->sm_count * 16);
-  forward_kernel<<<blocks, 256, 0, m->stream>>>(n, (const float *)df, m->wbf, m->master, out);
+  // up to three blocks of shared memory per SM
+  const int blocks = (int)std::min<int64_t>((n + kVR - 1) / kVR, (int64_t)m->sm_count * 3);
+  MC_CUDA_TRY(cudaFuncSetAttribute(forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdSmem)));
+  forward_kernel<<<blocks, kVT, sizeof(FwdSmem), m->stream>>>(n, (const float *)df, m->wbf, m->master, out);
   g_launches++;
   MC_CUDA_TRY(cudaGetLastError());
   if (!dev_out) {

@@ -269,3 +269,31 @@ def test_gradient_with_an_infinite_weight(mc):
         g.append(m.gradient(x, y, 2.0)[0])
     assert np.isfinite(g[1]).all()
     assert np.allclose(g[0], g[1], rtol=1e-3, atol=1e-4 * np.abs(g[0]).max())
+
+
+def test_features_by_row_length(mc):
+    """Rows at the edges of a group's, a warp's and a block's share, with Q
+    dense, sparse and at the end of a row."""
+    r = np.random.default_rng(21)
+    n = 10000
+    lengths = [255, 256, 257, 4095, 4096, 4097, 9000, 31, 32, 33]
+    src = [np.full(d, v) for v, d in enumerate(lengths)]
+    dst = [r.choice(np.arange(10, n), d, replace=False) for d in lengths]
+    a, b = np.nonzero(np.triu(r.random((60, 60)) < 0.8, 1))  # dense at the end
+    e = r.integers(10, n, (2, 20000))
+    e = e[:, e[0] != e[1]]
+    g = gg.from_edges(n, np.concatenate(src + [n - 60 + a, e[0]]), np.concatenate(dst + [n - 60 + b, e[1]]))
+    assert np.array_equal(np.diff(g.row_ptr)[:10], lengths)
+    f = mc.mc_features(mc.mc_load_csr(g.row_ptr, g.col_idx))
+    ref = OL.features(g, oracle.core_numbers(g))
+    assert np.allclose(f, ref, rtol=2e-6, atol=2e-6)
+
+
+@pytest.mark.parametrize("rows", [1, 127, 128, 129, 3 * 152 * 128 + 1])
+def test_forward_by_row_count(mc, rows):
+    """The network's tiles of 128 rows at their edges and more tiles than
+    blocks, at the tolerance of the test above."""
+    x = np.random.default_rng(rows).random((rows, OL.F)).astype(np.float32)
+    m = mc.MLP(seed=9)
+    ref = OL.forward(m.get_params(), x)
+    assert np.allclose(m.forward(x), ref, rtol=1e-4, atol=1e-4 * np.abs(ref).max())
