@@ -12,10 +12,9 @@
 //           and the candidates are filtered to that member's neighbours.  A
 //           stored clique stays valid while all its members are alive (the
 //           vertices that died were rejected candidates, whose removal
-//           changes no decision of the greedy scan).  Warps check 32
-//           vertices at a time and grow the stale ones one after the other;
-//           vertices of more than 4,096 neighbours are grown by a whole
-//           block, one candidate slice per warp.
+//           changes no decision of the greedy scan).  A thread per vertex
+//           checks that and lists the stale ones; warps grow them, whole
+//           blocks those of more than 512 neighbours.
 //   scatter key(v) = |C(v)| << 32 | (2^31 - 1 - rank(v)); every member u of
 //           C(v) takes the largest key of the cliques holding it (atomicMax).
 //   accept  C(v) is accepted iff it holds the largest key at every member;
@@ -26,8 +25,8 @@
 //           accepted clique writes its members ranked by decreasing degree
 //           (ties: smaller id) and marks them dead.
 //
-// Rounds repeat until every vertex is placed (the host reads the placed
-// count after each round).  Cliques live in one arena laid out like the
+// Rounds repeat until every vertex is placed (four are queued before the host
+// reads the placed count; a round after the last vertex changes nothing).  Cliques live in one arena laid out like the
 // CSR: vertex v's candidates occupy the front of [rp[v], rp[v+1]) while it
 // grows, and its members other than v end at the top of that range, so the
 // arena is nnz int32 and needs no per-warp buffers or size limits.
@@ -53,15 +52,19 @@ constexpr int kOT = 256;         // threads per block of the warp-per-vertex ker
 constexpr int kWarpSortMax = 1024;
 constexpr int kBlockSortMax = 16384;
 constexpr int kBigT = 1024;      // threads of the block sorter
-constexpr int kBG = 512;         // threads of the block grower
-constexpr int kBGW = kBG / 32;
-constexpr int64_t kBlockGrowMin = 4096;  // neighbours above which a block grows the clique
-constexpr int kTake = 4;                 // listed vertices a warp takes at a time
+constexpr int kGT = 256;         // threads of a growing block
+constexpr int kGW = kGT / 32;
+constexpr int64_t kBlockGrowMin = 512;  // neighbours above which a block grows the clique
+constexpr int kTake = 4;                // listed vertices a warp takes at a time while there are many
+constexpr int kNear = 256;              // candidates, and entries of a row, that a warp holds in shared memory
+constexpr int kFly = 4;                 // entries or candidates a lane has in flight
+constexpr int kRoundsPerSync = 4;       // rounds queued before the host looks at the placed count
 
 struct OA {
   int64_t n;
   const int64_t *rp;
   const int32_t *ci, *core;
+  const unsigned long long *kd;  // core number (high word) and degree per vertex
   const int32_t *rank;  // tie rank per vertex, nullptr: the vertex id
   uint8_t *alive;
   int32_t *csize;  // stored clique size; 0: grow; negative: accepted this round
@@ -89,118 +92,176 @@ __device__ __forceinline__ bool ahead(const CKey &a, const CKey &b) {
   if (a.d != b.d) return a.d > b.d;
   return a.id < b.id;
 }
-__device__ __forceinline__ CKey warp_first(CKey x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    CKey y{__shfl_xor_sync(FULL, x.k, o), __shfl_xor_sync(FULL, x.d, o), __shfl_xor_sync(FULL, x.id, o)};
-    if (ahead(y, x)) x = y;
-  }
-  return x;
+// The warp's first key (core numbers and degrees are not negative).
+__device__ __forceinline__ CKey warp_first(const CKey &x) {
+  const int k = __reduce_max_sync(FULL, x.k);
+  const int d = __reduce_max_sync(FULL, x.k == k ? x.d : INT_MIN);
+  return CKey{k, d, __reduce_min_sync(FULL, (x.k == k && x.d == d) ? x.id : INT_MAX)};
 }
 __device__ __forceinline__ CKey ckey(const OA &a, int u) {
-  return CKey{a.core[u], (int)(a.rp[u + 1] - a.rp[u]), u};
+  const unsigned long long x = __ldg(a.kd + u);
+  return CKey{(int)(x >> 32), (int)(x & 0xffffffffu), u};
 }
-__device__ __forceinline__ bool in_row(const int64_t *rp, const int32_t *ci, int x, int y) {
-  int64_t lo = rp[x], hi = rp[x + 1];
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (ci[mid] < y) lo = mid + 1; else hi = mid;
-  }
-  return lo < rp[x + 1] && ci[lo] == y;
+__global__ void key_kernel(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ core,
+                           unsigned long long *__restrict__ kd) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    kd[v] = ((unsigned long long)(unsigned)core[v] << 32) | (unsigned)(rp[v + 1] - rp[v]);
 }
 __device__ __forceinline__ unsigned long long key_of(const OA &a, int v, int size) {
   const int r = a.rank ? a.rank[v] : v;
   return ((unsigned long long)(unsigned)size << 32) | (unsigned)(0x7fffffff - r);
 }
 
-// Windowed merge step of a greedy filter (all 32 lanes): lane candidate x
-// (INT_MAX past the end; `last` = the last valid lane) against w's row from
-// pos, which only moves forward; true iff x is in the row.
-__device__ __forceinline__ bool merge_hit(const OA &a, int x, int last, int64_t &pos, int64_t r1) {
-  const int xmin = __shfl_sync(FULL, x, 0), xmax = __shfl_sync(FULL, x, last);
-  int64_t p = pos;
-  while (p < r1) {
-    const int64_t e = min(p + 31, r1 - 1);
-    if (a.ci[e] >= xmin) break;
-    p = e + 1;
-  }
-  bool hit = false;
-  while (p < r1) {
-    const int y = (p + (threadIdx.x & 31) < r1) ? a.ci[p + (threadIdx.x & 31)] : INT_MAX;
-    int l = -1;  // largest window index with y <= x
-#pragma unroll
-    for (int st = 32; st >= 1; st >>= 1) {
-      const int t = l + st;
-      const int yt = __shfl_sync(FULL, y, t & 31);
-      if (t < 32 && yt <= x) l = t;
-    }
-    const int yl = __shfl_sync(FULL, y, l & 31);
-    if (l >= 0 && yl == x) hit = true;
-    const int ymax = __shfl_sync(FULL, y, 31);
-    if (ymax >= xmax) break;
-    p += 32;
-  }
-  pos = p;
-  return hit;
+// Fence posts of w's row [r0, r1): every step-th entry, at most cap of them, to
+// `post` (by nt threads, this one t).  A row of at most cap entries is held
+// whole (step 1).
+struct Fence {
+  const int32_t *post, *row;
+  int posts, top, len, step;
+};
+__device__ __forceinline__ Fence set_fence(const OA &a, int64_t r0, int64_t r1, int32_t *post, int cap, int t, int nt) {
+  Fence f;
+  f.row = a.ci + r0;
+  f.post = post;
+  f.len = (int)(r1 - r0);
+  f.step = (f.len + cap - 1) / cap;
+  f.posts = f.step ? (f.len + f.step - 1) / f.step : 0;
+  f.top = f.posts ? 1 << (31 - __clz(f.posts)) : 0;
+  for (int i = t; i < f.posts; i += nt) post[i] = f.row[(int64_t)i * f.step];
+  return f;
 }
 
-// Greedy growth of C(v) by one warp (all lanes): v's alive neighbours to the
-// front of its arena range (row order: ascending id), then pick the first
-// candidate by (core, degree, id) and keep the candidates adjacent to it
-// (binary search per candidate when the candidates are few against w's row,
-// else a merge), until none is left.  Member j (from 1) goes to rp[v+1] - j
-// after its filter: with cnt candidates left, cnt + j <= deg(v), so it lies
-// past them.  Returns |C(v)|.
-__device__ __forceinline__ int warp_grow(const OA &a, int v, unsigned long long &tests) {
+// Greedy filter step of one warp: candidates in[i0, i1) other than w that are
+// in w's row go to out, in order; their first key to nb.  Each lane looks up
+// kFly candidates side by side: a binary search of the fence posts in shared
+// memory, then of the step - 1 entries behind one.  in and out may be the same
+// list (a tile is read before anything of it is written).
+__device__ __forceinline__ int filter(const OA &a, const Fence &f, int w, const int32_t *in, int i0, int i1,
+                                      int32_t *out, CKey &nb) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const CKey none{INT_MIN, INT_MIN, INT_MAX};
-  const int64_t e0 = a.rp[v], e1 = a.rp[v + 1];
-  int32_t *cand = a.arena + e0;
-  int cnt = 0;
-  CKey bk = none;
-  for (int64_t eb = e0; eb < e1; eb += 32) {
-    const int64_t e = eb + lane;
-    int u = -1;
-    bool ok = false;
-    if (e < e1) {
-      u = a.ci[e];
-      ok = a.alive[u] != 0;
+  int kept = 0;
+  for (int base = i0; base < i1; base += 32 * kFly) {
+    int x[kFly], lo[kFly], left[kFly];
+    bool keep[kFly];
+#pragma unroll
+    for (int q = 0; q < kFly; q++) {
+      const int i = base + 32 * q + lane;
+      x[q] = i < i1 ? in[i] : -1;
+      lo[q] = 0;  // posts <= x
     }
-    const unsigned m = __ballot_sync(FULL, ok);
-    if (ok) {
-      cand[cnt + __popc(m & lt)] = u;
-      const CKey k = ckey(a, u);
-      if (ahead(k, bk)) bk = k;
+    for (int st = f.top; st > 0; st >>= 1) {
+#pragma unroll
+      for (int q = 0; q < kFly; q++)
+        if (base + 32 * q < i1 && lo[q] + st <= f.posts && f.post[lo[q] + st - 1] <= x[q]) lo[q] += st;
     }
-    cnt += __popc(m);
+    int any = 0;
+#pragma unroll
+    for (int q = 0; q < kFly; q++) {
+      keep[q] = lo[q] > 0 && f.post[lo[q] - 1] == x[q];
+      const int at = (lo[q] - 1) * f.step + 1;
+      left[q] = (lo[q] > 0 && !keep[q]) ? min(f.step - 1, f.len - at) : 0;
+      lo[q] = at;
+      any |= left[q];
+    }
+    while (any) {
+      int y[kFly];
+#pragma unroll
+      for (int q = 0; q < kFly; q++) y[q] = left[q] ? f.row[lo[q] + (left[q] >> 1)] : 0;
+      any = 0;
+#pragma unroll
+      for (int q = 0; q < kFly; q++) {
+        if (left[q] == 0) continue;
+        const int h = left[q] >> 1;
+        if (y[q] == x[q]) {
+          keep[q] = true;
+          left[q] = 0;
+        } else if (y[q] < x[q]) {
+          lo[q] += h + 1;
+          left[q] -= h + 1;
+        } else {
+          left[q] = h;
+        }
+        any |= left[q];
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < kFly; q++) {
+      keep[q] = keep[q] && x[q] != w;
+      const unsigned m = __ballot_sync(FULL, keep[q]);
+      if (keep[q]) {
+        out[kept + __popc(m & lt)] = x[q];
+        const CKey k = ckey(a, x[q]);
+        if (ahead(k, nb)) nb = k;
+      }
+      kept += __popc(m);
+    }
+    __syncwarp();
   }
-  __syncwarp();
-  bk = warp_first(bk);
-  int j = 0;
+  return kept;
+}
+
+// A growing warp's shared memory.
+struct GrowSmem {
+  int32_t post[kGW][kNear], cand[kGW][kNear];
+};
+
+// Alive entries of v's row [s0, s1), one warp: to out (row order: ascending
+// id), their first key to bk.
+__device__ __forceinline__ int alive_of(const OA &a, int64_t s0, int64_t s1, int32_t *out, CKey &bk) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  int cnt = 0;
+  for (int64_t eb = s0; eb < s1; eb += 32 * kFly) {
+    int u[kFly];
+    bool ok[kFly];
+#pragma unroll
+    for (int q = 0; q < kFly; q++) {
+      const int64_t e = eb + 32 * q + lane;
+      u[q] = e < s1 ? a.ci[e] : -1;
+    }
+#pragma unroll
+    for (int q = 0; q < kFly; q++) ok[q] = u[q] >= 0 && a.alive[u[q]] != 0;
+#pragma unroll
+    for (int q = 0; q < kFly; q++) {
+      const unsigned m = __ballot_sync(FULL, ok[q]);
+      if (ok[q]) {
+        out[cnt + __popc(m & lt)] = u[q];
+        const CKey k = ckey(a, u[q]);
+        if (ahead(k, bk)) bk = k;
+      }
+      cnt += __popc(m);
+    }
+  }
+  return cnt;
+}
+
+// Greedy growth of C(v) by one warp (all lanes) from cnt candidates (in
+// ascending id) whose first key is bk, j members found so far: take the first
+// candidate, keep the candidates adjacent to it, until none is left.  The
+// candidates are in shared memory once they are at most kNear; before that at
+// the front of v's arena range, where member j (from 1) goes to rp[v+1] - j
+// after its filter: with cnt candidates left, cnt + j <= deg(v), so it lies
+// past them.  Returns |C(v)|.
+__device__ __forceinline__ int warp_steps(const OA &a, int64_t e1, int32_t *cand, int cnt, CKey bk, int j,
+                                          int32_t *post, int32_t *near, unsigned long long &tests) {
+  const int lane = threadIdx.x & 31;
+  const CKey none{INT_MIN, INT_MIN, INT_MAX};
   while (cnt > 0) {
+    if (cand != near && cnt <= kNear) {
+      for (int i = lane; i < cnt; i += 32) near[i] = cand[i];
+      cand = near;
+    }
     const int w = bk.id;
-    const int64_t r0 = a.rp[w], r1 = a.rp[w + 1];
-    const bool merge = (int64_t)cnt * 16 >= (r1 - r0);
     tests += (unsigned long long)cnt;
     int out = 0;
     CKey nb = none;
-    int64_t pos = r0;
-    for (int base = 0; base < cnt; base += 32) {
-      const int i = base + lane;
-      const int x = (i < cnt) ? cand[i] : INT_MAX;
-      bool keep;
-      if (!merge) keep = i < cnt && x != w && in_row(a.rp, a.ci, w, x);
-      else keep = merge_hit(a, x, min(31, cnt - 1 - base), pos, r1) && i < cnt && x != w;
-      const unsigned m = __ballot_sync(FULL, keep);
+    if (cnt > 1) {
       __syncwarp();
-      if (keep) {
-        cand[out + __popc(m & lt)] = x;
-        const CKey k = ckey(a, x);
-        if (ahead(k, nb)) nb = k;
-      }
-      out += __popc(m);
+      const Fence f = set_fence(a, a.rp[w], a.rp[w + 1], post, kNear, lane, 32);
       __syncwarp();
+      out = filter(a, f, w, cand, 0, cnt, cand, nb);
     }
     cnt = out;
     j++;
@@ -249,21 +310,126 @@ __global__ void check_kernel(OA a) {
   }
 }
 
-// grow: each warp takes the next kTake listed vertices as it frees up, so a
-// few long growths (the dense core's, every round) do not hold back the rest
-__global__ void __launch_bounds__(kOT) grow_kernel(OA a) {
-  const int lane = threadIdx.x & 31;
-  const unsigned total = *a.nstale;
+// First candidate over the block (contains two __syncthreads).
+__device__ __forceinline__ CKey block_first(CKey x, CKey *sk) {
+  x = warp_first(x);
+  if ((threadIdx.x & 31) == 0) sk[threadIdx.x >> 5] = x;
+  __syncthreads();
+  CKey r = sk[0];
+#pragma unroll
+  for (int i = 1; i < kGW; i++)
+    if (ahead(sk[i], r)) r = sk[i];
+  __syncthreads();
+  return r;
+}
+// This warp's place among the block's counts (contains a __syncthreads before
+// the read; the caller syncs before scnt is written again).
+__device__ __forceinline__ int block_place(int c, int *scnt, int *tot) {
+  const int wid = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) scnt[wid] = c;
+  __syncthreads();
+  int before = 0, all = 0;
+#pragma unroll
+  for (int i = 0; i < kGW; i++) {
+    const int x = scnt[i];
+    before += i < wid ? x : 0;
+    all += x;
+  }
+  *tot = all;
+  return before;
+}
+
+// The same growth by a whole block, for vertices of many neighbours: one slice
+// of the candidates per warp, filtered to a scratch row and packed back in
+// order; the fence posts are the block's.  What is left goes to the first warp
+// once it fits its shared memory.
+__device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt, CKey *sk,
+                          unsigned long long &tests) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const CKey none{INT_MIN, INT_MIN, INT_MAX};
+  const int64_t e0 = a.rp[v], e1 = a.rp[v + 1], len = e1 - e0;
+  int32_t *A = a.arena + e0;
+  int64_t s0 = len * wid / kGW, s1 = len * (wid + 1) / kGW;
+  CKey nb = none;
+  int c = alive_of(a, e0 + s0, e0 + s1, B + s0, nb);
+  int cnt, j = 0;
+  for (;;) {
+    __syncwarp();
+    const int at = block_place(c, scnt, &cnt);
+    for (int i = lane; i < c; i += 32) A[at + i] = B[s0 + i];
+    const CKey bk = block_first(nb, sk);
+    if (cnt <= kNear) {
+      int size = 0;
+      if (wid == 0) size = warp_steps(a, e1, A, cnt, bk, j, S.post[0], S.cand[0], tests);
+      __syncthreads();
+      return size;  // of the first warp
+    }
+    const int w = bk.id;
+    if (threadIdx.x == 0) tests += (unsigned long long)cnt;
+    const Fence f = set_fence(a, a.rp[w], a.rp[w + 1], &S.post[0][0], kGW * kNear, threadIdx.x, kGT);
+    __syncthreads();
+    s0 = (int64_t)cnt * wid / kGW;
+    s1 = (int64_t)cnt * (wid + 1) / kGW;
+    nb = none;
+    c = filter(a, f, w, A, (int)s0, (int)s1, B + s0, nb);
+    j++;
+    __syncthreads();  // A has been read
+    // cnt + j <= deg(v): the member's slot lies past the packed candidates
+    if (threadIdx.x == 0) a.arena[e1 - j] = w;
+  }
+}
+
+// grow: the listed vertices of many neighbours by the first blocks (those with
+// a scratch row), the others by warps, each taking the next as it frees up, so
+// that a few long growths (the dense core's, every round) do not hold back the
+// rest.  The longest chain of dependent loads is what a round takes: a step of
+// a growth is the next member's row bounds, its fence posts, at most
+// log2(length / 256) further entries of it and the kept candidates' keys.
+// R-MAT scale 16, all rounds: 5.1 ms with 8 warps per SM, rows searched or
+// merged in L2 and blocks only above 4,096 neighbours; 2.0 ms now (blocks above
+// 512; above 1,024 or 2,048: 3.56 or 3.95 ms per order instead of 3.70 at this
+// scale, 5.83 or 5.87 instead of 5.51 at scale 17).
+__global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, int64_t scratch_stride, int big_blocks) {
+  __shared__ GrowSmem S;
+  __shared__ CKey sk[kGW];
+  __shared__ int scnt[kGW];
+  __shared__ unsigned s_b;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const CKey none{INT_MIN, INT_MIN, INT_MAX};
   unsigned long long grows = 0, tests = 0;
+  const unsigned nbig = *a.nbig;
+  if ((int)blockIdx.x < big_blocks && nbig) {
+    for (;;) {
+      if (threadIdx.x == 0) s_b = atomicAdd(a.take_big, 1u);
+      __syncthreads();
+      const unsigned b = s_b;
+      __syncthreads();
+      if (b >= nbig) break;
+      const int v = a.big[b];
+      const int size = block_grow(a, v, scratch + blockIdx.x * scratch_stride, S, scnt, sk, tests);
+      if (threadIdx.x == 0) {
+        a.csize[v] = size;
+        grows++;
+      }
+    }
+  }
+  const unsigned total = *a.nstale;
+  const unsigned chunk = total > 8u * kGW * gridDim.x ? (unsigned)kTake : 1u;
   for (;;) {
     unsigned idx = 0;
-    if (lane == 0) idx = atomicAdd(a.take, (unsigned)kTake);
+    if (lane == 0) idx = atomicAdd(a.take, chunk);
     idx = __shfl_sync(FULL, idx, 0);
     if (idx >= total) break;
-    const unsigned end = min(total, idx + (unsigned)kTake);
+    const unsigned end = min(total, idx + chunk);
     for (unsigned t = idx; t < end; t++) {
       const int v = a.stale[t];
-      const int size = warp_grow(a, v, tests);
+      const int64_t e0 = a.rp[v], e1 = a.rp[v + 1];
+      int32_t *cand = e1 - e0 <= kNear ? S.cand[wid] : a.arena + e0;
+      CKey bk = none;
+      __syncwarp();
+      const int cnt = alive_of(a, e0, e1, cand, bk);
+      __syncwarp();
+      const int size = warp_steps(a, e1, cand, cnt, warp_first(bk), 0, S.post[wid], S.cand[wid], tests);
       if (lane == 0) {
         a.csize[v] = size;
         grows++;
@@ -272,129 +438,6 @@ __global__ void __launch_bounds__(kOT) grow_kernel(OA a) {
   }
   if (lane == 0 && grows) atomicAdd((unsigned long long *)(a.ctl + 2), grows);
   if (lane == 0 && tests) atomicAdd((unsigned long long *)(a.ctl + 3), tests);
-}
-
-// First candidate over the block (contains two __syncthreads).
-__device__ __forceinline__ CKey block_first(CKey x, CKey *sk) {
-  x = warp_first(x);
-  if ((threadIdx.x & 31) == 0) sk[threadIdx.x >> 5] = x;
-  __syncthreads();
-  CKey r = sk[0];
-#pragma unroll
-  for (int i = 1; i < kBGW; i++)
-    if (ahead(sk[i], r)) r = sk[i];
-  __syncthreads();
-  return r;
-}
-
-// The same greedy growth by a whole block, for vertices of many neighbours:
-// the candidates are split into one slice per warp, each warp merges its
-// slice against w's row from the slice's first candidate on and writes what
-// it keeps to a scratch row, and the kept runs are packed back in order.
-__global__ void __launch_bounds__(kBG) grow_big_kernel(OA a, int32_t *scratch, int64_t scratch_stride) {
-  __shared__ CKey sk[kBGW];
-  __shared__ int scnt[kBGW];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const unsigned lt = (1u << lane) - 1u;
-  const CKey none{INT_MIN, INT_MIN, INT_MAX};
-  __shared__ unsigned s_b;
-  const unsigned nbig = *a.nbig;
-  int32_t *B = scratch + blockIdx.x * scratch_stride;
-  unsigned long long grows = 0, tests = 0;
-  for (;;) {
-    // the next listed vertex, taken as the block frees up
-    if (threadIdx.x == 0) s_b = atomicAdd(a.take_big, 1u);
-    __syncthreads();
-    const unsigned b = s_b;
-    __syncthreads();
-    if (b >= nbig) break;
-    const int v = a.big[b];
-    const int64_t e0 = a.rp[v], e1 = a.rp[v + 1];
-    int32_t *A = a.arena + e0;
-    int cnt = 0;
-    CKey bk = none;
-    for (int64_t tb = e0; tb < e1; tb += kBG) {
-      const int64_t e = tb + threadIdx.x;
-      int u = -1;
-      bool ok = false;
-      if (e < e1) {
-        u = a.ci[e];
-        ok = a.alive[u] != 0;
-      }
-      const unsigned m = __ballot_sync(FULL, ok);
-      if (lane == 0) scnt[wid] = __popc(m);
-      __syncthreads();
-      int before = 0, tot = 0;
-#pragma unroll
-      for (int i = 0; i < kBGW; i++) {
-        const int c = scnt[i];
-        before += i < wid ? c : 0;
-        tot += c;
-      }
-      if (ok) {
-        A[cnt + before + __popc(m & lt)] = u;
-        const CKey k = ckey(a, u);
-        if (ahead(k, bk)) bk = k;
-      }
-      cnt += tot;
-      __syncthreads();
-    }
-    bk = block_first(bk, sk);
-    int j = 0;
-    while (cnt > 0) {
-      const int w = bk.id;
-      const int64_t r0 = a.rp[w], r1 = a.rp[w + 1];
-      if (threadIdx.x == 0) tests += (unsigned long long)cnt;
-      const int s0 = (int)((int64_t)cnt * wid / kBGW), s1 = (int)((int64_t)cnt * (wid + 1) / kBGW);
-      int out = 0;
-      CKey nb = none;
-      if (s0 < s1) {
-        // the row from its first entry >= A[s0]
-        const int x0 = A[s0];
-        int64_t lo = r0, hi = r1;
-        while (lo < hi) {
-          const int64_t mid = (lo + hi) >> 1;
-          if (a.ci[mid] < x0) lo = mid + 1; else hi = mid;
-        }
-        int64_t pos = lo;
-        for (int base = s0; base < s1; base += 32) {
-          const int i = base + lane;
-          const int x = i < s1 ? A[i] : INT_MAX;
-          const bool keep = merge_hit(a, x, min(31, s1 - 1 - base), pos, r1) && i < s1 && x != w;
-          const unsigned m = __ballot_sync(FULL, keep);
-          if (keep) {
-            B[s0 + out + __popc(m & lt)] = x;
-            const CKey k = ckey(a, x);
-            if (ahead(k, nb)) nb = k;
-          }
-          out += __popc(m);
-        }
-      }
-      if (lane == 0) scnt[wid] = out;
-      __syncthreads();
-      int before = 0, tot = 0;
-#pragma unroll
-      for (int i = 0; i < kBGW; i++) {
-        const int c = scnt[i];
-        before += i < wid ? c : 0;
-        tot += c;
-      }
-      for (int i = lane; i < out; i += 32) A[before + i] = B[s0 + i];
-      cnt = tot;
-      j++;
-      bk = block_first(nb, sk);
-      // cnt + j <= deg(v): the member slot lies past the packed candidates
-      if (threadIdx.x == 0) a.arena[e1 - j] = w;
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      a.csize[v] = 1 + j;
-      grows++;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && grows) atomicAdd((unsigned long long *)(a.ctl + 2), grows);
-  if (threadIdx.x == 0 && tests) atomicAdd((unsigned long long *)(a.ctl + 3), tests);
 }
 
 // scatter: every member takes the largest key of the cliques holding it
@@ -489,7 +532,7 @@ __global__ void advance_kernel(int64_t *ctl) {
   const int64_t t = ctl[5];
   ctl[0] += t & 0xffffffffLL;
   ctl[1] += t >> 32;
-  ctl[4] += 1;
+  ctl[4] += t != 0;  // (a round that was queued after the last vertex was placed has none)
   ((unsigned *)(ctl + 6))[0] = 0u;  // the growers' lists, empty for the next round
   ((unsigned *)(ctl + 6))[1] = 0u;
   ((unsigned *)(ctl + 7))[0] = 0u;
@@ -744,6 +787,10 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
     MC_CUDA_TRY(cudaStreamSynchronize(g->stream));
     if (*(int32_t *)g->h_small) return MC_ERR_ARG;
   }
+  MC_TRY(ws_get(g, "co.kd", (size_t)n * 8, &p));
+  a.kd = (const unsigned long long *)p;
+  key_kernel<<<grid_of(g, n, 256, 8), 256, 0, g->stream>>>(n, a.rp, a.core, (unsigned long long *)p);
+  g_launches++;
   MC_CUDA_TRY(cudaMemsetAsync(a.alive, 1, (size_t)n, g->stream));
   MC_CUDA_TRY(cudaMemsetAsync(a.csize, 0, (size_t)n * 4, g->stream));
   a.nbig = (unsigned *)(a.ctl + 6);
@@ -753,7 +800,7 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
   MC_TRY(ws_get(g, "co.stale", (size_t)n * 4, &p));
   a.stale = (int32_t *)p;
   int32_t *scratch = nullptr;
-  const int big_blocks = 2 * g->sm_count;
+  const int big_blocks = 2 * g->sm_count, grow_blocks = 4 * g->sm_count;
   const int64_t stride = std::max<int64_t>(g->max_degree, 1);
   const bool any_big = g->max_degree > kBlockGrowMin;
   if (any_big) {
@@ -765,23 +812,19 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
   const int gw = grid_of(g, (n + 31) / 32, kOT / 32, 8), gt = grid_of(g, n, 256, 8);
   int64_t *h = (int64_t *)((char *)g->h_small + 2560);
   int64_t placed = 0;
-  for (int32_t r = 0;; r++) {
-    a.round = r;
-    check_kernel<<<gt, 256, 0, g->stream>>>(a);
-    grow_kernel<<<gw, kOT, 0, g->stream>>>(a);
-    g_launches++;
-    if (any_big) {
-      grow_big_kernel<<<big_blocks, kBG, 0, g->stream>>>(a, scratch, stride);
-      g_launches++;
+  for (int32_t r = 0;;) {
+    for (int i = 0; i < kRoundsPerSync; i++) {
+      a.round = r++;
+      check_kernel<<<gt, 256, 0, g->stream>>>(a);
+      grow_kernel<<<grow_blocks, kGT, 0, g->stream>>>(a, scratch, stride, any_big ? big_blocks : 0);
+      scatter_kernel<<<gt, 256, 0, g->stream>>>(a);
+      accept_kernel<<<gt, 256, 0, g->stream>>>(a);
+      MC_CUDA_TRY(cudaGetLastError());
+      MC_TRY(device_scan(g, n, AccF{a.csize}, AccG{a.goff}, a.ctl + 5, "co.scan"));
+      place_kernel<<<gw, kOT, 0, g->stream>>>(a);
+      advance_kernel<<<1, 1, 0, g->stream>>>(a.ctl);
+      g_launches += 6;
     }
-    scatter_kernel<<<gt, 256, 0, g->stream>>>(a);
-    accept_kernel<<<gt, 256, 0, g->stream>>>(a);
-    g_launches += 3;
-    MC_CUDA_TRY(cudaGetLastError());
-    MC_TRY(device_scan(g, n, AccF{a.csize}, AccG{a.goff}, a.ctl + 5, "co.scan"));
-    place_kernel<<<gw, kOT, 0, g->stream>>>(a);
-    advance_kernel<<<1, 1, 0, g->stream>>>(a.ctl);
-    g_launches += 2;
     MC_CUDA_TRY(cudaGetLastError());
     MC_CUDA_TRY(cudaMemcpyAsync(h, a.ctl, 6 * sizeof(int64_t), cudaMemcpyDeviceToHost, g->stream));
     MC_CUDA_TRY(cudaStreamSynchronize(g->stream));

@@ -93,6 +93,35 @@ def test_clique_order_hub_beyond_4096_bit_exact(mc):
     h.close()
 
 
+def _rows_of(lengths, n=6000, seed=5):
+    """Vertices 0.. of the given degrees, over a sparse random graph with a
+    dense end (so that candidates remain in the last part of long rows)."""
+    rng = np.random.default_rng(seed)
+    h = len(lengths)
+    src = [np.full(d, v) for v, d in enumerate(lengths)] + [rng.integers(h, n, 2 * n)]
+    dst = [np.arange(n - d, n) for d in lengths] + [rng.integers(h, n, 2 * n)]
+    a, b = np.nonzero(np.triu(rng.random((70, 70)) < 0.7, 1))
+    src, dst = np.concatenate(src + [n - 70 + a]), np.concatenate(dst + [n - 70 + b])
+    keep = src != dst
+    return gg.from_edges(n, src[keep], dst[keep], name="rows%d" % h)
+
+
+@pytest.mark.parametrize("g", [
+    gg.complete(257), gg.complete(258), gg.complete(513), gg.complete(514), gg.turan(700, 20), gg.turan(400, 3),
+    gg.erdos_renyi(800, 0.75, planted=30, seed=4), _rows_of([255, 256, 257, 511, 512, 513, 2048, 2049, 4100, 5000]),
+    ], ids=lambda g: g.name)
+def test_clique_order_by_row_length_bit_exact(mc, g):
+    """Rows and candidate lists on both sides of what a warp holds in shared
+    memory (256) and of a block's share (512), rows longer than a block's
+    fence posts (2,048), candidate lists that a block hands to its first
+    warp at once, late, or never short of 256."""
+    want = OO.clique_order(g, oracle.core_numbers(g))
+    h = load(mc, g)
+    order, starts, rounds, _ = mc.mc_clique_order(h)
+    assert np.array_equal(order, want[0]) and np.array_equal(starts, want[1]) and np.array_equal(rounds, want[2])
+    h.close()
+
+
 @pytest.mark.parametrize("seed", [0, 1, 2])
 def test_clique_order_with_rank_bit_exact(mc, seed):
     g = [gg.path(64), gg.rmat(10, 8, planted=10, seed=9), gg.chung_lu(3000, 2.4, 8.0, 200.0, planted=9, seed=4)][seed]
