@@ -1015,24 +1015,14 @@ int mc_gap_bits(mc_graph *g, const int32_t *order, double *bits_out) {
   *bits_out = 0.0;
   if (g->nnz == 0) return MC_OK;
   void *p;
-  const int64_t *rp = g->row_ptr;
-  const int32_t *ci = g->col_idx;
-  if (order) {
-    MC_TRY(ws_get(g, "rl.nrp", (size_t)(g->n + 1) * 8, &p));
-    int64_t *d_nrp = (int64_t *)p;
-    MC_TRY(ws_get(g, "rl.nci", (size_t)g->nnz * 4, &p));
-    int32_t *d_nci = (int32_t *)p;
-    MC_TRY(relabel(g, order, d_nrp, d_nci));
-    rp = d_nrp;
-    ci = d_nci;
-  }
   MC_TRY(ws_get(g, "rl.sum", 8, &p));
-  double *d_sum = (double *)p;
-  MC_TRY(gap_bits(g, rp, ci, d_sum));
-  MC_CUDA_TRY(cudaMemcpyAsync(g->h_small, d_sum, 8, cudaMemcpyDeviceToHost, g->stream));
+  if (order) MC_TRY(gap_bits_of(g, order, (unsigned long long *)p));
+  else MC_TRY(gap_bits(g, g->row_ptr, g->col_idx, (double *)p));
+  MC_CUDA_TRY(cudaMemcpyAsync(g->h_small, p, 8, cudaMemcpyDeviceToHost, g->stream));
   MC_CUDA_TRY(cudaStreamSynchronize(g->stream));
   MC_TRY(check_device_error(g));
-  *bits_out = *(double *)g->h_small / (double)g->nnz;
+  const double sum = order ? (double)*(unsigned long long *)g->h_small / kGapUnit : *(double *)g->h_small;
+  *bits_out = sum / (double)g->nnz;
   return MC_OK;
 }
 

@@ -214,6 +214,10 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
 int relabel(mc_graph *g, const int32_t *order, int64_t *d_nrp, int32_t *d_nci);
 // *d_total = sum over the entries of a sorted CSR of log2(1 + gap).
 int gap_bits(mc_graph *g, const int64_t *d_nrp, const int32_t *d_nci, double *d_total);
+// The same for the graph relabelled by `order` (host or device), in units of 1 / kGapUnit; MC_ERR_ARG if it is
+// no permutation.
+constexpr float kGapUnit = 16777216.f;
+int gap_bits_of(mc_graph *g, const int32_t *order, unsigned long long *d_total);
 int launch_gid(mc_graph *g);
 // Stable radix sort of (key, value) pairs by decreasing key (sort.cu); the
 // result is back in keys / vals, ktmp / vtmp are n-entry scratch.

@@ -32,11 +32,12 @@
 // arena is nnz int32 and needs no per-warp buffers or size limits.
 //
 // The gap cost relabels the graph by an order (new id = position), sorts
-// every new row (bitonic networks: a warp in registers up to 32 entries, a
-// warp in shared memory up to 1,024, a block in shared memory up to 16,384,
-// a block over a global scratch row beyond), and sums log2(1 + gap) over the
-// entries, the first gap of row p taken from p itself: 1 + gap rounded once
-// to single precision, log2f (within 1 ulp), summed in double.
+// every new row (bitonic networks in a warp's registers up to 1,024 entries;
+// above, a block sets a bit per entry and reads the bits in order, or runs the
+// network in shared memory), and sums log2(1 + gap) over the entries, the
+// first gap of row p taken from p itself: 1 + gap rounded once to single
+// precision, log2f (within 1 ulp), summed exactly in units of 2^-24 (in double
+// for the graph as it was loaded).
 #include <algorithm>
 #include <climits>
 
@@ -571,60 +572,222 @@ struct RowG {
   __device__ void operator()(int64_t p, int64_t excl, int64_t) const { nrp[p] = excl; }
 };
 
-// a warp per new row: copy the old row through pos, sort rows of at most
-// kWarpSortMax entries at once (bitonic; registers up to 32, shared memory
-// above), and list the longer rows for the block sorter
-__global__ void __launch_bounds__(kOT) fill_sort_kernel(int64_t n, const int64_t *rp, const int32_t *ci,
-                                                        const int32_t *order, const int32_t *pos,
-                                                        const int64_t *nrp, int32_t *nci, int32_t *big,
-                                                        unsigned long long *nbig) {
-  __shared__ int32_t sm[kOT / 32][kWarpSortMax];
+// One term of the gap cost: log2(1 + gap) in single precision (one rounding of
+// 1 + gap, log2f within 1 ulp, so a relative error below 2^-22).
+__device__ __forceinline__ float gap_term(int x, int prev, bool first) {
+  const int gap = first ? abs(x - prev) : x - prev;
+  return log2f((float)(gap + 1));
+}
+
+// The term in units of 2^-24: exact, since a term of a sorted row without
+// repeats is log2f of at least 2, so above one half, and below 32; a repeat's
+// is 0.  The integer sum is exact as well, and cheaper than doubles on this
+// chip (gap cost of R-MAT scale 18: 345 us with doubles, 327 us with integers,
+// everything else alike).
+__device__ __forceinline__ int64_t gap_fixed(int x, int prev, bool first) {
+  return (int64_t)__float2int_rn(gap_term(x, prev, first) * kGapUnit);
+}
+
+struct RA {
+  int64_t n;
+  const int64_t *rp;
+  const int32_t *ci, *order, *pos;
+  // the rows' place in nci: nrp[p] (relabelling), or nullptr: the old row's own
+  // range (the gap cost, which needs memory for the long rows only)
+  const int64_t *nrp;
+  int32_t *nci;
+  int32_t *mid, *big;  // rows of 33 .. kWarpSortMax entries, and of more
+  unsigned *nmid;
+  unsigned long long *nbig;
+  unsigned long long *total;  // the gap cost's sum
+};
+
+// Bitonic sort of 32 R integers in a warp's registers; x[r] of lane l is item
+// l R + r, so only the stages across lanes need shuffles.  The merges are a
+// loop: unrolled over all sizes of R the code did not stay in the instruction
+// cache (134 us instead of 70 for the rows of 33 .. 1,024 entries of R-MAT
+// scale 18, 225 instead of 80 with the gap cost).
+template <int R>
+__device__ __forceinline__ void merge_lane(int (&x)[R], bool up) {
+#pragma unroll
+  for (int j = R / 2; j > 0; j >>= 1) {
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      if (r & j) continue;
+      const int lo = min(x[r], x[r | j]), hi = max(x[r], x[r | j]);
+      x[r] = up ? lo : hi;
+      x[r | j] = up ? hi : lo;
+    }
+  }
+}
+template <int R>
+__device__ __forceinline__ void sort_regs(int (&x)[R]) {
   const int lane = threadIdx.x & 31;
-  int32_t *buf = sm[threadIdx.x >> 5];
+#pragma unroll
+  for (int k = 2; k < R; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        if (r & j) continue;
+        const int lo = min(x[r], x[r | j]), hi = max(x[r], x[r | j]);
+        x[r] = (r & k) == 0 ? lo : hi;
+        x[r | j] = (r & k) == 0 ? hi : lo;
+      }
+    }
+  }
+#pragma unroll 1
+  for (int d = 1; d <= 32; d <<= 1) {  // sorts of d lanes' items
+    const bool up = (lane & d) == 0;
+#pragma unroll 1
+    for (int j = d >> 1; j > 0; j >>= 1) {
+      const bool keep_min = ((lane & j) == 0) == up;
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const int y = __shfl_xor_sync(FULL, x[r], j);
+        x[r] = keep_min ? min(x[r], y) : max(x[r], y);
+      }
+    }
+    merge_lane<R>(x, up);
+  }
+}
+
+// A row of 33 .. 32 R entries, sorted in registers and brought into row order
+// through shared memory.
+template <int R, bool GAP>
+__device__ __forceinline__ int64_t sort_row(const RA &a, int64_t p, int64_t e0, int L, int64_t o0, int32_t *buf) {
+  const int lane = threadIdx.x & 31;
+  int x[R];
+#pragma unroll
+  for (int r = 0; r < R; r++) x[r] = 32 * r + lane < L ? a.ci[e0 + 32 * r + lane] : -1;
+#pragma unroll
+  for (int r = 0; r < R; r++) x[r] = x[r] >= 0 ? a.pos[x[r]] : INT_MAX;
+  sort_regs<R>(x);
+  __syncwarp();
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int i = lane * R + r;
+    buf[i + (i >> 5)] = x[r];
+  }
+  __syncwarp();
+  int64_t s = 0;
+  for (int i = lane; i < L; i += 32) {
+    const int y = buf[i + (i >> 5)];
+    if (GAP) s += gap_fixed(y, i ? buf[i - 1 + ((i - 1) >> 5)] : (int)p, i == 0);
+    else a.nci[o0 + i] = y;
+  }
+  __syncwarp();
+  return s;
+}
+
+__device__ __forceinline__ void block_add(int64_t s, unsigned long long *total) {
+  __shared__ int64_t red[32];
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+  if (lane == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int64_t t = 0;
+    for (int w = 0; w < (int)blockDim.x / 32; w++) t += red[w];
+    if (t != 0) atomicAdd(total, (unsigned long long)t);
+  }
+}
+
+// The rows of at most 32 entries of the relabelled graph, written (GAP false) or
+// only summed up for the gap cost: a warp holds the bounds of up to 32 rows,
+// one per lane (rows far apart in the new order, which puts the long ones
+// together), and sorts four at a time -- the chain entry -> position is what
+// bounds them.  The longer rows are listed for the kernels below.  R-MAT scale
+// 18 (7.2 M entries): 0.60 ms for rows up to 1,024 entries with one row per
+// warp at a time and the sort in shared memory; now 30 us here and 70 us in
+// mid_rows_kernel (with the gap cost instead of the writes 39 and 80 us; that
+// was a pass of its own, 0.43 ms).  Both in one kernel took 183 us: the sort of
+// 1,024 entries left the short rows 16 warps per SM.
+template <bool GAP>
+__global__ void __launch_bounds__(kOT) short_rows_kernel(RA a) {
+  const int lane = threadIdx.x & 31;
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t p = gw; p < n; p += nw) {
-    const int v = order[p];
-    const int64_t e0 = rp[v], L = rp[v + 1] - e0, o0 = nrp[p];
-    if (L > kWarpSortMax) {
-      for (int64_t i = lane; i < L; i += 32) nci[o0 + i] = pos[ci[e0 + i]];
-      if (lane == 0) big[atomicAdd(nbig, 1ull)] = (int32_t)p;
-      continue;
+  int64_t s = 0;
+  for (int64_t base = gw; base < a.n; base += nw * 32) {
+    const int64_t mp = base + nw * lane;
+    int64_t me0 = 0, mo0 = 0, ml = 0;
+    if (mp < a.n) {
+      const int v = a.order[mp];
+      me0 = a.rp[v];
+      ml = a.rp[v + 1] - me0;
+      mo0 = a.nrp ? a.nrp[mp] : me0;
     }
-    if (L <= 32) {
-      int x = lane < L ? pos[ci[e0 + lane]] : INT_MAX;
-      // bitonic network over the 32 lanes
+    unsigned m = __ballot_sync(FULL, ml > 0 && ml <= 32);
+    while (m) {
+      int x[4], len[4], src[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        src[q] = m ? __ffs(m) - 1 : -1;
+        m &= m - 1;  // (0 stays 0)
+        const int64_t e0 = __shfl_sync(FULL, me0, max(src[q], 0));
+        len[q] = __shfl_sync(FULL, (int)ml, max(src[q], 0));
+        if (src[q] < 0) len[q] = 0;
+        x[q] = lane < len[q] ? a.ci[e0 + lane] : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; q++) x[q] = x[q] >= 0 ? a.pos[x[q]] : INT_MAX;
+#pragma unroll
       for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
         for (int j = k >> 1; j > 0; j >>= 1) {
-          const int y = __shfl_xor_sync(FULL, x, j);
-          const bool up = (lane & k) == 0, lower = (lane & j) == 0;
-          x = (lower == up) ? min(x, y) : max(x, y);
-        }
-      if (lane < L) nci[o0 + lane] = x;
-      continue;
-    }
-    int P = 64;
-    while (P < L) P <<= 1;
-    for (int i = lane; i < P; i += 32) buf[i] = i < L ? pos[ci[e0 + i]] : INT_MAX;
-    __syncwarp();
-    for (int k = 2; k <= P; k <<= 1)
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int i = lane; i < P; i += 32) {
-          const int l = i ^ j;
-          if (l > i) {
-            const int x = buf[i], y = buf[l];
-            const bool up = (i & k) == 0;
-            if ((x > y) == up) {
-              buf[i] = y;
-              buf[l] = x;
-            }
+          const bool keep_min = ((lane & j) == 0) == ((lane & k) == 0);
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            const int y = __shfl_xor_sync(FULL, x[q], j);
+            x[q] = keep_min ? min(x[q], y) : max(x[q], y);
           }
         }
-        __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        if (GAP) {
+          const int y = __shfl_up_sync(FULL, x[q], 1);
+          if (lane < len[q]) s += gap_fixed(x[q], lane ? y : (int)(base + nw * src[q]), lane == 0);
+        } else {
+          const int64_t o0 = __shfl_sync(FULL, mo0, max(src[q], 0));
+          if (lane < len[q]) a.nci[o0 + lane] = x[q];
+        }
       }
-    for (int i = lane; i < L; i += 32) nci[o0 + i] = buf[i];
-    __syncwarp();
+    }
+    // the longer ones are listed
+    const unsigned mid = __ballot_sync(FULL, ml > 32 && ml <= kWarpSortMax);
+    unsigned at = 0;
+    if (lane == 0 && mid) at = atomicAdd(a.nmid, (unsigned)__popc(mid));
+    at = __shfl_sync(FULL, at, 0);
+    if (ml > 32) {
+      if (ml <= kWarpSortMax) a.mid[at + __popc(mid & ((1u << lane) - 1u))] = (int32_t)mp;
+      else a.big[atomicAdd(a.nbig, 1ull)] = (int32_t)mp;
+    }
   }
+  if (GAP) block_add(s, a.total);
+}
+
+// The listed rows of 33 to kWarpSortMax entries, a warp each.
+template <bool GAP>
+__global__ void __launch_bounds__(kOT, 3) mid_rows_kernel(RA a) {
+  __shared__ int32_t sm[kOT / 32][kWarpSortMax + kWarpSortMax / 32];
+  int32_t *buf = sm[threadIdx.x >> 5];
+  const unsigned gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+  const unsigned total = *a.nmid;
+  int64_t s = 0;
+  for (unsigned t = gw; t < total; t += nw) {
+    const int64_t p = a.mid[t];
+    const int v = a.order[p];
+    const int64_t e0 = a.rp[v], o0 = a.nrp ? a.nrp[p] : e0;
+    const int L = (int)(a.rp[v + 1] - e0);
+    if (L <= 64) s += sort_row<2, GAP>(a, p, e0, L, o0, buf);
+    else if (L <= 128) s += sort_row<4, GAP>(a, p, e0, L, o0, buf);
+    else if (L <= 256) s += sort_row<8, GAP>(a, p, e0, L, o0, buf);
+    else if (L <= 512) s += sort_row<16, GAP>(a, p, e0, L, o0, buf);
+    else s += sort_row<32, GAP>(a, p, e0, L, o0, buf);
+  }
+  if (GAP) block_add(s, a.total);
 }
 
 // compare-exchange stages (k, j >= jlo) of a bitonic sort over buf[0..P) by
@@ -646,70 +809,139 @@ __device__ __forceinline__ void bitonic_stages(int32_t *buf, int P, int64_t base
   }
 }
 
-// a block per long row: shared memory up to kBlockSortMax entries, else a
-// scratch row of the next power of two in global memory whose stages with
-// j below kBlockSortMax run chunk by chunk in shared memory
-__global__ void __launch_bounds__(kBigT) block_sort_kernel(const int64_t *nrp, int32_t *nci, const int32_t *big,
-                                                           const unsigned long long *nbig, int32_t *scratch,
-                                                           int64_t scratch_stride) {
-  extern __shared__ int32_t sbuf[];
-  const int64_t cnt = (int64_t)*nbig;
-  for (int64_t b = blockIdx.x; b < cnt; b += gridDim.x) {
-    const int64_t p = big[b];
-    const int64_t o0 = nrp[p], L = nrp[p + 1] - o0;
-    int64_t P = 1;
-    while (P < L) P <<= 1;
-    if (P <= kBlockSortMax) {
-      for (int64_t i = threadIdx.x; i < P; i += blockDim.x) sbuf[i] = i < L ? nci[o0 + i] : INT_MAX;
-      __syncthreads();
-      for (int k = 2; k <= P; k <<= 1) bitonic_stages(sbuf, (int)P, 0, k, k >> 1, 1);
-      for (int64_t i = threadIdx.x; i < L; i += blockDim.x) nci[o0 + i] = sbuf[i];
-      __syncthreads();
-      continue;
-    }
-    int32_t *row = scratch + blockIdx.x * scratch_stride;
-    for (int64_t i = threadIdx.x; i < P; i += blockDim.x) row[i] = i < L ? nci[o0 + i] : INT_MAX;
+// Row [e0, e0 + L) of new ids sorted to out by bitonic stages (row: the block's
+// scratch row).
+__device__ void bitonic_row(const RA &a, int64_t e0, int64_t L, int32_t *out, int32_t *sbuf, int32_t *row) {
+  int64_t P = 1;
+  while (P < L) P <<= 1;
+  if (P <= kBlockSortMax) {
+    for (int64_t i = threadIdx.x; i < P; i += blockDim.x) sbuf[i] = i < L ? a.pos[a.ci[e0 + i]] : INT_MAX;
     __syncthreads();
-    const int C = kBlockSortMax;
-    // every stage with k <= C stays inside a chunk
+    for (int k = 2; k <= P; k <<= 1) bitonic_stages(sbuf, (int)P, 0, k, k >> 1, 1);
+    for (int64_t i = threadIdx.x; i < L; i += blockDim.x) out[i] = sbuf[i];
+    __syncthreads();
+    return;
+  }
+  for (int64_t i = threadIdx.x; i < P; i += blockDim.x) row[i] = i < L ? a.pos[a.ci[e0 + i]] : INT_MAX;
+  __syncthreads();
+  const int C = kBlockSortMax;
+  // every stage with k <= C stays inside a chunk
+  for (int64_t c = 0; c < P; c += C) {
+    for (int i = threadIdx.x; i < C; i += blockDim.x) sbuf[i] = row[c + i];
+    __syncthreads();
+    for (int k = 2; k <= C; k <<= 1) bitonic_stages(sbuf, C, c, k, k >> 1, 1);
+    for (int i = threadIdx.x; i < C; i += blockDim.x) row[c + i] = sbuf[i];
+    __syncthreads();
+  }
+  for (int64_t k = 2 * (int64_t)C; k <= P; k <<= 1) {
+    for (int64_t j = k >> 1; j >= C; j >>= 1) {
+      for (int64_t i = threadIdx.x; i < P; i += blockDim.x) {
+        const int64_t l = i ^ j;
+        if (l > i) {
+          const int x = row[i], y = row[l];
+          const bool up = (i & k) == 0;
+          if ((x > y) == up) {
+            row[i] = y;
+            row[l] = x;
+          }
+        }
+      }
+      __syncthreads();
+    }
     for (int64_t c = 0; c < P; c += C) {
       for (int i = threadIdx.x; i < C; i += blockDim.x) sbuf[i] = row[c + i];
       __syncthreads();
-      for (int k = 2; k <= C; k <<= 1) bitonic_stages(sbuf, C, c, k, k >> 1, 1);
+      bitonic_stages(sbuf, C, c, (int)k, C >> 1, 1);
       for (int i = threadIdx.x; i < C; i += blockDim.x) row[c + i] = sbuf[i];
       __syncthreads();
     }
-    for (int64_t k = 2 * (int64_t)C; k <= P; k <<= 1) {
-      for (int64_t j = k >> 1; j >= C; j >>= 1) {
-        for (int64_t i = threadIdx.x; i < P; i += blockDim.x) {
-          const int64_t l = i ^ j;
-          if (l > i) {
-            const int x = row[i], y = row[l];
-            const bool up = (i & k) == 0;
-            if ((x > y) == up) {
-              row[i] = y;
-              row[l] = x;
-            }
-          }
-        }
-        __syncthreads();
-      }
-      for (int64_t c = 0; c < P; c += C) {
-        for (int i = threadIdx.x; i < C; i += blockDim.x) sbuf[i] = row[c + i];
-        __syncthreads();
-        bitonic_stages(sbuf, C, c, (int)k, C >> 1, 1);
-        for (int i = threadIdx.x; i < C; i += blockDim.x) row[c + i] = sbuf[i];
-        __syncthreads();
-      }
-    }
-    for (int64_t i = threadIdx.x; i < L; i += blockDim.x) nci[o0 + i] = row[i];
-    __syncthreads();
   }
+  for (int64_t i = threadIdx.x; i < L; i += blockDim.x) out[i] = row[i];
+  __syncthreads();
 }
 
-// sum over the entries of the relabelled graph of log2(1 + gap): each term
-// in single precision (one rounding of 1 + gap, log2f within 1 ulp, so a
-// relative error below 2^-22), the sum in double
+// Row [e0, e0 + L) of distinct new ids, sorted to out, by the bits of a window of
+// 32 words new ids at a time: every entry sets its bit, and the set bits are
+// written in order.  words of shared memory to clear and read instead of
+// log^2 L passes over the row.  Returns whether all L entries were distinct
+// (else what is in out does not count).
+__device__ bool bitmap_row(const RA &a, int64_t e0, int64_t L, int32_t *out, unsigned *bm, int words, int *wsum) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t span = 32ll * words;
+  const int per = ((words + kBigT / 32 - 1) / (kBigT / 32) + 31) & ~31;  // words per warp
+  const int b0 = min(words, wid * per), b1 = min(words, b0 + per);
+  int64_t done = 0;
+  for (int64_t first = 0; first < a.n; first += span) {
+    for (int i = threadIdx.x; i < words; i += kBigT) bm[i] = 0u;
+    __syncthreads();
+    for (int64_t i = threadIdx.x; i < L; i += kBigT) {
+      const int64_t x = a.pos[a.ci[e0 + i]] - first;
+      if (x >= 0 && x < span) atomicOr(bm + (x >> 5), 1u << (x & 31));
+    }
+    __syncthreads();
+    int c = 0;
+    for (int i = b0 + lane; i < b1; i += 32) c += __popc(bm[i]);
+    c = __reduce_add_sync(FULL, c);
+    if (lane == 0) wsum[wid] = c;
+    __syncthreads();
+    int64_t at = done;
+    for (int w = 0; w < kBigT / 32; w++) {
+      at += w < wid ? wsum[w] : 0;
+      done += wsum[w];
+    }
+    for (int i = b0; i < b1; i += 32) {
+      unsigned y = i + lane < b1 ? bm[i + lane] : 0u;
+      int incl = __popc(y);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int z = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += z;
+      }
+      int32_t *o = out + at + incl - __popc(y);
+      while (y) {
+        *o++ = (int32_t)(first + 32ll * (i + lane) + __ffs(y) - 1);
+        y &= y - 1;
+      }
+      at += __shfl_sync(FULL, incl, 31);
+    }
+    __syncthreads();  // bm and wsum are free
+  }
+  return done == L;
+}
+
+// A block per long row: by bits where the words of all new ids are few for the
+// row (at most kBitWords per entry: equal there, 0.80 and 0.85 ms for 600 rows
+// of 4,100 entries among 4.2 M ids; at 64 words 0.61 against 0.45 ms, at 8 1.09
+// against 1.35 ms); otherwise, and for rows with an entry twice, a bitonic sort
+// in shared memory, above kBlockSortMax entries over a scratch row of the next
+// power of two in global memory whose stages with j below kBlockSortMax run
+// chunk by chunk in shared memory.  R-MAT scale 18: 0.50 ms with the bitonic
+// sort alone, 0.07 ms now.
+constexpr int kBitWords = 32;
+template <bool GAP>
+__global__ void __launch_bounds__(kBigT) long_rows_kernel(RA a, int words, int32_t *scratch, int64_t scratch_stride) {
+  extern __shared__ int32_t sbuf[];
+  __shared__ int wsum[kBigT / 32];
+  const int64_t cnt = (int64_t)*a.nbig;
+  int64_t s = 0;
+  for (int64_t b = blockIdx.x; b < cnt; b += gridDim.x) {
+    const int64_t p = a.big[b], e0 = a.rp[a.order[p]], L = a.rp[a.order[p] + 1] - e0;
+    const int64_t o0 = a.nrp ? a.nrp[p] : e0;
+    const bool bits = (a.n + 31) / 32 <= kBitWords * L;
+    if (!bits || !bitmap_row(a, e0, L, a.nci + o0, (unsigned *)sbuf, words, wsum))
+      bitonic_row(a, e0, L, a.nci + o0, sbuf, scratch + blockIdx.x * scratch_stride);
+    if (GAP) {
+      __syncthreads();
+      const int32_t *row = a.nci + o0;
+      for (int64_t i = threadIdx.x; i < L; i += kBigT)
+        s += gap_fixed(row[i], i ? row[i - 1] : (int)p, i == 0);
+    }
+  }
+  if (GAP) block_add(s, a.total);
+}
+
+// The gap cost of the graph as it is: sum over the entries of log2(1 + gap),
+// the sum in double.
 __global__ void __launch_bounds__(kOT) gap_kernel(int64_t n, const int64_t *nrp, const int32_t *nci, double *total) {
   __shared__ double red[kOT / 32];
   const int lane = threadIdx.x & 31;
@@ -718,12 +950,7 @@ __global__ void __launch_bounds__(kOT) gap_kernel(int64_t n, const int64_t *nrp,
   double s = 0.0;
   for (int64_t p = gw; p < n; p += nw) {
     const int64_t e0 = nrp[p], e1 = nrp[p + 1];
-    for (int64_t e = e0 + lane; e < e1; e += 32) {
-      const int64_t x = nci[e];
-      const int64_t prev = e == e0 ? p : (int64_t)nci[e - 1];
-      const int64_t gap = e == e0 ? (x > p ? x - p : p - x) : x - prev;
-      s += (double)log2f((float)(gap + 1));
-    }
+    for (int64_t e = e0 + lane; e < e1; e += 32) s += (double)gap_term(nci[e], e == e0 ? (int)p : nci[e - 1], e == e0);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
@@ -847,12 +1074,9 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
   return MC_OK;
 }
 
-int relabel(mc_graph *g, const int32_t *order, int64_t *d_nrp, int32_t *d_nci) {
+// The order on the device and its inverse; refused unless it is a permutation.
+static int load_order(mc_graph *g, const int32_t *order, RA &a) {
   const int64_t n = g->n;
-  if (n == 0) {
-    MC_CUDA_TRY(cudaMemsetAsync(d_nrp, 0, sizeof(int64_t), g->stream));
-    return MC_OK;
-  }
   if (!g->cores_valid) MC_TRY(launch_core_numbers(g, kDefaultSpinLimit));  // sets max_degree
   void *p;
   MC_TRY(ws_get(g, "rl.order", (size_t)n * 4, &p));
@@ -869,34 +1093,85 @@ int relabel(mc_graph *g, const int32_t *order, int64_t *d_nrp, int32_t *d_nci) {
   MC_CUDA_TRY(cudaMemcpyAsync(g->h_small, bad, 4, cudaMemcpyDeviceToHost, g->stream));
   MC_CUDA_TRY(cudaStreamSynchronize(g->stream));
   if (*(int32_t *)g->h_small) return MC_ERR_ARG;
-  MC_TRY(device_scan(g, n, DegF{g->row_ptr, d_order}, RowG{d_nrp}, d_nrp + n, "rl.scan"));
-  MC_TRY(ws_get(g, "rl.big", (size_t)n * 4, &p));
-  int32_t *big = (int32_t *)p;
-  MC_TRY(ws_get(g, "rl.nbig", 8, &p));
-  unsigned long long *nbig = (unsigned long long *)p;
-  MC_CUDA_TRY(cudaMemsetAsync(nbig, 0, 8, g->stream));
-  fill_sort_kernel<<<grid_of(g, n * 32, kOT, 8), kOT, 0, g->stream>>>(n, g->row_ptr, g->col_idx, d_order, pos,
-                                                                        d_nrp, d_nci, big, nbig);
+  a.n = n;
+  a.rp = g->row_ptr;
+  a.ci = g->col_idx;
+  a.order = d_order;
+  a.pos = pos;
+  return MC_OK;
+}
+
+// The rows of a (order, pos and where they go are set).
+template <bool GAP>
+static int launch_rows(mc_graph *g, RA a) {
+  void *p;
+  const bool any_mid = g->max_degree > 32, any_long = g->max_degree > kWarpSortMax;
+  if (any_mid) {
+    MC_TRY(ws_get(g, "rl.mid", 64 + (size_t)std::min<int64_t>(g->n, g->nnz / 33 + 1) * 4, &p));
+    a.nbig = (unsigned long long *)p;
+    a.nmid = (unsigned *)(a.nbig + 1);
+    a.mid = (int32_t *)((char *)p + 64);
+    MC_CUDA_TRY(cudaMemsetAsync(p, 0, 16, g->stream));
+  }
+  if (any_long) {
+    MC_TRY(ws_get(g, "rl.big", (size_t)(g->nnz / kWarpSortMax + 1) * 4, &p));
+    a.big = (int32_t *)p;
+  }
+  short_rows_kernel<GAP><<<grid_of(g, a.n * 8, kOT, 6), kOT, 0, g->stream>>>(a);
   g_launches++;
+  if (any_mid) {
+    mid_rows_kernel<GAP><<<grid_of(g, std::min<int64_t>(g->n, g->nnz / 33 + 1) * 32, kOT, 3), kOT, 0, g->stream>>>(a);
+    g_launches++;
+  }
   MC_CUDA_TRY(cudaGetLastError());
-  if (g->max_degree > kWarpSortMax) {
+  if (any_long) {
     int64_t P = 1;
     while (P < g->max_degree) P <<= 1;
-    const int blocks = g->sm_count;
     int32_t *scratch = nullptr;
     int64_t stride = 0;
-    if (P > kBlockSortMax) {
+    int blocks = 2 * g->sm_count;
+    if (P > kBlockSortMax) {  // the rows that may need a scratch row are megabytes
       stride = P;
+      blocks = g->sm_count;
       MC_TRY(ws_get(g, "rl.scratch", (size_t)blocks * P * 4, &p));
       scratch = (int32_t *)p;
     }
-    const int smem = kBlockSortMax * 4;
-    MC_CUDA_TRY(cudaFuncSetAttribute(block_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    block_sort_kernel<<<blocks, kBigT, smem, g->stream>>>(d_nrp, d_nci, big, nbig, scratch, stride);
+    // the window: all new ids if they fit 192 KiB of bits
+    const int words = (int)std::min<int64_t>((a.n + 31) / 32, 48 << 10);
+    const int smem = std::max(words, kBlockSortMax) * 4;
+    MC_CUDA_TRY(cudaFuncSetAttribute(long_rows_kernel<GAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    long_rows_kernel<GAP><<<blocks, kBigT, smem, g->stream>>>(a, words, scratch, stride);
     g_launches++;
     MC_CUDA_TRY(cudaGetLastError());
   }
   return MC_OK;
+}
+
+int relabel(mc_graph *g, const int32_t *order, int64_t *d_nrp, int32_t *d_nci) {
+  if (g->n == 0) {
+    MC_CUDA_TRY(cudaMemsetAsync(d_nrp, 0, sizeof(int64_t), g->stream));
+    return MC_OK;
+  }
+  RA a{};
+  MC_TRY(load_order(g, order, a));
+  MC_TRY(device_scan(g, g->n, DegF{g->row_ptr, a.order}, RowG{d_nrp}, d_nrp + g->n, "rl.scan"));
+  a.nrp = d_nrp;
+  a.nci = d_nci;
+  return launch_rows<false>(g, a);
+}
+
+int gap_bits_of(mc_graph *g, const int32_t *order, unsigned long long *d_total) {
+  MC_CUDA_TRY(cudaMemsetAsync(d_total, 0, sizeof(*d_total), g->stream));
+  if (g->n == 0) return MC_OK;
+  RA a{};
+  MC_TRY(load_order(g, order, a));
+  if (g->max_degree > kWarpSortMax) {
+    void *p;
+    MC_TRY(ws_get(g, "rl.nci", (size_t)std::max<int64_t>(g->nnz, 1) * 4, &p));
+    a.nci = (int32_t *)p;
+  }
+  a.total = d_total;
+  return launch_rows<true>(g, a);
 }
 
 int gap_bits(mc_graph *g, const int64_t *d_nrp, const int32_t *d_nci, double *d_total) {

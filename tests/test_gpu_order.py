@@ -219,3 +219,30 @@ def test_clique_order_rmat_s22_properties(mc):
     # the clique order is more local than the vertex ids of R-MAT
     assert mc.mc_gap_bits(h, order) < mc.mc_gap_bits(h)
     h.close()
+
+
+@pytest.mark.parametrize("n", [1 << 20, (1 << 20) + 33, 1700000])
+def test_relabel_by_row_length(mc, n):
+    """Rows at the edges of the sorters (32, 64, ..., 1,024 entries), long rows
+    on both sides of the rule between bits and the sorting network (n / 32
+    words against 32 per entry), and ids beyond one window of bits: rows as
+    numpy sorts them, the gap cost from those rows."""
+    rng = np.random.default_rng(n)
+    lengths = [1, 2, 31, 32, 33, 64, 65, 128, 129, 256, 257, 512, 513, 1023, 1024, 1025, 1100, 1600, 1700, 2048, 17000]
+    src = np.concatenate([np.full(d, v) for v, d in enumerate(lengths)])
+    dst = np.concatenate([100 + rng.choice(n - 100, d, replace=False) for d in lengths])
+    g = gg.from_edges(n, src, dst)
+    h = load(mc, g)
+    order = rng.permutation(n).astype(np.int32)
+    pos = np.empty(n, np.int64)
+    pos[order] = np.arange(n)
+    rp, ci = mc.mc_relabel(h, order)
+    old = np.repeat(np.arange(n), np.diff(g.row_ptr))
+    o = np.lexsort((pos[g.col_idx], pos[old]))
+    want = pos[g.col_idx][o]
+    assert np.array_equal(rp, np.r_[0, np.cumsum(np.diff(g.row_ptr)[order])]) and np.array_equal(ci, want)
+    row = pos[old][o]
+    gaps = np.where(np.r_[True, row[1:] != row[:-1]], np.abs(want - row), np.r_[0, np.diff(want)])
+    bits = float(np.log2(1.0 + gaps).mean())
+    assert abs(mc.mc_gap_bits(h, order) - bits) <= GAP_RTOL * bits
+    h.close()
