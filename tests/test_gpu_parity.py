@@ -653,3 +653,24 @@ def test_repeel_rebuilds_when_omega_rises(mc):
             mc.mc_max_clique(h, **bad)
         assert e.value.code == mc.MC_ERR_ARG
     h.close()
+
+
+def test_validate_by_row_length(mc):
+    """Rows on both sides of a warp's share (512 entries) and of a block's
+    step (2,048): accepted as they are, refused with one entry out of order,
+    repeated, missing its reverse or leaving the range, wherever it stands."""
+    g = _hubs(9000, [511, 512, 513, 2047, 2048, 2049, 5000], 8)
+    mc.mc_load_csr(g.row_ptr, g.col_idx, mc.MC_VALIDATE).close()
+    for v in (1, 2, 4, 6, 8000):
+        e0, e1 = int(g.row_ptr[v]), int(g.row_ptr[v + 1])
+        for e in sorted({e0, e0 + 1, (e0 + e1) // 2, e1 - 2, e1 - 1}):
+            for put in (lambda c: c[e - 1] if e > e0 else c[e + 1], lambda c: v, lambda c: g.n, lambda c: -1,
+                        lambda c: next(x for x in range(c[e] + 1, g.n + 1) if x == g.n or x not in set(c[e0:e1]))):
+                c = g.col_idx.copy()
+                c[e] = put(c)
+                with pytest.raises(mc.MCError):
+                    mc.mc_load_csr(g.row_ptr, c, mc.MC_VALIDATE)
+    rp = g.row_ptr.copy()
+    rp[5] -= 700  # a row and its neighbour overlap
+    with pytest.raises(mc.MCError):
+        mc.mc_load_csr(rp, g.col_idx, mc.MC_VALIDATE)
