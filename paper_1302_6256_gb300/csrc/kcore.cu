@@ -70,35 +70,36 @@ struct KcoreCtl {
 
 __device__ __forceinline__ long long ld_vol64(const long long *p) { return *(const volatile long long *)p; }
 
-// Grid barrier that also snapshots (otail, wtail) when every block has
-// arrived.  Bounded spin: on timeout the error word is set.
-__device__ __forceinline__ void barrier_snap(KcoreCtl *ctl, unsigned nblocks, int32_t *err, long long spin_limit,
-                                             long long *otail_out, long long *wtail_out, const int *live_src,
-                                             long long *live_out) {
+// Grid barrier number gen + 1 (every block counts them) that also snapshots
+// (otail, wtail) when every block has arrived.  Bounded spin: on timeout the
+// error word is set.
+__device__ __forceinline__ void barrier_snap(KcoreCtl *ctl, unsigned nblocks, unsigned &gen, int32_t *err,
+                                             long long spin_limit, long long *otail_out, long long *wtail_out,
+                                             const int *live_src, long long *live_out) {
   __shared__ long long s_o, s_w, s_l;
   __syncthreads();
+  gen++;
   if (threadIdx.x == 0) {
-    unsigned g0 = *(volatile unsigned *)&ctl->bar_gen;
     __threadfence();
     if (atomicAdd(&ctl->bar_count, 1u) == nblocks - 1) {
       __threadfence();
-      ctl->snap[(g0 + 1) & 1][0] = *(volatile int *)&ctl->otail;
-      ctl->snap[(g0 + 1) & 1][1] = ld_vol64(&ctl->wtail);
-      ctl->snap[(g0 + 1) & 1][2] = live_src ? *(volatile const int *)live_src : 0;
+      ctl->snap[gen & 1][0] = *(volatile int *)&ctl->otail;
+      ctl->snap[gen & 1][1] = ld_vol64(&ctl->wtail);
+      ctl->snap[gen & 1][2] = live_src ? *(volatile const int *)live_src : 0;
       *(volatile unsigned *)&ctl->bar_count = 0;
       __threadfence();
-      atomicAdd(&ctl->bar_gen, 1u);
+      *(volatile unsigned *)&ctl->bar_gen = gen;
     } else {
       long long it = 0;
-      while (*(volatile unsigned *)&ctl->bar_gen == g0) {
+      while (*(volatile unsigned *)&ctl->bar_gen != gen) {
         if (++it > spin_limit) { atomicExch(err, kDevTimeout); break; }
         __nanosleep(16);
       }
     }
     __threadfence();
-    s_o = ld_vol64(&ctl->snap[(g0 + 1) & 1][0]);
-    s_w = ld_vol64(&ctl->snap[(g0 + 1) & 1][1]);
-    s_l = ld_vol64(&ctl->snap[(g0 + 1) & 1][2]);
+    s_o = ld_vol64(&ctl->snap[gen & 1][0]);
+    s_w = ld_vol64(&ctl->snap[gen & 1][1]);
+    s_l = ld_vol64(&ctl->snap[gen & 1][2]);
   }
   __syncthreads();
   *otail_out = s_o;
@@ -381,6 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_peel_kernel(int64_t n, cons
                                                                  int32_t *err, long long spin_limit, int nocheck,
                                                                  const int32_t *skip) {
   if (skip && *skip) return;  // the order is made already
+  unsigned gen = 0;           // grid barriers passed
   __shared__ int bmin;
   extern __shared__ __align__(16) unsigned char s_pool[];
   BlockPool *bp = (BlockPool *)s_pool;
@@ -475,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_peel_kernel(int64_t n, cons
     __syncthreads();
     if (threadIdx.x == 0 && bmin != INT_MAX) atomicMin(&ctl->minrem[level % 3], bmin);
     long long live_next = 0;
-    barrier_snap(ctl, nblocks, err, spin_limit, &otail_now, &wtail_now, lout_n, &live_next);
+    barrier_snap(ctl, nblocks, gen, err, spin_limit, &otail_now, &wtail_now, lout_n, &live_next);
     if (*(volatile int32_t *)err) return;
     live_count = live_next;
     { int32_t *t = lin; lin = lout; lout = t; }
@@ -525,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_peel_kernel(int64_t n, cons
       }
       block_drain<false>(k, chk, rp, ci, deg, core, order, wq, ctl, bp, 0);
       long long e1 = 0;
-      barrier_snap(ctl, nblocks, err, spin_limit, &otail_now, &e1, nullptr, nullptr);
+      barrier_snap(ctl, nblocks, gen, err, spin_limit, &otail_now, &e1, nullptr, nullptr);
       if (*(volatile int32_t *)err) return;
       s0 = e0;
       e0 = e1;
@@ -598,8 +600,8 @@ constexpr int kLocalBlockBins = kLocalBins * kWarps;
 constexpr int kStage = 64;                      // listed vertices a warp holds back to append 32 at a time
 
 struct LocalCtl {
-  unsigned bar_count, bar_gen;
-  int pad[30];
+  unsigned bar_count;
+  int pad[31];
   int n[3][32];   // [counter set][class 0..2]: listed vertices
   int all[32];    // [0..1] vertices of class 1, 2; [2] vertices placed; [3] largest core number
 };
@@ -624,6 +626,7 @@ struct LocalShared {
   int stage[kWarps][kStage];
   int cnt[3], err;
   int red[4];
+  unsigned barriers;  // thread 0's
 };
 
 __device__ __forceinline__ int row_class(int64_t len) { return len <= 32 ? 0 : (len <= kLocalWarpRow ? 1 : 2); }
@@ -639,15 +642,13 @@ __device__ __forceinline__ int short_batch(int64_t n0, int64_t nwarps) {
 __device__ bool local_barrier(const LocalArgs &a, LocalShared &S, const int *src) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned g0 = *(volatile unsigned *)&a.ctl->bar_gen;
+    // arrivals are counted over the whole launch: the count itself says when
+    // all have reached this barrier, nothing is reset and no second word read
+    const unsigned all = (S.barriers += 1) * gridDim.x;
     __threadfence();
-    if (atomicAdd(&a.ctl->bar_count, 1u) == gridDim.x - 1) {
-      *(volatile unsigned *)&a.ctl->bar_count = 0;
-      __threadfence();
-      atomicAdd(&a.ctl->bar_gen, 1u);
-    } else {
+    if (atomicAdd(&a.ctl->bar_count, 1u) + 1 < all) {
       long long it = 0;
-      while (*(volatile unsigned *)&a.ctl->bar_gen == g0) {
+      while ((int)(*(volatile unsigned *)&a.ctl->bar_count - all) < 0) {
         if (++it > a.spin) {
           atomicExch(a.err, kDevTimeout);
           break;
@@ -919,6 +920,7 @@ __device__ __forceinline__ void local_walk(const LocalArgs &a, const int32_t *l0
 
 __global__ void __launch_bounds__(kThreads, 1) kcore_local_kernel(LocalArgs a) {
   __shared__ LocalShared S;
+  if (threadIdx.x == 0) S.barriers = 0;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int64_t gwarp = (int64_t)wib * gridDim.x + blockIdx.x;  // neighbouring items go to different blocks
   const int64_t nwarps = (int64_t)gridDim.x * kWarps;
