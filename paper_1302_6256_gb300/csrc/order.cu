@@ -14,7 +14,7 @@
 //           vertices that died were rejected candidates, whose removal
 //           changes no decision of the greedy scan).  A thread per vertex
 //           checks that and lists the stale ones; warps grow them, whole
-//           blocks those of more than 512 neighbours.
+//           blocks those of many neighbours.
 //   scatter key(v) = |C(v)| << 32 | (2^31 - 1 - rank(v)); every member u of
 //           C(v) takes the largest key of the cliques holding it (atomicMax).
 //   accept  C(v) is accepted iff it holds the largest key at every member;
@@ -55,7 +55,9 @@ constexpr int kBlockSortMax = 16384;
 constexpr int kBigT = 1024;      // threads of the block sorter
 constexpr int kGT = 256;         // threads of a growing block
 constexpr int kGW = kGT / 32;
-constexpr int64_t kBlockGrowMin = 512;  // neighbours above which a block grows the clique
+constexpr int64_t kBlockGrowMin = 4096;  // neighbours above which a block grows the clique
+constexpr int64_t kMidGrowMin = 512;     // ... while few vertices have more than these
+constexpr unsigned kMidPerBlock = 8;     // few: at most this many per growing block
 constexpr int kTake = 4;                // listed vertices a warp takes at a time while there are many
 constexpr int kNear = 256;              // candidates, and entries of a row, that a warp holds in shared memory
 constexpr int kFly = 4;                 // entries or candidates a lane has in flight
@@ -72,15 +74,16 @@ struct OA {
   int32_t *arena;
   unsigned long long *bestkey;
   int64_t *ctl;  // [0] placed, [1] groups, [2] grows, [3] candidate tests, [4] rounds, [5] scan total,
-                 // [6] the block grower's list length and next entry, [7] the warps' (two unsigned each)
+                 // [6] the blocks' list length and next entry, [7] the warps' (two unsigned each), [8] the
+                 // mid-size vertices' list length
   int64_t *goff;
   int32_t *order;
   int64_t *gstart;
   int32_t *ground;
   int32_t round;
   int32_t *err;
-  int32_t *big;     // vertices for the block grower this round
-  unsigned *nbig;
+  int32_t *big;     // vertices for the blocks this round; from the list's end on, those of mid-size
+  unsigned *nbig, *nmid;
   int32_t *stale;   // vertices for the warps this round
   unsigned *nstale, *take, *take_big;
 };
@@ -284,30 +287,30 @@ __device__ __forceinline__ bool needs_grow(const OA &a, int v) {
 }
 
 // check: a thread per vertex resets the alive vertices' keys and lists the
-// ones that need a clique (warp-aggregated appends): vertices of more than
-// kBlockGrowMin neighbours for the block grower, the rest for the warps
+// ones that need a clique (warp-aggregated appends) by their row's length
 __global__ void check_kernel(OA a) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < a.n; base += stride) {
     const int64_t vv = base + lane;
-    bool need = false, big = false;
+    int c = -1;  // 0: warps, 1: mid-size, 2: blocks
     if (vv < a.n && a.alive[vv]) {
       a.bestkey[vv] = 0ull;
-      need = needs_grow(a, (int)vv);
-      big = need && a.rp[vv + 1] - a.rp[vv] > kBlockGrowMin;
+      if (needs_grow(a, (int)vv)) {
+        const int64_t d = a.rp[vv + 1] - a.rp[vv];
+        c = d > kBlockGrowMin ? 2 : d > kMidGrowMin ? 1 : 0;
+      }
     }
-    const unsigned ms = __ballot_sync(FULL, need && !big), mb = __ballot_sync(FULL, big);
-    unsigned at_s = 0, at_b = 0;
-    if (lane == 0) {
-      if (ms) at_s = atomicAdd(a.nstale, (unsigned)__popc(ms));
-      if (mb) at_b = atomicAdd(a.nbig, (unsigned)__popc(mb));
-    }
-    at_s = __shfl_sync(FULL, at_s, 0);
-    at_b = __shfl_sync(FULL, at_b, 0);
-    if (need && !big) a.stale[at_s + __popc(ms & lt)] = (int32_t)vv;
-    if (big) a.big[at_b + __popc(mb & lt)] = (int32_t)vv;
+    const unsigned ms = __ballot_sync(FULL, c == 0), mm = __ballot_sync(FULL, c == 1), mb = __ballot_sync(FULL, c == 2);
+    unsigned at = 0;
+    if (lane == 0 && ms) at = atomicAdd(a.nstale, (unsigned)__popc(ms));
+    if (lane == 1 && mm) at = atomicAdd(a.nmid, (unsigned)__popc(mm));
+    if (lane == 2 && mb) at = atomicAdd(a.nbig, (unsigned)__popc(mb));
+    const unsigned as = __shfl_sync(FULL, at, 0), am = __shfl_sync(FULL, at, 1), ab = __shfl_sync(FULL, at, 2);
+    if (c == 0) a.stale[as + __popc(ms & lt)] = (int32_t)vv;
+    if (c == 1) a.big[a.n - 1 - (am + __popc(mm & lt))] = (int32_t)vv;
+    if (c == 2) a.big[ab + __popc(mb & lt)] = (int32_t)vv;
   }
 }
 
@@ -387,9 +390,12 @@ __device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt
 // a growth is the next member's row bounds, its fence posts, at most
 // log2(length / 256) further entries of it and the kept candidates' keys.
 // R-MAT scale 16, all rounds: 5.1 ms with 8 warps per SM, rows searched or
-// merged in L2 and blocks only above 4,096 neighbours; 2.0 ms now (blocks above
-// 512; above 1,024 or 2,048: 3.56 or 3.95 ms per order instead of 3.70 at this
-// scale, 5.83 or 5.87 instead of 5.51 at scale 17).
+// merged in L2 and blocks only above 4,096 neighbours; 2.0 ms now.  Vertices of
+// 513 .. 4,096 neighbours go to blocks while there are at most kMidPerBlock per
+// block, when the longest growth decides, and to warps otherwise, when all of
+// them do: whole order of scale 16 / 17 / 20 / 22 in 3.8 / 5.6 / 51 / 191 ms,
+// always blocks 3.8 / 5.8 / 55 / 342, never blocks 4.8 / 7.7 / 50 / 185
+// (before: 7.6 / 11.9 / 71 / 316).
 __global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, int64_t scratch_stride, int big_blocks) {
   __shared__ GrowSmem S;
   __shared__ CKey sk[kGW];
@@ -398,15 +404,18 @@ __global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, in
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const CKey none{INT_MIN, INT_MIN, INT_MAX};
   unsigned long long grows = 0, tests = 0;
-  const unsigned nbig = *a.nbig;
-  if ((int)blockIdx.x < big_blocks && nbig) {
+  const unsigned nbig = *a.nbig, nmid = *a.nmid, nstale = *a.nstale;
+  const bool mid_blocks = nmid <= kMidPerBlock * (unsigned)big_blocks;
+  if ((int)blockIdx.x < big_blocks) {
+    const unsigned total = nbig + (mid_blocks ? nmid : 0u);
     for (;;) {
+      if (total == 0) break;
       if (threadIdx.x == 0) s_b = atomicAdd(a.take_big, 1u);
       __syncthreads();
       const unsigned b = s_b;
       __syncthreads();
-      if (b >= nbig) break;
-      const int v = a.big[b];
+      if (b >= total) break;
+      const int v = b < nbig ? a.big[b] : a.big[a.n - 1 - (b - nbig)];
       const int size = block_grow(a, v, scratch + blockIdx.x * scratch_stride, S, scnt, sk, tests);
       if (threadIdx.x == 0) {
         a.csize[v] = size;
@@ -414,7 +423,7 @@ __global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, in
       }
     }
   }
-  const unsigned total = *a.nstale;
+  const unsigned mids = mid_blocks ? 0u : nmid, total = mids + nstale;
   const unsigned chunk = total > 8u * kGW * gridDim.x ? (unsigned)kTake : 1u;
   for (;;) {
     unsigned idx = 0;
@@ -423,7 +432,7 @@ __global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, in
     if (idx >= total) break;
     const unsigned end = min(total, idx + chunk);
     for (unsigned t = idx; t < end; t++) {
-      const int v = a.stale[t];
+      const int v = t < mids ? a.big[a.n - 1 - t] : a.stale[t - mids];
       const int64_t e0 = a.rp[v], e1 = a.rp[v + 1];
       int32_t *cand = e1 - e0 <= kNear ? S.cand[wid] : a.arena + e0;
       CKey bk = none;
@@ -538,6 +547,7 @@ __global__ void advance_kernel(int64_t *ctl) {
   ((unsigned *)(ctl + 6))[1] = 0u;
   ((unsigned *)(ctl + 7))[0] = 0u;
   ((unsigned *)(ctl + 7))[1] = 0u;
+  ((unsigned *)(ctl + 8))[0] = 0u;
 }
 
 // a caller's tie rank must be a permutation of [0, n): seen[] starts at 0
@@ -993,13 +1003,13 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
   a.bestkey = (unsigned long long *)p;
   MC_TRY(ws_get(g, "co.goff", (size_t)n * 8, &p));
   a.goff = (int64_t *)p;
-  MC_TRY(ws_get(g, "co.ctl", 64, &p));
+  MC_TRY(ws_get(g, "co.ctl", 128, &p));
   a.ctl = (int64_t *)p;
   a.err = g->err;
   a.order = d_order;
   a.gstart = d_gstart;
   a.ground = d_ground;
-  MC_CUDA_TRY(cudaMemsetAsync(a.ctl, 0, 64, g->stream));
+  MC_CUDA_TRY(cudaMemsetAsync(a.ctl, 0, 128, g->stream));
   if (rank) {
     MC_TRY(ws_get(g, "co.rank", (size_t)n * 4, &p));
     MC_CUDA_TRY(cudaMemcpyAsync(p, rank, (size_t)n * 4, cudaMemcpyDefault, g->stream));
@@ -1024,12 +1034,13 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
   a.take_big = a.nbig + 1;
   a.nstale = (unsigned *)(a.ctl + 7);
   a.take = a.nstale + 1;
+  a.nmid = (unsigned *)(a.ctl + 8);
   MC_TRY(ws_get(g, "co.stale", (size_t)n * 4, &p));
   a.stale = (int32_t *)p;
   int32_t *scratch = nullptr;
   const int big_blocks = 2 * g->sm_count, grow_blocks = 4 * g->sm_count;
   const int64_t stride = std::max<int64_t>(g->max_degree, 1);
-  const bool any_big = g->max_degree > kBlockGrowMin;
+  const bool any_big = g->max_degree > kMidGrowMin;
   if (any_big) {
     MC_TRY(ws_get(g, "co.big", (size_t)n * 4, &p));
     a.big = (int32_t *)p;

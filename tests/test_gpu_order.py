@@ -122,6 +122,19 @@ def test_clique_order_by_row_length_bit_exact(mc, g):
     h.close()
 
 
+@pytest.mark.parametrize("size,count", [(514, 3), (514, 6), (4098, 2)])
+def test_clique_order_of_equal_cliques(mc, size, count):
+    """Few vertices of 513 neighbours (blocks take them), more than eight per
+    growing block (warps do), and rows above 4,096: disjoint cliques, each
+    placed in the first round from its smallest vertex, ids ascending."""
+    g = gg.disjoint_cliques([size] * count)
+    h = load(mc, g)
+    order, starts, rounds, _ = mc.mc_clique_order(h)
+    assert np.array_equal(order, np.arange(g.n)) and np.array_equal(starts, np.arange(0, g.n + 1, size))
+    assert not rounds.any()
+    h.close()
+
+
 @pytest.mark.parametrize("seed", [0, 1, 2])
 def test_clique_order_with_rank_bit_exact(mc, seed):
     g = [gg.path(64), gg.rmat(10, 8, planted=10, seed=9), gg.chung_lu(3000, 2.4, 8.0, 200.0, planted=9, seed=4)][seed]
