@@ -62,104 +62,130 @@ __global__ void verify_set_kernel(int64_t n, const int64_t *rp, const int32_t *c
   if (threadIdx.x == 0) *ok = bad ? 0 : 1;
 }
 
-// Entries from, from + step, ... below e1 of v's row [e0, e1): in [lo, hi), not v,
-// above their predecessor, and v in their own row.  A lane's kValidFly searches
-// run side by side.  Row u is searched only inside [0, nnz): a broken row_ptr
-// is reported (by u's own warp too) instead of read out of bounds.
-constexpr int kValidT = 512, kValidW = kValidT / 32, kValidFly = 4;
-constexpr int64_t kValidLong = 512;  // entries above which a row is the block's
-__device__ __forceinline__ bool entries_ok(int64_t nnz, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                                           int v, int64_t e0, int64_t e1, int64_t from, int step, int64_t lo,
-                                           int64_t hi) {
-  bool ok = true;
-  for (int64_t eb = from; eb < e1; eb += (int64_t)step * kValidFly) {
-    int u[kValidFly], before[kValidFly];
-    int64_t at[kValidFly], left[kValidFly];
-    int missing = 0;
-#pragma unroll
-    for (int q = 0; q < kValidFly; q++) {
-      const int64_t e = eb + (int64_t)q * step;
-      u[q] = e < e1 ? ci[e] : 0;
-      before[q] = e < e1 && e > e0 ? ci[e - 1] : INT_MIN;
+// Sorted strictly increasing rows, no self-loop, columns in range (and inside
+// the vertex's graph for a batch), reverse edge present.  A warp per row of at
+// most kValidShort entries; longer rows are listed as (row, slice) units of
+// kValidSlice entries for validate_long_kernel, since one warp's walk through a
+// hub's row was what the check took.  R-MAT scale 15: 364 us with a warp per
+// row, 65 us now (152 us with the whole block for a long row, which cost graphs of
+// short rows its barriers: 5.0 instead of 2.6 ms for 2,000 of them).
+constexpr int kValidShort = 128, kValidSlice = 512, kValidFly = 4;
+struct ValidUnits {
+  unsigned long long n;
+  unsigned long long unit[1];  // row << 32 | slice, at most `cap` of them
+};
+__global__ void __launch_bounds__(256, 8) validate_kernel(int64_t n, int64_t nnz, const int64_t *rp,
+                                                          const int32_t *ci, const int32_t *gid,
+                                                          const int64_t *voff, ValidUnits *units,
+                                                          unsigned long long cap, int32_t *bad) {
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  if (gw == 0 && lane == 0 && (rp[0] != 0 || rp[n] != nnz)) atomicExch(bad, 1);
+  for (int64_t v = gw; v < n; v += nw) {
+    const int64_t e0 = rp[v], e1 = rp[v + 1];
+    if (e1 < e0 || e0 < 0 || e1 > nnz) {
+      if (lane == 0) atomicExch(bad, 1);
+      continue;
     }
-#pragma unroll
-    for (int q = 0; q < kValidFly; q++) {
-      at[q] = left[q] = 0;
-      if (eb + (int64_t)q * step >= e1) continue;
-      if (u[q] < lo || u[q] >= hi || u[q] == v || before[q] >= u[q]) {
-        ok = false;
+    if (e1 - e0 > kValidShort) {
+      const int64_t k = (e1 - e0 + kValidSlice - 1) / kValidSlice;
+      unsigned long long at = 0;
+      if (lane == 0) at = atomicAdd(&units->n, (unsigned long long)k);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      // rows that do not overlap never need more than cap units
+      if (at + k > cap) {
+        if (lane == 0) atomicExch(bad, 1);
         continue;
       }
-      const int64_t u0 = rp[u[q]], u1 = rp[u[q] + 1];
-      if (u0 < 0 || u1 <= u0 || u1 > nnz) {
-        ok = false;
-        continue;
-      }
-      at[q] = u0;
-      left[q] = u1 - u0;
-      missing |= 1 << q;
+      for (int64_t i = lane; i < k; i += 32) units->unit[at + i] = ((unsigned long long)v << 32) | (unsigned long long)i;
+      continue;
     }
-    while ((left[0] | left[1] | left[2] | left[3]) != 0) {
-      int x[kValidFly];
-#pragma unroll
-      for (int q = 0; q < kValidFly; q++) x[q] = left[q] ? ci[at[q] + (left[q] >> 1)] : 0;
-#pragma unroll
-      for (int q = 0; q < kValidFly; q++) {
-        if (left[q] == 0) continue;
-        const int64_t h = left[q] >> 1;
-        if (x[q] == v) {
-          missing &= ~(1 << q);
-          left[q] = 0;
-        } else if (x[q] < v) {
-          at[q] += h + 1;
-          left[q] -= h + 1;
-        } else {
-          left[q] = h;
-        }
+    const int64_t lo = gid ? voff[gid[v]] : 0, hi = gid ? voff[gid[v] + 1] : n;
+    bool ok = true;
+    for (int64_t e = e0 + lane; e < e1; e += 32) {
+      int u = ci[e];
+      if (u < lo || u >= hi || u == v) ok = false;
+      else if (e > e0 && ci[e - 1] >= u) ok = false;
+      else {
+        // row u is searched only inside [0, nnz): a broken row_ptr is
+        // reported (by u's own warp) instead of read out of bounds
+        const int64_t u0 = rp[u], u1 = rp[u + 1];
+        if (u0 < 0 || u1 < u0 || u1 > nnz || !adjacent(rp, ci, u, (int)v)) ok = false;
       }
     }
-    ok = ok && missing == 0;
+    if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicExch(bad, 1);
   }
-  return ok;
 }
 
-// Sorted strictly increasing rows, no self-loop, columns in range (and inside
-// the vertex's graph for a batch), reverse edge present.  A warp per row,
-// neighbouring rows in different blocks (an R-MAT graph's hubs are neighbours);
-// rows above kValidLong entries are left to the whole block, since one warp's
-// walk through a hub's row was what the check took: R-MAT scale 15 364
-// us, 152 us now.
-__global__ void __launch_bounds__(kValidT) validate_kernel(int64_t n, int64_t nnz, const int64_t *rp,
-                                                           const int32_t *ci, const int32_t *gid,
-                                                           const int64_t *voff, int32_t *bad) {
-  __shared__ int64_t wide[kValidW];  // this pass's long row of each warp, -1: none
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && (rp[0] != 0 || rp[n] != nnz)) atomicExch(bad, 1);
+// The listed slices, a warp each: the same checks, a lane's kValidFly searches
+// side by side.
+__global__ void __launch_bounds__(256) validate_long_kernel(int64_t n, int64_t nnz, const int64_t *__restrict__ rp,
+                                                            const int32_t *__restrict__ ci,
+                                                            const int32_t *__restrict__ gid,
+                                                            const int64_t *__restrict__ voff,
+                                                            const ValidUnits *__restrict__ units,
+                                                            unsigned long long cap, int32_t *bad) {
+  const int lane = threadIdx.x & 31;
+  const unsigned long long gw = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5;
+  const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+  if (units->n > cap) return;  // (reported already; some units were not written)
+  const unsigned long long total = units->n;
   bool ok = true;
-  for (int64_t base = 0; base < n; base += (int64_t)gridDim.x * kValidW) {
-    const int64_t v = base + (int64_t)wid * gridDim.x + blockIdx.x;
-    int64_t mine = -1;
-    if (v < n) {
-      const int64_t e0 = rp[v], e1 = rp[v + 1];
-      if (e1 < e0 || e0 < 0 || e1 > nnz) {
-        ok = false;
-      } else if (e1 - e0 > kValidLong) {
-        mine = v;
-      } else {
-        const int64_t lo = gid ? voff[gid[v]] : 0, hi = gid ? voff[gid[v] + 1] : n;
-        ok = entries_ok(nnz, rp, ci, (int)v, e0, e1, e0 + lane, 32, lo, hi) && ok;
+  for (unsigned long long t = gw; t < total; t += nw) {
+    const int v = (int)(units->unit[t] >> 32);
+    const int64_t e0 = rp[v], end = rp[v + 1];  // checked when it was listed
+    const int64_t s0 = e0 + (int64_t)(units->unit[t] & 0xffffffffull) * kValidSlice;
+    const int64_t s1 = min(end, s0 + kValidSlice);
+    const int64_t lo = gid ? voff[gid[v]] : 0, hi = gid ? voff[gid[v] + 1] : n;
+    for (int64_t eb = s0 + lane; eb < s1; eb += 32 * kValidFly) {
+      int u[kValidFly], before[kValidFly];
+      int64_t at[kValidFly], left[kValidFly];
+      int missing = 0;
+#pragma unroll
+      for (int q = 0; q < kValidFly; q++) {
+        const int64_t e = eb + 32 * q;
+        u[q] = e < s1 ? ci[e] : 0;
+        before[q] = e < s1 && e > e0 ? ci[e - 1] : INT_MIN;
       }
+#pragma unroll
+      for (int q = 0; q < kValidFly; q++) {
+        at[q] = left[q] = 0;
+        if (eb + 32 * q >= s1) continue;
+        if (u[q] < lo || u[q] >= hi || u[q] == v || before[q] >= u[q]) {
+          ok = false;
+          continue;
+        }
+        const int64_t u0 = rp[u[q]], u1 = rp[u[q] + 1];
+        if (u0 < 0 || u1 <= u0 || u1 > nnz) {
+          ok = false;
+          continue;
+        }
+        at[q] = u0;
+        left[q] = u1 - u0;
+        missing |= 1 << q;
+      }
+      while ((left[0] | left[1] | left[2] | left[3]) != 0) {
+        int x[kValidFly];
+#pragma unroll
+        for (int q = 0; q < kValidFly; q++) x[q] = left[q] ? ci[at[q] + (left[q] >> 1)] : 0;
+#pragma unroll
+        for (int q = 0; q < kValidFly; q++) {
+          if (left[q] == 0) continue;
+          const int64_t h = left[q] >> 1;
+          if (x[q] == v) {
+            missing &= ~(1 << q);
+            left[q] = 0;
+          } else if (x[q] < v) {
+            at[q] += h + 1;
+            left[q] -= h + 1;
+          } else {
+            left[q] = h;
+          }
+        }
+      }
+      ok = ok && missing == 0;
     }
-    if (lane == 0) wide[wid] = mine;
-    if (!__syncthreads_or(mine >= 0)) continue;
-    for (int w = 0; w < kValidW; w++) {
-      const int64_t x = wide[w];
-      if (x < 0) continue;
-      const int64_t e0 = rp[x], e1 = rp[x + 1];  // checked by its warp
-      const int64_t lo = gid ? voff[gid[x]] : 0, hi = gid ? voff[gid[x] + 1] : n;
-      ok = entries_ok(nnz, rp, ci, (int)x, e0, e1, e0 + threadIdx.x, kValidT, lo, hi) && ok;
-    }
-    __syncthreads();  // wide is free
   }
   if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicExch(bad, 1);
 }
@@ -245,8 +271,22 @@ int launch_verify_set(mc_graph *g, const int32_t *d_vs, int32_t k, int32_t *d_ok
 
 int launch_validate(mc_graph *g, int32_t *d_bad) {
   if (g->n == 0) return MC_OK;
-  const int blocks = (int)std::min<int64_t>((g->n + kValidW - 1) / kValidW, (int64_t)g->sm_count * 4);
-  validate_kernel<<<blocks, kValidT, 0, g->stream>>>(g->n, g->nnz, g->row_ptr, g->col_idx, g->gid, g->voff, d_bad);
+  const int blocks = (int)std::min<int64_t>((g->n * 32 + 255) / 256, (int64_t)g->sm_count * 16);
+  // a row of L > kValidShort entries has at most L / kValidShort units
+  const unsigned long long cap = (unsigned long long)(g->nnz / kValidShort);
+  void *p;
+  MC_TRY(ws_get(g, "va.units", (size_t)(cap + 1) * 8, &p));
+  ValidUnits *units = (ValidUnits *)p;
+  MC_CUDA_TRY(cudaMemsetAsync(units, 0, 8, g->stream));
+  validate_kernel<<<blocks, 256, 0, g->stream>>>(g->n, g->nnz, g->row_ptr, g->col_idx, g->gid, g->voff, units, cap,
+                                                 d_bad);
+  g_launches++;
+  if (cap == 0) {
+    MC_CUDA_TRY(cudaGetLastError());
+    return MC_OK;
+  }
+  validate_long_kernel<<<(int)std::min<int64_t>((int64_t)(cap + 7) / 8, (int64_t)g->sm_count * 8), 256, 0, g->stream>>>(
+      g->n, g->nnz, g->row_ptr, g->col_idx, g->gid, g->voff, units, cap, d_bad);
   g_launches++;
   MC_CUDA_TRY(cudaGetLastError());
   return MC_OK;

@@ -289,10 +289,10 @@ def test_features_by_row_length(mc):
     assert np.allclose(f, ref, rtol=2e-6, atol=2e-6)
 
 
-@pytest.mark.parametrize("rows", [1, 127, 128, 129, 3 * 152 * 128 + 1])
+@pytest.mark.parametrize("rows", [1, 31, 33, 4096, 4097, 4224, 4225, 3 * 152 * 128 + 1])
 def test_forward_by_row_count(mc, rows):
-    """The network's tiles of 128 rows at their edges and more tiles than
-    blocks, at the tolerance of the test above."""
+    """Eight lanes per row up to 4,096 rows, tiles of 128 rows above, at their
+    edges and with more tiles than blocks, at the tolerance of the test above."""
     x = np.random.default_rng(rows).random((rows, OL.F)).astype(np.float32)
     m = mc.MLP(seed=9)
     ref = OL.forward(m.get_params(), x)
