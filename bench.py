@@ -40,9 +40,9 @@ def load_peaks():
 # Per-solve DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of
 # the kernels on the R-MAT scale-22 solve, from one ncu capture of the
 # current kernels; None until captured (and again whenever a kernel changes).
-# search_block_kernel: its 512- and 1,024-candidate launches of one solve,
-# 122.81 + 3.45 MB and 25.36 + 0 MB.
-TRAFFIC_S22 = {"search_block_kernel": 151.62e6}
+# search_block_kernel: its 512-, 864- and 1,024-candidate launches of one solve,
+# 250.37 + 4.00 MB, 6.29 + 0 MB and 6.36 + 0 MB.
+TRAFFIC_S22 = {"search_block_kernel": 267.02e6}
 
 
 def roofline(stats, n, nnz, clk, dev):
@@ -89,7 +89,8 @@ def roofline(stats, n, nnz, clk, dev):
                 "traffic": TRAFFIC_S22.get(dom),
                 "peak_source": "derived: %d SMs x 32 lanes x %.0f MHz, one shared-memory probe per lane per clock"
                                % (sms, mhz),
-                "algorithmic_units": ent, "unit_note": "neighbour-list entries read in InitialBranch (Fact 3)",
+                "algorithmic_units": ent, "unit_note": "look-ups that build the matrices of InitialBranch (Fact 3): neighbour-list "
+                "entries read, or member pairs gathered from bit rows",
                 "kernel_ms": ms, "streaming": streaming, "_stages": kern}
     if dom == "heuristic_kernel":
         # Algorithm 1's reads: every row entry it scans and one 4-byte column

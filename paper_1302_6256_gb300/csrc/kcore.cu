@@ -588,8 +588,10 @@ __global__ void peel_pos_kernel(int64_t n, const int32_t *__restrict__ order, in
 //
 // The peel / this kernel: Chung-Lu 20,000 vertices 1.42 / 0.46 ms, R-MAT scale
 // 15 2.1 / 0.58, scale 18 (edge factor 12) 3.5 / 1.5, scale 20 5.7 / 5.0,
-// Chung-Lu 1,000,003 vertices (35 M entries, K(G) = 438) 14.8 / 4.3.  Above
-// kLocalMaxNnz the repeated reads cost more than the peel's barriers.
+// Chung-Lu 1,000,003 vertices (35 M entries, K(G) = 438) 14.8 / 4.3.  Barriers
+// that count arrivals over the launch took another 4 .. 10% off (calls of the
+// first three and the last: 0.58 -> 0.55, 0.67 -> 0.63, 2.01 -> 1.92, 5.1 -> 4.6
+// ms).  Above kLocalMaxNnz the repeated reads cost more than the peel's barriers.
 // ------------------------------------------------------------------------
 
 constexpr int64_t kLocalMaxNnz = 40000000;
