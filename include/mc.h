@@ -97,7 +97,8 @@ typedef struct {
   int32_t graph;
   /* 1 = every worker searches its root's whole tree itself (the warps of a
    * block worker still share it through the block's pool); 0 = (default) a
-   * root of at most 1,024 candidates whose colouring leaves branches copies
+   * root of at most 1,024 candidates whose colouring leaves branches (with at
+   * most 128 candidates: that a few Branch nodes do not decide) copies
    * its adjacency matrix to a device arena and becomes a task of one GPU-wide
    * queue, which every warp serves, so one hard neighbourhood spreads over
    * the GPU */

@@ -257,14 +257,15 @@ __device__ bool raise_incumbent(int32_t *best, int32_t *lock, int32_t *wit, cons
   const int lane = threadIdx.x & 31;
   int ok = 0;
   if (lane == 0) {
-    if (size > ld_volatile(best + gidx)) {
-      long long it = 0;
-      while (atomicCAS(lock + gidx, 0, 1) != 0) {
-        if (++it > spin_limit) { atomicExch(err, kDevTimeout); break; }
-        __nanosleep(64);
-      }
-      if (it <= spin_limit) ok = (size > ld_volatile(best + gidx)) ? 1 : 2;
+    // a warp whose clique is no longer larger stops waiting: thousands that
+    // find their first clique at once would each take the lock in turn
+    long long it = 0;
+    bool held = false;
+    while (size > ld_volatile(best + gidx) && !(held = atomicCAS(lock + gidx, 0, 1) == 0)) {
+      if (++it > spin_limit) { atomicExch(err, kDevTimeout); break; }
+      __nanosleep(64);
     }
+    if (held) ok = (size > ld_volatile(best + gidx)) ? 1 : 2;
   }
   ok = __shfl_sync(0xffffffffu, ok, 0);
   if (ok == 0) return false;

@@ -33,7 +33,8 @@
 //                shared-memory pool (a busy warp hands the shallowest untried
 //                branch to an idle one);
 //   big class    larger: as the block class with the matrix in global memory.
-// Task queue: a root whose colouring leaves branches copies its matrix to an
+// Task queue: a root whose colouring leaves branches (in the warp class, one
+// that a few nodes do not decide) copies its matrix to an
 // arena and becomes one task of a GPU-wide ring; the task kernel searches
 // tasks with single warps, which hand the untried branches of their
 // shallowest level to the ring while other warps wait for work, so one hard
@@ -94,6 +95,7 @@ struct SA {
   int64_t sort_stride;
   int32_t *overflow;             // roots too large for this launch's layout (or null)
   int64_t *noverflow;
+  int32_t task_warps;            // warps of the task kernel
   int32_t offer_nodes;           // Branch nodes of a task between two looks for waiting warps
 };
 
@@ -374,8 +376,8 @@ struct Root {
 // Take k consecutive queue positions, all or none; returns the first or -1.
 // The queue is a ring of task_cap slots: positions are taken only while
 // fewer than task_cap are taken and not yet handed out.  The positions count
-// as pending from here on (the caller still holds a task, or runs before the
-// task kernel, so the count cannot reach zero in between).  tries bounds the
+// as pending from here on (the caller still holds a task, so the count cannot
+// reach zero in between).  tries bounds the
 // compare-and-swap attempts: thousands of warps offer branches at once when
 // the queue runs dry, and one that loses goes on searching instead.
 __device__ int reserve_tasks(const SA &a, int k, long long tries) {
@@ -391,6 +393,21 @@ __device__ int reserve_tasks(const SA &a, int k, long long tries) {
     cur = prev;
   }
   return -1;
+}
+
+// One queue position for a root, before the task kernel starts; -1: the ring is
+// full.  Nothing is handed out yet, so the first task_cap takers have theirs for
+// good and a later one only takes back its own count.  (A compare-and-swap lets
+// one of thousands of warps through per round trip to L2: 90,000 roots took 115
+// ms.)
+__device__ int reserve_root_task(const SA &a) {
+  const int t = atomicAdd(a.ntasks, 1);
+  if (t >= a.task_cap) {
+    atomicSub(a.ntasks, 1);
+    return -1;
+  }
+  atomicAdd(a.pending, 1);
+  return t;
 }
 
 // Reserve arena room and a record for a root's matrix and P list.  Returns
@@ -466,17 +483,19 @@ __device__ void emit_task(const SA &a, const Root &r, const uint32_t *A, int Ws,
 
 // Depth-first Branch from one level (csize0 = |C| including the root u).
 // Stack levels above the start hold (P, B, omega-at-colouring, chosen).
-// If `pool` is not null, untried branches are handed to idle warps.
+// If `pool` is not null, untried branches are handed to idle warps.  After
+// `limit` nodes it stops: true if the search is done, else `rest` holds the
+// candidates of the first level without the branches that are.
 template <int WPL, bool SM>
-__device__ void dfs(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, uint32_t *stk, int csize0,
+__device__ bool dfs(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, uint32_t *stk, int csize0,
                     Bits<WPL> P, Bits<WPL> B, Bits<WPL> C, int wat, Pool<WPL> *pool, unsigned long long &nodes,
-                    unsigned long long &donations) {
+                    unsigned long long &donations, long long limit = LLONG_MAX, Bits<WPL> *rest = nullptr) {
   const int lane = threadIdx.x & 31;
   const int stride = 64 * WPL + 2;
   int d = 0, csize = csize0;
   long long spent = 0;
   for (;;) {
-    if (__shfl_sync(FULL, lane == 0 ? *(volatile int32_t *)a.err : 0, 0)) return;
+    if (__shfl_sync(FULL, lane == 0 ? *(volatile int32_t *)a.err : 0, 0)) return true;
     int om = read_best(a.best, r.g);
     if (om > wat) {
       color_ise<WPL, SM>(A, Ws, W, P, om - csize, B);
@@ -484,7 +503,7 @@ __device__ void dfs(const SA &a, const Root &r, const uint32_t *A, int Ws, int W
     }
     int v = bhighest(B);
     if (v < 0) {
-      if (d == 0) return;
+      if (d == 0) return true;
       d--;
       uint32_t *lv = stk + (int64_t)d * stride;
 #pragma unroll
@@ -497,6 +516,15 @@ __device__ void dfs(const SA &a, const Root &r, const uint32_t *A, int Ws, int W
       bclear(C, ch);
       csize--;
       continue;
+    }
+    if (spent >= limit) {
+      *rest = P;
+      if (d > 0) {
+#pragma unroll
+        for (int k = 0; k < WPL; k++) rest->w[k] = stk[k * 32 + lane];
+        bset(*rest, level_word(stk + 64 * WPL + 1));
+      }
+      return false;
     }
     bclear(B, v);
     bclear(P, v);
@@ -771,7 +799,7 @@ __device__ int open_record(const SA &a, const Root &r, int m, int *t_out) {
   *t_out = -1;
   const int rec = reserve_record(a, rm, Wsm, &off);
   if (rec < 0) return -1;
-  *t_out = reserve_tasks(a, 1, a.spin);
+  *t_out = reserve_root_task(a);
   RootRec rr;
   rr.u = r.u;
   rr.g = r.g;
@@ -802,12 +830,10 @@ __device__ __forceinline__ uint32_t permuted_row(const uint32_t *A, int Ws, cons
   return mine;
 }
 
-// A warp's root (at most kWarpCap candidates, those left by the core test in
-// al) as a task: its candidates in minimum-width order (see width_keys), its
-// matrix and P list copied to the arena once.  keys: kWarpCap words.  False,
-// publishing nothing, without room for the record or in the queue.
-__device__ bool publish_warp(const SA &a, const Root &r, const uint32_t *A, int Ws, int W, const uint32_t *al,
-                             uint32_t *keys) {
+// The candidates of a warp's root (at most kWarpCap) in bits al, in
+// minimum-width order (see width_keys); returns how many.  keys: kWarpCap
+// words.
+__device__ int width_keys_warp(const Root &r, const uint32_t *A, int Ws, int W, const uint32_t *al, uint32_t *keys) {
   const int lane = threadIdx.x & 31;
   int deg[4], m = 0;
 #pragma unroll
@@ -844,21 +870,35 @@ __device__ bool publish_warp(const SA &a, const Root &r, const uint32_t *A, int 
       }
   }
   __syncwarp();
+  bitonic_desc<false>((int *)keys, kWarpCap, lane, 32);
+  return m;
+}
+
+// The matrix and P list of those m candidates in that order, to dm (m rows of
+// Wsm words) and dp, by a warp.
+__device__ __forceinline__ void permute_rows_warp(const Root &r, const uint32_t *A, int Ws, const uint32_t *keys,
+                                                  int m, uint32_t *dm, int Wsm, int *dp) {
+  const int lane = threadIdx.x & 31;
+  for (int i = 0; i < m; i++) {
+    const uint32_t x = permuted_row(A, Ws, keys, m, i);
+    if (lane < Wsm) dm[i * Wsm + lane] = x;
+  }
+  for (int i = lane; i < m; i += 32) dp[i] = r.Pidx[0xffff - (int)(keys[i] & 0xffffu)];
+  __syncwarp();
+}
+
+// A warp's root as a task, its matrix copied to the arena once.  False,
+// publishing nothing, without room for the record or in the queue.
+__device__ bool publish_warp(const SA &a, const Root &r, const uint32_t *A, int Ws, const uint32_t *keys, int m) {
+  const int lane = threadIdx.x & 31;
   int rec = -1, t = -1;
   if (lane == 0) rec = open_record(a, r, m, &t);
   rec = __shfl_sync(FULL, rec, 0);
   t = __shfl_sync(FULL, t, 0);
   if (t < 0) return false;
-  bitonic_desc<false>((int *)keys, kWarpCap, lane, 32);
   uint32_t *dm = a.arena + __shfl_sync(FULL, lane == 0 ? a.recs[rec].off : 0ll, 0);
   const int Wsm = ((m + 31) >> 5) | 1;
-  for (int i = 0; i < m; i++) {
-    const uint32_t x = permuted_row(A, Ws, keys, m, i);
-    if (lane < Wsm) dm[i * Wsm + lane] = x;
-  }
-  int *dp = (int *)(dm + m * Wsm);
-  for (int i = lane; i < m; i += 32) dp[i] = r.Pidx[0xffff - (int)(keys[i] & 0xffffu)];
-  __syncwarp();
+  permute_rows_warp(r, A, Ws, keys, m, dm, Wsm, (int *)(dm + m * Wsm));
   __threadfence();
   Bits<1> C, P;
   bzero(C);
@@ -975,19 +1015,54 @@ __device__ __forceinline__ int edges_upto(const SA &a, const int *Pidx, int p, u
   return dev::warp_sum(hits);
 }
 
+// Branch nodes that a warp expands on its root before what is left becomes a
+// task: few while the task kernel's warps have no task each, many once they
+// have, or while no clique is known (a first clique lies deeper than a few
+// nodes, and every root would become a task under omega 0).  With every
+// branching root published at once, 300 graphs of 150-400 vertices took 130 ms
+// (now 2.6), 5,000 of 30-80 vertices 160 (4.5), a 300 x 300 grid without a lower
+// bound 118 (5.8, the search 0.2), R-MAT scale 17 (ef 12) without one 166 (7.6).
+// 16 nodes always: R-MAT scale 15 loaded and solved 6% slower, the 300 graphs
+// 3.2 ms; 32 instead of 64: 2.8 ms; 256: R-MAT 17 without a bound 10.3 ms.
+constexpr int kRootNodes = 4, kRootNodesBusy = 64;
+
 // Branching roots leave the kernel's registers to the others: their part is
-// kept out of line.
-__device__ __noinline__ void branch_warp_root(const SA &a, const Root &r, uint32_t *A, int Ws, int W,
-                                              const uint32_t *al, uint32_t *keys, uint32_t *stk, int om,
+// kept out of line.  What a root that needs more nodes has left becomes a
+// task; without room for one it is searched here, in the order that the task
+// would have had.
+__device__ __noinline__ void branch_warp_root(const SA &a, Root r, uint32_t *A, int Ws, int W, uint32_t *al,
+                                              uint32_t *keys, int *Pidx, uint32_t *stk, int om,
                                               unsigned long long *nodes) {
-  if (a.tasks && publish_warp(a, r, A, Ws, W, al, keys)) return;
   const int lane = threadIdx.x & 31;
-  Bits<1> P, B, C;
+  Bits<1> P, B, C, rest;
   P.w[0] = (lane < 4) ? al[lane] : 0u;
   bzero(C);
   unsigned long long n = 0, don = 0;
   color_ise<1, true>(A, Ws, W, P, om - 1, B);
-  dfs<1, true>(a, r, A, Ws, W, stk, 1, P, B, C, om, (Pool<1> *)nullptr, n, don);
+  long long limit = LLONG_MAX;
+  if (a.tasks) {
+    const int t = lane == 0 ? *(volatile int32_t *)a.ntasks : 0;
+    limit = om == 0 || __shfl_sync(FULL, t, 0) >= a.task_warps ? kRootNodesBusy : kRootNodes;
+  }
+  if (!dfs<1, true>(a, r, A, Ws, W, stk, 1, P, B, C, om, (Pool<1> *)nullptr, n, don, limit, &rest)) {
+    __syncwarp();
+    if (lane < 4) al[lane] = rest.w[0];
+    __syncwarp();
+    const int m = width_keys_warp(r, A, Ws, W, al, keys);
+    if (!publish_warp(a, r, A, Ws, keys, m)) {
+      const int Wm = (m + 31) >> 5, Wsm = Wm | 1;
+      int *dp = (int *)(stk + m * Wsm);  // the stack is free: it has room for more than m rows of 66 words
+      permute_rows_warp(r, A, Ws, keys, m, stk, Wsm, dp);
+      for (int i = lane; i < m * Wsm; i += 32) A[i] = stk[i];
+      for (int i = lane; i < m; i += 32) Pidx[i] = dp[i];
+      __syncwarp();
+      r.p = m;
+      om = read_best(a.best, r.g);
+      P.w[0] = first_bits(m);
+      color_ise<1, true>(A, Wsm, Wm, P, om - 1, B);
+      dfs<1, true>(a, r, A, Wsm, Wm, stk, 1, P, B, C, om, (Pool<1> *)nullptr, n, don);
+    }
+  }
   *nodes += n;
 }
 
@@ -1086,8 +1161,7 @@ __global__ void __launch_bounds__(kSW * 32, 6) search_warp_kernel(SA a) {
     color_ise<1, true>(S.A, Ws, W, al, om - 1, B);
     if (!bany(B)) continue;
     branched++;
-    const Root r{u, g, S.Pidx, p};
-    branch_warp_root(a, r, S.A, Ws, W, S.al, (uint32_t *)S.hk, stk, om, &nodes);
+    branch_warp_root(a, Root{u, g, S.Pidx, p}, S.A, Ws, W, S.al, (uint32_t *)S.hk, S.Pidx, stk, om, &nodes);
   }
   if (lane == 0) {
     atomicAdd(a.counters + 0, colored);
@@ -2351,6 +2425,7 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   const int blocks_b = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_b, small_cap);
   const int blocks_m = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_m, small_cap);
   const int blocks_t = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_t, std::max<int64_t>(1, (g->n + 15) / 16));
+  a.task_warps = blocks_t * kTW;
   const int64_t stride_b = (int64_t)(std::min(kbound, 1024) + 2) * (64 + 2);
   const int64_t stride_m = (int64_t)(std::min(kbound, kMidCap) + 2) * (64 + 2);
   // levels above the compact form, then those of the compact form (uint4)

@@ -674,3 +674,42 @@ def test_validate_by_row_length(mc):
     rp[5] -= 700  # a row and its neighbour overlap
     with pytest.raises(mc.MCError):
         mc.mc_load_csr(rp, g.col_idx, mc.MC_VALIDATE)
+
+
+def _grid(a, b):
+    i = np.arange(a * b).reshape(a, b)
+    return gg.from_edges(a * b, np.concatenate([i[:, :-1].ravel(), i[:-1].ravel()]),
+                         np.concatenate([i[:, 1:].ravel(), i[1:].ravel()]), "grid%dx%d" % (a, b))
+
+
+@pytest.mark.parametrize("g", [_grid(60, 70), gg.cycle(4001), gg.path(500), gg.complete_bipartite(4, 900)],
+                         ids=lambda g: g.name)
+def test_roots_of_few_nodes_stay_with_their_warp(mc, g):
+    """A root is published once its warp has expanded four Branch nodes on it.
+    In a triangle-free graph a root's tree has a node per candidate, and these
+    graphs have at most four later neighbours per vertex: without a lower
+    bound, where every root branches, none becomes a task."""
+    h = load(mc, g)
+    for opts in (dict(heuristic=2), dict(heuristic=2, no_neigh_cores=True), dict(heuristic=2, split_nodes=1)):
+        om, wit, st = mc.mc_max_clique(h, **opts)
+        assert om == 2 and oracle.is_clique(g, wit)
+        assert st["roots_branched"] > 0 and st["tasks"] == 0, opts
+    h.close()
+
+
+def test_batch_of_branching_roots(mc):
+    """Many small graphs whose roots nearly all branch, some for a few nodes
+    and some for long enough to become tasks: omega of each as the oracle's."""
+    gs = [gg.erdos_renyi(40 + 11 * i, (0.8, 0.7, 0.5, 0.3)[i % 4], seed=i) for i in range(12)]
+    voff = np.r_[0, np.cumsum([g.n for g in gs])].astype(np.int64)
+    rp = np.r_[0, np.cumsum(np.concatenate([np.diff(g.row_ptr) for g in gs]))].astype(np.int64)
+    ci = np.concatenate([g.col_idx + v for g, v in zip(gs, voff)]).astype(np.int32)
+    want = [oracle.max_clique(g)[0] for g in gs]
+    h = mc.mc_load_batch(voff, rp, ci, mc.MC_VALIDATE)
+    for opts in (dict(), dict(heuristic=2), dict(heuristic=2, split_nodes=1), dict(heuristic=2, no_split=True)):
+        om, wit, st = mc.mc_max_clique_batch(h, **opts)
+        assert list(om) == want, opts
+        for g, w in zip(gs, wit):
+            assert oracle.is_clique(g, w)
+        assert (st["tasks"] > 0) == (not opts.get("no_split"))
+    h.close()
