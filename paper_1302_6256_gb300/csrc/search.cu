@@ -414,6 +414,8 @@ __device__ int reserve_root_task(const SA &a) {
 // the record index (and the arena offset) or -1 without room.
 __device__ int reserve_record(const SA &a, const Root &r, int Ws, long long *off_out) {
   const long long need = ((long long)r.p * Ws + r.p + 31) & ~31ll;  // records start on 128-byte lines
+  // a root that does not fit takes nothing: smaller ones after it still may
+  if ((long long)*(volatile unsigned long long *)a.arena_used + need > a.arena_cap) return -1;
   const long long off = (long long)atomicAdd(a.arena_used, (unsigned long long)need);
   if (off + need > a.arena_cap) return -1;
   const int rec = atomicAdd(a.nrec, 1);
