@@ -91,7 +91,7 @@ struct SA {
   int32_t *task_next;            // tickets taken by the task kernel's warps (runs ahead of ntasks by the waiting ones)
   int32_t *pending;              // tasks published and not yet finished
   int32_t *progress;             // heartbeat: bumped every 256 Branch nodes
-  uint32_t *sort;                // per-block room for a sorted matrix (roots searched in place; or null)
+  uint32_t *sort;                // per-block room for a sorted matrix (roots searched in place)
   int64_t sort_stride;
   int32_t *overflow;             // roots too large for this launch's layout (or null)
   int64_t *noverflow;
@@ -1668,29 +1668,29 @@ __global__ void __launch_bounds__(kBT, (SM && (PC <= kMidCap || DENSE)) ? 2 : 1)
       // built); a task, or searched here: the matrix goes through global
       // memory, and the colouring test is taken again in the new order.  In
       // rank order the search in place took 1 to 10 s on 2 of 3 R-MAT scale-20
-      // graphs (5.7 and 9.4 ms sorted), 10-14 ms at scale 21 (9)
+      // graphs (5.7 and 9.4 ms sorted), 10-14 ms at scale 21 (9).  Where most
+      // roots of a dense graph find the arena full: G(1200, 0.4) 187 ms in
+      // rank order, 175 sorted; G(1500, 0.3), smaller trees, 90 and 100
       const int m = width_keys(A, p, Ws, W, al, (uint32_t *)hk, rm);
       if (a.tasks && publish_sorted(a, r, A, Ws, (uint32_t *)hk, m, ctl + 8)) continue;
-      if (a.sort) {
-        uint32_t *dm = a.sort + (int64_t)blockIdx.x * a.sort_stride;
-        Wr = (m + 31) >> 5;
-        Wsr = Wr | 1;
-        int *dp = (int *)(dm + (int64_t)m * Wsr);
-        permute_rows(A, Ws, Pidx, (uint32_t *)hk, m, dm, Wsr, dp);
-        __syncthreads();
-        for (int i = tid; i < m * Wsr; i += kBT) A[i] = dm[i];
-        for (int i = tid; i < m; i += kBT) Pidx[i] = dp[i];
-        __syncthreads();
-        r.p = m;
-        if (wid == 0) {
-          P.w[0] = first_bits(m);
-          color_ise<WPL, SM>(A, Wsr, Wr, P, om - 1, B);
-          have = bany(B);
-          if (lane == 0) ctl[4] = have ? 1 : 0;
-        }
-        __syncthreads();
-        if (!ctl[4]) continue;
+      uint32_t *dm = a.sort + (int64_t)blockIdx.x * a.sort_stride;
+      Wr = (m + 31) >> 5;
+      Wsr = Wr | 1;
+      int *dp = (int *)(dm + (int64_t)m * Wsr);
+      permute_rows(A, Ws, Pidx, (uint32_t *)hk, m, dm, Wsr, dp);
+      __syncthreads();
+      for (int i = tid; i < m * Wsr; i += kBT) A[i] = dm[i];
+      for (int i = tid; i < m; i += kBT) Pidx[i] = dp[i];
+      __syncthreads();
+      r.p = m;
+      if (wid == 0) {
+        P.w[0] = first_bits(m);
+        color_ise<WPL, SM>(A, Wsr, Wr, P, om - 1, B);
+        have = bany(B);
+        if (lane == 0) ctl[4] = have ? 1 : 0;
       }
+      __syncthreads();
+      if (!ctl[4]) continue;
     }
     block_search<WPL, SM>(a, r, A, Wsr, Wr, stk, pool, have, P, B, C, cs, wat, nodes, don);
     __syncthreads();
@@ -2442,7 +2442,7 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
     stk_t = (uint32_t *)p;
   }
 
-  if (no_split && kbound > wmax) {
+  if (kbound > wmax) {  // also for roots that find the queue or the arena full
     const int cap = std::min(kbound, 1024);
     a.sort_stride = (int64_t)cap * (((cap + 31) / 32) | 1) + cap;
     const int blocks = std::max({blocks_b, blocks_m, g->sm_count * 2});

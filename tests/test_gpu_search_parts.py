@@ -6,6 +6,9 @@ import subprocess
 
 import pytest
 
+import graphgen as gg
+import oracle
+
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
@@ -33,6 +36,10 @@ extern "C" int t_records(int n, const int *cand, int *out, uint32_t *arena, long
   a.nrec = nrec;
   records_kernel<<<1, 1>>>(a, n, cand, out);
   return (int)cudaDeviceSynchronize();
+}
+extern "C" long long t_ws_bytes(mc_graph *g, const char *name) {
+  auto it = g->ws.find(name);
+  return it == g->ws.end() ? -1 : (long long)it->second.bytes;
 }
 """
 
@@ -75,3 +82,19 @@ def test_record_that_does_not_fit_takes_nothing(lib):
                               ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]
     assert lib.t_records(7, _p(cand), _p(out), _p(arena), 512, _p(used), _p(recs), 64, _p(nrec)) == 0
     assert out.view(7, 2).tolist() == [[0, 0], [-1, -1], [1, 320], [2, 384], [-1, -1], [3, 448], [-1, -1]]
+
+
+def test_full_arena_keeps_the_search_order(mc, lib):
+    """Block roots of a dense graph overflow the arena (4 words per CSR entry;
+    a root of 400 candidates takes 5,600).  Those searched in place have the
+    room to be put in minimum-width order first, and omega is kept."""
+    g = gg.relabel(gg.erdos_renyi(1000, 0.4, planted=28, seed=1), 3)
+    h = mc.mc_load_csr(torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col_idx).cuda(), mc.MC_VALIDATE)
+    for opts in (dict(), dict(heuristic=2), dict(no_bitmap=True), dict(layout=1)):
+        om, wit, st = mc.mc_max_clique(h, **opts)
+        assert om == 28 and oracle.is_clique(g, wit)
+        assert st["max_core"] > 256 and st["roots_branched"] > 100
+    lib.t_ws_bytes.argtypes, lib.t_ws_bytes.restype = [ctypes.c_void_p, ctypes.c_char_p], ctypes.c_longlong
+    cap = st["max_core"]
+    assert lib.t_ws_bytes(h.handle, b"se.sort") >= 4 * (cap * (((cap + 31) // 32) | 1) + cap)
+    h.close()
