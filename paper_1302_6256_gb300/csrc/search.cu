@@ -1893,8 +1893,10 @@ __device__ void write_task_clique(int32_t *base, const SA &a, const TaskCtx &T, 
 }
 
 // Hand the untried branches of the shallowest level that has some to the
-// queue, one task each; that level keeps none.  All or nothing: without room
-// in the queue nothing changes.  Returns the tasks written.
+// queue, one task each; that level keeps none, also among its candidates, so
+// that a colouring under a higher omega does not bring them back.  All or
+// nothing: without room in the queue nothing changes.  Returns the tasks
+// written.
 template <int NW>
 __device__ int offer_level(const SA &a, const TaskCtx &T, TaskSmem &S, uint32_t *stk, int d, Set<NW> &P, Set<NW> &B) {
   const int lane = threadIdx.x & 31;
@@ -1957,10 +1959,12 @@ __device__ int offer_level(const SA &a, const TaskCtx &T, TaskSmem &S, uint32_t 
       Set<NW> none;
 #pragma unroll
       for (int q = 0; q < NW; q++) none.w[q] = 0;
+      sstore<NW>(stk + l * kTStk, Pl);
       sstore<NW>(stk + l * kTStk + 8, none);
     }
     __syncwarp();
   } else {
+    P = Pl;
 #pragma unroll
     for (int q = 0; q < NW; q++) B.w[q] = 0;
   }
@@ -1992,6 +1996,7 @@ __device__ __noinline__ int offer_big(const SA &a, const TaskCtx &T, int chosen)
       bclear(Pl, x);
       emit_task(a, r, T.A, T.Ws, T.W, T.rec, t + i, Cl, T.cs - (chosen - l), Pl, x);
     }
+    q[lane] = Pl.w[0];
     q[32 + lane] = 0;
     __syncwarp();
     return k;

@@ -4,6 +4,7 @@ import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 import graphgen as gg
@@ -35,6 +36,57 @@ extern "C" int t_records(int n, const int *cand, int *out, uint32_t *arena, long
   a.rec_cap = rec_cap;
   a.nrec = nrec;
   records_kernel<<<1, 1>>>(a, n, cand, out);
+  return (int)cudaDeviceSynchronize();
+}
+
+// One warp's task on a compact matrix A (m rows of 4 words), d levels in stk,
+// the sets P, B of the current one in pb: what offer_level leaves of them, and
+// what it returns.
+__global__ void offer_kernel(SA a, const uint32_t *A, int m, uint32_t *stk, int d, uint32_t *pb, int *k) {
+  __shared__ __align__(16) TaskSmem S;
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < 4 * m; i += 32) S.A[i] = A[i];
+  for (int i = lane; i < m; i += 32) S.mem[i] = i;
+  __syncwarp();
+  TaskCtx T{};
+  T.cs = 1;
+  Set<4> P = sload<4>(pb), B = sload<4>(pb + 4);
+  __syncwarp();
+  const int r = offer_level<4>(a, T, S, stk, d, P, B);
+  if (lane == 0) {
+    sstore<4>(pb, P);
+    sstore<4>(pb + 4, B);
+    *k = r;
+  }
+}
+// The same for offer_big: levels of 66 words in lev, matrix of ws words a row.
+__global__ void offer_big_kernel(SA a, const uint32_t *A, int m, int ws, uint32_t *lev, int nlev, int *k) {
+  TaskCtx T{};
+  T.cs = 1 + nlev;
+  T.p = m;
+  T.W = (m + 31) / 32;
+  T.Ws = ws;
+  T.A = A;
+  T.lev = lev;
+  T.nlev = nlev;
+  const int r = offer_big(a, T, nlev);
+  if ((threadIdx.x & 31) == 0) *k = r;
+}
+// ctr: best, tasks, tickets, pending, error; the queue has 256 places
+extern "C" int t_offer(int big, const uint32_t *A, int m, int ws, uint32_t *stk, int d, uint32_t *pb, int *k, int *ctr,
+                       uint32_t *tasks, int *ready) {
+  SA a{};
+  a.best = ctr;
+  a.ntasks = ctr + 1;
+  a.task_next = ctr + 2;
+  a.pending = ctr + 3;
+  a.err = ctr + 4;
+  a.tasks = tasks;
+  a.ready = ready;
+  a.task_cap = 256;
+  a.spin = 1000;
+  if (big) offer_big_kernel<<<1, 32>>>(a, A, m, ws, stk, d, k);
+  else offer_kernel<<<1, 32>>>(a, A, m, stk, d, pb, k);
   return (int)cudaDeviceSynchronize();
 }
 extern "C" long long t_ws_bytes(mc_graph *g, const char *name) {
@@ -98,3 +150,65 @@ def test_full_arena_keeps_the_search_order(mc, lib):
     cap = st["max_core"]
     assert lib.t_ws_bytes(h.handle, b"se.sort") >= 4 * (cap * (((cap + 31) // 32) | 1) + cap)
     h.close()
+
+
+def _words(members, n):
+    w = np.zeros(n, np.uint32)
+    for x in members:
+        w[x >> 5] |= np.uint32(1) << np.uint32(x & 31)
+    return w
+
+
+def _members(words):
+    return {32 * i + b for i, w in enumerate(words) for b in range(32) if (int(w) >> b) & 1}
+
+
+@pytest.mark.parametrize("big", [False, True])
+@pytest.mark.parametrize("level", [0, 2, 3])
+def test_handed_over_branches_leave_their_level(lib, big, level):
+    """Four levels (three stored and the current one; in the large form all
+    stored), of which those from `level` on have untried branches.  The first
+    of these hands over every branch x with its candidates (x's neighbours
+    among the candidates that no branch before x took), and keeps neither the
+    branches nor, as candidates, the vertices: a later colouring of the level
+    cannot bring them back.  The other levels stay as they are."""
+    rng = np.random.default_rng(10 * level + big)
+    m, ws, sw = (300, 11, 32) if big else (100, 4, 4)
+    adj = np.triu(rng.random((m, m)) < 0.5, 1)
+    adj |= adj.T
+    A = np.stack([_words(np.nonzero(r)[0], ws) for r in adj])
+    P = [set(rng.choice(m, m // 2, replace=False).tolist()) for _ in range(4)]
+    B = [set(rng.choice(sorted(p), 9 + l, replace=False).tolist()) if l >= level else set() for l, p in enumerate(P)]
+    chosen = [int(v) for v in rng.choice(m, 4, replace=False)]
+    if big:
+        stk = np.zeros((4, 66), np.uint32)
+        for l in range(4):
+            stk[l, :32], stk[l, 32:64], stk[l, 65] = _words(P[l], 32), _words(B[l], 32), chosen[l]
+        pb = np.zeros(8, np.uint32)
+    else:
+        stk = np.zeros((3, 20), np.uint32)
+        for l in range(3):
+            stk[l, :4], stk[l, 8:12], stk[l, 17] = _words(P[l], 4), _words(B[l], 4), chosen[l]
+        pb = np.concatenate([_words(P[3], 4), _words(B[3], 4)])
+    dev = [torch.from_numpy(x.view(np.int32)).cuda() for x in (A.reshape(-1), stk.reshape(-1), pb)]
+    k, ctr = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(5, dtype=torch.int32, device="cuda")
+    ctr[0] = 1000  # no clique found here is larger
+    tasks, ready = torch.zeros(256 * 66, dtype=torch.int32, device="cuda"), torch.zeros(256, dtype=torch.int32, device="cuda")
+    i, p = ctypes.c_int, ctypes.c_void_p
+    lib.t_offer.argtypes = [i, p, i, i, p, i, p, p, p, p, p]
+    assert lib.t_offer(int(big), _p(dev[0]), m, ws, _p(dev[1]), 4 if big else 3, _p(dev[2]), _p(k), _p(ctr), _p(tasks),
+                       _p(ready)) == 0
+    assert int(k) == len(B[level]) and ctr.tolist() == [1000, len(B[level]), 0, len(B[level]), 0]
+    got, q = dev[1].cpu().numpy().view(np.uint32).reshape(stk.shape), dev[2].cpu().numpy().view(np.uint32)
+    for l in range(4):
+        if big:
+            g = _members(got[l, :32]), _members(got[l, 32:64])
+        else:
+            g = (_members(got[l, :4]), _members(got[l, 8:12])) if l < 3 else (_members(q[:4]), _members(q[4:]))
+        assert g == ((P[l] - B[l], set()) if l == level else (P[l], B[l])), l
+    t = tasks.cpu().numpy().view(np.uint32).reshape(256, 66)
+    left = set(P[level])
+    for n, x in enumerate(sorted(B[level], reverse=True)):
+        left.discard(x)
+        assert _members(t[n, 34:]) == left & set(np.nonzero(adj[x])[0].tolist())
+        assert x in _members(t[n, 2:34])
