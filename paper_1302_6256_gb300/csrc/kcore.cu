@@ -1,5 +1,5 @@
 // Core numbers.  Graphs of up to kLocalMaxNnz entries: kcore_local_kernel
-// (below); larger ones, and small ones of long cascades:
+// (below); larger ones, and small ones of few levels or of long cascades:
 // a bucketed parallel peel (Section 3: K(v) is the largest k
 // such that v lies in the k-core; the peel removes, level by level, every
 // vertex whose remaining degree is at most k).
@@ -562,7 +562,7 @@ __global__ void peel_pos_kernel(int64_t n, const int32_t *__restrict__ order, in
 // ------------------------------------------------------------------------
 // Core numbers by local updates, then the order shell by shell.
 //
-// Up to kLocalMaxNnz entries the level-by-level peel is bound by latency: a
+// The level-by-level peel of a graph of many levels is bound by latency: a
 // level costs a grid barrier and a chain of dependent steps per generation of
 // its cascade, and graphs have hundreds of levels (258 at R-MAT scale 22).
 // This kernel runs all levels at once, in two parts (the H-index operator
@@ -573,12 +573,12 @@ __global__ void peel_pos_kernel(int64_t n, const int32_t *__restrict__ order, in
 //           with a bound of at least h) may have fallen below h takes the
 //           largest k with at least k neighbours of bound >= k.  A step
 //           evaluates the listed vertices, and after a barrier the lowered
-//           ones list the neighbours they no longer support.  18 to 45 steps.
+//           ones list the neighbours they no longer support.  8 to 70 steps.
 //   order   with K known, the shells are peeled side by side: a vertex leaves
 //           in the first round in which at most K(v) of its neighbours of core
 //           number >= K(v) have not left in an earlier round; positions go by
 //           shell, then by round.  Each vertex has at most K(v) neighbours
-//           after it, so this is a degeneracy order.  13 to 43 rounds.
+//           after it, so this is a degeneracy order.  7 to 68 rounds.
 // Rows of at most 32 entries are read by a warp four at a time, rows of up to
 // kLocalWarpRow by a warp, longer ones by a block; a new value is found in
 // one pass over the row from a histogram of the values just below h.  A step
@@ -591,11 +591,16 @@ __global__ void peel_pos_kernel(int64_t n, const int32_t *__restrict__ order, in
 // Chung-Lu 1,000,003 vertices (35 M entries, K(G) = 438) 14.8 / 4.3.  Barriers
 // that count arrivals over the launch took another 4 .. 10% off (calls of the
 // first three and the last: 0.58 -> 0.55, 0.67 -> 0.63, 2.01 -> 1.92, 5.1 -> 4.6
-// ms).  Above kLocalMaxNnz the repeated reads cost more than the peel's barriers.
+// ms).  Above kLocalMaxNnz the repeated reads cost more than the peel's barriers,
+// and so they do below it where the levels are few for the rows (local_pays).
 // ------------------------------------------------------------------------
 
 constexpr int64_t kLocalMaxNnz = 40000000;
-constexpr int kLocalSteps = 256;
+// Steps (rounds) after which the graph is left to the peel.  R-MAT, Chung-Lu and
+// G(n, p) graphs of 10^3 .. 2 x 10^6 vertices need 8 to 70; what a graph with a long
+// cascade besides (a path of thousands at R-MAT scale 15: 5.7 ms by the peel
+// alone) pays on top is 128 steps of 9 us, 2.4 ms with 256 of them.
+constexpr int kLocalSteps = 128;
 constexpr int kLocalWarpRow = 2048;
 constexpr int kLocalBins = 256;                 // per warp; a block uses all its warps' bins
 constexpr int kLocalBlockBins = kLocalBins * kWarps;
@@ -606,10 +611,39 @@ struct LocalCtl {
   int pad[31];
   int n[3][32];   // [counter set][class 0..2]: listed vertices
   int all[32];    // [0..1] vertices of class 1, 2; [2] vertices placed; [3] largest core number
+  int hist[256];  // vertices by degree (degree_bin)
 };
 
+// Degrees in bins: one each below 32, then eight per power of two.
+__device__ __forceinline__ int degree_bin(int d) {
+  const int e = 31 - __clz(d | 1);
+  return d < 32 ? d : 32 + (e - 5) * 8 + ((d >> (e - 3)) & 7);
+}
+__device__ __forceinline__ int bin_degree(int b) {  // the bin's smallest degree
+  return b < 32 ? b : (8 + ((b - 32) & 7)) << (2 + ((b - 32) >> 3));
+}
+
+// Whether this kernel beats the peel, from the degrees alone.  The peel pays per
+// level, of which there are at most H - L: no core number is above the largest H
+// with H vertices of degree >= H, and few are below L, the degree that 1/64 of
+// the vertices do not reach.  This kernel pays per row entry, about 17 reads
+// each.  Up to 4.5 M entries the reads are in L2 and 16 levels are enough; above,
+// the line of equal times is at 28 levels per million entries.  This kernel /
+// the peel, in ms with loading (0.5): H - L = 15, 4.0 M entries 1.39 / 0.81;
+// 16, 0.1 M 0.80 / 0.86; 29, 0.9 M 1.53 / 2.47; 35, 4.0 M 2.20 / 2.65; 19, 8.0 M
+// 2.00 / 1.00; 52, 10 M 1.80 / 1.19; 251, 6.0 M 3.04 / 2.97; 333, 12 M 4.10 / 3.43;
+// 596, 20 M 3.95 / 4.85; 650, 30 M 8.39 / 6.73; 1,058, 32 M 4.71 / 6.61; 1,386, 31
+// M 5.75 / 6.27.  Grids, paths, trees and stars have H - L of 0 to 8: 2.5 / 1.1 (a
+// 100 x 100 grid), 25.6 / 9.0 (a star of 10^7).  Dense graphs of nearly one degree
+// and no hubs are decided in a step or two here (K(300, 5000) 0.65 / 0.78).
+__device__ __forceinline__ bool local_pays(int high, int low, int maxdeg, int64_t nnz) {
+  const int levels = high - low;
+  if (levels < 16) return low >= 64 && nnz < 8000000 && maxdeg <= 8192;
+  return nnz < 4500000 || levels * (int64_t)1000000 >= 28 * nnz;
+}
+
 struct LocalArgs {
-  int64_t n;
+  int64_t n, nnz;
   int cap;  // sqrt(entries)
   const int64_t *rp;
   const int32_t *ci;
@@ -931,7 +965,9 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_local_kernel(LocalArgs a) {
   int *bin = S.bins + wib * kLocalBins, *buf = S.stage[wib];
   const int64_t n = a.n;
 
-  // ---- bounds, and the vertices of longer rows
+  // ---- bounds, the vertices of longer rows, and the degrees
+  for (int i = threadIdx.x; i < 256; i += kThreads) S.bins[i] = 0;
+  __syncthreads();
   int top = 0;
   for (int64_t b = gwarp * 32; b < n; b += nwarps * 32) {
     const int64_t v = b + lane;
@@ -942,6 +978,12 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_local_kernel(LocalArgs a) {
       a.h[v] = x;
       a.stamp[v] = 0;
       top = max(top, d);
+    }
+    const int db = v < n ? degree_bin(d) : -1;
+    if (__all_sync(0xffffffffu, db == __shfl_sync(0xffffffffu, db, 0))) {
+      if (lane == 0) atomicAdd(&S.bins[db], 32);
+    } else if (db >= 0) {
+      atomicAdd(&S.bins[db], 1);
     }
 #pragma unroll
     for (int q = 1; q < 3; q++) {
@@ -956,7 +998,34 @@ __global__ void __launch_bounds__(kThreads, 1) kcore_local_kernel(LocalArgs a) {
   }
   top = dev::warp_max(top);
   if (lane == 0) atomicMax(a.maxdeg, top);
+  __syncthreads();
+  for (int i = threadIdx.x; i < 256; i += kThreads)
+    if (S.bins[i]) atomicAdd(&a.ctl->hist[i], S.bins[i]);
   if (!local_barrier(a, S, nullptr)) return;
+  if (wib == 0) {
+    int c[8], sum = 0, high = 0, low = INT_MAX;
+#pragma unroll
+    for (int q = 0; q < 8; q++) sum += c[q] = __ldcg(&a.ctl->hist[8 * lane + q]);
+    int below = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, below, o);
+      if (lane >= o) below += y;
+    }
+    below -= sum;
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      const int d = 8 * lane + q < 240 ? bin_degree(8 * lane + q) : INT_MAX;
+      if (n - below >= d) high = max(high, d);
+      below += c[q];
+      if (below > n / 64) low = min(low, d);
+    }
+    high = __reduce_max_sync(0xffffffffu, high);
+    low = __reduce_min_sync(0xffffffffu, low);
+    if (lane == 0) S.red[0] = local_pays(high, low, __ldcg(a.maxdeg), a.nnz);
+  }
+  __syncthreads();
+  if (!S.red[0]) return;  // done stays 0: left to the peel
   const int all1 = __ldcg(&a.ctl->all[0]), all2 = __ldcg(&a.ctl->all[1]);
 
   // ---- values
@@ -1300,6 +1369,7 @@ static int launch_local(mc_graph *g, long long spin_limit, const int32_t **out) 
   const int64_t n = g->n;
   LocalArgs a{};
   a.n = n;
+  a.nnz = g->nnz;
   a.cap = (int)std::sqrt((double)g->nnz) + 1;
   a.rp = g->row_ptr;
   a.ci = g->col_idx;
@@ -1310,7 +1380,7 @@ static int launch_local(mc_graph *g, long long spin_limit, const int32_t **out) 
   a.spin = spin_limit;
   const int64_t c1 = std::min<int64_t>(n, g->nnz / 33 + 1), c2 = std::min<int64_t>(n, g->nnz / kLocalWarpRow + 1);
   void *p;
-  MC_TRY(ws_get(g, "kl.v", (size_t)(4 * n + 3 * (c1 + c2) + 2 * (a.cap + 2)) * sizeof(int32_t), &p));
+  MC_TRY(ws_get(g, "kl.v", (size_t)(4 * n + 3 * (c1 + c2) + a.cap + 2) * sizeof(int32_t), &p));
   int32_t *w = (int32_t *)p;
   auto take = [&](int64_t k) {
     int32_t *r = w;
@@ -1327,14 +1397,14 @@ static int launch_local(mc_graph *g, long long spin_limit, const int32_t **out) 
   a.all[0] = take(c1);
   a.all[1] = take(c2);
   a.start = take(a.cap + 2);
-  a.taken = take(a.cap + 2);
-  MC_CUDA_TRY(cudaMemsetAsync(a.taken, 0, (size_t)(a.cap + 2) * sizeof(int32_t), g->stream));
-  MC_TRY(ws_get(g, "kl.ctl", sizeof(LocalCtl) + 64, &p));
-  MC_CUDA_TRY(cudaMemsetAsync(p, 0, sizeof(LocalCtl) + 64, g->stream));
+  const size_t ctl_bytes = sizeof(LocalCtl) + 64 + (size_t)(a.cap + 2) * sizeof(int32_t);
+  MC_TRY(ws_get(g, "kl.ctl", ctl_bytes, &p));
+  MC_CUDA_TRY(cudaMemsetAsync(p, 0, ctl_bytes, g->stream));
   a.ctl = (LocalCtl *)p;
   a.done = (int32_t *)((char *)p + sizeof(LocalCtl));
   a.maxdeg = a.done + 1;
   a.maxcore = a.done + 2;
+  a.taken = (int32_t *)((char *)p + sizeof(LocalCtl) + 64);
   *out = a.done;
   int per_sm = 0;
   MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kcore_local_kernel, kThreads, 0));
@@ -1382,8 +1452,8 @@ int launch_core_numbers(mc_graph *g, long long spin_limit) {
     g->cores_valid = true;
     return MC_OK;
   }
-  // mid-size graphs: all levels at once; the peel below is then a fallback,
-  // skipped on the device in a captured solve and not launched otherwise
+  // mid-size graphs: all levels at once, if that pays; the peel below is
+  // skipped on the device then in a captured solve and not launched otherwise
   const int32_t *skip = nullptr;
   if (g->nnz <= kLocalMaxNnz) {
     MC_TRY(launch_local(g, spin_limit, &skip));

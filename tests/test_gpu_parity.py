@@ -713,3 +713,35 @@ def test_batch_of_branching_roots(mc):
             assert oracle.is_clique(g, w)
         assert (st["tasks"] > 0) == (not opts.get("no_split"))
     h.close()
+
+
+def _random_graph(n, degree, seed):
+    r = np.random.default_rng(seed)
+    s, t = r.integers(0, n, (2, n * degree // 2))
+    return gg.from_edges(n, s[s != t], t[s != t], "random%d_%d" % (n, degree))
+
+
+@pytest.mark.parametrize("g,local", [
+    (_random_graph(300000, 4, 1), False), (_random_graph(100000, 60, 2), False), (_grid(150, 150), False),
+    (gg.path(40), False), (gg.star(5000), False), (gg.complete_bipartite(40, 20000), False),
+    (gg.disjoint_cliques([10] * 3000), False), (gg.rmat(13, 16, planted=20, seed=3), True),
+    (gg.chung_lu(20000, 2.5, 8.0, 300.0, planted=15, seed=3), True), (gg.complete(400), True),
+    (gg.complete_bipartite(200, 1000), True), (_random_graph(5000, 30, 3), True)], ids=lambda x: getattr(x, "name", str(x)))
+def test_core_numbers_go_to_the_cheaper_kernel(mc, g, local):
+    """Graphs of few levels (by their degrees) are left to the peel at once, which
+    takes three launches more than the local updates; those of many levels, and
+    small dense ones of nearly one degree, are not.  Core numbers and order hold
+    either way, also when the call is repeated by a captured solve."""
+    ref = oracle.core_numbers(g)
+    h = load(mc, g, flags=0)
+    n0 = mc.mc_launch_count()
+    core, kmax = mc.mc_core_numbers(h)
+    assert mc.mc_launch_count() - n0 == (1 if local else 4)
+    assert np.array_equal(core, ref) and kmax == int(ref.max())
+    assert _is_degeneracy_order(g, mc.mc_peel_order(h).copy(), core)
+    first = mc.mc_max_clique(h)
+    for _ in range(3):
+        om, wit, st = mc.mc_max_clique(h, graph=True)
+        assert om == first[0] and oracle.is_clique(g, wit) and st["max_core"] == kmax
+        assert np.array_equal(mc.mc_core_numbers(h)[0], ref)
+    h.close()
