@@ -25,8 +25,9 @@
 //           accepted clique writes its members ranked by decreasing degree
 //           (ties: smaller id) and marks them dead.
 //
-// Rounds repeat until every vertex is placed (four are queued before the host
-// reads the placed count; a round after the last vertex changes nothing).  Cliques live in one arena laid out like the
+// Rounds repeat until every vertex is placed (two are queued before the host
+// reads the placed count, four from the fifth on; a round after the last vertex
+// changes nothing).  Cliques live in one arena laid out like the
 // CSR: vertex v's candidates occupy the front of [rp[v], rp[v+1]) while it
 // grows, and its members other than v end at the top of that range, so the
 // arena is nnz int32 and needs no per-warp buffers or size limits.
@@ -61,7 +62,7 @@ constexpr unsigned kMidPerBlock = 8;     // few: at most this many per growing b
 constexpr int kTake = 4;                // listed vertices a warp takes at a time while there are many
 constexpr int kNear = 256;              // candidates, and entries of a row, that a warp holds in shared memory
 constexpr int kFly = 4;                 // entries or candidates a lane has in flight
-constexpr int kRoundsPerSync = 4;       // rounds queued before the host looks at the placed count
+constexpr int kRoundsPerSync = 4;       // rounds queued before the host looks at the placed count (half of them at first)
 
 struct OA {
   int64_t n;
@@ -1051,7 +1052,8 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
   int64_t *h = (int64_t *)((char *)g->h_small + 2560);
   int64_t placed = 0;
   for (int32_t r = 0;;) {
-    for (int i = 0; i < kRoundsPerSync; i++) {
+    const int rounds = r < kRoundsPerSync ? kRoundsPerSync / 2 : kRoundsPerSync;
+    for (int i = 0; i < rounds; i++) {
       a.round = r++;
       check_kernel<<<gt, 256, 0, g->stream>>>(a);
       grow_kernel<<<grow_blocks, kGT, 0, g->stream>>>(a, scratch, stride, any_big ? big_blocks : 0);

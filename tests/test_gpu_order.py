@@ -259,3 +259,19 @@ def test_relabel_by_row_length(mc, n):
     bits = float(np.log2(1.0 + gaps).mean())
     assert abs(mc.mc_gap_bits(h, order) - bits) <= GAP_RTOL * bits
     h.close()
+
+
+def test_clique_order_of_few_rounds_queues_few(mc):
+    """Rounds are queued two at first, then two, then four: an order of one
+    round launches less than one of three, one of three less than one of five,
+    and one of five as much as one of eight."""
+    count = []
+    for g, rounds in ((gg.disjoint_cliques([5] * 4), 1), (gg.path(6), 3), (gg.path(9), 5), (gg.path(16), 8)):
+        h = load(mc, g)
+        mc.mc_core_numbers(h)
+        n0 = mc.mc_launch_count()
+        got = mc.mc_clique_order(h)[2]
+        count.append(mc.mc_launch_count() - n0)
+        assert got.max() + 1 == rounds
+        h.close()
+    assert count[0] < count[1] < count[2] == count[3]
