@@ -61,7 +61,7 @@ constexpr int64_t kMidGrowMin = 512;     // ... while few vertices have more tha
 constexpr unsigned kMidPerBlock = 8;     // few: at most this many per growing block
 constexpr int kTake = 4;                // listed vertices a warp takes at a time while there are many
 constexpr int kNear = 256;              // candidates, and entries of a row, that a warp holds in shared memory
-constexpr int kFly = 4;                 // entries or candidates a lane has in flight
+constexpr int64_t kManyVertices = 50000;  // ten per growing warp; above, throughput is the bound (grow_kernel)
 constexpr int kRoundsPerSync = 4;       // rounds queued before the host looks at the placed count (half of them at first)
 
 struct OA {
@@ -138,31 +138,32 @@ __device__ __forceinline__ Fence set_fence(const OA &a, int64_t r0, int64_t r1, 
 
 // Greedy filter step of one warp: candidates in[i0, i1) other than w that are
 // in w's row go to out, in order; their first key to nb.  Each lane looks up
-// kFly candidates side by side: a binary search of the fence posts in shared
+// FLY candidates side by side: a binary search of the fence posts in shared
 // memory, then of the step - 1 entries behind one.  in and out may be the same
 // list (a tile is read before anything of it is written).
+template <int FLY>
 __device__ __forceinline__ int filter(const OA &a, const Fence &f, int w, const int32_t *in, int i0, int i1,
                                       int32_t *out, CKey &nb) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   int kept = 0;
-  for (int base = i0; base < i1; base += 32 * kFly) {
-    int x[kFly], lo[kFly], left[kFly];
-    bool keep[kFly];
+  for (int base = i0; base < i1; base += 32 * FLY) {
+    int x[FLY], lo[FLY], left[FLY];
+    bool keep[FLY];
 #pragma unroll
-    for (int q = 0; q < kFly; q++) {
+    for (int q = 0; q < FLY; q++) {
       const int i = base + 32 * q + lane;
       x[q] = i < i1 ? in[i] : -1;
       lo[q] = 0;  // posts <= x
     }
     for (int st = f.top; st > 0; st >>= 1) {
 #pragma unroll
-      for (int q = 0; q < kFly; q++)
+      for (int q = 0; q < FLY; q++)
         if (base + 32 * q < i1 && lo[q] + st <= f.posts && f.post[lo[q] + st - 1] <= x[q]) lo[q] += st;
     }
     int any = 0;
 #pragma unroll
-    for (int q = 0; q < kFly; q++) {
+    for (int q = 0; q < FLY; q++) {
       keep[q] = lo[q] > 0 && f.post[lo[q] - 1] == x[q];
       const int at = (lo[q] - 1) * f.step + 1;
       left[q] = (lo[q] > 0 && !keep[q]) ? min(f.step - 1, f.len - at) : 0;
@@ -170,12 +171,12 @@ __device__ __forceinline__ int filter(const OA &a, const Fence &f, int w, const 
       any |= left[q];
     }
     while (any) {
-      int y[kFly];
+      int y[FLY];
 #pragma unroll
-      for (int q = 0; q < kFly; q++) y[q] = left[q] ? f.row[lo[q] + (left[q] >> 1)] : 0;
+      for (int q = 0; q < FLY; q++) y[q] = left[q] ? f.row[lo[q] + (left[q] >> 1)] : 0;
       any = 0;
 #pragma unroll
-      for (int q = 0; q < kFly; q++) {
+      for (int q = 0; q < FLY; q++) {
         if (left[q] == 0) continue;
         const int h = left[q] >> 1;
         if (y[q] == x[q]) {
@@ -192,7 +193,7 @@ __device__ __forceinline__ int filter(const OA &a, const Fence &f, int w, const 
     }
     __syncwarp();
 #pragma unroll
-    for (int q = 0; q < kFly; q++) {
+    for (int q = 0; q < FLY; q++) {
       keep[q] = keep[q] && x[q] != w;
       const unsigned m = __ballot_sync(FULL, keep[q]);
       if (keep[q]) {
@@ -214,22 +215,23 @@ struct GrowSmem {
 
 // Alive entries of v's row [s0, s1), one warp: to out (row order: ascending
 // id), their first key to bk.
+template <int FLY>
 __device__ __forceinline__ int alive_of(const OA &a, int64_t s0, int64_t s1, int32_t *out, CKey &bk) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   int cnt = 0;
-  for (int64_t eb = s0; eb < s1; eb += 32 * kFly) {
-    int u[kFly];
-    bool ok[kFly];
+  for (int64_t eb = s0; eb < s1; eb += 32 * FLY) {
+    int u[FLY];
+    bool ok[FLY];
 #pragma unroll
-    for (int q = 0; q < kFly; q++) {
+    for (int q = 0; q < FLY; q++) {
       const int64_t e = eb + 32 * q + lane;
       u[q] = e < s1 ? a.ci[e] : -1;
     }
 #pragma unroll
-    for (int q = 0; q < kFly; q++) ok[q] = u[q] >= 0 && a.alive[u[q]] != 0;
+    for (int q = 0; q < FLY; q++) ok[q] = u[q] >= 0 && a.alive[u[q]] != 0;
 #pragma unroll
-    for (int q = 0; q < kFly; q++) {
+    for (int q = 0; q < FLY; q++) {
       const unsigned m = __ballot_sync(FULL, ok[q]);
       if (ok[q]) {
         out[cnt + __popc(m & lt)] = u[q];
@@ -249,6 +251,7 @@ __device__ __forceinline__ int alive_of(const OA &a, int64_t s0, int64_t s1, int
 // the front of v's arena range, where member j (from 1) goes to rp[v+1] - j
 // after its filter: with cnt candidates left, cnt + j <= deg(v), so it lies
 // past them.  Returns |C(v)|.
+template <int FLY>
 __device__ __forceinline__ int warp_steps(const OA &a, int64_t e1, int32_t *cand, int cnt, CKey bk, int j,
                                           int32_t *post, int32_t *near, unsigned long long &tests) {
   const int lane = threadIdx.x & 31;
@@ -266,7 +269,7 @@ __device__ __forceinline__ int warp_steps(const OA &a, int64_t e1, int32_t *cand
       __syncwarp();
       const Fence f = set_fence(a, a.rp[w], a.rp[w + 1], post, kNear, lane, 32);
       __syncwarp();
-      out = filter(a, f, w, cand, 0, cnt, cand, nb);
+      out = filter<FLY>(a, f, w, cand, 0, cnt, cand, nb);
     }
     cnt = out;
     j++;
@@ -348,6 +351,7 @@ __device__ __forceinline__ int block_place(int c, int *scnt, int *tot) {
 // of the candidates per warp, filtered to a scratch row and packed back in
 // order; the fence posts are the block's.  What is left goes to the first warp
 // once it fits its shared memory.
+template <int FLY>
 __device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt, CKey *sk,
                           unsigned long long &tests) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -356,7 +360,7 @@ __device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt
   int32_t *A = a.arena + e0;
   int64_t s0 = len * wid / kGW, s1 = len * (wid + 1) / kGW;
   CKey nb = none;
-  int c = alive_of(a, e0 + s0, e0 + s1, B + s0, nb);
+  int c = alive_of<FLY>(a, e0 + s0, e0 + s1, B + s0, nb);
   int cnt, j = 0;
   for (;;) {
     __syncwarp();
@@ -365,7 +369,7 @@ __device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt
     const CKey bk = block_first(nb, sk);
     if (cnt <= kNear) {
       int size = 0;
-      if (wid == 0) size = warp_steps(a, e1, A, cnt, bk, j, S.post[0], S.cand[0], tests);
+      if (wid == 0) size = warp_steps<FLY>(a, e1, A, cnt, bk, j, S.post[0], S.cand[0], tests);
       __syncthreads();
       return size;  // of the first warp
     }
@@ -376,7 +380,7 @@ __device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt
     s0 = (int64_t)cnt * wid / kGW;
     s1 = (int64_t)cnt * (wid + 1) / kGW;
     nb = none;
-    c = filter(a, f, w, A, (int)s0, (int)s1, B + s0, nb);
+    c = filter<FLY>(a, f, w, A, (int)s0, (int)s1, B + s0, nb);
     j++;
     __syncthreads();  // A has been read
     // cnt + j <= deg(v): the member's slot lies past the packed candidates
@@ -397,7 +401,15 @@ __device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt
 // them do: whole order of scale 16 / 17 / 20 / 22 in 3.8 / 5.6 / 51 / 191 ms,
 // always blocks 3.8 / 5.8 / 55 / 342, never blocks 4.8 / 7.7 / 50 / 185
 // (before: 7.6 / 11.9 / 71 / 316).
-__global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, int64_t scratch_stride, int big_blocks) {
+// FLY: candidates that a lane has in flight.  Four side by side, with 32 warps
+// per SM, are right for the latency of long growths; where no vertex has more than
+// kMidGrowMin neighbours and many are left, warps are what is short: one at a time
+// with 48 warps per SM.  Whole order of 50,000 cliques of 20 in 5.0 ms (7.3 with four;
+// 5.3 with 64 warps that searched the rows in L2), 50,000 of 50 in 39.9 (56.1;
+// 43.9), G(10^6, 16) 2.47 (3.07; 2.74); 64 warps per SM spill (5.1, 39.8, 2.56).
+// R-MAT scale 20, which has longer rows, would take 49 ms instead of 41.
+template <int FLY, int BLOCKS>
+__global__ void __launch_bounds__(kGT, BLOCKS) grow_kernel(OA a, int32_t *scratch, int64_t scratch_stride, int big_blocks) {
   __shared__ GrowSmem S;
   __shared__ CKey sk[kGW];
   __shared__ int scnt[kGW];
@@ -417,7 +429,7 @@ __global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, in
       __syncthreads();
       if (b >= total) break;
       const int v = b < nbig ? a.big[b] : a.big[a.n - 1 - (b - nbig)];
-      const int size = block_grow(a, v, scratch + blockIdx.x * scratch_stride, S, scnt, sk, tests);
+      const int size = block_grow<FLY>(a, v, scratch + blockIdx.x * scratch_stride, S, scnt, sk, tests);
       if (threadIdx.x == 0) {
         a.csize[v] = size;
         grows++;
@@ -438,9 +450,9 @@ __global__ void __launch_bounds__(kGT, 4) grow_kernel(OA a, int32_t *scratch, in
       int32_t *cand = e1 - e0 <= kNear ? S.cand[wid] : a.arena + e0;
       CKey bk = none;
       __syncwarp();
-      const int cnt = alive_of(a, e0, e1, cand, bk);
+      const int cnt = alive_of<FLY>(a, e0, e1, cand, bk);
       __syncwarp();
-      const int size = warp_steps(a, e1, cand, cnt, warp_first(bk), 0, S.post[wid], S.cand[wid], tests);
+      const int size = warp_steps<FLY>(a, e1, cand, cnt, warp_first(bk), 0, S.post[wid], S.cand[wid], tests);
       if (lane == 0) {
         a.csize[v] = size;
         grows++;
@@ -1039,7 +1051,7 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
   MC_TRY(ws_get(g, "co.stale", (size_t)n * 4, &p));
   a.stale = (int32_t *)p;
   int32_t *scratch = nullptr;
-  const int big_blocks = 2 * g->sm_count, grow_blocks = 4 * g->sm_count;
+  const int big_blocks = 2 * g->sm_count;
   const int64_t stride = std::max<int64_t>(g->max_degree, 1);
   const bool any_big = g->max_degree > kMidGrowMin;
   if (any_big) {
@@ -1056,7 +1068,10 @@ int clique_order(mc_graph *g, const int32_t *rank, int32_t *d_order, int64_t *d_
     for (int i = 0; i < rounds; i++) {
       a.round = r++;
       check_kernel<<<gt, 256, 0, g->stream>>>(a);
-      grow_kernel<<<grow_blocks, kGT, 0, g->stream>>>(a, scratch, stride, any_big ? big_blocks : 0);
+      if (!any_big && n - placed > kManyVertices)
+        grow_kernel<1, 6><<<6 * g->sm_count, kGT, 0, g->stream>>>(a, scratch, stride, any_big ? big_blocks : 0);
+      else
+        grow_kernel<4, 4><<<4 * g->sm_count, kGT, 0, g->stream>>>(a, scratch, stride, any_big ? big_blocks : 0);
       scatter_kernel<<<gt, 256, 0, g->stream>>>(a);
       accept_kernel<<<gt, 256, 0, g->stream>>>(a);
       MC_CUDA_TRY(cudaGetLastError());

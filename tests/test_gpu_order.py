@@ -261,6 +261,37 @@ def test_relabel_by_row_length(mc, n):
     h.close()
 
 
+def _uniform(n, degree, seed):
+    r = np.random.default_rng(seed)
+    s, t = r.integers(0, n, (2, n * degree // 2))
+    return gg.from_edges(n, s[s != t], t[s != t], "uniform%d_%d" % (n, degree))
+
+
+@pytest.mark.parametrize("g", [_uniform(60000, 7, 1), _uniform(50001, 2, 2),
+                               gg.disjoint_cliques([31, 33, 1, 2] * 800)], ids=lambda g: g.name[:20])
+def test_clique_order_of_many_vertices_bit_exact(mc, g):
+    """More than 50,000 vertices left and none of more than 512 neighbours: the
+    growths with one candidate per lane in flight, and the change over to the
+    others as fewer are left."""
+    want = OO.clique_order(g, oracle.core_numbers(g))
+    h = load(mc, g)
+    order, starts, rounds, _ = mc.mc_clique_order(h)
+    assert np.array_equal(order, want[0]) and np.array_equal(starts, want[1]) and np.array_equal(rounds, want[2])
+    h.close()
+
+
+@pytest.mark.parametrize("size,count", [(40, 1300), (257, 200), (300, 170), (513, 98)])
+def test_clique_order_of_many_equal_cliques(mc, size, count):
+    """The same kernel with candidate lists on both sides of the 256 a warp holds
+    in shared memory, up to the 512 neighbours it is used for."""
+    g = gg.disjoint_cliques([size] * count)
+    h = load(mc, g)
+    order, starts, rounds, _ = mc.mc_clique_order(h)
+    assert np.array_equal(order, np.arange(g.n)) and np.array_equal(starts, np.arange(0, g.n + 1, size))
+    assert not rounds.any()
+    h.close()
+
+
 def test_clique_order_of_few_rounds_queues_few(mc):
     """Rounds are queued two at first, then two, then four: an order of one
     round launches less than one of three, one of three less than one of five,
