@@ -85,24 +85,24 @@ constexpr int kRowFly = 4;
 // Number of u in ci[e0, e1) with core[u] >= kv, counted by LANES lanes (gl =
 // the lane's place among them, shift = their first lane, gm = their mask); the
 // first kQ of them go to qs.
-template <int LANES>
+template <int LANES, int FLY>
 __device__ int count_row(const int32_t *__restrict__ ci, const int32_t *__restrict__ core, int kv, int64_t e0,
                          int64_t e1, unsigned gm, int shift, int gl, int *qs) {
   constexpr unsigned all = LANES == 32 ? 0xffffffffu : (1u << (LANES & 31)) - 1u;
   const unsigned below = (1u << gl) - 1u;
   int c = 0;
-  for (int64_t eb = e0; eb < e1; eb += LANES * kRowFly) {
-    int u[kRowFly];
-    bool ok[kRowFly];
+  for (int64_t eb = e0; eb < e1; eb += LANES * FLY) {
+    int u[FLY];
+    bool ok[FLY];
 #pragma unroll
-    for (int i = 0; i < kRowFly; i++) {
+    for (int i = 0; i < FLY; i++) {
       const int64_t e = eb + i * LANES + gl;
       u[i] = e < e1 ? ci[e] : -1;
     }
 #pragma unroll
-    for (int i = 0; i < kRowFly; i++) ok[i] = u[i] >= 0 && core[u[i]] >= kv;
+    for (int i = 0; i < FLY; i++) ok[i] = u[i] >= 0 && core[u[i]] >= kv;
 #pragma unroll
-    for (int i = 0; i < kRowFly; i++) {
+    for (int i = 0; i < FLY; i++) {
       const unsigned m = (__ballot_sync(gm, ok[i]) >> shift) & all;
       const int pos = c + __popc(m & below);
       if (ok[i] && pos < kQ) qs[pos] = u[i];
@@ -110,6 +110,19 @@ __device__ int count_row(const int32_t *__restrict__ ci, const int32_t *__restri
     }
   }
   return c;
+}
+
+// The features from the row's length and count c, the edges t of G[Q] and its
+// colours chi.
+__device__ __forceinline__ void write_features(float kmax, float ldmax, int64_t deg, int kv, int c, int t, int chi,
+                                               float f[kF]) {
+  const float d = (float)deg;
+  f[0] = log1pf(d) / ldmax;
+  f[1] = (float)kv / kmax;
+  f[2] = (float)t / (float)(kQ * (kQ - 1) / 2);
+  f[3] = (float)(chi + 1) / (float)(kQ + 1);
+  f[4] = (float)c / fmaxf(d, 1.f);
+  f[5] = log1pf((float)c) / ldmax;
 }
 
 // The six features of vertex v (row [e0, e1), core number kv) from its count c
@@ -177,14 +190,65 @@ __device__ void vertex_features(const int64_t *__restrict__ rp, const int32_t *_
     const int k = __ffs(~clash) - 1;
     if (gl == k) cls |= 1u << i;
   }
-  const int chi = __popc(group_ballot(gm, cls != 0u, grp));
-  const float d = (float)deg;
-  f[0] = log1pf(d) / ldmax;
-  f[1] = (float)kv / kmax;
-  f[2] = (float)t / (float)(kQ * (kQ - 1) / 2);
-  f[3] = (float)(chi + 1) / (float)(kQ + 1);
-  f[4] = (float)c / fmaxf(d, 1.f);
-  f[5] = log1pf((float)c) / ldmax;
+  write_features(kmax, ldmax, deg, kv, c, t, __popc(group_ballot(gm, cls != 0u, grp)), f);
+}
+
+// The same for Q of at most kFewQ members: a pair per lane, and every lane colours
+// from the six bits.  For four vertices per warp that all have so few, which is
+// most of a sparse graph, the form above lost to the one-search-per-pair form
+// before it: 1,000 x 1,000 grid 0.22 ms then, 0.30 with it alone, 0.17 now; 200,000
+// cliques of five 0.21, 0.30, 0.16; 10^6 vertices of degree one 0.13, 0.21, 0.13.
+constexpr int kFewQ = 4;
+__device__ __forceinline__ void few_features(const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
+                                             float kmax, float ldmax, int64_t deg, int kv, int c, const int *qs,
+                                             float f[kF]) {
+  const int lane = threadIdx.x & 31, grp = lane >> 3, gl = lane & 7;
+  const unsigned gm = 0xFFu << (grp * 8);
+  const int q = c;
+  // pairs (0, 1), (0, 2), (0, 3), (1, 2), (1, 3), (2, 3)
+  const int i = gl < 3 ? 0 : (gl < 5 ? 1 : 2), j = gl < 3 ? gl + 1 : (gl < 5 ? gl - 1 : 3);
+  bool adj = false;
+  if (gl < 6 && j < q) {
+    int x = qs[i], y = qs[j];
+    int64_t lo = rp[x], r0 = rp[y];
+    int left = (int)(rp[x + 1] - lo);
+    const int other = (int)(rp[y + 1] - r0);
+    if (other < left) {  // the shorter of the two rows
+      left = other;
+      lo = r0;
+      y = x;
+    }
+    while (left) {
+      const int h = left >> 1, z = ci[lo + h];
+      if (z == y) {
+        adj = true;
+        left = 0;
+      } else if (z < y) {
+        lo += h + 1;
+        left -= h + 1;
+      } else {
+        left = h;
+      }
+    }
+  }
+  __syncwarp(gm);
+  const unsigned p = group_ballot(gm, adj, grp);
+  // greedy colouring in index order; rows[v]: the earlier neighbours of member v
+  const unsigned rows[4] = {0u, p & 1u, ((p >> 1) & 1u) | ((p >> 2) & 2u), ((p >> 2) & 1u) | ((p >> 3) & 6u)};
+  unsigned cls[4] = {0u, 0u, 0u, 0u};
+  int chi = 0;
+#pragma unroll
+  for (int v = 0; v < 4; v++) {
+    bool placed = v >= q;
+#pragma unroll
+    for (int k = 0; k <= v; k++)
+      if (!placed && !(cls[k] & rows[v])) {
+        cls[k] |= 1u << v;
+        chi = max(chi, k + 1);
+        placed = true;
+      }
+  }
+  write_features(kmax, ldmax, deg, kv, c, __popc(p), chi, f);
 }
 
 struct FA {
@@ -308,14 +372,16 @@ __global__ void __launch_bounds__(256) features_kernel(FA a) {
       wide &= wide - 1;
       const int64_t f0 = __shfl_sync(0xffffffffu, e0, src), f1 = __shfl_sync(0xffffffffu, e1, src);
       const int fk = __shfl_sync(0xffffffffu, kv, src);
-      const int fc = count_row<32>(a.ci, a.core, fk, f0, f1, 0xffffffffu, 0, lane, Q[src >> 3]);
+      const int fc = count_row<32, kRowFly>(a.ci, a.core, fk, f0, f1, 0xffffffffu, 0, lane, Q[src >> 3]);
       if (grp == (src >> 3)) c = fc;
     }
-    if (len <= kGroupRow) c = count_row<8>(a.ci, a.core, kv, e0, e1, gm, grp * 8, gl, Q[grp]);
-    __syncwarp();
+    if (__all_sync(0xffffffffu, len <= 8)) c = count_row<8, 1>(a.ci, a.core, kv, e0, e1, gm, grp * 8, gl, Q[grp]);
+    else if (len <= kGroupRow) c = count_row<8, kRowFly>(a.ci, a.core, kv, e0, e1, gm, grp * 8, gl, Q[grp]);
+    const bool few = __all_sync(0xffffffffu, hub || c <= kFewQ);
     if (r < total && !hub) {
       float x[kF];
-      vertex_features(a.rp, a.ci, a.kmax, a.ldmax, len, kv, c, Q[grp], x);
+      if (few) few_features(a.rp, a.ci, a.kmax, a.ldmax, len, kv, c, Q[grp], x);
+      else vertex_features(a.rp, a.ci, a.kmax, a.ldmax, len, kv, c, Q[grp], x);
       if (SCORE) {
         const float s = mlp_logit_group(S[0], x);
         if (gl == 0) a.out[v] = s;
@@ -341,7 +407,7 @@ __global__ void __launch_bounds__(kUT) hub_kernel(FA a) {
     const int64_t v = a.hubs[h], e0 = a.rp[v], e1 = a.rp[v + 1], len = e1 - e0;
     const int kv = a.core[v];
     const int64_t s0 = e0 + len * wid / (kUT / 32), s1 = e0 + len * (wid + 1) / (kUT / 32);
-    const int c = count_row<32>(a.ci, a.core, kv, s0, s1, 0xffffffffu, 0, lane, qs[wid]);
+    const int c = count_row<32, kRowFly>(a.ci, a.core, kv, s0, s1, 0xffffffffu, 0, lane, qs[wid]);
     if (lane == 0) cs[wid] = c;
     __syncthreads();
     if (threadIdx.x < 8) {

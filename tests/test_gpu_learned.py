@@ -297,3 +297,28 @@ def test_forward_by_row_count(mc, rows):
     m = mc.MLP(seed=9)
     ref = OL.forward(m.get_params(), x)
     assert np.allclose(m.forward(x), ref, rtol=1e-4, atol=1e-4 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("extra", [0, 1, 6])
+def test_features_of_few_neighbours(mc, extra):
+    """All 1,024 labelled graphs on five vertices side by side: every pattern of
+    edges among up to four neighbours, in warps of few such neighbours only (a
+    pair per lane) and, with a K6 between each two of them (extra 6) or isolated
+    vertices (1), in mixed warps."""
+    pairs = [(a, b) for a in range(5) for b in range(a)]
+    src, dst, n = [], [], 0
+    for bits in range(1024):
+        for i, (a, b) in enumerate(pairs):
+            if bits >> i & 1:
+                src.append(n + a)
+                dst.append(n + b)
+        n += 5
+        if extra > 1:
+            for a in range(extra):
+                for b in range(a):
+                    src.append(n + a)
+                    dst.append(n + b)
+        n += extra
+    g = gg.from_edges(n, np.array(src), np.array(dst))
+    f = mc.mc_features(mc.mc_load_csr(g.row_ptr, g.col_idx))
+    assert np.allclose(f, OL.features(g, oracle.core_numbers(g)), rtol=2e-6, atol=2e-6)
