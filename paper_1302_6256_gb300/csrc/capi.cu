@@ -253,7 +253,7 @@ static int load_common(int32_t count, const int64_t *voff_in, int64_t n, const i
   }
   if (flags & MC_VALIDATE) {
     int32_t *bad = g->err + 8;
-    cudaMemsetAsync(bad, 0, 4, g->stream);
+    cudaMemsetAsync(bad, 0, kValidCount * 4 + 8, g->stream);
     if ((rc = launch_validate(g, bad)) != MC_OK) return fail(rc);
     if (cudaMemcpyAsync(g->h_small, bad, 4, cudaMemcpyDeviceToHost, g->stream) != cudaSuccess ||
         cudaStreamSynchronize(g->stream) != cudaSuccess)

@@ -199,6 +199,7 @@ int launch_verify_set(mc_graph *g, const int32_t *d_vs, int32_t k, int32_t *d_ok
 // Replace the peel order by the caller's (host or device) after checking that
 // it is a degeneracy order of the graph (MC_ERR_ARG otherwise).
 int use_order(mc_graph *g, const int32_t *order);
+constexpr int kValidCount = 4;  // words from the validation's flag to its (64-bit) counter
 int launch_validate(mc_graph *g, int32_t *d_bad);
 // Candidates of pruned root j (original ids, padding dropped), read to the host.
 int gather_root_row(mc_graph *g, const Pruned &pg, int32_t j, std::vector<int32_t> *out);

@@ -69,14 +69,15 @@ __global__ void verify_set_kernel(int64_t n, const int64_t *rp, const int32_t *c
 // hub's row was what the check took.  R-MAT scale 15: 364 us with a warp per
 // row, 65 us now (152 us with the whole block for a long row, which cost graphs of
 // short rows its barriers: 5.0 instead of 2.6 ms for 2,000 of them).
+// Rows of up to four times the mean length stay with a warp as well: where most
+// rows are long, one search per lane and 64 warps per SM do more than slices do
+// (2,000 cliques of 200: 1.25 ms with a warp per row, 2.4 by slices).
 constexpr int kValidShort = 128, kValidSlice = 512, kValidFly = 4;
-struct ValidUnits {
-  unsigned long long n;
-  unsigned long long unit[1];  // row << 32 | slice, at most `cap` of them
-};
+// units: row << 32 | slice, *count of them, at most cap.
 __global__ void __launch_bounds__(256, 8) validate_kernel(int64_t n, int64_t nnz, const int64_t *rp,
                                                           const int32_t *ci, const int32_t *gid,
-                                                          const int64_t *voff, ValidUnits *units,
+                                                          const int64_t *voff, int64_t longest,
+                                                          unsigned long long *units, unsigned long long *count,
                                                           unsigned long long cap, int32_t *bad) {
   const int lane = threadIdx.x & 31;
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -88,17 +89,17 @@ __global__ void __launch_bounds__(256, 8) validate_kernel(int64_t n, int64_t nnz
       if (lane == 0) atomicExch(bad, 1);
       continue;
     }
-    if (e1 - e0 > kValidShort) {
+    if (e1 - e0 > longest) {
       const int64_t k = (e1 - e0 + kValidSlice - 1) / kValidSlice;
       unsigned long long at = 0;
-      if (lane == 0) at = atomicAdd(&units->n, (unsigned long long)k);
+      if (lane == 0) at = atomicAdd(count, (unsigned long long)k);
       at = __shfl_sync(0xffffffffu, at, 0);
       // rows that do not overlap never need more than cap units
       if (at + k > cap) {
         if (lane == 0) atomicExch(bad, 1);
         continue;
       }
-      for (int64_t i = lane; i < k; i += 32) units->unit[at + i] = ((unsigned long long)v << 32) | (unsigned long long)i;
+      for (int64_t i = lane; i < k; i += 32) units[at + i] = ((unsigned long long)v << 32) | (unsigned long long)i;
       continue;
     }
     const int64_t lo = gid ? voff[gid[v]] : 0, hi = gid ? voff[gid[v] + 1] : n;
@@ -124,18 +125,19 @@ __global__ void __launch_bounds__(256) validate_long_kernel(int64_t n, int64_t n
                                                             const int32_t *__restrict__ ci,
                                                             const int32_t *__restrict__ gid,
                                                             const int64_t *__restrict__ voff,
-                                                            const ValidUnits *__restrict__ units,
+                                                            const unsigned long long *__restrict__ units,
+                                                            const unsigned long long *__restrict__ count,
                                                             unsigned long long cap, int32_t *bad) {
   const int lane = threadIdx.x & 31;
   const unsigned long long gw = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5;
   const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  if (units->n > cap) return;  // (reported already; some units were not written)
-  const unsigned long long total = units->n;
+  const unsigned long long total = *count;
+  if (total > cap) return;  // (reported already; some units were not written)
   bool ok = true;
   for (unsigned long long t = gw; t < total; t += nw) {
-    const int v = (int)(units->unit[t] >> 32);
+    const int v = (int)(units[t] >> 32);
     const int64_t e0 = rp[v], end = rp[v + 1];  // checked when it was listed
-    const int64_t s0 = e0 + (int64_t)(units->unit[t] & 0xffffffffull) * kValidSlice;
+    const int64_t s0 = e0 + (int64_t)(units[t] & 0xffffffffull) * kValidSlice;
     const int64_t s1 = min(end, s0 + kValidSlice);
     const int64_t lo = gid ? voff[gid[v]] : 0, hi = gid ? voff[gid[v] + 1] : n;
     for (int64_t eb = s0 + lane; eb < s1; eb += 32 * kValidFly) {
@@ -269,25 +271,26 @@ int launch_verify_set(mc_graph *g, const int32_t *d_vs, int32_t k, int32_t *d_ok
   return MC_OK;
 }
 
+// *d_bad and the count of the units, kValidCount words on, are zero.
 int launch_validate(mc_graph *g, int32_t *d_bad) {
   if (g->n == 0) return MC_OK;
   const int blocks = (int)std::min<int64_t>((g->n * 32 + 255) / 256, (int64_t)g->sm_count * 16);
   // a row of L > kValidShort entries has at most L / kValidShort units
   const unsigned long long cap = (unsigned long long)(g->nnz / kValidShort);
-  void *p;
-  MC_TRY(ws_get(g, "va.units", (size_t)(cap + 1) * 8, &p));
-  ValidUnits *units = (ValidUnits *)p;
-  MC_CUDA_TRY(cudaMemsetAsync(units, 0, 8, g->stream));
-  validate_kernel<<<blocks, 256, 0, g->stream>>>(g->n, g->nnz, g->row_ptr, g->col_idx, g->gid, g->voff, units, cap,
-                                                 d_bad);
+  const int64_t longest = std::max<int64_t>(kValidShort, 4 * (g->nnz / g->n));
+  // the core numbers' array is free until they are computed
+  void *p = g->core;
+  if (8 * cap > 4 * (unsigned long long)g->n) MC_TRY(ws_get(g, "va.units", (size_t)cap * 8, &p));
+  unsigned long long *units = (unsigned long long *)p, *count = (unsigned long long *)(d_bad + kValidCount);
+  validate_kernel<<<blocks, 256, 0, g->stream>>>(g->n, g->nnz, g->row_ptr, g->col_idx, g->gid, g->voff, longest, units,
+                                                 count, cap, d_bad);
   g_launches++;
-  if (cap == 0) {
-    MC_CUDA_TRY(cudaGetLastError());
-    return MC_OK;
+  if (g->nnz > longest) {
+    validate_long_kernel<<<(int)std::min<int64_t>((int64_t)(cap + 7) / 8, (int64_t)g->sm_count * 5), 256, 0,
+                           g->stream>>>(g->n, g->nnz, g->row_ptr, g->col_idx, g->gid, g->voff, units, count, cap,
+                                        d_bad);
+    g_launches++;
   }
-  validate_long_kernel<<<(int)std::min<int64_t>((int64_t)(cap + 7) / 8, (int64_t)g->sm_count * 8), 256, 0, g->stream>>>(
-      g->n, g->nnz, g->row_ptr, g->col_idx, g->gid, g->voff, units, cap, d_bad);
-  g_launches++;
   MC_CUDA_TRY(cudaGetLastError());
   return MC_OK;
 }

@@ -745,3 +745,41 @@ def test_core_numbers_go_to_the_cheaper_kernel(mc, g, local):
         assert om == first[0] and oracle.is_clique(g, wit) and st["max_core"] == kmax
         assert np.array_equal(mc.mc_core_numbers(h)[0], ref)
     h.close()
+
+
+def _refused(mc, g, e, x):
+    c = g.col_idx.copy()
+    c[e] = x
+    with pytest.raises(mc.MCError) as err:
+        mc.mc_load_csr(torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(c).cuda(), mc.MC_VALIDATE)
+    assert err.value.code == mc.MC_ERR_INVALID_GRAPH
+
+
+@pytest.mark.parametrize("g", [
+    _hubs(9000, [100, 127, 128, 129, 256, 500, 512, 513, 1000, 1024, 1025, 1537], 8), gg.disjoint_cliques([130] * 40),
+    gg.disjoint_cliques([513] * 4), gg.disjoint_cliques([2600]), gg.complete_bipartite(129, 70),
+    gg.complete_bipartite(520, 3)], ids=lambda g: "%s n=%d" % (g.name[:24], g.n))
+def test_validate_at_the_edges_of_slices(mc, g):
+    """Rows of a warp (at most 128 entries, or four times the mean length) and of
+    slices of 512: accepted as they are; refused with one entry repeated, equal
+    to its row or without its reverse, at the row's ends and on both sides of
+    every slice."""
+    rp = torch.from_numpy(g.row_ptr).cuda()
+    mc.mc_load_csr(rp, torch.from_numpy(g.col_idx).cuda(), mc.MC_VALIDATE).close()
+    d = g.degrees()
+    rows = sorted({int(np.nonzero(d == x)[0][k]) for x in np.unique(d)[-6:] for k in (0, -1)} | {g.n - 1})
+    for v in rows:
+        e0, e1 = int(g.row_ptr[v]), int(g.row_ptr[v + 1])
+        row = set(g.col_idx[e0:e1].tolist())
+        for e in sorted({e0, e1 - 1} | {e0 + x + k for x in range(512, e1 - e0, 512) for k in (-1, 0, 1)}):
+            if not e0 <= e < e1:
+                continue
+            _refused(mc, g, e, g.col_idx[e - 1] if e > e0 else g.col_idx[min(e + 1, e1 - 1)] + (e1 - e0 == 1))
+            _refused(mc, g, e, v)
+            # a value that keeps the row sorted but is no neighbour's reverse
+            lo = g.col_idx[e - 1] + 1 if e > e0 else 0
+            hi = g.col_idx[e + 1] if e + 1 < e1 else g.n
+            for x in range(int(lo), int(hi)):
+                if x not in row and x != v:
+                    _refused(mc, g, e, x)
+                    break
