@@ -783,3 +783,58 @@ def test_validate_at_the_edges_of_slices(mc, g):
                 if x not in row and x != v:
                     _refused(mc, g, e, x)
                     break
+
+
+def _root_tests(g, order, core, om, keep=None):
+    """roots_colored and roots_branched of a search whose omega stays as it is:
+    the roots whose (omega - 1)-core of G[P] has omega vertices left, and those of
+    them that omega - 1 greedy colours (latest vertex first) do not cover.  keep:
+    the edges that the matrices of G[P] hold (a planted mistake)."""
+    pos = np.empty(g.n, np.int64)
+    pos[order] = np.arange(g.n)
+    adj = np.zeros((g.n, g.n), bool)
+    adj[np.repeat(np.arange(g.n), g.degrees()), g.col_idx] = True
+    mat = adj if keep is None else adj & keep
+    colored = branched = 0
+    for u in order:
+        P = np.nonzero(adj[u] & (pos > pos[u]) & (core >= om))[0]
+        if core[u] < om or len(P) < om:
+            continue
+        P = P[np.argsort(-pos[P])]
+        S, live = mat[np.ix_(P, P)], np.ones(len(P), bool)
+        while True:
+            low = live & (S[:, live].sum(1) < om - 1)
+            if not low.any():
+                break
+            live &= ~low
+        if live.sum() < om:
+            continue
+        colored += 1
+        for _ in range(om - 1):
+            free = live.copy()
+            while free.any():
+                i = np.argmax(free)
+                live[i] = free[i] = False
+                free &= ~S[i]
+        branched += bool(live.any())
+    return colored, branched
+
+
+@pytest.mark.parametrize("n,p,k", [(700, 0.4, 30), (1100, 0.55, 70), (1760, 0.58, 120)])
+def test_block_matrices_root_for_root(mc, n, p, k):
+    """Bit rows, bitmap and hash lookups build the same matrices as numpy: with
+    omega known from the heuristic (a planted clique) and the vertex order given,
+    the number of roots that pass each of the two tests on them is fixed.  K(G) of
+    about 250, 560 and 970 covers the layouts of 512, 864 and 1,024 candidates.  A
+    loss of 1% of the edges, planted in numpy's matrices, changes the numbers."""
+    g = gg.relabel(gg.erdos_renyi(n, p, planted=k, seed=n), 7)
+    core, order = oracle.core_numbers(g, with_order=True)
+    want = _root_tests(g, order, core, k)
+    lost = np.triu(np.random.default_rng(1).random((n, n)) < 0.01, 1)
+    assert _root_tests(g, order, core, k, ~(lost | lost.T)) != want
+    h = load(mc, g, flags=0)
+    for opts in (dict(), dict(no_bitmap=True), dict(layout=1), dict(no_split=True), dict(layout=1, no_bitmap=True)):
+        om, wit, st = mc.mc_max_clique(h, warp_max=1, order=order.astype(np.int32), **opts)
+        assert om == k == st["heuristic_size"] and oracle.is_clique(g, wit)
+        assert (st["roots_colored"], st["roots_branched"]) == want, opts
+    h.close()
