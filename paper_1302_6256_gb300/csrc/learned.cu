@@ -584,12 +584,14 @@ __global__ void __launch_bounds__(kVT) forward_kernel(int64_t n, const float *__
 // the first layer are register tiles of 4 x 4 outputs per thread over operands
 // in shared memory, each operand in the layout that the product reads as
 // float4; sums over rows stay in registers over all tiles of a block and reach
-// memory once per block.  FP32 throughout, as the bound on precision asks: the
-// activations are not BF16, so the tensor pipe's types would round them.
+// memory once per block.  FP32 throughout: the activations are not BF16, so the
+// tensor pipe's types would round them.  Every sum has a fixed order.
 // 16,384 rows: 190 us with a thread per row (128 rows per block, serial
 // 64-long chains per thread, 6% of the warps, sums by atomics), 36 us now with
 // 5 us for the sum over the blocks; its error against 64 bits is a third of
-// what it was (the blocks' sums are added in order, not by atomics).
+// what it was (the blocks' sums are added in order, not by atomics).  Two blocks
+// fit an SM (106 KB each), so 16,384 rows are one tile for each of 256 blocks: a
+// call takes 71 us, 80 with one block of 124 KB per SM and two tiles in turn.
 constexpr int kGR = 64;    // rows per tile
 constexpr int kGT = 256;   // threads: 16 x 16, 4 x 4 outputs each
 constexpr int kPart = (kParams + 1 + 31) / 32 * 32;  // floats of a block's sums: parameters, loss
@@ -599,7 +601,6 @@ struct GradSmem {
   float d2[kGR][kGS], d2t[kH][kGS];
   float w1t[kF][kH], x[kF][kGR];
   float b1[kH], b2[kH], w3[kH], y[kGR], b3;
-  float sum[kParams + 1];  // the block's gradient and loss
 };
 // what is read as float4 starts on 16 bytes, in every row (columns and rows are
 // taken at multiples of four)
@@ -642,7 +643,6 @@ __global__ void __launch_bounds__(kGT, 2) grad_kernel(int64_t n, const float *__
     S.w3[j] = bf16_to_f32(wbf[kOffW3 + j]);
   }
   if (t == 0) S.b3 = master[kOffB3];
-  for (int e = t; e <= kParams; e += kGT) S.sum[e] = 0.f;
   // a unit that is off passes nothing back, also where a weight is infinite
   const bool odd = __syncthreads_or(bad);
   const float inv_n = 1.f / (float)n;
@@ -743,36 +743,57 @@ __global__ void __launch_bounds__(kGT, 2) grad_kernel(int64_t n, const float *__
         for (int f = 0; f < kF; f++) gw1[j][f] = fmaf(d, S.x[f][r0 + i], gw1[j][f]);
       }
   }
-  // the two halves of a warp hold other rows of the same units
+  // The block's sums, to its place.  W2's gradient is whole in each thread; the
+  // others are spread over the 16 threads of a column: the two halves of a warp
+  // are added here, the eight warps pairwise, through the tiles' space.
+  float *out = part + (int64_t)blockIdx.x * kPart;
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+    *reinterpret_cast<float4 *>(out + kOffW2 + (r0 + i) * kH + c0) =
+        make_float4(gw2[i][0], gw2[i][1], gw2[i][2], gw2[i][3]);
+  __syncthreads();  // the tiles are free
+  constexpr int kWarps = kGT / 32, kUnit = kF + 3;  // warps; sums per unit
+  float *red = &S.w2[0][0], *ends = &S.h1[0][0];
+  static_assert(kWarps * kUnit * kH <= 2 * kH * kGS && kGT / 16 == 16, "room for the sums");
 #pragma unroll
   for (int j = 0; j < 4; j++) {
-    float v[kF + 3];
+    float v[kUnit];
 #pragma unroll
     for (int f = 0; f < kF; f++) v[f] = gw1[j][f];
     v[kF] = gb1[j];
     v[kF + 1] = gb2[j];
     v[kF + 2] = gw3[j];
 #pragma unroll
-    for (int f = 0; f < kF + 3; f++) {
+    for (int f = 0; f < kUnit; f++) {
       v[f] += __shfl_xor_sync(0xffffffffu, v[f], 16);
-      const int at = f < kF ? kOffW1 + (c0 + j) * kF + f
-                            : (f == kF ? kOffB1 : (f == kF + 1 ? kOffB2 : kOffW3)) + c0 + j;
-      if ((t & 16) == 0) atomicAdd(&S.sum[at], v[f]);
+      if ((t & 16) == 0) red[((t >> 5) * kUnit + f) * kH + c0 + j] = v[f];
     }
   }
   if (tx == 0) {
-    atomicAdd(&S.sum[kOffB3], gb3);
-    atomicAdd(&S.sum[kParams], lsum);
+    ends[ty] = gb3;
+    ends[kGT / 16 + ty] = lsum;
   }
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) S.sum[kOffW2 + (r0 + i) * kH + c0 + j] = gw2[i][j];
   __syncthreads();
-  for (int e = t; e <= kParams; e += kGT) part[(int64_t)blockIdx.x * kPart + e] = S.sum[e];
+  for (int e = t; e < kUnit * kH; e += kGT) {
+    float v[kWarps];
+#pragma unroll
+    for (int w = 0; w < kWarps; w++) v[w] = red[w * kUnit * kH + e];
+#pragma unroll
+    for (int o = kWarps / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int w = 0; w < o; w++) v[w] += v[w + o];
+    const int f = e / kH, c = e % kH;
+    out[f < kF ? kOffW1 + c * kF + f : (f == kF ? kOffB1 : (f == kF + 1 ? kOffB2 : kOffW3)) + c] = v[0];
+  }
+  if (t < 32) {  // b3 in the first half of the warp, the loss in the second
+    float v = ends[t];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((t & 15) == 0) out[t == 0 ? kOffB3 : kParams] = v;
+  }
 }
 
-// The blocks' sums, added in a fixed order (the gradient is the same bits on
+// The blocks' sums, added in a fixed order too (the gradient is the same bits on
 // every call): a warp's lanes are 32 parameters, its eight warps an eighth of
 // the blocks each.
 constexpr int kRT = 256;
@@ -1272,9 +1293,9 @@ static int run_grad(mc_mlp *m, const float *feat, const float *label, int64_t n,
     df = m->buf;
     dl = (char *)m->buf + fb;
   }
+  MC_CUDA_TRY(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
   const int64_t tiles = (n + kGR - 1) / kGR;
   const int blocks = (int)std::min<int64_t>(tiles, m->part_blocks);
-  MC_CUDA_TRY(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
   grad_kernel<<<blocks, kGT, sizeof(GradSmem), m->stream>>>(n, (const float *)df, (const float *)dl, pos_weight, m->wbf,
                                                             m->master, m->part);
   grad_sum_kernel<<<kPart / 32, kRT, 0, m->stream>>>(blocks, m->part, m->grad, m->loss);

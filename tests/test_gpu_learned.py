@@ -322,3 +322,20 @@ def test_features_of_few_neighbours(mc, extra):
     g = gg.from_edges(n, np.array(src), np.array(dst))
     f = mc.mc_features(mc.mc_load_csr(g.row_ptr, g.col_idx))
     assert np.allclose(f, OL.features(g, oracle.core_numbers(g)), rtol=2e-6, atol=2e-6)
+
+
+@pytest.mark.parametrize("rows", [1, 64, 1000, 16384, 60000])
+def test_gradient_is_the_same_bits_on_every_call(mc, rows):
+    """All sums of the gradient and the loss have a fixed order."""
+    r = np.random.default_rng(rows)
+    x = r.random((rows, OL.F)).astype(np.float32)
+    y = (r.random(rows) < 0.2).astype(np.float32)
+    m = mc.MLP(seed=5)
+    g0, loss0 = m.gradient(x, y, 5.0)
+    g0 = np.array(g0)
+    for _ in range(20):
+        g, loss = m.gradient(x, y, 5.0)
+        assert loss == loss0 and np.array_equal(np.asarray(g).view(np.uint32), g0.view(np.uint32))
+    other = mc.MLP(seed=5)
+    g, loss = other.gradient(x, y, 5.0)
+    assert loss == loss0 and np.array_equal(np.asarray(g), g0)
