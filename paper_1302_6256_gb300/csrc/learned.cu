@@ -1157,21 +1157,17 @@ int mc_mlp_create(uint64_t seed, void *cuda_stream, mc_mlp **out) {
   mc_mlp *m = new mc_mlp();
   m->stream = (cudaStream_t)cuda_stream;
   auto fail = [&](int rc) {
-    cudaFree(m->master); cudaFree(m->wbf); cudaFree(m->part); cudaFree(m->m); cudaFree(m->v);
+    cudaFree(m->master); cudaFree(m->wbf); cudaFree(m->m); cudaFree(m->v);
     if (m->h_small) cudaFreeHost(m->h_small);
     delete m;
     return rc;
   };
   if (cudaGetDevice(&m->device) != cudaSuccess) return fail(MC_ERR_CUDA);
   cudaDeviceGetAttribute(&m->sm_count, cudaDevAttrMultiProcessorCount, m->device);
-  m->part_blocks = 2 * std::max(m->sm_count, 1);  // the blocks of grad_kernel that run at once
-  if (cudaMalloc(&m->part, (size_t)(m->part_blocks + 2) * kPart * 4) != cudaSuccess ||
-      cudaMalloc(&m->master, kParams * 4) != cudaSuccess || cudaMalloc(&m->wbf, kParams * 2) != cudaSuccess ||
+  if (cudaMalloc(&m->master, kParams * 4) != cudaSuccess || cudaMalloc(&m->wbf, kParams * 2) != cudaSuccess ||
       cudaMalloc(&m->m, kParams * 4) != cudaSuccess || cudaMalloc(&m->v, kParams * 4) != cudaSuccess ||
       cudaMallocHost(&m->h_small, 4096) != cudaSuccess)
     return fail(MC_ERR_OOM);
-  m->grad = m->part + (size_t)m->part_blocks * kPart;
-  m->loss = m->grad + kPart;
   // He-uniform initial weights from a counter-based generator, zero biases
   std::vector<float> p(kParams, 0.f);
   uint64_t ctr = seed * 0x9E3779B97F4A7C15ULL + 1;
@@ -1294,6 +1290,15 @@ static int run_grad(mc_mlp *m, const float *feat, const float *label, int64_t n,
     dl = (char *)m->buf + fb;
   }
   MC_CUDA_TRY(cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
+  if (!m->part) {  // made by the first gradient: a network that only scores needs none
+    int per_sm = 0;
+    MC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grad_kernel, kGT, sizeof(GradSmem)));
+    const int most = std::max(per_sm, 1) * std::max(m->sm_count, 1);  // the blocks that run at once
+    MC_CUDA_TRY(cudaMalloc(&m->part, (size_t)(most + 2) * kPart * 4));
+    m->part_blocks = most;
+    m->grad = m->part + (size_t)most * kPart;
+    m->loss = m->grad + kPart;
+  }
   const int64_t tiles = (n + kGR - 1) / kGR;
   const int blocks = (int)std::min<int64_t>(tiles, m->part_blocks);
   grad_kernel<<<blocks, kGT, sizeof(GradSmem), m->stream>>>(n, (const float *)df, (const float *)dl, pos_weight, m->wbf,

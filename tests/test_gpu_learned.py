@@ -339,3 +339,24 @@ def test_gradient_is_the_same_bits_on_every_call(mc, rows):
     other = mc.MLP(seed=5)
     g, loss = other.gradient(x, y, 5.0)
     assert loss == loss0 and np.array_equal(np.asarray(g), g0)
+
+
+def test_a_network_that_only_scores_holds_no_gradient_sums(mc):
+    """The room for the gradient's partial sums (megabytes) is made by the first
+    gradient, not with the network."""
+    def used():
+        torch.cuda.synchronize()
+        free, total = torch.cuda.mem_get_info()
+        return total - free
+
+    x = np.random.default_rng(0).random((100, OL.F)).astype(np.float32)
+    keep = [mc.MLP(seed=i) for i in range(4)]
+    base = used()
+    nets = [mc.MLP(seed=i) for i in range(16)]
+    for m in nets:
+        m.forward(x)
+    scoring = used() - base
+    for m in nets:
+        m.gradient(x, np.zeros(100, np.float32), 1.0)
+    assert scoring <= 16 << 20 < used() - base
+    del keep, nets
