@@ -404,7 +404,7 @@ static int search_in_ranges(mc_graph *g, const mc_options &o, Pruned *pg, Search
   g->repeel_rebuilds = 0;
   g->repeel_roots = 0;
   const int R = o.repeel;
-  bool searched = false;
+  bool searched = false, same = false;  // same: the last search was of this pruned graph
   for (int c = 0; c < R; c++) {
     const int64_t hi = g->n - n0 * c / R, lo = g->n - n0 * (c + 1) / R;
     if (hi <= lo) continue;
@@ -416,12 +416,13 @@ static int search_in_ranges(mc_graph *g, const mc_options &o, Pruned *pg, Search
       bound = *h;
       MC_TRY(launch_prune(g, 0, nullptr, g->warp_max_used, pg, spin, pr, pc, lo, hi));
       g->repeel_rebuilds++;
+      same = false;
     } else {
       MC_TRY(relaunch_roots(g, g->warp_max_used, pg, pr, pc, lo, hi));
     }
-    MC_TRY(launch_search(g, *pg, o.no_neigh_cores, o.no_split, o.split_nodes, spin, sc, o.layout, o.no_bitmap));
+    MC_TRY(launch_search(g, *pg, o.no_neigh_cores, o.no_split, o.split_nodes, spin, sc, o.layout, o.no_bitmap, same));
     MC_TRY(search_huge_roots(g, o, pg));
-    searched = true;
+    searched = same = true;
     MC_TRY(read_search_counters(g, sc));
     MC_TRY(read_pruned_counts(g, pg));
     g->repeel_roots += pg->nroots_small + pg->nroots_block + pg->nroots_big;

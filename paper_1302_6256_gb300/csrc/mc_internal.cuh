@@ -136,8 +136,11 @@ int read_search_counters(mc_graph *g, SearchCounters *cnt);
 int record_event(mc_graph *g, int i);
 // layout 1: every block-class root in the 1,024-candidate layout; no_bitmap:
 // member lookups by hash table only.
+// same_graph: the last search of this handle had the same pruned graph (with other
+// root lists), so its dense rows are there.
 int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_split, int split_nodes,
-                  long long spin_limit, SearchCounters *counters, int layout = 0, int no_bitmap = 0);
+                  long long spin_limit, SearchCounters *counters, int layout = 0, int no_bitmap = 0,
+                  bool same_graph = false);
 
 }  // namespace mc
 

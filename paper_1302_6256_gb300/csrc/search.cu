@@ -2345,7 +2345,7 @@ __global__ void __launch_bounds__(kTW * 32, 4) branch_task_kernel(SA a) {
 }  // namespace
 
 int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_split, int split_nodes,
-                  long long spin_limit, SearchCounters *cnt, int layout, int no_bitmap) {
+                  long long spin_limit, SearchCounters *cnt, int layout, int no_bitmap, bool same_graph) {
   // Persistent kernels with fixed grids; the root counts are read on the
   // device (pg.d_counts), and sizes are bounded by K(G) >= |N+(u)|, so the
   // launches need no host synchronisation.
@@ -2467,7 +2467,7 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   // block class first (largest trees), then big, then warp class, then the
   // tasks the first and last of these published; events 8-12 time each
   MC_TRY(record_event(g, 8));
-  if (dense) {
+  if (dense && !same_graph) {
     const size_t smem = (size_t)kDW * a.dense_stride * 4;
     MC_CUDA_TRY(cudaFuncSetAttribute(dense_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dense_rows_kernel<<<(int)std::min<int64_t>((int64_t)g->sm_count * 4, (g->n + kDW - 1) / kDW), kDW * 32, smem,

@@ -838,3 +838,21 @@ def test_block_matrices_root_for_root(mc, n, p, k):
         assert om == k == st["heuristic_size"] and oracle.is_clique(g, wit)
         assert (st["roots_colored"], st["roots_branched"]) == want, opts
     h.close()
+
+
+def test_repeel_builds_the_bit_rows_once_per_pruned_graph(mc):
+    """The search over bit rows launches their builder besides what the search over
+    lookups launches (K(G) is below 513: no second layout): once while the pruned
+    graph stays the same, whatever the number of ranges."""
+    g = gg.rmat(13, 16, planted=60, seed=9)
+    h = load(mc, g)
+    want = mc.mc_max_clique(h)[0]
+    for repeel in (2, 5, 9):
+        launches = []
+        for no_bitmap in (False, True):
+            n0 = mc.mc_launch_count()
+            om, wit, st = mc.mc_max_clique(h, repeel=repeel, warp_max=16, no_bitmap=no_bitmap)
+            launches.append(mc.mc_launch_count() - n0)
+            assert om == want and oracle.is_clique(g, wit) and st["rebuilds"] == 0 and st["pruned_n"] > 9
+        assert launches[0] - launches[1] == 1
+    h.close()
