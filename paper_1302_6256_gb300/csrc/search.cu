@@ -2458,7 +2458,10 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   // builder's time counts with theirs
   const bool dense = g->count == 1 && !no_bitmap && kbound > wmax;
   if (dense) {
-    a.dense_cap = (int32_t)std::min<int64_t>(kDenseCap, (g->n + 31) & ~(int64_t)31);
+    // a block root has more than wmax later neighbours, so K > wmax from its rank on:
+    // at most one vertex per wmax + 1 entries
+    const int64_t useful = std::min(g->n, g->nnz / (wmax + 1) + 1);
+    a.dense_cap = (int32_t)std::min(kDenseCap, (useful + 31) & ~(int64_t)31);
     a.dense_stride = a.dense_cap / 32;
     MC_TRY(ws_get(g, "se.dense", (size_t)a.dense_cap * a.dense_stride * 4, &p));
     a.dense = (const uint32_t *)p;

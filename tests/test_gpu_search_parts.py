@@ -212,3 +212,25 @@ def test_handed_over_branches_leave_their_level(lib, big, level):
         left.discard(x)
         assert _members(t[n, 34:]) == left & set(np.nonzero(adj[x])[0].tolist())
         assert x in _members(t[n, 2:34])
+
+
+def test_bit_rows_take_room_for_ranks_that_can_use_them(mc, lib):
+    """A root of more than warp_max candidates has K > warp_max, and so have all
+    later ranks; those are at most one vertex per warp_max + 1 entries.  60,000
+    vertices of 8 neighbours and a dense part take rows for 4,036 ranks (2 MB), not
+    for 40,960 (210 MB); the search is the same as over lookups."""
+    r = np.random.default_rng(3)
+    s, t = r.integers(0, 60000, (2, 220000))
+    d = gg.erdos_renyi(400, 0.5, planted=30, seed=2)
+    ds = np.repeat(np.arange(400), d.degrees())
+    g = gg.from_edges(60000, np.r_[s[s != t], ds], np.r_[t[s != t], d.col_idx])
+    h = mc.mc_load_csr(torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col_idx).cuda(), mc.MC_VALIDATE)
+    for wm in (128, 16):
+        om, wit, st = mc.mc_max_clique(h, warp_max=wm, heuristic=2)
+        assert om == 30 == mc.mc_max_clique(h, warp_max=wm, no_bitmap=True)[0] and oracle.is_clique(g, wit)
+        if wm == 128:
+            assert st["max_core"] > 128
+            ranks = g.nnz // 129 + 1 + 31
+            assert lib.t_ws_bytes(h.handle, b"se.dense") <= 2 * (ranks * ranks // 8)
+    h.close()
+
