@@ -105,7 +105,11 @@ typedef struct {
   int32_t no_split;
   /* Branch nodes a warp expands on a task between two looks at the queue:
    * when other warps wait, it hands them the untried branches of its
-   * shallowest level; 0 = default (8) */
+   * shallowest level; 0 = default (8).  4 to 32 make sense.  Once these were the
+   * nodes after which a worker gave up its whole tree, with values of 1,024 to
+   * 16,384: such a value is still taken, and leaves waiting warps idle (R-MAT
+   * scale 17, edge factor 12: 6.3 ms by default, 9.0 with 64, 44 with 1,024, 87
+   * with 4,096) */
   int32_t split_nodes;
   /* The learned form (an extension; the paper has no learned part): a
    * scoring network from mc_mlp_create, or NULL.  With a network, the solve
