@@ -62,7 +62,7 @@ struct HA {
   int64_t cand_stride;
   int32_t *cl;              // per-warp clique buffers
   int64_t cl_stride;
-  int32_t *next;
+  unsigned long long *next;    // next visiting position of the launch, from begin on
   unsigned long long *detkey;  // per graph (mode 1)
   const int32_t *seeds;
   int64_t nseeds;
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(kWT, 2) heuristic_warm_kernel(HA a) {
   int32_t *cl = a.cl + (int64_t)blockIdx.x * a.cl_stride;
   for (;;) {
     __syncthreads();
-    if (threadIdx.x == 0) s_i = *(volatile int32_t *)a.err ? a.limit : a.begin + atomicAdd(a.next, 1);
+    if (threadIdx.x == 0) s_i = *(volatile int32_t *)a.err ? a.limit : a.begin + (int64_t)atomicAdd(a.next, 1ull);
     __syncthreads();
     const int64_t i = s_i;
     if (i >= a.limit) break;
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kHT, 5) heuristic_kernel(HA a) {
   bool end = false;
   while (!end) {
     int64_t i0 = 0;
-    if (lane == 0) i0 = *(volatile int32_t *)a.err ? total : a.begin + atomicAdd(a.next, take);
+    if (lane == 0) i0 = *(volatile int32_t *)a.err ? total : a.begin + (int64_t)atomicAdd(a.next, (unsigned long long)take);
     i0 = __shfl_sync(FULL, (long long)i0, 0);
     if (i0 >= total) break;
     const int64_t i = i0 + lane;
@@ -708,9 +708,10 @@ int launch_heuristic(mc_graph *g, int mode, long long spin_limit, const int32_t 
   MC_TRY(ws_get(g, "he.cl", (size_t)std::max({warps_s, warps_b, warm_blocks}) * lstride * 4, &p));
   int32_t *cl = (int32_t *)p;
   MC_TRY(ws_get(g, "he.ctl", 64 + (size_t)g->count * 8, &p));
-  int32_t *next = (int32_t *)p;  // [0] warm-up, [2] main launch, [1] deferred launch; [4..5] deferred count
-  unsigned long long *ndefer = (unsigned long long *)((char *)p + 16);
-  unsigned long long *hctr = (unsigned long long *)((char *)p + 24);  // three counters, bytes 24..47
+  // 64 bits: a batch visits as many positions as its count times its largest graph
+  unsigned long long *next = (unsigned long long *)p;  // [0] warm-up, [1] main launch, [2] deferred launch
+  unsigned long long *ndefer = next + 3;               // deferred count
+  unsigned long long *hctr = next + 4;                 // three counters
   unsigned long long *detkey = (unsigned long long *)((char *)p + 64);
   MC_CUDA_TRY(cudaMemsetAsync(p, 0, 64 + (size_t)g->count * 8, g->stream));
   int32_t *defer = nullptr;
@@ -791,7 +792,7 @@ int launch_heuristic(mc_graph *g, int mode, long long spin_limit, const int32_t 
   if (warm < main_end) {
     a.begin = warm;
     a.limit = main_end;
-    a.next = next + 2;
+    a.next = next + 1;
     heuristic_kernel<<<(int)((warps_s * 32 + kHT - 1) / kHT), kHT, 0, g->stream>>>(a);
     g_launches++;
     MC_CUDA_TRY(cudaGetLastError());
@@ -804,7 +805,7 @@ int launch_heuristic(mc_graph *g, int mode, long long spin_limit, const int32_t 
   if (two && warm < main_end) {
     a.list = defer;
     a.nlist = ndefer;
-    a.next = next + 1;
+    a.next = next + 2;
     heuristic_kernel<<<blocks_b, kHT, 0, g->stream>>>(a);
     g_launches++;
     MC_CUDA_TRY(cudaGetLastError());

@@ -856,3 +856,25 @@ def test_repeel_builds_the_bit_rows_once_per_pruned_graph(mc):
             assert om == want and oracle.is_clique(g, wit) and st["rebuilds"] == 0 and st["pruned_n"] > 9
         assert launches[0] - launches[1] == 1
     h.close()
+
+
+def test_batch_of_more_than_two_billion_visiting_positions(mc):
+    """The heuristic visits the j-th highest vertex of every graph before the next:
+    530,000 graphs, the largest of 4,096 vertices, have 2.17 x 10^9 positions, more
+    than 32 bits count.  A path of 4,096 vertices with a K5 and two isolated
+    edges stand among single vertices."""
+    n, src, dst = 0, [], []
+    sizes = np.ones(530000, np.int64)
+    sizes[[7, 264999, 529999]] = 4096, 2, 2
+    voff = np.r_[0, np.cumsum(sizes)]
+    p = int(voff[7])
+    src = np.r_[np.arange(p, p + 4095), [p + a for a in range(5) for b in range(a)], voff[264999], voff[529999]]
+    dst = np.r_[np.arange(p + 1, p + 4096), [p + b for a in range(5) for b in range(a)], voff[264999] + 1, voff[529999] + 1]
+    g = gg.from_edges(int(voff[-1]), src, dst)
+    want = np.ones(530000, np.int32)
+    want[[7, 264999, 529999]] = 5, 2, 2
+    h = mc.mc_load_batch(voff, torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col_idx).cuda(), mc.MC_VALIDATE)
+    for opts in (dict(), dict(heuristic=1)):
+        om, wit, st = mc.mc_max_clique_batch(h, **opts)
+        assert np.array_equal(om, want) and sorted(wit[7].tolist()) == [0, 1, 2, 3, 4]
+    h.close()
