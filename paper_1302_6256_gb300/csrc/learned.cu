@@ -794,25 +794,25 @@ __global__ void __launch_bounds__(kGT, 2) grad_kernel(int64_t n, const float *__
 }
 
 // The blocks' sums, added in a fixed order too (the gradient is the same bits on
-// every call): a warp's lanes are 32 parameters, its eight warps an eighth of
-// the blocks each.
+// every call) and in double, so that each parameter is rounded once here: a
+// warp's lanes are 32 parameters, its eight warps an eighth of the blocks each.
 constexpr int kRT = 256;
 __global__ void __launch_bounds__(kRT) grad_sum_kernel(int blocks, const float *__restrict__ part,
                                                        float *__restrict__ grad, float *__restrict__ loss) {
-  __shared__ float sm[kRT / 32][32];
+  __shared__ double sm[kRT / 32][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
-  float v = 0.f;
+  double v = 0.0;
   if (e <= kParams) {
 #pragma unroll 8
-    for (int b = wid; b < blocks; b += kRT / 32) v += part[(int64_t)b * kPart + e];
+    for (int b = wid; b < blocks; b += kRT / 32) v += (double)part[(int64_t)b * kPart + e];
   }
   sm[wid][lane] = v;
   __syncthreads();
   if (wid == 0 && e <= kParams) {
 #pragma unroll
     for (int i = 1; i < kRT / 32; i++) v += sm[i][lane];
-    if (e < kParams) grad[e] = v;
-    else *loss = v;
+    if (e < kParams) grad[e] = (float)v;
+    else *loss = (float)v;
   }
 }
 
