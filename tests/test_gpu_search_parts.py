@@ -1,5 +1,6 @@
-"""Single device functions of the search, called by themselves: a small library
-that includes search.cu is compiled here and linked against libmc.so."""
+"""Single device functions of the search and the heuristic, called by themselves: a
+small library that includes search.cu and heuristic.cu is compiled here and linked
+against libmc.so."""
 import ctypes
 import os
 import subprocess
@@ -234,3 +235,37 @@ def test_bit_rows_take_room_for_ranks_that_can_use_them(mc, lib):
             assert lib.t_ws_bytes(h.handle, b"se.dense") <= 2 * (ranks * ranks // 8)
     h.close()
 
+
+TOP = r"""
+#include "%s"
+using namespace mc;
+extern "C" int t_top(long long n, int ntop, const int *order, const int *core, const int64_t *rp, int *top) {
+  top_kernel<<<kTop / kTopKeys, kTopT>>>(n, ntop, order, core, rp, top);
+  return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+@pytest.mark.parametrize("n,ntop,degrees", [(4096, 4096, 5), (9000, 4096, 3000), (9000, 4095, 1 << 30), (50, 50, 4), (1, 1, 1)])
+def test_front_of_the_visiting_order(mc, tmp_path, n, ntop, degrees):
+    """The last ntop positions of the order by core number, then degree, then the
+    later position: as numpy sorts them, ties and the largest degrees included."""
+    from paper_1302_6256_gb300 import _build
+    src, out = str(tmp_path / "top.cu"), str(tmp_path / "libtop.so")
+    with open(src, "w") as f:
+        f.write(TOP % os.path.join(_build.CSRC, "heuristic.cu"))
+    subprocess.run([_build._nvcc(), *_build.ARCH, *_build.FLAGS, "-shared", src, "-o", out, _build.LIB, "-lcudart",
+                    "-Xlinker", "-rpath=" + _build.BUILD], check=True)
+    lib = ctypes.CDLL(out)
+    r = np.random.default_rng(n + ntop)
+    order, core = r.permutation(n).astype(np.int32), r.integers(0, 7, n).astype(np.int32)
+    core[r.integers(0, n, 5)] = 270000
+    deg = r.integers(0, degrees, n)
+    rp = np.r_[0, np.cumsum(deg)].astype(np.int64)
+    last = order[::-1][:ntop]
+    want = last[np.lexsort((np.arange(ntop), -deg[last], -core[last]))]
+    dev = [torch.from_numpy(x).cuda() for x in (order, core, rp)]
+    top = torch.zeros(ntop, dtype=torch.int32, device="cuda")
+    lib.t_top.argtypes = [ctypes.c_longlong, ctypes.c_int] + [ctypes.c_void_p] * 4
+    assert lib.t_top(n, ntop, *(_p(x) for x in dev), _p(top)) == 0
+    assert np.array_equal(top.cpu().numpy(), want)
