@@ -90,7 +90,7 @@ struct SA {
   int32_t *ntasks;               // positions taken (the queue's tail, monotonic)
   int32_t *task_next;            // tickets taken by the task kernel's warps (runs ahead of ntasks by the waiting ones)
   int32_t *pending;              // tasks published and not yet finished
-  int32_t *progress;             // heartbeat: bumped every 256 Branch nodes
+  int32_t *progress;             // heartbeat: bumped every 256 Branch nodes, and at every one above the compact form
   uint32_t *sort;                // per-block room for a sorted matrix (roots searched in place)
   int64_t sort_stride;
   int32_t *overflow;             // roots too large for this launch's layout (or null)
@@ -2239,7 +2239,7 @@ __device__ void run_task(const SA &a, TaskCtx &T, Bits<1> P, TaskSmem &S, uint32
         P = LP;
         band_row<1, false>(P, T.A, T.Ws, T.W, v);
         nodes++;
-        if (lane == 0 && (nodes & 15) == 0) atomicAdd(a.progress, 1);
+        if (lane == 0) atomicAdd(a.progress, 1);  // (a node of this size takes 10 us and more)
         Bits<1> C;
         C.w[0] = T.C;
         bset(C, v);

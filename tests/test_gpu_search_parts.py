@@ -90,6 +90,37 @@ extern "C" int t_offer(int big, const uint32_t *A, int m, int ws, uint32_t *stk,
   else offer_kernel<<<1, 32>>>(a, A, m, stk, d, pb, k);
   return (int)cudaDeviceSynchronize();
 }
+// One task of m candidates on the matrix A (ws words a row): run_task by one warp.
+__global__ void run_kernel(SA a, const uint32_t *A, int m, int ws, uint32_t *lev, uint32_t *stk,
+                           unsigned long long *out) {
+  __shared__ __align__(16) TaskSmem S;
+  TaskCtx T{};
+  T.cs = 1;
+  T.p = m;
+  T.W = (m + 31) / 32;
+  T.Ws = ws;
+  T.A = A;
+  T.lev = lev;
+  Bits<1> P;
+  P.w[0] = first_bits(m);
+  unsigned long long nodes = 0, don = 0;
+  run_task(a, T, P, S, stk, nodes, don);
+  if ((threadIdx.x & 31) == 0) out[0] = nodes;
+}
+// ctr: best, tasks, tickets, error, progress
+extern "C" int t_run(const uint32_t *A, int m, int ws, uint32_t *lev, uint32_t *stk, int *ctr,
+                     unsigned long long *out) {
+  SA a{};
+  a.best = ctr;
+  a.ntasks = ctr + 1;
+  a.task_next = ctr + 2;
+  a.err = ctr + 3;
+  a.progress = ctr + 4;
+  a.spin = 1000;
+  a.offer_nodes = 8;
+  run_kernel<<<1, 32>>>(a, A, m, ws, lev, stk, out);
+  return (int)cudaDeviceSynchronize();
+}
 extern "C" long long t_ws_bytes(mc_graph *g, const char *name) {
   auto it = g->ws.find(name);
   return it == g->ws.end() ? -1 : (long long)it->second.bytes;
@@ -234,6 +265,26 @@ def test_bit_rows_take_room_for_ranks_that_can_use_them(mc, lib):
             ranks = g.nnz // 129 + 1 + 31
             assert lib.t_ws_bytes(h.handle, b"se.dense") <= 2 * (ranks * ranks // 8)
     h.close()
+
+
+def test_every_large_node_is_a_sign_of_life(lib):
+    """A task of 60 disjoint five-cycles (300 candidates) with omega 3: two colours
+    leave one vertex of each cycle to branch on, and its two neighbours, which are
+    not adjacent, are dropped at once.  60 nodes above the compact form, and as many
+    heartbeats for the warps that wait."""
+    m, ws = 300, 11
+    A = np.zeros((m, ws), np.uint32)
+    for v in range(m):
+        c = v - v % 5
+        A[v] = _words([c + (v + 1) % 5, c + (v + 4) % 5], ws)
+    dev = [torch.from_numpy(A.reshape(-1).view(np.int32)).cuda()]
+    dev += [torch.zeros(k, dtype=torch.int32, device="cuda") for k in (66 * 304, 20 * 304)]
+    ctr = torch.tensor([3, 0, 0, 0, 0], dtype=torch.int32, device="cuda")
+    out = torch.zeros(1, dtype=torch.int64, device="cuda")
+    i, p = ctypes.c_int, ctypes.c_void_p
+    lib.t_run.argtypes = [p, i, i, p, p, p, p]
+    assert lib.t_run(_p(dev[0]), m, ws, _p(dev[1]), _p(dev[2]), _p(ctr), _p(out)) == 0
+    assert int(out) == 60 and ctr.tolist() == [3, 0, 0, 0, 60]
 
 
 TOP = r"""
