@@ -95,7 +95,7 @@ struct SA {
   int64_t sort_stride;
   int32_t *overflow;             // roots too large for this launch's layout (or null)
   int64_t *noverflow;
-  int32_t task_warps;            // warps of the task kernel
+  int32_t task_warps;            // warps of a task kernel that fills the chip
   int32_t offer_nodes;           // Branch nodes of a task between two looks for waiting warps
 };
 
@@ -1018,9 +1018,11 @@ __device__ __forceinline__ int edges_upto(const SA &a, const int *Pidx, int p, u
 }
 
 // Branch nodes that a warp expands on its root before what is left becomes a
-// task: few while the task kernel's warps have no task each, many once they
-// have, or while no clique is known (a first clique lies deeper than a few
-// nodes, and every root would become a task under omega 0).  With every
+// task: few while there are not as many tasks as the chip has warps for, many once
+// there are, or while no clique is known (a first clique lies deeper than a few
+// nodes, and every root would become a task under omega 0); none where the launch
+// has fewer roots than that (a node takes 35 us here on a dense graph: G(150, 0.8)
+// 8.9 ms, 9.5 with four).  With every
 // branching root published at once, 300 graphs of 150-400 vertices took 130 ms
 // (now 2.6), 5,000 of 30-80 vertices 160 (4.5), a 300 x 300 grid without a lower
 // bound 118 (5.8, the search 0.2), R-MAT scale 17 (ef 12) without one 166 (7.6).
@@ -1033,7 +1035,7 @@ constexpr int kRootNodes = 4, kRootNodesBusy = 64;
 // task; without room for one it is searched here, in the order that the task
 // would have had.
 __device__ __noinline__ void branch_warp_root(const SA &a, Root r, uint32_t *A, int Ws, int W, uint32_t *al,
-                                              uint32_t *keys, int *Pidx, uint32_t *stk, int om,
+                                              uint32_t *keys, int *Pidx, uint32_t *stk, int om, bool few_roots,
                                               unsigned long long *nodes) {
   const int lane = threadIdx.x & 31;
   Bits<1> P, B, C, rest;
@@ -1044,7 +1046,7 @@ __device__ __noinline__ void branch_warp_root(const SA &a, Root r, uint32_t *A, 
   long long limit = LLONG_MAX;
   if (a.tasks) {
     const int t = lane == 0 ? *(volatile int32_t *)a.ntasks : 0;
-    limit = om == 0 || __shfl_sync(FULL, t, 0) >= a.task_warps ? kRootNodesBusy : kRootNodes;
+    limit = om == 0 || __shfl_sync(FULL, t, 0) >= a.task_warps ? kRootNodesBusy : few_roots ? 0 : kRootNodes;
   }
   if (!dfs<1, true>(a, r, A, Ws, W, stk, 1, P, B, C, om, (Pool<1> *)nullptr, n, don, limit, &rest)) {
     __syncwarp();
@@ -1163,7 +1165,8 @@ __global__ void __launch_bounds__(kSW * 32, 6) search_warp_kernel(SA a) {
     color_ise<1, true>(S.A, Ws, W, al, om - 1, B);
     if (!bany(B)) continue;
     branched++;
-    branch_warp_root(a, Root{u, g, S.Pidx, p}, S.A, Ws, W, S.al, (uint32_t *)S.hk, S.Pidx, stk, om, &nodes);
+    branch_warp_root(a, Root{u, g, S.Pidx, p}, S.A, Ws, W, S.al, (uint32_t *)S.hk, S.Pidx, stk, om, nroots <= a.task_warps,
+                     &nodes);
   }
   if (lane == 0) {
     atomicAdd(a.counters + 0, colored);
@@ -2432,7 +2435,7 @@ int launch_search(mc_graph *g, const Pruned &pg, int no_neigh_cores, int no_spli
   const int blocks_b = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_b, small_cap);
   const int blocks_m = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_m, small_cap);
   const int blocks_t = (int)std::min<int64_t>((int64_t)g->sm_count * per_sm_t, std::max<int64_t>(1, (g->n + 15) / 16));
-  a.task_warps = blocks_t * kTW;
+  a.task_warps = g->sm_count * per_sm_t * kTW;
   const int64_t stride_b = (int64_t)(std::min(kbound, 1024) + 2) * (64 + 2);
   const int64_t stride_m = (int64_t)(std::min(kbound, kMidCap) + 2) * (64 + 2);
   // levels above the compact form, then those of the compact form (uint4)

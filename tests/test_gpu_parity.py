@@ -685,7 +685,7 @@ def _grid(a, b):
 @pytest.mark.parametrize("g", [_grid(60, 70), gg.cycle(4001), gg.path(500), gg.complete_bipartite(4, 900)],
                          ids=lambda g: g.name)
 def test_roots_of_few_nodes_stay_with_their_warp(mc, g):
-    """A root is published once its warp has expanded four Branch nodes on it.
+    """A root is published once its warp has expanded a few Branch nodes on it.
     In a triangle-free graph a root's tree has a node per candidate, and these
     graphs have at most four later neighbours per vertex: without a lower
     bound, where every root branches, none becomes a task."""
@@ -877,4 +877,18 @@ def test_batch_of_more_than_two_billion_visiting_positions(mc):
     for opts in (dict(), dict(heuristic=1)):
         om, wit, st = mc.mc_max_clique_batch(h, **opts)
         assert np.array_equal(om, want) and sorted(wit[7].tolist()) == [0, 1, 2, 3, 4]
+    h.close()
+
+
+@pytest.mark.parametrize("n,p", [(125, 0.85), (150, 0.75), (400, 0.25)])
+def test_few_roots_become_tasks_at_once(mc, n, p):
+    """A launch of fewer roots than the chip has warps for (all of at most 128
+    candidates here) publishes every root that branches, with a clique known: the
+    other tasks are branches handed over."""
+    g = gg.erdos_renyi(n, p, seed=2)
+    h = load(mc, g)
+    om, wit, st = mc.mc_max_clique(h)
+    assert om == oracle.max_clique(g)[0] and oracle.is_clique(g, wit)
+    assert st["max_core"] <= 128 and st["roots_branched"] > 20
+    assert st["tasks"] - st["donations"] == st["roots_branched"]
     h.close()
