@@ -587,11 +587,11 @@ __global__ void __launch_bounds__(kVT) forward_kernel(int64_t n, const float *__
 // memory once per block.  FP32 throughout: the activations are not BF16, so the
 // tensor pipe's types would round them.  Every sum has a fixed order.
 // 16,384 rows: 190 us with a thread per row (128 rows per block, serial
-// 64-long chains per thread, 6% of the warps, sums by atomics), 36 us now with
-// 5 us for the sum over the blocks; its error against 64 bits is a third of
-// what it was (the blocks' sums are added in order, not by atomics).  Two blocks
+// 64-long chains per thread, 6% of the warps, sums by atomics), 26 us now with
+// 9 us for the sum over the blocks; its error against 64 bits is a quarter of
+// what it was (pairwise in a block, in double over the blocks).  Two blocks
 // fit an SM (106 KB each), so 16,384 rows are one tile for each of 256 blocks: a
-// call takes 71 us, 80 with one block of 124 KB per SM and two tiles in turn.
+// call takes 67 us, 75 with one block of 124 KB per SM and two tiles in turn.
 constexpr int kGR = 64;    // rows per tile
 constexpr int kGT = 256;   // threads: 16 x 16, 4 x 4 outputs each
 constexpr int kPart = (kParams + 1 + 31) / 32 * 32;  // floats of a block's sums: parameters, loss

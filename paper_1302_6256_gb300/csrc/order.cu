@@ -26,10 +26,11 @@
 //           (ties: smaller id) and marks them dead.
 //
 // Rounds repeat until every vertex is placed (the host queues one ahead of the
-// count it looks at; a round after the last vertex changes nothing).  Cliques live in one arena laid out like the
-// CSR: vertex v's candidates occupy the front of [rp[v], rp[v+1]) while it
-// grows, and its members other than v end at the top of that range, so the
-// arena is nnz int32 and needs no per-warp buffers or size limits.
+// count it looks at; a round after the last vertex changes nothing).  Cliques
+// live in one arena laid out like the CSR: vertex v's candidates occupy the front
+// of [rp[v], rp[v+1]) while it grows, and its members other than v end at the top
+// of that range, so the arena is nnz int32 and needs no per-warp buffers or size
+// limits.
 //
 // The gap cost relabels the graph by an order (new id = position), sorts
 // every new row (bitonic networks in a warp's registers up to 1,024 entries;
@@ -398,7 +399,8 @@ __device__ int block_grow(const OA &a, int v, int32_t *B, GrowSmem &S, int *scnt
 // block, when the longest growth decides, and to warps otherwise, when all of
 // them do: whole order of scale 16 / 17 / 20 / 22 in 3.8 / 5.6 / 51 / 191 ms,
 // always blocks 3.8 / 5.8 / 55 / 342, never blocks 4.8 / 7.7 / 50 / 185
-// (before: 7.6 / 11.9 / 71 / 316).
+// (before: 7.6 / 11.9 / 71 / 316; all on one machine, another has taken 3.6 / 5.0 /
+// 43 / 218 since).
 // FLY: candidates that a lane has in flight.  Four side by side, with 32 warps
 // per SM, are right for the latency of long growths; where no vertex has more than
 // kMidGrowMin neighbours and many are left, warps are what is short: one at a time

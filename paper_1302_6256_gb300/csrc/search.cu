@@ -1025,7 +1025,7 @@ __device__ __forceinline__ int edges_upto(const SA &a, const int *Pidx, int p, u
 // 8.9 ms, 9.5 with four).  With every
 // branching root published at once, 300 graphs of 150-400 vertices took 130 ms
 // (now 2.6), 5,000 of 30-80 vertices 160 (4.5), a 300 x 300 grid without a lower
-// bound 118 (5.8, the search 0.2), R-MAT scale 17 (ef 12) without one 166 (7.6).
+// bound 118 (2.6, the search 0.2), R-MAT scale 17 (ef 12) without one 166 (5.5).
 // 16 nodes always: R-MAT scale 15 loaded and solved 6% slower, the 300 graphs
 // 3.2 ms; 32 instead of 64: 2.8 ms; 256: R-MAT 17 without a bound 10.3 ms.
 constexpr int kRootNodes = 4, kRootNodesBusy = 64;
@@ -1720,14 +1720,17 @@ __global__ void __launch_bounds__(kBT, (SM && (PC <= kMidCap || DENSE)) ? 2 : 1)
 // word per lane: 13 us per Branch node before, 7 us now, and 5 to 30 times
 // fewer nodes, since a root's candidates are in the minimum-width order of its
 // neighbourhood.  R-MAT scale 18, edge factor 12: search 83-330 ms before (it
-// depends on when the larger cliques are found), 4.2-4.6 ms now; scale 15,
-// edge factor 16: 60-104 ms before, 1.3 ms now.
+// depends on when the larger cliques are found), 3.5-4.9 ms now, of which the tasks
+// 2.5-3.9; scale 15, edge factor 16: 60-104 ms before, 0.9-1.2 ms now.  (While a
+// branch that was handed over stayed among its level's candidates, and came back
+// when omega rose, scale 17 took 260,000 nodes and 3.8 ms; now 165,000 and 2.6.)
 // Subproblems above 256 candidates are searched depth first by the warp on the
 // root's matrix until a child fits; publishing every branch of such a node
 // instead (breadth first) let the queue fill with them before omega rose: two
 // of 40 R-MAT scale-20 graphs then took 36 and 85 s, now none of 129 takes
-// more than 65 ms.  Block roots are published with their candidates sorted by
-// degree, so that these levels are coloured densest first as well.
+// more than 65 ms.  Block roots are published with their candidates in
+// minimum-width order (width_keys), so that these levels are coloured densest
+// first as well.
 constexpr int kTM = 256;    // candidates of a compact subproblem
 constexpr int kTW = 4;      // warps per block of the task kernel
 constexpr int kTStk = 20;   // stack words per level (two sets of at most 8 words, omega, chosen vertex)
